@@ -169,7 +169,7 @@ void drop_graph(swale_ctx* ctx) {
 void free_tiles(swale_ctx* ctx) {
   for (void* p : ctx->tile_allocs) cudaFree(p);
   ctx->tile_allocs.clear();
-  ctx->D.rtiles = ctx->D.utiles = ctx->D.mtiles = ctx->D.ftiles = nullptr;
+  ctx->D.rtiles = ctx->D.utiles = ctx->D.mtiles = ctx->D.ftiles = ctx->D.rftiles = nullptr;
 }
 
 void free_alpha_log(swale_ctx* ctx) {
@@ -210,20 +210,21 @@ swale_status dalloc(swale_ctx* ctx, std::vector<void*>& list, T** p, size_t n) {
 swale_status alloc_state(swale_ctx* ctx, int64_t B, int64_t Ntot, DevState& D) {
   const size_t nc = (size_t)Ntot, nn = nc + B, ne = nc + 2 * B;
   double** cells[] = {&D.E0, &D.M0, &D.B0, &D.Ea, &D.Ma, &D.Ba, &D.Eb, &D.Mb, &D.Bb,
-                      &D.YE, &D.YM, &D.YB, &D.J0, &D.J1, &D.J2, &D.bE, &D.bM, &D.bB, &D.bJ};
+                      &D.YE, &D.YM, &D.YB, &D.J0, &D.J1, &D.J2, &D.bE, &D.bM, &D.bB, &D.bJ, &D.iJ1, &D.iJ2};
   for (double** p : cells)
     if (swale_status s = dalloc(ctx, ctx->allocs, p, nc)) return s;
   double** nodes[] = {&D.x, &D.w, &D.P, &D.bx};
   for (double** p : nodes)
     if (swale_status s = dalloc(ctx, ctx->allocs, p, nn)) return s;
-  double** edges[] = {&D.eEL, &D.eER, &D.eBL, &D.eBR, &D.ehL, &D.ehR, &D.euL, &D.euR, &D.ipair, &D.itri};
+  double** edges[] = {&D.eEL, &D.eER, &D.eBL, &D.eBR, &D.ehL, &D.ehR, &D.euL, &D.euR, &D.ipair, &D.itri,
+                      &D.dE, &D.dH, &D.H};
   for (double** p : edges)
     if (swale_status s = dalloc(ctx, ctx->allocs, p, ne)) return s;
   if (ctx->cfg.scheme == SWALE_SCHEME_SPECIAL) {
     if (swale_status s = dalloc(ctx, ctx->allocs, &D.eG1, ne)) return s;
     if (swale_status s = dalloc(ctx, ctx->allocs, &D.eG2, ne)) return s;
   }
-  if (swale_status s = dalloc(ctx, ctx->allocs, &D.geo, (size_t)SWALE_GEO_ARRAYS * ne)) return s;
+  if (swale_status s = dalloc(ctx, ctx->allocs, &D.geo, (size_t)GEO_ARRAYS * ne)) return s;
   D.geo_stride = (int64_t)ne;
   if (swale_status s = dalloc(ctx, ctx->allocs, &D.flags, ne)) return s;
   if (swale_status s = dalloc(ctx, ctx->allocs, &D.IC, (size_t)B)) return s;
@@ -287,42 +288,49 @@ swale_status build_tiles(swale_ctx* ctx, std::vector<InstConst>& ic) {
   const int64_t B = ctx->B;
   const int Tr = ctx->Tr, Tu = ctx->Tu, Tm = kMeshNodes;
   const int Tf = Tu - 1;  // cells of a forward update tile (its Tu interfaces take one pass)
-  std::vector<Tile> rt, ut, mt, ft;
+  const int Trf = Tr - 4; // cells of a forward reconstruction tile (its Tr stencil cells take one pass)
+  std::vector<Tile> rt, ut, mt, ft, rf;
   for (int64_t i = 0; i < B; ++i) {
     const int64_t N = ic[i].N;
     const int64_t nr = (N + 2 + Tr - 1) / Tr, nu = (N + Tu - 1) / Tu, nm = (N + 1 + Tm - 1) / Tm;
-    const int64_t nf = (N + Tf - 1) / Tf;
-    ic[i].ntiles_r = (int32_t)nr;
+    const int64_t nf = (N + Tf - 1) / Tf, nrf = (N + 2 + Trf - 1) / Trf;
+    ic[i].ntiles_r = (int32_t)nrf;
     if (B > 1) {
       for (int64_t t = 0; t < nr; ++t) rt.push_back(Tile{(int32_t)i, (int32_t)(t * Tr - 1)});
       for (int64_t t = 0; t < nu; ++t) ut.push_back(Tile{(int32_t)i, (int32_t)(t * Tu)});
       for (int64_t t = 0; t < nm; ++t) mt.push_back(Tile{(int32_t)i, (int32_t)(t * Tm)});
       for (int64_t t = 0; t < nf; ++t) ft.push_back(Tile{(int32_t)i, (int32_t)(t * Tf)});
+      for (int64_t t = 0; t < nrf; ++t) rf.push_back(Tile{(int32_t)i, (int32_t)(t * Trf - 1)});
     } else {
       ctx->D.nr = (int32_t)nr;
       ctx->D.nu = (int32_t)nu;
       ctx->D.nm = (int32_t)nm;
       ctx->D.nf = (int32_t)nf;
+      ctx->D.nrf = (int32_t)nrf;
     }
   }
   if (B > 1) {
-    Tile *dr, *du, *dm, *df;
+    Tile *dr, *du, *dm, *df, *drf;
     if (swale_status s = dalloc(ctx, ctx->tile_allocs, &dr, rt.size())) return s;
     if (swale_status s = dalloc(ctx, ctx->tile_allocs, &du, ut.size())) return s;
     if (swale_status s = dalloc(ctx, ctx->tile_allocs, &dm, mt.size())) return s;
     if (swale_status s = dalloc(ctx, ctx->tile_allocs, &df, ft.size())) return s;
+    if (swale_status s = dalloc(ctx, ctx->tile_allocs, &drf, rf.size())) return s;
     SW_CUDA(ctx, cudaMemcpyAsync(dr, rt.data(), rt.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
     SW_CUDA(ctx, cudaMemcpyAsync(du, ut.data(), ut.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
     SW_CUDA(ctx, cudaMemcpyAsync(dm, mt.data(), mt.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
     SW_CUDA(ctx, cudaMemcpyAsync(df, ft.data(), ft.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
+    SW_CUDA(ctx, cudaMemcpyAsync(drf, rf.data(), rf.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
     ctx->D.rtiles = dr;
     ctx->D.utiles = du;
     ctx->D.mtiles = dm;
     ctx->D.ftiles = df;
+    ctx->D.rftiles = drf;
     ctx->D.nr = (int32_t)rt.size();
     ctx->D.nu = (int32_t)ut.size();
     ctx->D.nm = (int32_t)mt.size();
     ctx->D.nf = (int32_t)ft.size();
+    ctx->D.nrf = (int32_t)rf.size();
   }
   SW_CUDA(ctx, cudaMemcpyAsync(ctx->D.IC, ic.data(), B * sizeof(InstConst), cudaMemcpyHostToDevice, ctx->stream));
   SW_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -360,59 +368,49 @@ swale_status timed_launch(swale_ctx* ctx, int family, F&& launch) {
   return SWALE_OK;
 }
 
+template <int STAGE, int SCHEME, bool STOREK>
+void launch_recon_as(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
+                     const double* M, const double* B, const double* J) {
+  if (T == 64) k_recon<STAGE, 64, SCHEME, STOREK><<<grid, 64, 0, s>>>(K, D, E, M, B, J);
+  else if (T == 256) k_recon<STAGE, 256, SCHEME, STOREK><<<grid, 256, 0, s>>>(K, D, E, M, B, J);
+  else k_recon<STAGE, 128, SCHEME, STOREK><<<grid, 128, 0, s>>>(K, D, E, M, B, J);
+}
+
 template <int STAGE>
 void launch_recon(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                   const double* M, const double* B, const double* J) {
-  if (K.scheme == SWALE_SCHEME_NONWB) {
-    if (T == 64) k_recon<STAGE, 64, 1><<<grid, 64, 0, s>>>(K, D, E, M, B, J);
-    else if (T == 256) k_recon<STAGE, 256, 1><<<grid, 256, 0, s>>>(K, D, E, M, B, J);
-    else k_recon<STAGE, 128, 1><<<grid, 128, 0, s>>>(K, D, E, M, B, J);
-    return;
+  if (K.scheme == SWALE_SCHEME_NONWB) launch_recon_as<STAGE, 1, false>(K, D, T, grid, s, E, M, B, J);
+  else if (K.scheme == SWALE_SCHEME_SPECIAL) launch_recon_as<STAGE, 2, false>(K, D, T, grid, s, E, M, B, J);
+  else if (D.gK) launch_recon_as<STAGE, 0, true>(K, D, T, grid, s, E, M, B, J);  // the adjoint's recomputes
+  else launch_recon_as<STAGE, 0, false>(K, D, T, grid, s, E, M, B, J);
+}
+
+template <int STAGE, int MODE, int SCHEME, bool BOT, bool STOREK>
+void launch_update_as(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
+                      const double* M, const double* B, const double* J, const RhsOut& ro) {
+  if (T == 64) k_update<STAGE, MODE, 64, SCHEME, BOT, STOREK><<<grid, 64, 0, s>>>(K, D, E, M, B, J, ro);
+  else if (T == 256) k_update<STAGE, MODE, 256, SCHEME, BOT, STOREK><<<grid, 256, 0, s>>>(K, D, E, M, B, J, ro);
+  else k_update<STAGE, MODE, 128, SCHEME, BOT, STOREK><<<grid, 128, 0, s>>>(K, D, E, M, B, J, ro);
+}
+
+template <int STAGE, int MODE, int SCHEME>
+void launch_update_scheme(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
+                          const double* M, const double* B, const double* J, const RhsOut& ro) {
+  if (MODE == 0 && K.bot_pieces > 0) {
+    launch_update_as<STAGE, MODE, SCHEME, MODE == 0, false>(K, D, T, grid, s, E, M, B, J, ro);
+  } else if (MODE == 0 && SCHEME == 0 && D.gK) {  // the adjoint's recomputes
+    launch_update_as<STAGE, MODE, SCHEME, false, MODE == 0 && SCHEME == 0>(K, D, T, grid, s, E, M, B, J, ro);
+  } else {
+    launch_update_as<STAGE, MODE, SCHEME, false, false>(K, D, T, grid, s, E, M, B, J, ro);
   }
-  if (K.scheme == SWALE_SCHEME_SPECIAL) {
-    if (T == 64) k_recon<STAGE, 64, 2><<<grid, 64, 0, s>>>(K, D, E, M, B, J);
-    else if (T == 256) k_recon<STAGE, 256, 2><<<grid, 256, 0, s>>>(K, D, E, M, B, J);
-    else k_recon<STAGE, 128, 2><<<grid, 128, 0, s>>>(K, D, E, M, B, J);
-    return;
-  }
-  if (D.gK) {  // the adjoint's recomputes: also store the smooth-class linear form
-    if (T == 64) k_recon<STAGE, 64, 0, false, true><<<grid, 64, 0, s>>>(K, D, E, M, B, J);
-    else if (T == 256) k_recon<STAGE, 256, 0, false, true><<<grid, 256, 0, s>>>(K, D, E, M, B, J);
-    else k_recon<STAGE, 128, 0, false, true><<<grid, 128, 0, s>>>(K, D, E, M, B, J);
-    return;
-  }
-  if constexpr (STAGE == 1) {
-    if (D.geo) {  // stage 1 reads the cached geometry: more resident warps
-      if (T == 64) k_recon<STAGE, 64, 0, true><<<grid, 64, 0, s>>>(K, D, E, M, B, J);
-      else if (T == 256) k_recon<STAGE, 256, 0, true><<<grid, 256, 0, s>>>(K, D, E, M, B, J);
-      else k_recon<STAGE, 128, 0, true><<<grid, 128, 0, s>>>(K, D, E, M, B, J);
-      return;
-    }
-  }
-  if (T == 64) k_recon<STAGE, 64><<<grid, 64, 0, s>>>(K, D, E, M, B, J);
-  else if (T == 256) k_recon<STAGE, 256><<<grid, 256, 0, s>>>(K, D, E, M, B, J);
-  else k_recon<STAGE, 128><<<grid, 128, 0, s>>>(K, D, E, M, B, J);
 }
 
 template <int STAGE, int MODE>
 void launch_update(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                    const double* M, const double* B, const double* J, RhsOut ro) {
-  if (MODE == 0 && K.scheme == SWALE_SCHEME_HYDROSTATIC && K.bot_pieces == 0 && D.gK) {
-    // the adjoint's recomputes: also store the source form's entries
-    if (T == 64) k_update<STAGE, MODE, 64, true, true><<<grid, 64, 0, s>>>(K, D, E, M, B, J, ro);
-    else if (T == 256) k_update<STAGE, MODE, 256, true, true><<<grid, 256, 0, s>>>(K, D, E, M, B, J, ro);
-    else k_update<STAGE, MODE, 128, true, true><<<grid, 128, 0, s>>>(K, D, E, M, B, J, ro);
-    return;
-  }
-  if (MODE == 0 && K.scheme == SWALE_SCHEME_HYDROSTATIC && K.bot_pieces == 0) {
-    if (T == 64) k_update<STAGE, MODE, 64, true><<<grid, 64, 0, s>>>(K, D, E, M, B, J, ro);
-    else if (T == 256) k_update<STAGE, MODE, 256, true><<<grid, 256, 0, s>>>(K, D, E, M, B, J, ro);
-    else k_update<STAGE, MODE, 128, true><<<grid, 128, 0, s>>>(K, D, E, M, B, J, ro);
-    return;
-  }
-  if (T == 64) k_update<STAGE, MODE, 64><<<grid, 64, 0, s>>>(K, D, E, M, B, J, ro);
-  else if (T == 256) k_update<STAGE, MODE, 256><<<grid, 256, 0, s>>>(K, D, E, M, B, J, ro);
-  else k_update<STAGE, MODE, 128><<<grid, 128, 0, s>>>(K, D, E, M, B, J, ro);
+  if (K.scheme == SWALE_SCHEME_NONWB) launch_update_scheme<STAGE, MODE, 1>(K, D, T, grid, s, E, M, B, J, ro);
+  else if (K.scheme == SWALE_SCHEME_SPECIAL) launch_update_scheme<STAGE, MODE, 2>(K, D, T, grid, s, E, M, B, J, ro);
+  else launch_update_scheme<STAGE, MODE, 0>(K, D, T, grid, s, E, M, B, J, ro);
 }
 
 unsigned grid_of(int32_t ntiles, int persistent) {
@@ -430,7 +428,7 @@ swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, 
   const DevState& D1 = stageD ? stageD[0] : D;
   const DevState& D2 = stageD ? stageD[1] : D;
   const DevState& D3 = stageD ? stageD[2] : D;
-  const unsigned gr = grid_of(D.nr, ctx->grid_r), gu = grid_of(D.nf, ctx->grid_u);
+  const unsigned gr = grid_of(D.nrf, ctx->grid_r), gu = grid_of(D.nf, ctx->grid_u);
   const int Tr = ctx->Tr, Tu = ctx->Tu;
   const RhsOut none{nullptr, nullptr, nullptr, 0.0};
   swale_status st = SWALE_OK;
@@ -1179,7 +1177,7 @@ swale_status swale_rhs(swale_ctx* ctx, int64_t N, const double* E, const double*
   K.t_end = 0.0;
   K.mesh = SWALE_MESH_STATIC;
   k_widths_max<<<64, 256, 0, st>>>(D.J0, N, D.S);
-  launch_recon<1>(K, D, tmp.Tr, grid_of(D.nr, 0), st, D.E0, D.M0, D.B0, D.J0);
+  launch_recon<1>(K, D, tmp.Tr, grid_of(D.nrf, 0), st, D.E0, D.M0, D.B0, D.J0);
   unsigned long long Abits = 0;
   e = cudaGetLastError();
   e = e ? e : cudaMemcpyAsync(&Abits, &D.S->A[0], 8, cudaMemcpyDeviceToHost, st);
@@ -1482,9 +1480,13 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
       if (!s) s = carve(p, (size_t)Nt);
     if (!s) s = carve(&X.x, (size_t)NN);
     if (!s) s = carve(&X.w, (size_t)NN);
-    double** edges[] = {&X.eEL, &X.eER, &X.eBL, &X.eBR, &X.ehL, &X.ehR, &X.euL, &X.euR, &X.ipair, &X.itri};
+    double** edges[] = {&X.eEL, &X.eER, &X.eBL, &X.eBR, &X.ehL, &X.ehR, &X.euL, &X.euR, &X.ipair, &X.itri,
+                        &X.dE, &X.dH, &X.H};
+    // (with the tape every step's edge arrays are its slot's; the set keeps only what the slots share)
     for (double** p : edges)
-      if (!s) s = carve(p, (size_t)NE);
+      if (!s && !(tape && p != &X.dE && p != &X.dH && p != &X.H)) s = carve(p, (size_t)NE);
+    if (!s) s = carve(&X.iJ1, (size_t)Nt);
+    if (!s) s = carve(&X.iJ2, (size_t)Nt);
     if (!s) s = carve(&X.flags, (size_t)NE);
     if (!s) s = carve(&X.S, (size_t)B);
   };
@@ -1515,7 +1517,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   // Snapshot buffers of two segments (one when a single segment covers every step).
   const int64_t nbuf = nseg == 1 ? 1 : 2;
   std::vector<StateCopy> ckpt(nseg), seg(C), seg2(nbuf == 2 ? C : 0);
-  StateCopy fin, snapR[2];
+  StateCopy fin;
   for (auto& c : ckpt) alloc_copy(c);
   for (auto& c : seg) alloc_copy(c);
   for (auto& c : seg2) alloc_copy(c);
@@ -1544,10 +1546,6 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
     }
   }
   alloc_copy(fin);
-  if (!tape) {
-    alloc_copy(snapR[0]);
-    alloc_copy(snapR[1]);
-  }
   double *gx = nullptr, *obs = nullptr, *Jacc = nullptr, *alog = nullptr;
   if (!s) s = carve(&gx, (size_t)B * G);
   if (!s) s = carve(&obs, (size_t)nsteps * B * G);
@@ -1556,14 +1554,6 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   int64_t* gcell = nullptr;  // last cell of each gauge (searched from, the mesh moves little per step)
   if (!s) s = carve(&gcell, (size_t)B * G);
   if (s) return release(s);
-  // q^n and J^n of the step being reversed, per state set.
-  AdjState AR[2] = {A, A};
-  for (int k = 0; k < 2; ++k) {
-    AR[k].sE = snapR[k].E;
-    AR[k].sM = snapR[k].M;
-    AR[k].sB = snapR[k].B;
-    AR[k].sJ = snapR[k].J;
-  }
   cudaError_t e = cudaSuccess;
   e = e ? e : cudaMemcpyAsync(gx, gauges_x, (size_t)B * G * sizeof(double), cudaMemcpyDefault, st);
   e = e ? e : cudaMemcpyAsync(obs, h_obs, (size_t)nsteps * B * G * sizeof(double), cudaMemcpyDefault, st);
@@ -1775,27 +1765,29 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
       if (used[k]) e = cudaStreamWaitEvent(st3, ev[7 + k], 0);
       used[k] = true;
       e = e ? e : load_into(c, X, st3);
-      e = e ? e : cudaMemcpyAsync(snapR[k].E, c.E, Nt * sizeof(double), cudaMemcpyDeviceToDevice, st3);
-      e = e ? e : cudaMemcpyAsync(snapR[k].M, c.M, Nt * sizeof(double), cudaMemcpyDeviceToDevice, st3);
-      e = e ? e : cudaMemcpyAsync(snapR[k].B, c.B, Nt * sizeof(double), cudaMemcpyDeviceToDevice, st3);
-      e = e ? e : cudaMemcpyAsync(snapR[k].J, c.J, Nt * sizeof(double), cudaMemcpyDeviceToDevice, st3);
       if (e) break;
       if ((s = enqueue_step_on(ctx, X, st3, Ds[k], 0))) break;
       if ((e = cudaEventRecord(ev[5 + k], st3))) break;
       // Reverse sweep of step m on the context's stream.
       if ((e = cudaStreamWaitEvent(st, ev[5 + k], 0))) break;
+      AdjState AR = A;  // with q^n, J^n of the step: the segment's snapshot
+      AR.sE = c.E;
+      AR.sM = c.M;
+      AR.sB = c.B;
+      AR.sJ = c.J;
       k_misfit<1><<<gg, 128, 0, st>>>(X, A, (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
-      launch_adj_rk<3>(ctx, X, AR[k]);
-      launch_adj_stage<3>(ctx, Ds[k][2], K, AR[k], X.Eb, X.Mb, X.Bb, X.J2);
-      launch_adj_rk<2>(ctx, X, AR[k]);
-      launch_adj_stage<2>(ctx, Ds[k][1], K, AR[k], X.Ea, X.Ma, X.Ba, X.J1);
-      launch_adj_rk<1>(ctx, X, AR[k]);
-      launch_adj_stage<1>(ctx, Ds[k][0], K, AR[k], snapR[k].E, snapR[k].M, snapR[k].B, snapR[k].J);
-      launch_adj_rk<0>(ctx, X, AR[k]);
+      launch_adj_rk<3>(ctx, X, AR);
+      launch_adj_stage<3>(ctx, Ds[k][2], K, AR, X.Eb, X.Mb, X.Bb, X.J2);
+      launch_adj_rk<2>(ctx, X, AR);
+      launch_adj_stage<2>(ctx, Ds[k][1], K, AR, X.Ea, X.Ma, X.Ba, X.J1);
+      launch_adj_rk<1>(ctx, X, AR);
+      launch_adj_stage<1>(ctx, Ds[k][0], K, AR, c.E, c.M, c.B, c.J);
+      launch_adj_rk<0>(ctx, X, AR);
       e = cudaGetLastError();
       if (!e) e = cudaEventRecord(ev[7 + k], st);
     }
-    if (!s && !e) e = cudaEventRecord(ev[3 + (sg & 1)], st3);
+    // The segment's snapshots are free once its reverse sweep, which reads them, is done.
+    if (!s && !e) e = cudaEventRecord(ev[3 + (sg & 1)], st);
   }
   if (!s && !e) e = load(fin);
   restore_ctx();
@@ -1833,7 +1825,8 @@ constexpr int kNoAllocMaxDevices = 64;
 constexpr int kNoAllocTile = 128;
 
 struct NoAllocScratch {
-  double edges[12][kNoAllocMaxCells + 2];  // 8 edge arrays, 2 reciprocals, 2 point-value arrays
+  // 8 edge arrays, 2 reciprocals, 2 point-value arrays, differences of eta and h, the depth
+  double edges[15][kNoAllocMaxCells + 2];
   uint8_t flags[kNoAllocMaxCells + 2];
   InstConst ic;
   DevScalars S;
@@ -1853,7 +1846,7 @@ __global__ void k_noalloc_init(InstConst* ic, DevScalars* S, int64_t N, int32_t 
   *S = z;
 }
 
-// Fixed scratch of the allocation-free entry point (about 6.3 MB per device).
+// Fixed scratch of the allocation-free entry point (about 7.9 MB per device).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocScratch)];
 
 // Device address of g_noalloc_scratch per device, obtained once with that device current.
@@ -1921,6 +1914,9 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
     D.eG1 = scr->edges[10];
     D.eG2 = scr->edges[11];
   }
+  D.dE = scr->edges[12];
+  D.dH = scr->edges[13];
+  D.H = scr->edges[14];
   D.flags = scr->flags;
   D.IC = &scr->ic;
   D.S = &scr->S;
@@ -1928,6 +1924,7 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   D.nr = (int32_t)((N + 2 + kNoAllocTile - 1) / kNoAllocTile);
   D.nu = (int32_t)((N + kNoAllocTile - 1) / kNoAllocTile);
   D.nf = (int32_t)((N + kNoAllocTile - 2) / (kNoAllocTile - 1));
+  D.nrf = (int32_t)((N + 2 + kNoAllocTile - 5) / (kNoAllocTile - 4));
   StepConst K;
   K.sc.g = cfg->g;
   K.sc.eps_weno = cfg->eps_weno;
@@ -1956,16 +1953,11 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   K.geo_epoch = 0;  // no geometry cache here (D.geo is null)
   K.wave_rel = cfg->alpha_bound ? 0 : 1;  // the largest |u - w| + sqrt(g h) (Eq. alpha2D) in A_out
   // The scalars keep the previous call's contents: start them from zero.
-  k_noalloc_init<<<1, 32, 0, st>>>(&scr->ic, &scr->S, N, D.nr);
+  k_noalloc_init<<<1, 32, 0, st>>>(&scr->ic, &scr->S, N, D.nrf);
   k_widths_max<<<64, 256, 0, st>>>(J, N, &scr->S);
-  if (cfg->scheme == SWALE_SCHEME_NONWB)
-    k_recon<1, kNoAllocTile, 1><<<(unsigned)D.nr, kNoAllocTile, 0, st>>>(K, D, E, M, B, J);
-  else if (cfg->scheme == SWALE_SCHEME_SPECIAL)
-    k_recon<1, kNoAllocTile, 2><<<(unsigned)D.nr, kNoAllocTile, 0, st>>>(K, D, E, M, B, J);
-  else
-    k_recon<1, kNoAllocTile><<<(unsigned)D.nr, kNoAllocTile, 0, st>>>(K, D, E, M, B, J);
-  RhsOut ro{RE, RM, RB, alpha};
-  k_update<2, 1, kNoAllocTile><<<(unsigned)D.nf, kNoAllocTile, 0, st>>>(K, D, E, M, B, J, ro);
+  launch_recon<1>(K, D, kNoAllocTile, (unsigned)D.nrf, st, E, M, B, J);
+  const RhsOut ro{RE, RM, RB, alpha};
+  launch_update<2, 1>(K, D, kNoAllocTile, (unsigned)D.nf, st, E, M, B, J, ro);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && flags) e = cudaMemcpyAsync(flags, scr->flags + 1, (size_t)N, cudaMemcpyDefault, st);
   if (e == cudaSuccess && A_out) {

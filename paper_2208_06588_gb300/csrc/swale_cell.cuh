@@ -156,14 +156,16 @@ SWALE_HD float f32_trunc(double x) {
 // The indicator factors of indicator_factors in FP32 from the widths h[5] and the length dx
 // (truncated to FP32): every term of F[0], F[1], -F[2], c4 and c3 is positive, so they come out
 // within 6 u (F), 8 u (c4) and 12 u (c3) of their values.
+SWALE_HD void indicator_factors_f32(const float h[5], float d, float F[3], float& c4, float& c3) {
+  F[0] = fmaf(1.5f, h[2], (h[0] + h[1]) + h[1]);
+  F[1] = fmaf(0.5f, h[2], h[1]);
+  F[2] = -fmaf(0.5f, h[2], h[3]);
+  c4 = (4.0f * d) * h[2];
+  c3 = (fmaf(3.0f * h[2], h[2], 36.0f * d * d) * d) * h[2];
+}
 SWALE_HD void indicator_factors_f32(const double h[5], double dx, float F[3], float& c4, float& c3) {
-  const float h0 = f32_trunc(h[0]), h1 = f32_trunc(h[1]), h2 = f32_trunc(h[2]), h3 = f32_trunc(h[3]);
-  const float d = f32_trunc(dx);
-  F[0] = fmaf(1.5f, h2, (h0 + h1) + h1);
-  F[1] = fmaf(0.5f, h2, h1);
-  F[2] = -fmaf(0.5f, h2, h3);
-  c4 = (4.0f * d) * h2;
-  c3 = (fmaf(3.0f * h2, h2, 36.0f * d * d) * d) * h2;
+  const float hf[5] = {f32_trunc(h[0]), f32_trunc(h[1]), f32_trunc(h[2]), f32_trunc(h[3]), f32_trunc(h[4])};
+  indicator_factors_f32(hf, f32_trunc(dx), F, c4, c3);
 }
 
 // ------------------------------------------------------------------------------------
@@ -231,6 +233,45 @@ SWALE_HD bool sure_smooth1_f32(const float F[3], float c4, float c3, const float
   const float den = (b[0] + b[1] + b[2]) * (1.0f / 3.0f) + eps;
   const float E = (96.0f * u) * msum + 1e-30f;
   return tau * (1.0f + 8.0f * u) + E <= 0.5f * (den * (1.0f - 8.0f * u) - E);
+}
+
+// The test for a cell of the non-well-balanced scheme: both characteristic fields and the bottom
+// surely smooth, from the FP32 pair differences of eta, hu and h and the cell's averages hb, mb. The
+// rows of R^-1 (nonwb_proj) are formed in FP32 too: u = mb / hb within 5 u, c within 4 u, 1 / (2c)
+// within 5 u, so the rows' entries within 12 u of (|u| + c) / (2c) and 5 u of 1 / (2c), and a
+// field's differences within 16 u of their magnitudes; the test gets three times these
+// magnitudes, which keeps the error within the 6 u that sure_smooth1_f32 allows. A smooth
+// cell then needs no projection: with linear weights in every field, mapping to the fields and
+// back is the identity.
+SWALE_HD bool sure_smooth_nonwb_f32(double g, double h_dry, double hb, double mb, const float F[3], float c4, float c3,
+                                    const float d2e[4], const float d2m[4], const float d2h[4], const float it[3],
+                                    float eps) {
+  float a11 = 1.0f, a12 = 0.0f, a21 = 0.0f, a22 = 1.0f, m1 = 1.0f, m12 = 0.0f, m21 = 0.0f, m2 = 1.0f;
+  if (hb > h_dry) {
+    const float hf = f32_trunc(hb), uf = f32_trunc(mb) / hf, cf = sqrtf(f32_trunc(g) * hf), i2c = 0.5f / cf;
+    a11 = (uf + cf) * i2c;
+    a12 = -i2c;
+    a21 = (cf - uf) * i2c;
+    a22 = i2c;
+    m1 = m21 = (fabsf(uf) + cf) * i2c;
+    m12 = m2 = i2c;
+  }
+  float fd[4], fm[4];
+  for (int a = 0; a < 4; ++a) {
+    fd[a] = fmaf(a11, d2e[a], a12 * d2m[a]);
+    fm[a] = 3.0f * fmaf(m1, fabsf(d2e[a]), m12 * fabsf(d2m[a]));
+  }
+  if (!sure_smooth1_f32(F, c4, c3, fd, fm, it, eps)) return false;
+  for (int a = 0; a < 4; ++a) {
+    fd[a] = fmaf(a21, d2e[a], a22 * d2m[a]);
+    fm[a] = 3.0f * fmaf(m21, fabsf(d2e[a]), m2 * fabsf(d2m[a]));
+  }
+  if (!sure_smooth1_f32(F, c4, c3, fd, fm, it, eps)) return false;
+  for (int a = 0; a < 4; ++a) {
+    fd[a] = d2e[a] - d2h[a];
+    fm[a] = fabsf(d2e[a]) + fabsf(d2h[a]);
+  }
+  return sure_smooth1_f32(F, c4, c3, fd, fm, it, eps);
 }
 
 // Wave speed |u| + sqrt(g max(h, 0)) of one limited edge state (Eq. alpha2D).
@@ -409,6 +450,21 @@ SWALE_HD real edge_value(const CellGeom& G, const real phi[2][3], const real v0[
   return s;
 }
 
+// Whether the limiter below surely leaves the cell alone, told on the integer and FP32 pipes: both
+// edge depths and the Gauss-Lobatto mean delta = (12 hbar - hL - hR) / 10 at or above eps_pp (>= the
+// limiter's floor). delta is formed in FP32 from copies truncated to 23 bits: its error stays
+// below 2^-21 (12 hbar + |hL| + |hR|), and the test asks for four times that and twice the floor.
+SWALE_HD bool surely_unlimited(const SchemeConst& P, real hbar, real hL, real hR) {
+#if defined(SWALE_REAL)
+  return false;
+#else
+  if (dlt(hL, P.eps_pp) || dlt(hR, P.eps_pp)) return false;
+  const float b = f32_trunc(hbar), l = f32_trunc(hL), r = f32_trunc(hR), e = f32_trunc(P.eps_pp);
+  const float m = 12.0f * b + (l + r);
+  return 12.0f * b - (l + r) > fmaf(20.0f, e, 2e-6f * m) + 1e-36f && m < 1e30f;
+#endif
+}
+
 // Limiter on h = eta - b with the Gauss-Lobatto mean delta (Eq. modifiedhjn, xd in 1D; hu scaled
 // by the same theta only if P.limit_hu), b re-derived as eta - h (Remark in Sec. 4.3), velocities.
 //   ev[v][e]  edge values of (eta, hu, h);  hbar0, mbar  the cell's depth and discharge means
@@ -418,17 +474,19 @@ SWALE_HD void limit_cell(const SchemeConst& P, const real ev[3][2], real hbar0, 
   if (dlt(hbar, -P.eps_pp)) st |= ST_NEGDEPTH;
   hbar = pos0(hbar);
   real hL = ev[2][0], hR = ev[2][1];
-  const real delta = (12.0 * hbar - hL - hR) * 0.1;
-  const real mn = dmin(dmin(hL, hR), delta);
-  const real epsv = dmin(P.eps_pp, hbar);
   real mL = ev[1][0], mR = ev[1][1];
-  if (dlt(mn, epsv)) {
-    const real theta = (hbar - epsv) * recip(hbar - mn);
-    hL = theta * (hL - hbar) + hbar;
-    hR = theta * (hR - hbar) + hbar;
-    if (P.limit_hu) {
-      mL = theta * (mL - mbar) + mbar;
-      mR = theta * (mR - mbar) + mbar;
+  if (!surely_unlimited(P, hbar, hL, hR)) {
+    const real delta = (12.0 * hbar - hL - hR) * 0.1;
+    const real mn = dmin(dmin(hL, hR), delta);
+    const real epsv = dmin(P.eps_pp, hbar);
+    if (dlt(mn, epsv)) {
+      const real theta = (hbar - epsv) * recip(hbar - mn);
+      hL = theta * (hL - hbar) + hbar;
+      hR = theta * (hR - hbar) + hbar;
+      if (P.limit_hu) {
+        mL = theta * (mL - mbar) + mbar;
+        mR = theta * (mR - mbar) + mbar;
+      }
     }
   }
   o.EL = ev[0][0];
@@ -499,6 +557,46 @@ SWALE_HD void recon_cell(const SchemeConst& P, const real h[5], const real it[3]
   cell_geom(h, P.beta_dx_global ? dxmax : h[2], G, st);
   smooth_edge_coeffs(h, it, G);
   recon_cell_g(P, G, v0, DD, o, flag, st);
+}
+
+// Edge values of the smooth class (linear weights) straight from the divided differences. With the
+// linear weights the combination of the three sub-stencils is the derivative of the big stencil's
+// quintic primitive P at the edge, and in Newton form with the nodes taken from the edge outwards
+// every basis polynomial but the last factors of each order vanishes there:
+//   P'(y3) = v_j + h2 (D2[j,j+1] - h3 (D3[j] + p12 (D4[j-1..j+2] - p34 D5)))
+//   P'(y2) = v_j - h2 (D2[j-1,j] + h1 (D3[j] - p23 (D4[j-2..j+1] + p01 D5)))
+// (p_ab = h_a + h_b). The factors are widths and pair sums that the divided differences need
+// anyway, so the class costs no mesh geometry: four FMAs per value, and two operations per value
+// for each order of differences (shared by the pairs, triples, quadruples that use them), with
+// four reciprocals per cell, against about 75 FP64 operations per cell and stage for the weights
+// and the linear form of smooth_edge_coeffs. Equal to it in exact arithmetic, exact for constants.
+struct SmoothWidths {
+  real h1, h2, h3, p01, p12, p23, p34;
+};
+SWALE_HD real smooth_right(const SmoothWidths& w, real v, real d2r, real d3, real d4r, real d5) {
+  return v + w.h2 * (d2r - w.h3 * (d3 + w.p12 * (d4r - w.p34 * d5)));
+}
+SWALE_HD real smooth_left(const SmoothWidths& w, real v, real d2l, real d3, real d4l, real d5) {
+  return v - w.h2 * (d2l + w.h1 * (d3 - w.p23 * (d4l + w.p01 * d5)));
+}
+// The same interpolant at the offset t h2 (0 < t < 1) from the cell's left edge: the nodes in the
+// order y2, y3, y4, y1, y5, y0 with the basis polynomials N_k and their derivatives.
+SWALE_HD real smooth_point(const SmoothWidths& w, real h4, real t, real v, real d2r, real d3, real d4r, real d5) {
+  const real n2 = (t * (t - 1.0)) * (w.h2 * w.h2), e2 = (2.0 * t - 1.0) * w.h2;
+  const real a4 = (t - 1.0) * w.h2 - w.h3, a1 = t * w.h2 + w.h1, a5 = a4 - h4;
+  const real n3 = n2 * a4, e3 = e2 * a4 + n2;
+  const real n4 = n3 * a1, e4 = e3 * a1 + n3;
+  const real e5 = e4 * a5 + n4;
+  return v + (d2r * e2 + (d3 * e3 + (d4r * e4 + d5 * e5)));
+}
+// Whether the five widths are positive, normal floats within a factor of 2^20 of each other (h32:
+// truncated to FP32). Then both middle linear weights d_1 are positive beyond any rounding: with
+// A = y3 - y0 >= B = y3 - y1, E = y5 - y3 >= D = y4 - y3, d_1 = 1 - DE / ((A+D)(A+E)) - AB / ((B+E)(A+E))
+// is at least about 2^-22 there, so the ST_EWEIGHT check of cell_geom needs no weights. Other cells
+// take the path that forms them.
+SWALE_HD bool moderate_widths(float a, float b, float c, float d, float e) {
+  const float mn = fminf(fminf(fminf(a, b), fminf(c, d)), e), mx = fmaxf(fmaxf(fmaxf(a, b), fmaxf(c, d)), e);
+  return mn > 1e-30f && mx < 1e30f && mx < 1048576.0f * mn;
 }
 
 // Reconstruction of cell j for the non-well-balanced scheme (Eq. se2D / s2D; Sec. 2.2, last
@@ -867,6 +965,95 @@ SWALE_HD real source_cell_special(real g, real etabar, const real eta4[4], const
   const real b2L = 0.5 * (bLm * bLm + u[3] * u[3]), b2R = 0.5 * (u[4] * u[4] + bRp * bRp);
   return (0.5 * g) * (b2R - b2L) - g * etabar * (bR - bL) - g * S2;
 }
+
+// The interface fluxes at twice their value, with each side's own edge pressure left out of the
+// momentum: with M = mL (uL - w) + mR (uR - w) - alpha (mR - mL) and Q = (g/2) (sR^2 - sL^2),
+//   2 FMm = M + Q + g hL^2,  2 FMp = M - Q + g hR^2  (interface_flux; s = h in the plain flux),
+// and a cell's own g (hR^2 - hL^2) joins its source term (source_pressure_form). FMl = M + Q is what the
+// left cell sees, FMr = M - Q the right one. The special scheme keeps the whole plain flux in both.
+struct Flux2 {
+  real FE, FMl, FMr, FB;
+};
+template <int SCHEME>
+SWALE_HD Flux2 interface_flux2(real g, real alpha, real w, real EL, real ER, real BL, real BR, real hL, real hR,
+                               real uL, real uR) {
+  real sL = hL, sR = hR;
+  if (SCHEME == 0) {
+    const real bstar = dmax(BL, BR);
+    sL = pos0(EL - bstar);
+    sR = pos0(ER - bstar);
+  }
+  const real mL = sL * uL, mR = sR * uR;
+  Flux2 f;
+  f.FE = ((mL + mR) - w * (EL + ER)) - alpha * (ER - EL);
+  const real M = (mL * (uL - w) + mR * (uR - w)) - alpha * (mR - mL);
+  const real hg = 0.5 * g;
+  if (SCHEME == 2) {
+    f.FMl = M + hg * (sL * sL + sR * sR);
+    f.FMr = f.FMl;
+  } else {
+    const real q = (sR - sL) * (sR + sL);
+    f.FMl = M + hg * q;
+    f.FMr = M - hg * q;
+  }
+  f.FB = w * (BL + BR) + alpha * (BR - BL);
+  return f;
+}
+
+// Width ratios at the interface of two cells (l, r) with ip = 1 / (J_l + J_r): rho = J_l ip, sig = J_r ip
+// and their squares, which the source terms of both cells use.
+struct PairRatio {
+  real rho, sig, rho2, sig2;
+};
+SWALE_HD PairRatio pair_ratio(real Jl, real Jr, real ip) {
+  const real rho = Jl * ip, sig = Jr * ip;
+  return {rho, sig, rho * rho, sig * sig};
+}
+
+// The source term of source_form in factored form, joined with the cell's own edge pressures.
+// With dv_k = v_k - v_j the differences of the five data of v from the cell average, de = dh + db,
+// A the antisymmetric matrix of source_form and K = A + (e_R e_R^T - e_L e_L^T) / 2,
+//   h^T K b + (h_R^2 - h_L^2) / 2 = h_j (de_R - de_L) + (dh_R de_R - dh_L de_L) / 2 + dh^T A de
+// (the terms in dh alone cancel: A is antisymmetric), a sum of differences of eta that is
+// exactly zero at rest, whatever the bottom. And A has rank-two structure: the functionals
+//   X = d_L + rho_l d_R + sig_l^2 (v_j - v_{j-1}),  Y = d_R + sig_r d_L - rho_r^2 (v_{j+1} - v_j)
+// (fourth differences of the confluent primitive, scaled), c = d_L + d_R, give
+//   2 dh^T A de = (G_h c_e - c_h G_e) + K3 (X_h Y_e - Y_h X_e),  G = d_R + GX X + GY Y,
+//   GX = -(2/5) (J_p + J_j/2) z / J_m,  GY = (2/5) (J_m + J_j/2) z / J_p,
+//   K3 = -(2/35) J_j^2 z / (J_m J_p),   z = J_j / (J_m + J_j + J_p)
+// (the six entries multiplied out; exact). Per cell 27 FP64 operations and 12 for the mesh-only
+// values (four more per interface), against 28 and 43 for source_form with its entries.
+struct SourceRatio {
+  real GX, GY, K3;
+};
+SWALE_HD SourceRatio source_ratio(real Jm, real Jc, real Jp, real iJm, real iJp, real itc) {
+  const real z = Jc * itc, a = z * iJm, b = z * iJp, e = -0.2 * Jc;
+  SourceRatio s;
+  s.GX = (e - 0.4 * Jp) * a;
+  s.GY = (0.4 * Jm - e) * b;
+  s.K3 = ((2.0 / 7.0) * e * Jc) * (a * iJp);
+  return s;
+}
+//   hc, hL, hR  depth average and limited edge depths;  deL, deR  edge values of eta less its average;
+//   dE*, dH*  eta_j - eta_{j-1}, h_j - h_{j-1} at the left (l) and right (r) interface.
+// Returns twice the value above (the momentum source and pressure difference is -g/2 times it).
+SWALE_HD real source_pressure_form(real hc, real hL, real hR, real deL, real deR, real dEl, real dHl, real dEr, real dHr,
+                                   real rho_l, real sig2_l, real sig_r, real rho2_r, const SourceRatio& s) {
+  const real dhL = hL - hc, dhR = hR - hc;
+  const real Xe = (deL + rho_l * deR) + sig2_l * dEl, Ye = (deR + sig_r * deL) - rho2_r * dEr;
+  const real Xh = (dhL + rho_l * dhR) + sig2_l * dHl, Yh = (dhR + sig_r * dhL) - rho2_r * dHr;
+  const real Ge = (deR + s.GX * Xe) + s.GY * Ye, Gh = (dhR + s.GX * Xh) + s.GY * Yh;
+  const real ce = deL + deR, ch = dhL + dhR;
+  real acc = deR * (hc + hR);
+  acc = acc - deL * (hc + hL);
+  acc = acc + Gh * ce;
+  acc = acc - ch * Ge;
+  return acc + s.K3 * (Xh * Ye - Yh * Xe);
+}
+
+// q + (a R - q dJ) / J' with inv = 1 / J': a cell average advanced by an increment a R of J q while
+// its width grows by dJ.
+SWALE_HD real rk_advance(real q, real a, real R, real dJ, real inv) { return q + (a * R - q * dJ) * inv; }
 
 // Flux differences and source of cell j: R = (R_E, R_M, R_B) of Eq. hydro2D / bottomrk.
 struct CellRhs {

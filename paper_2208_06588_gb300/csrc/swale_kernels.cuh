@@ -31,14 +31,14 @@
 
 namespace swale_dev {
 
-static_assert(sizeof(swale::CellGeom) == SWALE_GEOM_VALUES * sizeof(double), "CellGeom holds SWALE_GEOM_VALUES doubles");
-static_assert(sizeof(swale::SourceGeom) == 6 * sizeof(double), "SourceGeom holds 6 doubles");
 static_assert(sizeof(swale::SourceForm) == 6 * sizeof(double), "SourceForm holds 6 doubles");
 
 using swale::EdgeState;
 using swale::SchemeConst;
 
 constexpr int kMaxGaussHalf = 64;
+// Resident threads per SM that the launch bounds of the stage kernels ask for.
+constexpr int kReconThreads = 768, kUpdateThreads = 1024;
 constexpr int kMeshThreads = 256;
 constexpr int kMeshNodes = kMeshThreads - 1;  // nodes a mesh-velocity tile advances by
 constexpr double kTwoPi = 6.283185307179586476925286766559;
@@ -52,7 +52,7 @@ struct DevScalars {
   unsigned long long A[3];           // max edge wave speed per stage
   unsigned long long Jmax[3];        // max width of the stage meshes J^n, J^(1), J^(2)
   unsigned long long Jmin0;          // min J^n
-  unsigned long long JmaxN, JminN;   // of J^{n+1}, accumulated by stage 3
+  unsigned long long JmaxN, JminN;   // of J^{n+1} (the minimum accumulated by stage 1)
   unsigned long long Wabs, dWabs;    // fluid-driven motion: max |w|, max |w_{j+1} - w_j|
   long long steps;
   long long step_idx;                // index of the step in progress (set by the prologue)
@@ -60,8 +60,8 @@ struct DevScalars {
   unsigned int counter;              // reconstruction tiles finished in stage 1
   int done;
   int clipped;
-  // Mesh geometry cache: stage 2 stores the per-cell reconstruction geometry of the t_{n+1} mesh,
-  // which the next step's stage 1 reuses when the tag (context epoch, step index) matches.
+  // Mesh cache: stage 2 stores the mesh-only values (GEO_*) of the t_{n+1} mesh, which the next
+  // step's stage 1 reuses when the tag (context epoch, step index) matches.
   unsigned long long geo_tag;
 };
 
@@ -72,7 +72,7 @@ struct InstConst {
                        // edge arrays: coff + 2 i)
   double cfl;
   double Wbar_profile; // (2 pi / T) max |P| of the prescribed motion
-  int32_t ntiles_r;    // reconstruction tiles of the instance
+  int32_t ntiles_r;    // forward reconstruction tiles of the instance
   int32_t pad_;
 };
 
@@ -121,6 +121,11 @@ __device__ __forceinline__ double stage_alpha(const StepConst& K, int i, int s, 
   return computed;
 }
 
+// Mesh-only values that stage 2 keeps for the next step's stage 1, which runs on the same mesh: the
+// reciprocal sums of the widths (see k_recon) and the source term's ratios (per interface, at the
+// edge index of its left cell, and per cell).
+enum { GEO_IP, GEO_IT, GEO_IQ, GEO_IV, GEO_RHO, GEO_SIG, GEO_RHO2, GEO_SIG2, GEO_GX, GEO_GY, GEO_K3, GEO_ARRAYS };
+
 // Device arrays of a batch (concatenated over instances).
 struct DevState {
   double *E0, *M0, *B0;        // q^n (updated in place by stage 3)
@@ -137,9 +142,14 @@ struct DevState {
   // the step, restored by k_commit if that update raised an error (null: no roll-back).
   double *bE, *bM, *bB, *bJ, *bx;
   double *eG1, *eG2;           // eta at the interior Gauss-Lobatto points (special source scheme only)
-  // Geometry cache: SWALE_GEOM_VALUES arrays in the edge layout, geo[k * geo_stride + idx].
+  // Mesh cache: GEO_ARRAYS arrays in the edge layout, geo[k * geo_stride + idx] (null: every stage forms
+  // these values, bit for bit the same).
   double* geo;
   int64_t geo_stride;
+  // Per cell of the stage input in the edge layout, written by the reconstruction for the update of
+  // the same stage: differences of eta and h to the next cell, and the depth.
+  double *dE, *dH, *H;
+  double *iJ1, *iJ2;           // 1 / J^(1), 1 / J^(2) (cells)
   // Per cell of the stage mesh, 14 arrays in the edge layout (gK[k * geo_stride + idx]): the
   // smooth class's linear form K[2][4] (k < 8), stored by the hydrostatic reconstruction, and the
   // source term's six form entries (k = 8..13), stored by the update; set only for the adjoint's
@@ -154,6 +164,10 @@ struct DevState {
   // take one pass (utiles, of T cells, serve the adjoint's kernels).
   const Tile* ftiles;
   int32_t nf;
+  // The forward reconstruction's tiles: T - 4 cells for a block of T threads (rtiles, of T cells,
+  // serve the adjoint's kernels).
+  const Tile* rftiles;
+  int32_t nrf;
 };
 
 __constant__ double c_gauss_w[2 * kMaxGaussHalf + 1];
@@ -467,72 +481,80 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
 }
 
 // ------------------------------------------------------------------------------------
-// Reconstruction + limiter of cells -1..N_i (rows a2-a7) for stage STAGE. A tile is T
-// consecutive cells; the block stages their 5-cell stencils (tile plus a 2-cell halo each
-// side) in shared memory, computes each pair's and each triple's reciprocal width and divided
-// differences once, then reconstructs one cell per thread. It stores the pair / triple
-// reciprocals for the update kernel of the same stage, reduces the wave speed, and in stage 1
-// the instance's last tile computes its dt (and the secant factor of the prescribed motion).
+// Reconstruction + limiter of cells -1..N_i (rows a2-a7) for stage STAGE. A block of T threads
+// holds T consecutive cells, one per thread, and reconstructs the T - 4 inner ones: the
+// differences of order two to five that the stencils share (pairs, triples, quadruples,
+// quintuples of cells) are formed once each, one per thread and order, through shared memory, so
+// that every phase is a single pass of the block (a tile of T cells with a halo would leave four
+// entries of each phase to a second pass of one warp). It stores the edge states, the pair / triple reciprocals and
+// pair differences that the update kernel of the same stage reads, reduces the wave speed, and in
+// stage 1 the instance's last tile computes its dt (and the secant factor of the prescribed motion).
+// What bounds it: FP64 instructions, each of which holds its SM sub-partition for 64 cycles.
 // ------------------------------------------------------------------------------------
-// A cell of the well-balanced scheme whose smooth class the FP32 test leaves open, out of line:
-// the rest of its cached geometry (stage 1), the indicator factors and triple differences, the
-// FP64 detector and the edge values of its class. A call, not inlined, so that this rare path's
-// registers do not weigh on the smooth cells' code; its inputs are copies.
-struct OpenCell {
-  swale::CellGeom G;
-  swale::StencilDD DD;
-  double h[5], it[3], v0[3][3], dxe;
+// Shared-memory rows of a tile that the out-of-line path of an open cell reads (row i: cell, pair,
+// triple starting at cell c0 - 2 + i).
+struct TileRows {
+  const double *J, *E, *M, *H, *D2, *D3;
+  int ld;  // distance between the rows of the three variables in D2, D3
 };
 struct OpenOut {
   EdgeState o;
+  double etaG[2];
   uint32_t st;
   uint8_t flag;
 };
-__device__ __noinline__ OpenOut recon_open_cell(const SchemeConst P, OpenCell c, const double* geo, int64_t geo_stride,
-                                                int64_t idx) {
-  double* gv = reinterpret_cast<double*>(&c.G);
-  constexpr int kF0 = offsetof(swale::CellGeom, F) / sizeof(double), kF1 = kF0 + 5;
-  if (geo) {
+// A cell whose smooth class the FP32 test leaves open (or whose widths are not moderate), out of
+// line: the mesh geometry with its checks, the FP64 detector and the edge values of its class.
+// A call, not inlined, so that this rare path's registers do not weigh on the smooth cells' code.
+template <int SCHEME>
+__device__ __noinline__ OpenOut recon_open_cell(const SchemeConst P, const TileRows R, int i, double dxe) {
+  swale::CellGeom G;
+  swale::StencilDD DD;
+  double h[5], v0[3][3];
+  const double* V[3] = {R.E, R.M, R.H};
 #pragma unroll
-    for (int k = 0; k < SWALE_GEOM_BASE; ++k)
-      if (k < kF0 || k >= kF1) gv[k] = geo[k * geo_stride + idx];
+  for (int k = 0; k < 5; ++k) h[k] = R.J[i - 2 + k];
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) v0[v][a] = V[v][i - 2 + a];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) DD.D2[v][a] = R.D2[v * R.ld + i - 2 + a];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) DD.D3[v][a] = R.D3[v * R.ld + i - 2 + a];
   }
-  swale::indicator_factors(c.h, c.dxe, c.G);
-#pragma unroll
-  for (int v = 0; v < 3; ++v)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) c.DD.D3[v][a] = swale::triple_dd(c.DD.D2[v][a], c.DD.D2[v][a + 1], c.it[a]);
   OpenOut r;
   r.st = 0;
-  swale::recon_cell_g(P, c.G, c.v0, c.DD, r.o, r.flag, r.st, false);
+  r.etaG[0] = r.etaG[1] = 0.0;
+  swale::cell_geom(h, dxe, G, r.st);
+  if (SCHEME == 1) {
+    swale::recon_cell_nonwb_g(P, G, v0, DD, r.o, r.flag, r.st, swale::nonwb_proj(P, v0));
+  } else if (SCHEME == 2) {
+    swale::recon_cell_special_g(P, G, h, v0, DD, r.o, r.flag, r.st, r.etaG);
+  } else {
+    const double it[3] = {swale::triple_recip(h[0], h[1], h[2]), swale::triple_recip(h[1], h[2], h[3]),
+                          swale::triple_recip(h[2], h[3], h[4])};
+    swale::smooth_edge_coeffs(h, it, G);
+    swale::recon_cell_g(P, G, v0, DD, r.o, r.flag, r.st, false);
+  }
   return r;
 }
 
-// Launch bounds (resident threads per SM): HIOCC, 8 blocks of 128 threads (64 registers), for
-// stage 1 of the well-balanced scheme when it reads the cached mesh geometry: its per-cell work is
-// light enough there that more resident warps win (measured: 0.8 % of the dam-break step), while
-// every instantiation that computes the geometry itself spills heavily under that bound. The
-// other well-balanced instantiations take 768 threads (6 blocks of 128, 80 registers, a few
-// spilled doubles; 1.2 % faster per step than 4 blocks of 128 registers), the other schemes 512.
 // STOREK: an instantiation of the hydrostatic scheme that also stores each cell's smooth-class
 // linear form in D.gK (the adjoint's recomputes), so that the forward's own instantiations keep
 // their registers.
-template <int STAGE, int T, int SCHEME = 0, bool HIOCC = false, bool STOREK = false>
-__global__ void __launch_bounds__(T, (HIOCC ? 1024 : (SCHEME == 0 ? 768 : 512)) / T) k_recon(StepConst K, DevState D, const double* __restrict__ Eg,
+template <int STAGE, int T, int SCHEME = 0, bool STOREK = false>
+__global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, DevState D, const double* __restrict__ Eg,
                                              const double* __restrict__ Mg, const double* __restrict__ Bg,
                                              const double* __restrict__ Jg) {
-  __shared__ double sJ[T + 4], sV[3][T + 4];    // cells c0-2 .. c0+T+1
-  __shared__ double sIP[T + 3], sD2[3][T + 3];  // pairs starting at those cells
-  // Triples centred at cells c0-1 .. c0+T. The well-balanced scheme forms the second differences
-  // per cell, and only where the FP32 smooth-class test cannot decide (the smooth class needs
-  // none); the other schemes form them here.
-  constexpr int TD3 = SCHEME == 0 ? 0 : T;
-  __shared__ double sIT[T + 2], sD3[3][TD3 + 2];
-  // FP32 copies of the pair differences (hu, h, and for the non-well-balanced scheme eta) and of
-  // the triple reciprocals for the FP32 smooth-class tests
+  constexpr int TO = T - 4;                        // cells reconstructed
+  __shared__ __align__(16) double sRaw[4][T + 8];  // E, M, B, J of cells c0-2 .. c0+T-3 as bulk-copied
+  __shared__ double sH[T], sP[T], sQ[T];           // depths; pair and quadruple sums of widths
+  __shared__ double sD2[3][T], sD3[3][T], sD4[3][T];
+  // FP32 copies for the smooth-class test: widths, triple reciprocals, pair differences (hu, h, and
+  // for the non-well-balanced scheme eta)
   constexpr int NV32 = SCHEME == 1 ? 3 : 2;
-  __shared__ float sD2f[NV32][T + 3], sITf[T + 2];
-  __shared__ __align__(16) double sRaw[4][T + 8];  // E, M, B, J of those cells as bulk-copied
+  __shared__ float sJf[T], sITf[T], sD2f[NV32][T];
   __shared__ __align__(8) uint64_t sBar;           // completion of the tile's bulk copies
   __shared__ __align__(8) uint64_t sPad;           // test hook: a barrier no copy completes
   __shared__ bool last;
@@ -545,8 +567,8 @@ __global__ void __launch_bounds__(T, (HIOCC ? 1024 : (SCHEME == 0 ? 768 : 512)) 
   }
   __syncthreads();
   uint32_t phase = 0;
-  for (int t = blockIdx.x; t < D.nr; t += gridDim.x) {
-    const Tile tl = D.rtiles ? D.rtiles[t] : Tile{0, t * T - 1};
+  for (int t = blockIdx.x; t < D.nrf; t += gridDim.x) {
+    const Tile tl = D.rftiles ? D.rftiles[t] : Tile{0, t * TO - 1};
     DevScalars* S = D.S + tl.inst;
     // every thread reads the flags once, then the block agrees (the status may change meanwhile)
     if (__syncthreads_or(inst_idle(S))) continue;
@@ -557,15 +579,14 @@ __global__ void __launch_bounds__(T, (HIOCC ? 1024 : (SCHEME == 0 ? 768 : 512)) 
     const double* B = Bg + ic.coff;
     const double* J = Jg + ic.coff;
     const int64_t eb = ic.coff + 2 * (int64_t)tl.inst;  // edge-array base of the instance
-    __syncthreads();
-    // The stencil cells of the tile that lie in the instance, [cs, ce], arrive by four bulk
-    // copies (E, M, B, J). The copied span [ga, ge] (global element indices) is widened to
-    // 16-byte boundaries: one element before cs where needed (it exists: ga >= 1), one after ce
-    // when that element is in the arrays (the instance is not the last one, or ce < N - 1),
-    // else one fewer (that cell is loaded directly). Shared rows are shifted by `off` so that
-    // the first copied element lands on a 16-byte boundary as well. Ghost cells and anything
-    // not copied take the direct loads below.
-    const int64_t cs = c0 - 2 < 0 ? 0 : c0 - 2, ce = c0 + T + 1 < N - 1 ? c0 + T + 1 : N - 1;
+    // The cells of the tile that lie in the instance, [cs, ce], arrive by four bulk copies (E, M,
+    // B, J). The copied span [ga, ge] (global element indices) is widened to 16-byte boundaries:
+    // one element before cs where needed (it exists: ga >= 1), one after ce when that element is
+    // in the arrays (the instance is not the last one, or ce < N - 1), else one fewer (that cell
+    // is loaded directly). Shared rows are shifted by `off` so that the first copied element
+    // lands on a 16-byte boundary as well. Ghost cells and anything not copied take the direct
+    // loads below.
+    const int64_t cs = c0 - 2 < 0 ? 0 : c0 - 2, ce = c0 + T - 3 < N - 1 ? c0 + T - 3 : N - 1;
     int64_t ga = (ic.coff + cs) & ~(int64_t)1, ge = ic.coff + ce;
     if (!(ge & 1)) ge += (ce + 1 < N || tl.inst + 1 < K.B) ? 1 : -1;
     const int rel = (int)(ga - ic.coff - (c0 - 2));  // shared index of ga before the shift
@@ -573,6 +594,24 @@ __global__ void __launch_bounds__(T, (HIOCC ? 1024 : (SCHEME == 0 ? 768 : 512)) 
     const uint32_t bytes = ge >= ga ? (uint32_t)((ge - ga + 1) * 8) : 0u;
     const bool bulk = bytes >= 16 && ((((uintptr_t)(Eg + ga)) | ((uintptr_t)(Mg + ga)) | ((uintptr_t)(Bg + ga)) |
                                        ((uintptr_t)(Jg + ga))) & 15) == 0;
+    const int64_t c = c0 - 2 + tid;       // this thread's cell
+    const int64_t idx = eb + c + 1;       // its edge-array index
+    const unsigned long long geo_now =
+        ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)(S->step_idx & 0xffffffffLL);
+    // Reciprocal sums of the widths: as the previous step's stage 2 stored them (the same mesh), or
+    // formed below. Those that lie at cells -1..N are in the cache: the pair starting at c, the triple
+    // and quadruple whose second cell is c + 1, the quintuple centred at c.
+    const bool use_geo = STAGE == 1 && D.geo != nullptr && S->geo_tag == geo_now;
+    const bool g_pair = use_geo && c >= -1 && c <= N, g_next = use_geo && c >= -2 && c + 1 <= N;
+    double gip = 0.0, git = 0.0, giq = 0.0, giv = 0.0;
+    if (g_pair) {
+      gip = D.geo[GEO_IP * D.geo_stride + idx];
+      giv = D.geo[GEO_IV * D.geo_stride + idx];
+    }
+    if (g_next) {
+      git = D.geo[GEO_IT * D.geo_stride + idx + 1];
+      giq = D.geo[GEO_IQ * D.geo_stride + idx + 1];
+    }
     if (bulk) {
       if (tid == 0) {
         fence_proxy_async();  // the previous tile's reads of sRaw come before these writes
@@ -596,188 +635,158 @@ __global__ void __launch_bounds__(T, (HIOCC ? 1024 : (SCHEME == 0 ? 768 : 512)) 
         return;
       }
     }
-    const int64_t gs = ga - ic.coff, gl = ge - ic.coff;  // copied cells (instance indices)
-    for (int i = tid; i < T + 4; i += T) {
-      const int64_t c = c0 - 2 + i;
-      double jv = 1.0, ev = 0.0, mv = 0.0, bv = 0.0;  // filler beyond the last ghost cell
-      if (bulk && c >= 0 && c < N && c >= gs && c <= gl) {
-        const int k = i + off;
-        ev = sRaw[0][k];
-        mv = sRaw[1][k];
-        bv = sRaw[2][k];
-        jv = sRaw[3][k];
-      } else if (c >= -3 && c <= N + 2) {
+    double* const sE = &sRaw[0][off];
+    double* const sM = &sRaw[1][off];
+    double* const sJ = &sRaw[3][off];
+    double jv = 1.0, ev = 0.0, mv = 0.0, hv = 0.0;  // filler beyond the last ghost cell
+    if (bulk && c >= 0 && c < N && c >= ga - ic.coff && c <= ge - ic.coff) {
+      ev = sE[tid];
+      mv = sM[tid];
+      jv = sJ[tid];
+      hv = ev - sRaw[2][off + tid];
+    } else {
+      if (c >= -3 && c <= N + 2) {
         const int64_t s = ghost(c, N, K.bc);
         jv = J[s];
         ev = E[s];
-        bv = B[s];
         mv = M[s];
         if (refl && (c < 0 || c >= N)) mv = -mv;
+        hv = ev - B[s];
       }
-      sJ[i] = jv;
-      sV[0][i] = ev;
-      sV[1][i] = mv;
-      sV[2][i] = ev - bv;  // the depth is reconstructed in place of the bottom
+      sE[tid] = ev;
+      sM[tid] = mv;
+      sJ[tid] = jv;
     }
+    sH[tid] = hv;  // the depth is reconstructed in place of the bottom
+    sJf[tid] = swale::f32_trunc(jv);
     __syncthreads();
-    for (int i = tid; i < T + 3; i += T) {
-      const double ip = swale::pair_recip(sJ[i], sJ[i + 1]);
-      sIP[i] = ip;
-      double d2[3];
+    // Cells of the tile that are reconstructed and stored.
+    const bool mine = tid >= 2 && tid < 2 + TO && c <= N;
+    const bool next_mine = tid >= 1 && tid < 1 + TO && c + 1 <= N;  // cell c + 1 is
+    // Order 2: the pair (c, c+1).
+    double p = 0.0, d2[3] = {0.0, 0.0, 0.0};
+    if (tid < T - 1) {
+      const double jn = sJ[tid + 1], de = sE[tid + 1] - ev, dm = sM[tid + 1] - mv, dh = sH[tid + 1] - hv;
+      p = jv + jn;
+      const double ip = g_pair ? gip : swale::recip(p);
+      d2[0] = de * ip;
+      d2[1] = dm * ip;
+      d2[2] = dh * ip;
+      sP[tid] = p;
 #pragma unroll
-      for (int v = 0; v < 3; ++v) sD2[v][i] = d2[v] = swale::pair_dd(sV[v][i], sV[v][i + 1], ip);
-      sD2f[0][i] = swale::f32_trunc(d2[1]);
-      sD2f[1][i] = swale::f32_trunc(d2[2]);
-      if (SCHEME == 1) sD2f[NV32 - 1][i] = swale::f32_trunc(d2[0]);
-    }
-    __syncthreads();
-    for (int i = tid; i < T + 2; i += T) {
-      const double it = swale::triple_recip(sJ[i], sJ[i + 1], sJ[i + 2]);
-      sIT[i] = it;
-      if (SCHEME != 0) {
-#pragma unroll
-        for (int v = 0; v < 3; ++v) sD3[v][i] = swale::triple_dd(sD2[v][i], sD2[v][i + 1], it);
+      for (int v = 0; v < 3; ++v) sD2[v][tid] = d2[v];
+      sD2f[0][tid] = swale::f32_trunc(d2[1]);
+      sD2f[1][tid] = swale::f32_trunc(d2[2]);
+      if (SCHEME == 1) sD2f[NV32 - 1][tid] = swale::f32_trunc(d2[0]);
+      if (mine) {
+        if (SCHEME == 2 || !use_geo) D.ipair[idx] = ip;  // (on the cache the update needs neither)
+        D.dE[idx] = de;
+        D.dH[idx] = dh;
+        D.H[idx] = hv;
+        if (STAGE == 2 && D.geo) D.geo[GEO_IP * D.geo_stride + idx] = ip;
       }
-      sITf[i] = swale::f32_trunc(it);
     }
     __syncthreads();
-    const int64_t c = c0 + tid;
-    const unsigned long long geo_now =
-        ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)(S->step_idx & 0xffffffffLL);
-    const bool use_geo = STAGE == 1 && D.geo != nullptr && S->geo_tag == geo_now;
+    // Order 3: the triple (c, c+1, c+2).
+    double d3[3] = {0.0, 0.0, 0.0};
+    if (tid < T - 2) {
+      const double it = g_next ? git : swale::recip(p + sJ[tid + 2]);
+#pragma unroll
+      for (int v = 0; v < 3; ++v) sD3[v][tid] = d3[v] = (sD2[v][tid + 1] - d2[v]) * it;
+      sITf[tid] = swale::f32_trunc(it);
+      if (next_mine) {
+        if (SCHEME == 2 || !use_geo) D.itri[idx + 1] = it;
+        if (STAGE == 2 && D.geo) D.geo[GEO_IT * D.geo_stride + idx + 1] = it;
+      }
+    }
+    __syncthreads();
+    // Order 4: the quadruple (c .. c+3).
+    if (tid < T - 3) {
+      const double q = p + sP[tid + 2];
+      const double iq = g_next ? giq : swale::recip(q);
+      sQ[tid] = q;
+#pragma unroll
+      for (int v = 0; v < 3; ++v) sD4[v][tid] = (sD3[v][tid + 1] - d3[v]) * iq;
+      if (STAGE == 2 && D.geo && next_mine) D.geo[GEO_IQ * D.geo_stride + idx + 1] = iq;
+    }
+    __syncthreads();
     if (STAGE == 2 && D.geo != nullptr && c0 == -1 && tid == 0)
       S->geo_tag = ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)((S->step_idx + 1) & 0xffffffffLL);
     double wave = 0.0, ehL = 0.0, euL = 0.0, ehR = 0.0, euR = 0.0;
     bool useL = false, useR = false;
     uint32_t st = 0;
-    if (c <= N) {
-      double h[5], v0[3][3];
-      swale::StencilDD DD;
+    if (mine) {
+      const double dxmax = bitsd(S->Jmax[STAGE - 1]);
+      const double dxe = K.sc.beta_dx_global ? dxmax : jv;
+      if (!swale::gt0(jv)) st |= swale::ST_EMESH;
+      EdgeState o;
+      uint8_t flag = 0;
+      double etaG[2] = {0.0, 0.0};
+      // The smooth class, when FP32 can tell it for sure; else the FP64 detector decides.
+      bool smooth;
+      {
+        const float hf[5] = {sJf[tid - 2], sJf[tid - 1], sJf[tid], sJf[tid + 1], sJf[tid + 2]};
+        float F32[3], itf[3], c4f, c3f, d2h[4], d2m[4];
+        swale::indicator_factors_f32(hf, swale::f32_trunc(dxe), F32, c4f, c3f);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) h[k] = sJ[tid + k];
-      // The well-balanced scheme reads its stencil data from shared memory where its class is
-      // known (below): fewer values live across the mesh geometry.
-      if (SCHEME != 0) {
+        for (int a = 0; a < 3; ++a) itf[a] = sITf[tid - 2 + a];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          d2h[a] = sD2f[1][tid - 2 + a];
+          d2m[a] = sD2f[0][tid - 2 + a];
+        }
+        const float epsf = swale::f32_trunc(K.sc.eps_weno);
+        if (SCHEME == 1) {
+          float d2e[4];
+#pragma unroll
+          for (int a = 0; a < 4; ++a) d2e[a] = sD2f[NV32 - 1][tid - 2 + a];
+          smooth = swale::sure_smooth_nonwb_f32(K.sc.g, K.sc.h_dry, hv, mv, F32, c4f, c3f, d2e, d2m, d2h, itf, epsf);
+        } else {
+          smooth = swale::sure_smooth_f32(F32, c4f, c3f, d2h, d2m, itf, epsf);
+        }
+        smooth = smooth && swale::moderate_widths(hf[0], hf[1], hf[2], hf[3], hf[4]);
+      }
+      if (smooth) {
+        // Order 5, the quintuple centred at c, and the edge values.
+        const swale::SmoothWidths w = {sJ[tid - 1], jv, sJ[tid + 1], sP[tid - 2], sP[tid - 1], p, sP[tid + 1]};
+        const double iv = g_pair ? giv : swale::recip(sQ[tid - 2] + sJ[tid + 2]);
+        if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = iv;
+        const double vj[3] = {ev, mv, hv};
+        double evl[3][2];
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
-#pragma unroll
-          for (int a = 0; a < 3; ++a) v0[v][a] = sV[v][tid + a];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) DD.D2[v][a] = sD2[v][tid + a];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) DD.D3[v][a] = sD3[v][tid + a];
-        }
-      }
-      const double dxmax = bitsd(S->Jmax[STAGE - 1]);
-      const int64_t idx = eb + c + 1;
-      // Mesh geometry of the cell: from the cache that the previous step's stage 2 filled on the
-      // same mesh (t_{n+1}), else computed; stage 2 fills the cache.
-      swale::CellGeom G;
-      double* gv = reinterpret_cast<double*>(&G);
-      constexpr int kGeo = SCHEME == 0 ? SWALE_GEOM_VALUES : SWALE_GEOM_BASE;  // values cached
-      // The indicator factors (F, c4, c3) are not cached: they are formed below, in FP32 for the
-      // smooth-class test and in FP64 only where that test cannot decide.
-      constexpr int kF0 = offsetof(swale::CellGeom, F) / sizeof(double), kF1 = kF0 + 5;
-      static_assert(offsetof(swale::CellGeom, c4) / sizeof(double) == kF0 + 4, "F, c3, c4 are adjacent");
-      const double dxe = K.sc.beta_dx_global ? dxmax : h[2];
-      // The well-balanced scheme reads only the smooth-class form K here; the rest of the cached
-      // geometry (sub-stencil factors and linear weights) only for a cell whose class the FP32
-      // test leaves open.
-      constexpr int kLoad0 = SCHEME == 0 ? SWALE_GEOM_BASE : 0;
-      if (use_geo) {
-#pragma unroll
-        for (int k = kLoad0; k < kGeo; ++k)
-          if (k < kF0 || k >= kF1) gv[k] = D.geo[k * D.geo_stride + idx];
-        if (!swale::gt0(h[2])) st |= swale::ST_EMESH;
-      } else {
-        swale::cell_geom(h, dxe, G, st, false);
-        if (SCHEME == 0) {
-          const double it3[3] = {sIT[tid], sIT[tid + 1], sIT[tid + 2]};
-          swale::smooth_edge_coeffs(h, it3, G);
-        }
-      }
-      if (STAGE == 2 && D.geo) {
-#pragma unroll
-        for (int k = 0; k < kGeo; ++k)
-          if (k < kF0 || k >= kF1) D.geo[k * D.geo_stride + idx] = gv[k];
-      }
-      if (STOREK && SCHEME == 0) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) D.gK[k * D.geo_stride + idx] = G.K[k >> 2][k & 3];
-      }
-      EdgeState o;
-      uint8_t flag;
-      double etaG[2] = {0.0, 0.0};
-      // Indicator factors in FP32 from the FP32 widths.
-      float F32[3], itf[3], c4f, c3f;
-      swale::indicator_factors_f32(h, dxe, F32, c4f, c3f);
-#pragma unroll
-      for (int a = 0; a < 3; ++a) itf[a] = sITf[tid + a];
-      const float epsf = swale::f32_trunc(K.sc.eps_weno);
-      if (SCHEME == 1) {
-        // Each characteristic field and the bottom: its smooth class in FP32 when that can be
-        // told for sure, from the FP32 pair differences of eta, hu, h and the projection rows.
-        const swale::NonwbProj pr = swale::nonwb_proj(K.sc, v0);
-        const float a11 = swale::f32_trunc(pr.a11), a12 = swale::f32_trunc(pr.a12);
-        const float a21 = swale::f32_trunc(pr.a21), a22 = swale::f32_trunc(pr.a22);
-        float fd[3][4], fm[3][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const float e2 = sD2f[NV32 - 1][tid + a], m2 = sD2f[0][tid + a], h2 = sD2f[1][tid + a];
-          fd[0][a] = fmaf(a11, e2, a12 * m2);
-          fm[0][a] = fmaf(fabsf(a11), fabsf(e2), fabsf(a12) * fabsf(m2));
-          fd[1][a] = fmaf(a21, e2, a22 * m2);
-          fm[1][a] = fmaf(fabsf(a21), fabsf(e2), fabsf(a22) * fabsf(m2));
-          fd[2][a] = e2 - h2;
-          fm[2][a] = fabsf(e2) + fabsf(h2);
-        }
-        bool known[3];
-#pragma unroll
-        for (int f = 0; f < 3; ++f) known[f] = swale::sure_smooth1_f32(F32, c4f, c3f, fd[f], fm[f], itf, epsf);
-        if (!(known[0] && known[1] && known[2])) swale::indicator_factors(h, dxe, G);
-        swale::recon_cell_nonwb_g(K.sc, G, v0, DD, o, flag, st, pr, known);
-      } else {
-        // The smooth class, when FP32 can tell it for sure; else the FP64 detector decides.
-        float d2h[4], d2m[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          d2h[a] = sD2f[1][tid + a];
-          d2m[a] = sD2f[0][tid + a];
-        }
-        const bool smooth32 = swale::sure_smooth_f32(F32, c4f, c3f, d2h, d2m, itf, epsf);
-        if (SCHEME == 0) {
-          if (smooth32) {  // the cell's averages and pair differences are all the smooth class needs
-#pragma unroll
-            for (int v = 0; v < 3; ++v) {
-              v0[v][2] = sV[v][tid + 2];
-#pragma unroll
-              for (int a = 0; a < 4; ++a) DD.D2[v][a] = sD2[v][tid + a];
-            }
-            swale::recon_cell_g(K.sc, G, v0, DD, o, flag, st, true);
-          } else {  // the FP64 detector decides, out of line
-            OpenCell oc;
-            oc.G = G;
-            oc.dxe = dxe;
-#pragma unroll
-            for (int k = 0; k < 5; ++k) oc.h[k] = h[k];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) oc.it[a] = sIT[tid + a];
-#pragma unroll
-            for (int v = 0; v < 3; ++v) {
-#pragma unroll
-              for (int a = 0; a < 3; ++a) oc.v0[v][a] = sV[v][tid + a];
-#pragma unroll
-              for (int a = 0; a < 4; ++a) oc.DD.D2[v][a] = sD2[v][tid + a];
-            }
-            const OpenOut r = recon_open_cell(K.sc, oc, use_geo ? D.geo : nullptr, D.geo_stride, idx);
-            o = r.o;
-            flag = r.flag;
-            st |= r.st;
+          const double d4l = sD4[v][tid - 2], d4r = sD4[v][tid - 1], d3c = sD3[v][tid - 1];
+          const double d5 = (d4r - d4l) * iv;
+          evl[v][0] = swale::smooth_left(w, vj[v], sD2[v][tid - 1], d3c, d4l, d5);
+          evl[v][1] = swale::smooth_right(w, vj[v], d2[v], d3c, d4r, d5);
+          if (SCHEME == 2 && v == 0) {
+            etaG[0] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T1, ev, d2[v], d3c, d4r, d5);
+            etaG[1] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T2, ev, d2[v], d3c, d4r, d5);
           }
-        } else {
-          if (!smooth32) swale::indicator_factors(h, dxe, G);  // the FP64 detector needs them
-          swale::recon_cell_special_g(K.sc, G, h, v0, DD, o, flag, st, etaG, smooth32);
         }
+        swale::limit_cell(K.sc, evl, hv, mv, o, st);
+      } else {
+        if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = swale::recip(sQ[tid - 2] + sJ[tid + 2]);
+        const TileRows R = {sJ, sE, sM, sH, &sD2[0][0], &sD3[0][0], T};
+        const OpenOut r = recon_open_cell<SCHEME>(K.sc, R, tid, dxe);
+        o = r.o;
+        flag = r.flag;
+        etaG[0] = r.etaG[0];
+        etaG[1] = r.etaG[1];
+        st |= r.st;
+      }
+      if (STOREK) {
+        double h[5], K8[2][4];
+        swale::CellGeom G;
+        uint32_t stk = 0;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) h[k] = sJ[tid - 2 + k];
+        const double it3[3] = {swale::triple_recip(h[0], h[1], h[2]), swale::triple_recip(h[1], h[2], h[3]),
+                               swale::triple_recip(h[2], h[3], h[4])};
+        swale::cell_geom(h, dxe, G, stk, false);
+        swale::linear_edge_form(G.d, G.G1, G.G2, h, it3, K8);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) D.gK[k * D.geo_stride + idx] = K8[k >> 2][k & 3];
       }
       D.eEL[idx] = o.EL;
       D.eER[idx] = o.ER;
@@ -791,8 +800,6 @@ __global__ void __launch_bounds__(T, (HIOCC ? 1024 : (SCHEME == 0 ? 768 : 512)) 
         D.eG1[idx] = etaG[0];
         D.eG2[idx] = etaG[1];
       }
-      D.ipair[idx] = sIP[tid + 2];  // pair (c, c+1)
-      D.itri[idx] = sIT[tid + 1];   // triple centred at c
       if (STAGE == 1) D.flags[idx] = flag;
       // Edges that touch interfaces 0..N only.
       useL = (c != -1);
@@ -867,27 +874,33 @@ __global__ void __launch_bounds__(T, (HIOCC ? 1024 : (SCHEME == 0 ? 768 : 512)) 
 // ------------------------------------------------------------------------------------
 // Fluxes, source and the RK combination of stage STAGE for cells 0..N_i-1 (rows a1, a8, a9;
 // MODE 0), or the bare right-hand side of one instance (MODE 1, used by swale_rhs). A tile is
-// T - 1 consecutive cells for a block of T threads: its T interfaces' fluxes are computed once,
-// one per thread, into shared memory (a tile of T cells would leave its last interface to a
-// second pass of a single thread); the widths, their reciprocals and the depth / bottom
-// averages of the tile plus one halo cell each side are staged there too.
+// T - 1 consecutive cells for a block of T threads: thread i forms the fluxes of interface
+// j0 + i, once, and passes them to the cell on its left through shared memory (a tile of T cells
+// would leave its last interface to a second pass of a single thread). Bound by FP64
+// instructions like the reconstruction, so everything is at twice its value (the halves of the
+// Lax-Friedrichs flux are then free) and the pressure terms are combined with the source in the
+// cell (source_pressure_form in swale_cell.cuh).
+//
+// The three stages advance increments instead of the products J q: with the width recursion of
+// Eq. Jacobi2D in closed form, J^(1) = J^{n+1} = J + dt dw and J^(2) = J + dt dw / 2, the
+// combination of Eq. RK32D reads J^(s) q^(s) = J q + dt (b_s . R), so
+//   q^(s) = q + (dt (b_s . R) - q (J^(s) - J)) / J^(s),  b = (1), (1/4, 1/4), (1/6, 1/6, 2/3):
+// fewer operations, and the rounding of the products J q stays out of the state.
 // ------------------------------------------------------------------------------------
 struct RhsOut {
   double *RE, *RM, *RB;
   double alpha;
 };
 
-// PLAIN: an instantiation for the hydrostatic scheme without the L2-projection bottom (the
-// common case), in which the other schemes' branches are compiled out; it is held to 64
-// registers (8 blocks of 128 threads per SM: without the bound stage 1 takes 71 and 7 blocks,
-// measured slower). STOREK: one that also stores the source form's entries in D.gK (the
+// SCHEME: 0 hydrostatic, 1 non-well-balanced, 2 special source. BOT: an instantiation with the
+// L2-projection bottom. STOREK: one that also stores the old source form's entries in D.gK (the
 // adjoint's recomputes).
-template <int STAGE, int MODE, int T, bool PLAIN = false, bool STOREK = false>
-__global__ void __launch_bounds__(T, PLAIN ? 1024 / T : 1) k_update(StepConst K, DevState D, const double* __restrict__ Eg,
+template <int STAGE, int MODE, int T, int SCHEME = 0, bool BOT = false, bool STOREK = false>
+__global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, DevState D, const double* __restrict__ Eg,
                                               const double* __restrict__ Mg, const double* __restrict__ Bg,
                                               const double* __restrict__ Jsg, RhsOut ro) {
-  __shared__ double sF[4][T], sW[T];                              // interfaces / nodes j0 .. j0+T-1
-  __shared__ double sJ[T + 1], siJ[T + 1], sH[T + 1], sB[T + 1];  // cells j0-1 .. j0+T-1
+  __shared__ double sF[3][T], sW[T];      // interfaces / nodes j0 .. j0+T-1: fluxes FE, FMl, FB
+  __shared__ double sG[2][T], sDe[2][T];  // their sig and rho^2 (PairRatio); differences of eta and h
   const int tid = threadIdx.x;
   (void)Mg;
   constexpr int TC = T - 1;  // cells of a tile; its T interfaces j0 .. j0 + TC, one per thread
@@ -921,188 +934,195 @@ __global__ void __launch_bounds__(T, PLAIN ? 1024 / T : 1) k_update(StepConst K,
       dt = S->dt;
     }
     const bool fresh_w = (MODE == 0 && STAGE == 1 && K.mesh == SWALE_MESH_PROFILE);
-    // The source geometry of the cells (width ratios) is cached beside the reconstruction's
-    // mesh geometry: stage 2 stores it and the next step's stage 1, on the same mesh, reads it
-    // under the same tag.
+    // The source's mesh-only values are cached beside the reconstruction's reciprocals: stage 2
+    // stores them and the next step's stage 1, on the same mesh, reads them under the same tag.
     const unsigned long long geo_now =
         ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)(S->step_idx & 0xffffffffLL);
     const bool use_sgeo = STAGE == 1 && MODE == 0 && D.geo != nullptr && S->geo_tag == geo_now;
+    const bool put_sgeo = STAGE == 2 && MODE == 0 && D.geo != nullptr;
     const double sdiff = fresh_w ? S->sdiff : 0.0;
-    __syncthreads();
-    {
-      const int i = tid;
-      const int64_t k = j0 + i;  // node / interface index
-      if (k <= N) {
-        double wk;
-        if (fresh_w) {
-          wk = D.P[nb + k] * sdiff;
-          if (i < TC || k == N) D.w[nb + k] = wk;
-        } else if (MODE == 0 && K.mesh == SWALE_MESH_STATIC) {
-          wk = 0.0;
-        } else if (MODE == 0 && K.mesh == SWALE_MESH_LINEAR) {
-          wk = D.P[nb + k];  // constant node velocity (Eq. velocity)
-          if (STAGE == 1 && (i < TC || k == N)) D.w[nb + k] = wk;
-        } else {
-          wk = D.w[nb + k];
-        }
-        sW[i] = wk;
-        // Interface k: left state = right edge of cell k-1 (edge index k), right state = left
-        // edge of cell k (edge index k+1).
-        const int64_t el = eb + k, er = eb + k + 1;
-        const swale::Flux F =
-            (!PLAIN && K.scheme != 0) ? swale::interface_flux_plain(K.sc.g, alpha, wk, D.eER[el], D.eEL[er], D.eBR[el], D.eBL[er],
-                                                        D.ehR[el], D.ehL[er], D.euR[el], D.euL[er])
-                          : swale::interface_flux(K.sc.g, alpha, wk, D.eER[el], D.eEL[er], D.eBR[el], D.eBL[er],
-                                                  D.ehR[el], D.ehL[er], D.euR[el], D.euL[er]);
-        sF[0][i] = F.FE;
-        sF[1][i] = F.FMm;
-        sF[2][i] = F.FMp;
-        sF[3][i] = F.FB;
+    __syncthreads();  // the previous tile's reads of the shared rows
+    const int64_t k = j0 + tid;  // this thread's node / interface and cell
+    const int64_t el = eb + k, er = eb + k + 1;
+    swale::Flux2 F{0.0, 0.0, 0.0, 0.0};
+    swale::PairRatio pr{0.0, 0.0, 0.0, 0.0};
+    double wk = 0.0, ELj = 0.0, BLj = 0.0, hLj = 0.0, dE = 0.0, dH = 0.0;
+    if (k <= N) {
+      if (fresh_w) {
+        wk = D.P[nb + k] * sdiff;
+        if (tid < TC || k == N) D.w[nb + k] = wk;
+      } else if (MODE == 0 && K.mesh == SWALE_MESH_STATIC) {
+        wk = 0.0;
+      } else if (MODE == 0 && K.mesh == SWALE_MESH_LINEAR) {
+        wk = D.P[nb + k];  // constant node velocity (Eq. velocity)
+        if (STAGE == 1 && (tid < TC || k == N)) D.w[nb + k] = wk;
+      } else {
+        wk = D.w[nb + k];
       }
-    }
-    for (int i = tid; i < TC + 2; i += T) {
-      const int64_t c = j0 - 1 + i;
-      if (c >= -1 && c <= N) {
-        const int64_t s = ghost(c, N, K.bc);
-        const double jv = Js[s];
-        sJ[i] = jv;
-        if (!use_sgeo) siJ[i] = swale::recip(jv);  // only the source geometry needs it
-        sH[i] = E[s] - B[s];
-        sB[i] = B[s];
+      // Interface k: left state = right edge of cell k-1 (edge index k), right state = left
+      // edge of cell k (edge index k+1).
+      ELj = D.eEL[er];
+      BLj = D.eBL[er];
+      hLj = D.ehL[er];
+      dE = D.dE[el];  // eta_k - eta_{k-1}
+      dH = D.dH[el];
+      if (use_sgeo) {
+        pr.rho = D.geo[GEO_RHO * D.geo_stride + el];
+        pr.sig = D.geo[GEO_SIG * D.geo_stride + el];
+        pr.rho2 = D.geo[GEO_RHO2 * D.geo_stride + el];
+        pr.sig2 = D.geo[GEO_SIG2 * D.geo_stride + el];
+      } else {
+        const double Jl = Js[ghost(k - 1, N, K.bc)], Jr = Js[ghost(k, N, K.bc)];
+        pr = swale::pair_ratio(Jl, Jr, D.ipair[el]);
       }
+      if (put_sgeo) {
+        D.geo[GEO_RHO * D.geo_stride + el] = pr.rho;
+        D.geo[GEO_SIG * D.geo_stride + el] = pr.sig;
+        D.geo[GEO_RHO2 * D.geo_stride + el] = pr.rho2;
+        D.geo[GEO_SIG2 * D.geo_stride + el] = pr.sig2;
+      }
+      F = swale::interface_flux2<SCHEME>(K.sc.g, alpha, wk, D.eER[el], ELj, D.eBR[el], BLj, D.ehR[el], hLj, D.euR[el],
+                                         D.euL[er]);
+      sF[0][tid] = F.FE;
+      sF[1][tid] = F.FMl;
+      sF[2][tid] = F.FB;
+      sW[tid] = wk;
+      sG[0][tid] = pr.sig;
+      sG[1][tid] = pr.rho2;
+      sDe[0][tid] = dE;
+      sDe[1][tid] = dH;
     }
     __syncthreads();
-    const int64_t j = j0 + tid;
+    const int64_t j = k;
     double jmaxa = 0.0, jmaxb = 0.0, jminb = INFINITY;
     uint32_t st = 0;
     if (tid < TC && j < N) {
-      const swale::Flux Fl = {sF[0][tid], sF[1][tid], sF[2][tid], sF[3][tid]};
-      const swale::Flux Fr = {sF[0][tid + 1], sF[1][tid + 1], sF[2][tid + 1], sF[3][tid + 1]};
-      const int64_t ic_e = eb + j + 1;  // edge-array index of cell j
-      const double hd[5] = {sH[tid], sH[tid + 1], sH[tid + 2], D.ehL[ic_e], D.ehR[ic_e]};
-      const double bd[5] = {sB[tid], sB[tid + 1], sB[tid + 2], D.eBL[ic_e], D.eBR[ic_e]};
-      // Six mesh-only values of the source per cell: the antisymmetric form (SourceForm), or the
-      // width ratios (SourceGeom) for the special scheme's point-wise source.
-      double Sj;
-      if (!PLAIN && K.scheme == 2) {
-        swale::SourceGeom sg;
-        double* const src6 = reinterpret_cast<double*>(&sg);
-        if (use_sgeo) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) src6[k] = D.geo[(SWALE_GEOM_VALUES + k) * D.geo_stride + ic_e];
-        } else {
-          sg = swale::source_geom(sJ[tid], sJ[tid + 1], siJ[tid], siJ[tid + 1], siJ[tid + 2], D.ipair[eb + j],
-                                  D.ipair[eb + j + 1], D.itri[eb + j + 1]);
-        }
-        if (STAGE == 2 && MODE == 0 && D.geo) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) D.geo[(SWALE_GEOM_VALUES + k) * D.geo_stride + ic_e] = src6[k];
-        }
-        const double eta4[4] = {D.eEL[ic_e], D.eG1[ic_e], D.eG2[ic_e], D.eER[ic_e]};
-        Sj = swale::source_cell_special(K.sc.g, E[j], eta4, bd, sg, D.eBR[ic_e - 1],
-                                        D.eBL[ic_e + 1]);
+      const double ERj = D.eER[er], BRj = D.eBR[er], hRj = D.ehR[er];
+      const double hj = D.H[er], Ej = E[j];
+      double Sp;  // twice the pressure and source terms of the momentum (the source alone: special scheme)
+      const double Jm = use_sgeo && SCHEME != 2 ? 0.0 : Js[ghost(j - 1, N, K.bc)];
+      const double Jc = use_sgeo && SCHEME != 2 ? 0.0 : Js[j];
+      const double Jp = use_sgeo && SCHEME != 2 ? 0.0 : Js[ghost(j + 1, N, K.bc)];
+      if (SCHEME == 2) {
+        const double bd[5] = {B[ghost(j - 1, N, K.bc)], B[j], B[ghost(j + 1, N, K.bc)], BLj, BRj};
+        const swale::SourceGeom sg =
+            swale::source_geom(Jm, Jc, swale::recip(Jm), swale::recip(Jc), swale::recip(Jp), D.ipair[el], D.ipair[er], D.itri[er]);
+        const double eta4[4] = {ELj, D.eG1[er], D.eG2[er], ERj};
+        Sp = 2.0 * swale::source_cell_special(K.sc.g, Ej, eta4, bd, sg, D.eBR[er - 1], D.eBL[er + 1]);
       } else {
-        swale::SourceForm sf;
-        double* const src6 = reinterpret_cast<double*>(&sf);
+        swale::SourceRatio sr;
         if (use_sgeo) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) src6[k] = D.geo[(SWALE_GEOM_VALUES + k) * D.geo_stride + ic_e];
+          sr.GX = D.geo[GEO_GX * D.geo_stride + er];
+          sr.GY = D.geo[GEO_GY * D.geo_stride + er];
+          sr.K3 = D.geo[GEO_K3 * D.geo_stride + er];
         } else {
-          sf = swale::source_form(sJ[tid], sJ[tid + 1], sJ[tid + 2], siJ[tid], siJ[tid + 1], siJ[tid + 2],
-                                  D.ipair[eb + j], D.ipair[eb + j + 1], D.itri[eb + j + 1]);
+          // 1 / J of the stage mesh: stored by the previous stage's update, or formed here
+          double iJm, iJp;
+          if (MODE == 0 && STAGE > 1) {
+            const double* iJ = (STAGE == 2 ? D.iJ1 : D.iJ2) + cb;
+            iJm = iJ[ghost(j - 1, N, K.bc)];
+            iJp = iJ[ghost(j + 1, N, K.bc)];
+          } else {
+            iJm = swale::recip(Jm);
+            iJp = swale::recip(Jp);
+          }
+          sr = swale::source_ratio(Jm, Jc, Jp, iJm, iJp, D.itri[er]);
         }
-        if (STAGE == 2 && MODE == 0 && D.geo) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) D.geo[(SWALE_GEOM_VALUES + k) * D.geo_stride + ic_e] = src6[k];
+        if (put_sgeo) {
+          D.geo[GEO_GX * D.geo_stride + er] = sr.GX;
+          D.geo[GEO_GY * D.geo_stride + er] = sr.GY;
+          D.geo[GEO_K3 * D.geo_stride + er] = sr.K3;
         }
         if (STOREK) {
+          const swale::SourceForm sf = swale::source_form(Jm, Jc, Jp, swale::recip(Jm), swale::recip(Jc), swale::recip(Jp),
+                                                          D.ipair[el], D.ipair[er], D.itri[er]);
+          const double* const src6 = reinterpret_cast<const double*>(&sf);
 #pragma unroll
-          for (int k = 0; k < 6; ++k) D.gK[(8 + k) * D.geo_stride + ic_e] = src6[k];
+          for (int q = 0; q < 6; ++q) D.gK[(8 + q) * D.geo_stride + er] = src6[q];
         }
-        Sj = swale::source_cell_form(K.sc.g, hd, bd, sf);
+        const double acc = swale::source_pressure_form(hj, hLj, hRj, ELj - Ej, ERj - Ej, dE, dH, sDe[0][tid + 1],
+                                                       sDe[1][tid + 1], pr.rho, pr.sig2, sG[0][tid + 1],
+                                                       sG[1][tid + 1], sr);
+        Sp = -K.sc.g * acc;
       }
-      const swale::CellRhs R = swale::cell_rhs(Fl, Fr, Sj);
-      const double RE = R.RE, RM = R.RM, RB = R.RB;
+      // Twice the right-hand sides.
+      const double R2[3] = {F.FE - sF[0][tid + 1], (F.FMr - sF[1][tid + 1]) + Sp, sF[2][tid + 1] - F.FB};
       if (MODE == 1) {
-        ro.RE[j] = RE;
-        ro.RM[j] = RM;
-        ro.RB[j] = RB;
+        ro.RE[j] = 0.5 * R2[0];
+        ro.RM[j] = 0.5 * R2[1];
+        ro.RB[j] = 0.5 * R2[2];
       } else {
         const int64_t g = cb + j;  // global cell index
-        const double wl = sW[tid], wr = sW[tid + 1];
+        const double wl = wk, wr = sW[tid + 1];
         const double J0 = D.J0[g];
-        const double dw = wr - wl;
+        const double dJ = dt * (wr - wl);
+        const double q0[3] = {D.E0[g], D.M0[g], D.B0[g]};
         if (STAGE == 1) {
-          const double J1 = J0 + dt * dw;
-          const double J2 = 0.75 * J0 + 0.25 * J1 + 0.25 * dt * dw;
-          // J^{n+1} of the recursion, checked here already so that a step that would invert a
-          // cell fails before its stages run (stage 3 recomputes it from the stored J^(2)).
-          const double J3c = (1.0 / 3.0) * J0 + (2.0 / 3.0) * J2 + (2.0 / 3.0) * dt * dw;
+          const double J1 = J0 + dJ, J2 = J0 + 0.5 * dJ;
           D.J1[g] = J1;
           D.J2[g] = J2;
           jmaxa = J1;
           jmaxb = J2;
-          if (!swale::gt0(J1) || !swale::gt0(J2) || !swale::gt0(J3c)) st |= swale::ST_EMESH;
-          const double yE = J0 * D.E0[g] + dt * RE, yM = J0 * D.M0[g] + dt * RM, yB = J0 * D.B0[g] + dt * RB;
-          D.YE[g] = yE;
-          D.YM[g] = yM;
-          D.YB[g] = yB;
+          jminb = J1;
+          if (!swale::gt0(J1) || !swale::gt0(J2)) st |= swale::ST_EMESH;
           const double inv = swale::recip(J1);
-          D.Ea[g] = yE * inv;
-          D.Ma[g] = yM * inv;
-          D.Ba[g] = yB * inv;
-          if (!PLAIN && K.bot_pieces > 0)  // bottom of stage 2: projection onto the mesh at t_{n+1}
+          D.iJ1[g] = inv;
+          D.YE[g] = R2[0];
+          D.YM[g] = R2[1];
+          D.YB[g] = R2[2];
+          const double hdt = 0.5 * dt;
+          D.Ea[g] = swale::rk_advance(q0[0], hdt, R2[0], dJ, inv);
+          D.Ma[g] = swale::rk_advance(q0[1], hdt, R2[1], dJ, inv);
+          if (!BOT) D.Ba[g] = swale::rk_advance(q0[2], hdt, R2[2], dJ, inv);
+          else  // bottom of stage 2: projection onto the mesh at t_{n+1}
             D.Ba[g] = bottom_average(K, D.x[nb + j] + dt * wl, D.x[nb + j + 1] + dt * wr);
         } else if (STAGE == 2) {
-          const double yE = 0.75 * (J0 * D.E0[g]) + 0.25 * (D.YE[g] + dt * RE);
-          const double yM = 0.75 * (J0 * D.M0[g]) + 0.25 * (D.YM[g] + dt * RM);
-          const double yB = 0.75 * (J0 * D.B0[g]) + 0.25 * (D.YB[g] + dt * RB);
-          D.YE[g] = yE;
-          D.YM[g] = yM;
-          D.YB[g] = yB;
+          const double Y[3] = {D.YE[g] + R2[0], D.YM[g] + R2[1], D.YB[g] + R2[2]};
+          D.YE[g] = Y[0];
+          D.YM[g] = Y[1];
+          D.YB[g] = Y[2];
           const double inv = swale::recip(D.J2[g]);
-          D.Eb[g] = yE * inv;
-          D.Mb[g] = yM * inv;
-          D.Bb[g] = yB * inv;
-          if (!PLAIN && K.bot_pieces > 0) {  // bottom of stage 3: projection onto the mesh at t_{n+1/2}
+          D.iJ2[g] = inv;
+          const double edt = 0.125 * dt, hdJ = 0.5 * dJ;
+          D.Eb[g] = swale::rk_advance(q0[0], edt, Y[0], hdJ, inv);
+          D.Mb[g] = swale::rk_advance(q0[1], edt, Y[1], hdJ, inv);
+          if (!BOT) {
+            D.Bb[g] = swale::rk_advance(q0[2], edt, Y[2], hdJ, inv);
+          } else {  // bottom of stage 3: projection onto the mesh at t_{n+1/2}
             const double xl = D.x[nb + j], xr = D.x[nb + j + 1];
             D.Bb[g] = bottom_average(K, xl + 0.5 * dt * wl, xr + 0.5 * dt * wr);
             D.xn[nb + j] = xl + dt * wl;  // nodes at t_{n+1} for the projection after the step
             if (j == N - 1) D.xn[nb + N] = xr + dt * wr;
           }
         } else {
-          const double J3 = (1.0 / 3.0) * J0 + (2.0 / 3.0) * D.J2[g] + (2.0 / 3.0) * dt * dw;
-          if (!swale::gt0(J3)) st |= swale::ST_EMESH;
-          const double E0v = D.E0[g], M0v = D.M0[g], B0v = D.B0[g];
+          const double J3 = D.J1[g], inv = D.iJ1[g];  // J^{n+1} = J^(1)
           if (D.bE) {  // q^n, J^n, x^n kept for a roll-back by k_commit
-            D.bE[g] = E0v;
-            D.bM[g] = M0v;
-            D.bB[g] = B0v;
+            D.bE[g] = q0[0];
+            D.bM[g] = q0[1];
+            D.bB[g] = q0[2];
             D.bJ[g] = J0;
             D.bx[nb + j] = D.x[nb + j];
             if (j == N - 1) D.bx[nb + N] = D.x[nb + N];
           }
-          const double yE = (1.0 / 3.0) * (J0 * E0v) + (2.0 / 3.0) * (D.YE[g] + dt * RE);
-          const double yM = (1.0 / 3.0) * (J0 * M0v) + (2.0 / 3.0) * (D.YM[g] + dt * RM);
-          const double yB = (1.0 / 3.0) * (J0 * B0v) + (2.0 / 3.0) * (D.YB[g] + dt * RB);
-          const double inv = swale::recip(J3);
-          const double En = yE * inv, Mn = yM * inv, Bn = yB * inv;
-          D.E0[g] = En;
-          D.M0[g] = Mn;
-          D.B0[g] = Bn;
-          D.J0[g] = J3;
-          jmaxb = J3;
-          jminb = J3;
-          if (!PLAIN && K.bot_pieces > 0) {  // bottom after the step: projection onto the mesh at t_{n+1}
+          const double tdt = dt * (1.0 / 12.0);
+          const double En = swale::rk_advance(q0[0], tdt, 4.0 * R2[0] + D.YE[g], dJ, inv);
+          const double Mn = swale::rk_advance(q0[1], tdt, 4.0 * R2[1] + D.YM[g], dJ, inv);
+          double Bn = swale::rk_advance(q0[2], tdt, 4.0 * R2[2] + D.YB[g], dJ, inv);
+          if (BOT) {  // bottom after the step: projection onto the mesh at t_{n+1}
             const double xl = D.xn[nb + j], xr = D.xn[nb + j + 1];
-            D.B0[g] = bottom_average(K, xl, xr);
+            if (swale::bad(Bn)) st |= swale::ST_NONFINITE;
+            Bn = bottom_average(K, xl, xr);
             D.x[nb + j] = xl;
             if (j == N - 1) D.x[nb + N] = xr;
           } else {
             D.x[nb + j] += dt * wl;
             if (j == N - 1) D.x[nb + N] += dt * wr;
           }
-          if (swale::bad(En) || swale::bad(Mn) || swale::bad(Bn)) st |= swale::ST_NONFINITE;
+          D.E0[g] = En;
+          D.M0[g] = Mn;
+          D.B0[g] = Bn;
+          D.J0[g] = J3;
+          if (swale::bad(En) || swale::bad(Mn) || (!BOT && swale::bad(Bn))) st |= swale::ST_NONFINITE;
         }
       }
     }
@@ -1111,8 +1131,6 @@ __global__ void __launch_bounds__(T, PLAIN ? 1024 / T : 1) k_update(StepConst K,
       if (STAGE == 1) {
         block_max_to(&S->Jmax[1], jmaxa);
         block_max_to(&S->Jmax[2], jmaxb);
-      } else if (STAGE == 3) {
-        block_max_to(&S->JmaxN, jmaxb);
         block_min_to(&S->JminN, jminb);
       }
     }
@@ -1148,6 +1166,7 @@ __global__ void k_commit(StepConst K, DevState D) {
       if (!before && !bad3) {
         S->t = S->clipped ? K.t_end : S->t + S->dt;
         S->steps += 1;
+        S->JmaxN = S->Jmax[1];  // J^{n+1} = J^(1)
       } else {  // the widths stay those of J^n
         S->JmaxN = S->Jmax[0];
         S->JminN = S->Jmin0;

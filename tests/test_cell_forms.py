@@ -1,0 +1,280 @@
+"""Host checks of the per-cell forms that the stage kernels evaluate (a g++ build of
+swale_cell.cuh): the smooth class's edge and point values from divided differences, the fluxes at
+twice their value, the factored source with the edge pressures, the RK increment, and the FP32 and
+integer pre-tests, each against the plain form or the property it has to imply.
+
+Tolerances: rounding of a few dozen operations on data of order one, 1e-12 of the data's scale times
+the largest factor that the mesh brings in.
+"""
+import ctypes
+import os
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+G = 9.812
+
+SRC = r"""
+#include "swale_cell.cuh"
+using namespace swale;
+extern "C" {
+// dd[v]: D2[4], D3[3] of v on the widths h; out: left, right, two interior points, then the linear form's edges.
+void t_edges(const double* h, const double* v, double t1, double t2, double* out) {
+  double ip[4], it[3], iq[2], d2[4], d3[3], d4[2];
+  for (int a = 0; a < 4; ++a) { ip[a] = 1.0 / (h[a] + h[a + 1]); d2[a] = (v[a + 1] - v[a]) * ip[a]; }
+  for (int a = 0; a < 3; ++a) { it[a] = 1.0 / (h[a] + h[a + 1] + h[a + 2]); d3[a] = (d2[a + 1] - d2[a]) * it[a]; }
+  for (int a = 0; a < 2; ++a) { iq[a] = 1.0 / (h[a] + h[a + 1] + h[a + 2] + h[a + 3]); d4[a] = (d3[a + 1] - d3[a]) * iq[a]; }
+  const double d5 = (d4[1] - d4[0]) / (h[0] + h[1] + h[2] + h[3] + h[4]);
+  const SmoothWidths w = {h[1], h[2], h[3], h[0] + h[1], h[1] + h[2], h[2] + h[3], h[3] + h[4]};
+  out[0] = smooth_left(w, v[2], d2[1], d3[1], d4[0], d5);
+  out[1] = smooth_right(w, v[2], d2[2], d3[1], d4[1], d5);
+  out[2] = smooth_point(w, h[4], t1, v[2], d2[2], d3[1], d4[1], d5);
+  out[3] = smooth_point(w, h[4], t2, v[2], d2[2], d3[1], d4[1], d5);
+  CellGeom Gm; uint32_t st = 0;
+  cell_geom(h, h[2], Gm, st, false);
+  smooth_edge_coeffs(h, it, Gm);
+  for (int e = 0; e < 2; ++e)
+    out[4 + e] = v[2] + Gm.K[e][0] * d2[0] + Gm.K[e][1] * d2[1] + Gm.K[e][2] * d2[2] + Gm.K[e][3] * d2[3];
+}
+int t_eweight(const double* h) { CellGeom Gm; uint32_t st = 0; cell_geom(h, h[2], Gm, st, false); return (int)st; }
+int t_moderate(const double* h) {
+  return moderate_widths(f32_trunc(h[0]), f32_trunc(h[1]), f32_trunc(h[2]), f32_trunc(h[3]), f32_trunc(h[4]));
+}
+void t_flux(int scheme, double g, double al, double w, const double* e, double* two, double* one) {
+  Flux2 f = scheme == 0 ? interface_flux2<0>(g, al, w, e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7])
+            : scheme == 1 ? interface_flux2<1>(g, al, w, e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7])
+                          : interface_flux2<2>(g, al, w, e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7]);
+  Flux p = scheme == 0 ? interface_flux(g, al, w, e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7])
+                       : interface_flux_plain(g, al, w, e[0], e[1], e[2], e[3], e[4], e[5], e[6], e[7]);
+  const double pl = scheme == 2 ? 0.0 : g * e[4] * e[4], pr = scheme == 2 ? 0.0 : g * e[5] * e[5];
+  two[0] = f.FE; two[1] = f.FMl + pl; two[2] = f.FMr + pr; two[3] = f.FB;
+  one[0] = p.FE; one[1] = p.FMm; one[2] = p.FMp; one[3] = p.FB;
+}
+// J[3] widths; eta[5], hd[5] in the data order (j-1, j, j+1, L, R). out: the factored form, the antisymmetric one + pressures
+void t_source(const double* J, const double* eta, const double* hd, double* out) {
+  const PairRatio l = pair_ratio(J[0], J[1], 1.0 / (J[0] + J[1])), r = pair_ratio(J[1], J[2], 1.0 / (J[1] + J[2]));
+  const double itc = 1.0 / (J[0] + J[1] + J[2]);
+  const SourceRatio s = source_ratio(J[0], J[1], J[2], 1.0 / J[0], 1.0 / J[2], itc);
+  out[0] = source_pressure_form(hd[1], hd[3], hd[4], eta[3] - eta[1], eta[4] - eta[1], eta[1] - eta[0], hd[1] - hd[0],
+                                eta[2] - eta[1], hd[2] - hd[1], l.rho, l.sig2, r.sig, r.rho2, s);
+  const SourceForm f = source_form(J[0], J[1], J[2], 1.0 / J[0], 1.0 / J[1], 1.0 / J[2], 1.0 / (J[0] + J[1]),
+                                   1.0 / (J[1] + J[2]), itc);
+  double bd[5];
+  for (int k = 0; k < 5; ++k) bd[k] = eta[k] - hd[k];
+  out[1] = 2.0 * source_cell_form(-1.0, hd, bd, f) + (hd[4] * hd[4] - hd[3] * hd[3]);
+}
+double t_rk(double q, double a, double R, double dJ, double J) { return rk_advance(q, a, R, dJ, 1.0 / (J + dJ)); }
+// 1: the pre-test says the limiter is inactive; bit 1: it is active
+int t_limit(double eps, double hbar, double hL, double hR) {
+  SchemeConst P{9.812, 1e-6, eps, 1e-6, 1, 0};
+  const double delta = (12.0 * hbar - hL - hR) * 0.1, mn = dmin(dmin(hL, hR), delta), ev = dmin(eps, hbar);
+  return (surely_unlimited(P, hbar, hL, hR) ? 1 : 0) | (dlt(mn, ev) ? 2 : 0);
+}
+// 1: surely smooth in FP32; bit 1: the FP64 class is not 0
+int t_nonwb(const double* h, const double* eta, const double* hu, const double* hh, double dx, double hdry) {
+  SchemeConst P{9.812, 1e-6, 1e-11, hdry, 1, 0};
+  double v0[3][3]; StencilDD DD; const double* V[3] = {eta, hu, hh};
+  float d2f[3][4], itf[3], hf[5], F[3], c4, c3;
+  for (int k = 0; k < 5; ++k) hf[k] = f32_trunc(h[k]);
+  for (int a = 0; a < 3; ++a) itf[a] = f32_trunc(1.0 / (h[a] + h[a + 1] + h[a + 2]));
+  for (int v = 0; v < 3; ++v) {
+    for (int a = 0; a < 3; ++a) v0[v][a] = V[v][a];
+    for (int a = 0; a < 4; ++a) { DD.D2[v][a] = (V[v][a + 1] - V[v][a]) / (h[a] + h[a + 1]); d2f[v][a] = f32_trunc(DD.D2[v][a]); }
+    for (int a = 0; a < 3; ++a) DD.D3[v][a] = (DD.D2[v][a + 1] - DD.D2[v][a]) / (h[a] + h[a + 1] + h[a + 2]);
+  }
+  indicator_factors_f32(hf, f32_trunc(dx), F, c4, c3);
+  const bool s = sure_smooth_nonwb_f32(P.g, P.h_dry, hh[2], hu[2], F, c4, c3, d2f[0], d2f[1], d2f[2], itf, 1e-6f);
+  CellGeom Gm; uint32_t st = 0; cell_geom(h, dx, Gm, st);
+  EdgeState o; uint8_t flag;
+  recon_cell_nonwb_g(P, Gm, v0, DD, o, flag, st, nonwb_proj(P, v0));
+  return (s ? 1 : 0) | (flag ? 2 : 0);
+}
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("forms")
+    src, out = d / "forms.cpp", d / "forms.so"
+    src.write_text(SRC)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-fPIC", "-shared", "-I",
+                    os.path.join(ROOT, "paper_2208_06588_gb300", "csrc"), "-o", str(out), str(src)], check=True)
+    L = ctypes.CDLL(str(out))
+    for n, r in (("t_eweight", ctypes.c_int), ("t_moderate", ctypes.c_int), ("t_rk", ctypes.c_double),
+                 ("t_limit", ctypes.c_int), ("t_nonwb", ctypes.c_int)):
+        getattr(L, n).restype = r
+    return L
+
+
+def _p(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def _d(x):
+    return ctypes.c_double(float(x))
+
+
+@pytest.mark.parametrize("spread", [0.0, 0.5, 3.0])
+def test_smooth_values_are_the_big_stencils_polynomial(lib, spread):
+    """Equal to the linear form of the weights, exact for random quartics' averages, exact (bit for
+    bit) for constants."""
+    rng = np.random.default_rng(3)
+    for _ in range(300):
+        h = np.exp(rng.uniform(-spread, spread, 5))
+        y = np.concatenate([[0.0], np.cumsum(h)]) - h[0] - h[1]
+        y /= h[2]
+        c = rng.uniform(-1, 1, 5)
+        P = np.polynomial.Polynomial(c)
+        I = P.integ()
+        v = np.array([(I(y[k + 1]) - I(y[k])) / (y[k + 1] - y[k]) for k in range(5)])
+        out = np.zeros(6)
+        t = rng.uniform(0.01, 0.99, 2)
+        lib.t_edges(_p(h), _p(v), _d(t[0]), _d(t[1]), _p(out))
+        scale = np.abs(v).max() * (1.0 + np.exp(2.0 * spread))
+        assert abs(out[0] - P(0.0)) <= 1e-12 * scale and abs(out[1] - P(1.0)) <= 1e-12 * scale
+        assert abs(out[2] - P(t[0])) <= 1e-12 * scale and abs(out[3] - P(t[1])) <= 1e-12 * scale
+        assert np.abs(out[:2] - out[4:]).max() <= 1e-12 * scale
+        k = np.full(5, v[0])
+        lib.t_edges(_p(h), _p(k), _d(t[0]), _d(t[1]), _p(out))
+        assert np.all(out[:4] == v[0])
+
+
+def test_moderate_widths_never_hide_a_weight(lib):
+    """Where the FP32 test calls the widths moderate, cell_geom raises no status; extreme, zero,
+    negative and non-finite widths are not called moderate."""
+    rng = np.random.default_rng(4)
+    for _ in range(4000):
+        h = np.exp(rng.uniform(-8.0, 8.0, 5)) * 10.0 ** rng.uniform(-12, 6)
+        if lib.t_moderate(_p(h)):
+            assert lib.t_eweight(_p(h)) == 0
+    for bad in (0.0, -1.0, np.nan, np.inf, 1e-40, 1e12):
+        for k in range(5):
+            h = np.ones(5)
+            h[k] = bad
+            assert not lib.t_moderate(_p(h))
+
+
+@pytest.mark.parametrize("scheme", [0, 1, 2])
+def test_flux_at_twice_its_value(lib, scheme):
+    rng = np.random.default_rng(5)
+    for _ in range(300):
+        h = rng.uniform(0.0, 3.0, 2) * (rng.uniform(size=2) > 0.1)
+        E = rng.uniform(-1.0, 3.0, 2)
+        e = np.array([E[0], E[1], E[0] - h[0], E[1] - h[1], h[0], h[1], *rng.uniform(-4, 4, 2)])
+        two, one = np.zeros(4), np.zeros(4)
+        lib.t_flux(scheme, _d(G), _d(9.0), _d(rng.uniform(-2, 2)), _p(e), _p(two), _p(one))
+        assert np.abs(two - 2.0 * one).max() <= 1e-12 * 400.0
+        # at rest with equal surfaces the two sides' momentum terms vanish exactly, whatever the bottom
+    e = np.array([2.0, 2.0, 0.3, 0.7, 1.7, 1.3, 0.0, 0.0])
+    lib.t_flux(scheme, _d(G), _d(9.0), _d(0.4), _p(e), _p(two), _p(one))
+    if scheme == 0:
+        assert two[1] == G * 1.7 * 1.7 and two[2] == G * 1.3 * 1.3
+
+
+def _exact_source(J, eta, hd):
+    """2 h^T K b + h_R^2 - h_L^2 in rationals, the quartics by their Newton form."""
+    J = [Fraction(float(x)) for x in J]
+    rm, rp = J[0] / J[1], J[2] / J[1]
+
+    def poly(u):  # coefficients of v(t), t in the unit cell; u in the data order
+        u = [Fraction(float(x)) for x in u]
+        o = [None, None]
+        o2a, o2b, o2c, o2d = (u[3] - u[0]) / rm, u[1] - u[3], u[4] - u[1], (u[2] - u[4]) / rp
+        o3a, o3b, o3c = (o2b - o2a) / (1 + rm), o2c - o2b, (o2d - o2c) / (1 + rp)
+        o4a, o4b = (o3b - o3a) / (1 + rm), (o3c - o3b) / (1 + rp)
+        cb = [u[0], o2a, o3a, o4a, (o4b - o4a) / (1 + rm + rp)]
+        m = [[1], [0, 1], [0, 0, 1], [0, 0, -1, 1], [0, 0, 1, -2, 1]]
+        prim = [Fraction(0)] * 6
+        for ck, mk in zip(cb, m):
+            for d, a in enumerate(mk):  # ck (t + rm) a t^d
+                prim[d + 1] += ck * a
+                prim[d] += ck * a * rm
+        return [(d + 1) * prim[d + 1] for d in range(5)]
+
+    eta = [Fraction(float(x)) for x in eta]
+    hd = [Fraction(float(x)) for x in hd]
+    h, b = poly(hd), poly([x - y for x, y in zip(eta, hd)])
+    db = [(d + 1) * b[d + 1] for d in range(4)]
+    s = sum(h[i] * db[k] / (i + k + 1) for i in range(5) for k in range(4))
+    return 2 * s + hd[4] ** 2 - hd[3] ** 2
+
+
+@pytest.mark.parametrize("spread", [0.0, 0.4, 2.0])
+def test_source_with_pressures_is_the_exact_integral(lib, spread):
+    rng = np.random.default_rng(6)
+    for _ in range(100):
+        J = np.exp(rng.uniform(-spread, spread, 3))
+        eta, hd = rng.uniform(1.0, 2.0, 5), rng.uniform(0.0, 1.0, 5)
+        out = np.zeros(2)
+        lib.t_source(_p(J), _p(eta), _p(hd), _p(out))
+        ref = float(_exact_source(J, eta, hd))
+        scale = 4.0 * (1.0 + np.exp(4.0 * spread))
+        assert abs(out[0] - ref) <= 1e-13 * scale and abs(out[1] - ref) <= 1e-13 * scale
+        eta[:] = 1.3  # at rest: zero, exactly, whatever the bottom
+        lib.t_source(_p(J), _p(eta), _p(hd), _p(out))
+        assert out[0] == 0.0
+
+
+def test_rk_increment(lib):
+    rng = np.random.default_rng(7)
+    for _ in range(200):
+        q, a, R, J = rng.uniform(-2, 2), rng.uniform(0, 0.1), rng.uniform(-3, 3), rng.uniform(0.1, 1.0)
+        dJ = rng.uniform(-0.05, 0.05)
+        got = lib.t_rk(_d(q), _d(a), _d(R), _d(dJ), _d(J))
+        assert abs(got - (J * q + a * R) / (J + dJ)) <= 1e-14 * (abs(q) + 10.0)
+
+
+@pytest.mark.parametrize("eps", [0.0, 1e-11, 1e-3])
+def test_limiter_pretest_never_skips_an_active_limiter(lib, eps):
+    rng = np.random.default_rng(8)
+    told = 0
+    for _ in range(6000):
+        hbar = 10.0 ** rng.uniform(-14, 3) if rng.uniform() > 0.05 else rng.choice([0.0, eps])
+        s = rng.choice([1e-9, 1e-3, 1.0, 8.0])
+        hL, hR = hbar * (1.0 + s * rng.uniform(-1, 1, 2))
+        if rng.uniform() < 0.2:  # the Gauss-Lobatto mean right at its floor
+            hR = 12.0 * hbar - hL - 10.0 * eps * (1.0 + 1e-7 * rng.uniform(-1, 1))
+        r = lib.t_limit(_d(eps), _d(hbar), _d(hL), _d(hR))
+        assert r != 3, (eps, hbar, hL, hR)
+        told += r == 1
+    assert told > 1000
+    for bad in (np.nan, np.inf, -np.inf):
+        assert lib.t_limit(_d(eps), _d(1.0), _d(bad), _d(1.0)) != 3
+
+
+def test_nonwb_fp32_test_implies_the_smooth_class(lib):
+    """Random cells over many scales and near-threshold ones found by bisection: the FP32 test never
+    claims the smooth class where one of the three FP64 fields is not smooth."""
+    rng = np.random.default_rng(9)
+    told = smooth = 0
+
+    def ask(h, e, m, hh, dx, hdry=1e-6):
+        return lib.t_nonwb(_p(h), _p(e), _p(m), _p(hh), _d(dx), _d(hdry))
+
+    for i in range(6000):
+        sc = 10.0 ** rng.uniform(-4, 0)
+        h = sc * np.exp(rng.uniform(-0.7, 0.7, 5))
+        amp = 10.0 ** rng.uniform(-9, 0.5)
+        hh = np.abs(rng.choice([1.0, 1e-3, 1e-7]) + amp * rng.uniform(-1, 1, 5))
+        e = hh + amp * rng.uniform(-1, 1, 5) + rng.uniform(-1, 1)
+        m = rng.choice([0.0, 1.0, 3.1]) * hh + amp * rng.uniform(-1, 1, 5)
+        r = ask(h, e, m, hh, h.max())
+        assert r != 3
+        told += r == 1
+        smooth += r in (0, 1)
+        if i % 6 == 0 and r == 2:  # shrink the variation until the class turns smooth; test around it
+            lo, hi = 0.0, 1.0
+            f = lambda s: (h, e.mean() + s * (e - e.mean()), m.mean() + s * (m - m.mean()), hh.mean() + s * (hh - hh.mean()), h.max())  # noqa: E731,E501
+            for _ in range(50):
+                mid = 0.5 * (lo + hi)
+                if ask(*f(mid)) & 2:
+                    hi = mid
+                else:
+                    lo = mid
+            for s in (lo, hi, hi * (1 + 1e-12), hi * (1 + 1e-9), hi * (1 + 1e-6)):
+                assert ask(*f(s)) != 3
+    assert told > 1000 and told > 0.8 * smooth

@@ -124,6 +124,7 @@ StepConst step_const(const swale_ctx* ctx) {
   K.t_end = ctx->cfg.t_end;
   K.dt_fixed = ctx->cfg.dt_fixed;
   K.mesh_T = ctx->cfg.mesh_T;
+  K.inv_T = 1.0 / ctx->cfg.mesh_T;
   K.gauss_wsum = ctx->gauss_wsum;
   K.gauss_iwsum = 1.0 / ctx->gauss_wsum;
   K.bc = ctx->cfg.bc;
@@ -332,6 +333,7 @@ swale_status build_tiles(swale_ctx* ctx, std::vector<InstConst>& ic) {
     ctx->D.nf = (int32_t)ft.size();
     ctx->D.nrf = (int32_t)rf.size();
   }
+  ctx->D.ic1 = ic[0];
   SW_CUDA(ctx, cudaMemcpyAsync(ctx->D.IC, ic.data(), B * sizeof(InstConst), cudaMemcpyHostToDevice, ctx->stream));
   SW_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   return SWALE_OK;
@@ -1925,6 +1927,9 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   D.nu = (int32_t)((N + kNoAllocTile - 1) / kNoAllocTile);
   D.nf = (int32_t)((N + kNoAllocTile - 2) / (kNoAllocTile - 1));
   D.nrf = (int32_t)((N + 2 + kNoAllocTile - 5) / (kNoAllocTile - 4));
+  D.ic1.N = N;
+  D.ic1.cfl = 1.0;
+  D.ic1.ntiles_r = D.nrf;
   StepConst K;
   K.sc.g = cfg->g;
   K.sc.eps_weno = cfg->eps_weno;
@@ -1934,7 +1939,7 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   K.sc.limit_hu = cfg->limit_hu;
   K.t_end = 0.0;
   K.dt_fixed = 0.0;
-  K.mesh_T = 1.0;
+  K.mesh_T = K.inv_T = 1.0;
   K.gauss_wsum = 1.0;
   K.gauss_iwsum = 1.0;
   K.bc = cfg->bc;

@@ -94,6 +94,9 @@ SWALE_HD bool dlt(double a, double b) { return okey(a) < okey(b); }
 SWALE_HD double pos0(double a) { return __double_as_longlong(a) < 0 ? 0.0 : a; }
 // a > 0.
 SWALE_HD bool gt0(double a) { return __double_as_longlong(a) > 0; }
+// a < t and t < a for a bound t >= +0: the bit patterns compared as signed integers.
+SWALE_HD bool lt_pos(double a, double t) { return __double_as_longlong(a) < __double_as_longlong(t); }
+SWALE_HD bool gt_pos(double a, double t) { return __double_as_longlong(t) < __double_as_longlong(a); }
 // a <= b for a, b >= +0.
 SWALE_HD bool le_nn(double a, double b) {
   return (unsigned long long)__double_as_longlong(a) <= (unsigned long long)__double_as_longlong(b);
@@ -110,20 +113,45 @@ SWALE_HD double recip(double x) {
   return fma(fma(e, e, e), y, y);
 }
 SWALE_HD double dsqrt(double a) { return sqrt(a); }
+// Square root of a >= 0 for the wave speeds: the hardware's 20-bit reciprocal square root y refined
+// by one third-order step, a y (1 + e/2 + 3 e^2 / 8) with e = 1 - a y^2 (the binomial series of
+// (1 - e)^(-1/2)): 5 FP64 operations, within about one unit in the last place. Zero, subnormal and
+// huge arguments take sqrt().
+SWALE_HD double wave_sqrt(double a) {
+  if (!(a > 1e-300 && a < 1e300)) return sqrt(a);
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double r = a * y, e = fma(-r, y, 1.0);
+  return fma(r * e, fma(0.375, e, 0.5), r);
+}
+// NaN, infinite or of magnitude above 1e300, any of six (the high words first).
+SWALE_HD bool bad6(double a, double b, double c, double d, double e, double f) {
+  const int m = 0x7fffffff;
+  const int h = max(max(max(__double2hiint(a) & m, __double2hiint(b) & m), max(__double2hiint(c) & m, __double2hiint(d) & m)),
+                    max(__double2hiint(e) & m, __double2hiint(f) & m));
+  return h >= 0x7e37e43c && (bad(a) || bad(b) || bad(c) || bad(d) || bad(e) || bad(f));
+}
 #else
 SWALE_HD real dmax(real a, real b) { return (b > a) ? b : a; }
 SWALE_HD real dmin(real a, real b) { return (b < a) ? b : a; }
 SWALE_HD bool dlt(real a, real b) { return a < b; }
 SWALE_HD real pos0(real a) { return (real(0.0) > a) ? real(0.0) : a; }
 SWALE_HD bool gt0(real a) { return a > 0.0; }
+SWALE_HD bool lt_pos(real a, real t) { return a < t; }
+SWALE_HD bool gt_pos(real a, real t) { return t < a; }
 SWALE_HD bool le_nn(real a, real b) { return a <= b; }
 SWALE_HD real dabs(real a) { return a < 0.0 ? -a : a; }
 SWALE_HD bool bad(real a) { return !(a == a) || dabs(a) > 1.0e300; }
 SWALE_HD real recip(real x) { return 1.0 / x; }
+SWALE_HD bool bad6(real a, real b, real c, real d, real e, real f) {
+  return bad(a) || bad(b) || bad(c) || bad(d) || bad(e) || bad(f);
+}
 #ifdef SWALE_REAL
 SWALE_HD real dsqrt(real a) { return swale_sqrt(a); }
+SWALE_HD real wave_sqrt(real a) { return swale_sqrt(a); }
 #else
 SWALE_HD real dsqrt(real a) { return sqrt(a); }
+SWALE_HD real wave_sqrt(real a) { return sqrt(a); }
 #endif
 #endif
 
@@ -195,12 +223,19 @@ SWALE_HD bool sure_smooth_f32(const float F[3], float c4, float c3, const float 
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     const int a = 2 - r;
-    const float d3h = (d2h[a + 1] - d2h[a]) * it[a], d3m = (d2m[a + 1] - d2m[a]) * it[a];
     const float Mh = (fabsf(d2h[a + 1]) + fabsf(d2h[a])) * it[a], Mm = (fabsf(d2m[a + 1]) + fabsf(d2m[a])) * it[a];
-    const float qh = fmaf(d3h, F[a], d2h[a]), qm = fmaf(d3m, F[a], d2m[a]);
     const float Qh = fmaf(Mh, fabsf(F[a]), fabsf(d2h[a])), Qm = fmaf(Mm, fabsf(F[a]), fabsf(d2m[a]));
-    b[r] = fmaf(c4, fmaf(qh, qh, qm * qm), c3 * fmaf(d3h, d3h, d3m * d3m));
     msum += fmaf(c4, fmaf(Qh, Qh, Qm * Qm), c3 * fmaf(Mh, Mh, Mm * Mm));
+  }
+  // tau <= max(beta) <= the magnitudes' sum, den >= eps: below 0.4 eps nothing else is needed (most
+  // cells of a fine mesh).
+  if (msum <= 0.4f * eps) return true;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int a = 2 - r;
+    const float d3h = (d2h[a + 1] - d2h[a]) * it[a], d3m = (d2m[a + 1] - d2m[a]) * it[a];
+    const float qh = fmaf(d3h, F[a], d2h[a]), qm = fmaf(d3m, F[a], d2m[a]);
+    b[r] = fmaf(c4, fmaf(qh, qh, qm * qm), c3 * fmaf(d3h, d3h, d3m * d3m));
   }
   constexpr float u = 5.9604645e-8f;  // 2^-24
   const float tau = fabsf(b[0] - b[2]);
@@ -275,7 +310,7 @@ SWALE_HD bool sure_smooth_nonwb_f32(double g, double h_dry, double hb, double mb
 }
 
 // Wave speed |u| + sqrt(g max(h, 0)) of one limited edge state (Eq. alpha2D).
-SWALE_HD real wave_speed(real g, real h, real u) { return dabs(u) + dsqrt(g * pos0(h)); }
+SWALE_HD real wave_speed(real g, real h, real u) { return dabs(u) + wave_sqrt(g * pos0(h)); }
 
 // ------------------------------------------------------------------------------------
 // Shared per-pair and per-triple terms (Step 1): reciprocal widths and divided differences.
@@ -309,11 +344,6 @@ struct CellGeom {
   // hydrostatic scheme only).
   real K[2][4];
 };
-#define SWALE_GEOM_BASE 25    // doubles of a CellGeom before K (what every scheme uses)
-#define SWALE_GEOM_VALUES 33  // doubles in a CellGeom
-// cached per cell: a CellGeom and the source's six mesh-only values (a SourceForm; a SourceGeom
-// for the special scheme)
-#define SWALE_GEO_ARRAYS (SWALE_GEOM_VALUES + 6)
 // Indicator factors of Step 2 (F, c4, c3 of CellGeom) for the widths h[5] and the length dx.
 SWALE_HD void indicator_factors(const real h[5], real dx, CellGeom& G) {
   const real h1 = h[1], h2 = h[2], h3 = h[3];
@@ -458,7 +488,7 @@ SWALE_HD bool surely_unlimited(const SchemeConst& P, real hbar, real hL, real hR
 #if defined(SWALE_REAL)
   return false;
 #else
-  if (dlt(hL, P.eps_pp) || dlt(hR, P.eps_pp)) return false;
+  if (lt_pos(hL, P.eps_pp) || lt_pos(hR, P.eps_pp)) return false;
   const float b = f32_trunc(hbar), l = f32_trunc(hL), r = f32_trunc(hR), e = f32_trunc(P.eps_pp);
   const float m = 12.0f * b + (l + r);
   return 12.0f * b - (l + r) > fmaf(20.0f, e, 2e-6f * m) + 1e-36f && m < 1e30f;
@@ -496,13 +526,13 @@ SWALE_HD void limit_cell(const SchemeConst& P, const real ev[3][2], real hbar0, 
   o.BL = ev[0][0] - hL;
   o.BR = ev[0][1] - hR;
   // Velocities with one division: u_L = m_L h_R' / (h_L' h_R'), dry edges (h <= h_dry) -> 0.
-  const bool wetL = dlt(P.h_dry, hL), wetR = dlt(P.h_dry, hR);
+  const bool wetL = gt_pos(hL, P.h_dry), wetR = gt_pos(hR, P.h_dry);
   const real hLs = wetL ? hL : real(1.0), hRs = wetR ? hR : real(1.0);
   const real ihh = recip(hLs * hRs);
   o.uL = wetL ? mL * hRs * ihh : real(0.0);
   o.uR = wetR ? mR * hLs * ihh : real(0.0);
   // NaN propagates into the comparisons as false: catch it explicitly.
-  if (bad(o.EL) || bad(o.ER) || bad(hL) || bad(hR) || bad(mL) || bad(mR)) st |= ST_NONFINITE;
+  if (bad6(o.EL, o.ER, hL, hR, mL, mR)) st |= ST_NONFINITE;
 }
 
 // Reconstruction of cell j (Steps 1-4 of Sec. 2.2 with the shared indicators of
@@ -589,14 +619,14 @@ SWALE_HD real smooth_point(const SmoothWidths& w, real h4, real t, real v, real 
   const real e5 = e4 * a5 + n4;
   return v + (d2r * e2 + (d3 * e3 + (d4r * e4 + d5 * e5)));
 }
-// Whether the five widths are positive, normal floats within a factor of 2^20 of each other (h32:
-// truncated to FP32). Then both middle linear weights d_1 are positive beyond any rounding: with
+// Whether the five widths (truncated to FP32) are above 1e-9, so that the FP32 indicator factors (up
+// to the fourth power of a width) are normal numbers, and within a factor of 2^20 of each other. Then both middle linear weights d_1 are positive beyond any rounding: with
 // A = y3 - y0 >= B = y3 - y1, E = y5 - y3 >= D = y4 - y3, d_1 = 1 - DE / ((A+D)(A+E)) - AB / ((B+E)(A+E))
 // is at least about 2^-22 there, so the ST_EWEIGHT check of cell_geom needs no weights. Other cells
 // take the path that forms them.
 SWALE_HD bool moderate_widths(float a, float b, float c, float d, float e) {
   const float mn = fminf(fminf(fminf(a, b), fminf(c, d)), e), mx = fmaxf(fmaxf(fmaxf(a, b), fmaxf(c, d)), e);
-  return mn > 1e-30f && mx < 1e30f && mx < 1048576.0f * mn;
+  return mn > 1e-9f && mx < 1e30f && mx < 1048576.0f * mn;
 }
 
 // Reconstruction of cell j for the non-well-balanced scheme (Eq. se2D / s2D; Sec. 2.2, last

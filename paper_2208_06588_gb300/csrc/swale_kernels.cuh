@@ -38,10 +38,10 @@ using swale::SchemeConst;
 
 constexpr int kMaxGaussHalf = 64;
 // Resident threads per SM that the launch bounds of the stage kernels ask for.
-constexpr int kReconThreads = 768, kUpdateThreads = 1024;
+constexpr int kReconThreads = 896, kUpdateThreads = 896;
 constexpr int kMeshThreads = 256;
 constexpr int kMeshNodes = kMeshThreads - 1;  // nodes a mesh-velocity tile advances by
-constexpr double kTwoPi = 6.283185307179586476925286766559;
+constexpr double kTwoPi = 6.283185307179586476925286766559;  // (the host's bound on the node speeds)
 
 // Per-instance device scalars. Maxima of non-negative doubles are kept as their bit patterns
 // (unsigned order equals numeric order for non-negative IEEE doubles).
@@ -83,7 +83,7 @@ struct Tile {
 // Constants of the whole launch.
 struct StepConst {
   SchemeConst sc;
-  double t_end, dt_fixed, mesh_T;
+  double t_end, dt_fixed, mesh_T, inv_T;
   double gauss_wsum;  // sum of the full Gaussian window, summed from -H to H
   double gauss_iwsum; // its reciprocal
   int32_t bc, mesh, gauss_half, B;
@@ -168,6 +168,7 @@ struct DevState {
   // serve the adjoint's kernels).
   const Tile* rftiles;
   int32_t nrf;
+  InstConst ic1;  // the constants of a single instance (the stage kernels need no load for them)
 };
 
 __constant__ double c_gauss_w[2 * kMaxGaussHalf + 1];
@@ -187,14 +188,13 @@ __device__ __forceinline__ const double* node_velocities(const StepConst& K, con
   return K.mesh == SWALE_MESH_LINEAR ? D.P : D.w;
 }
 
-__device__ __forceinline__ int64_t ghost(int64_t i, int64_t N, int bc) {
+__device__ __forceinline__ int32_t ghost(int32_t i, int32_t N, int bc) {
+  if (i >= 0 && i < N) return i;
   if (bc == SWALE_BC_PERIODIC) {
     i %= N;
     return i < 0 ? i + N : i;
   }
-  if (i < 0) return -1 - i;
-  if (i >= N) return 2 * N - 1 - i;
-  return i;
+  return i < 0 ? -1 - i : N - 1 - (i - N);
 }
 
 // L2 projection of the bottom onto one cell [a, c] (Eq. baverage): on each piece the cell
@@ -238,11 +238,10 @@ __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned
 
 __device__ __forceinline__ double bitsd(unsigned long long b) { return __longlong_as_double((long long)b); }
 
-// Block-wide max / min of non-negative doubles, one atomicMax / atomicMin per block. The bit
+// Block-wide max of non-negative doubles, one atomicMax per block. The bit
 // patterns of doubles >= +0 order like unsigned integers, so the reductions run on the integer
 // pipe (the FP64 pipe is the bottleneck of the stage kernels). A NaN wins the max.
 __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
-__device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b) { return a < b ? a : b; }
 
 __device__ __forceinline__ void block_max_to(unsigned long long* dst, double v) {
   __shared__ unsigned long long red[32];
@@ -260,72 +259,92 @@ __device__ __forceinline__ void block_max_to(unsigned long long* dst, double v) 
   __syncthreads();
 }
 
-__device__ __forceinline__ void block_min_to(unsigned long long* dst, double v) {
-  __shared__ unsigned long long red[32];
-  unsigned long long b = dbits(v);
-  for (int o = 16; o > 0; o >>= 1) b = umin64(b, __shfl_xor_sync(0xffffffffu, b, o));
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = b;
-  __syncthreads();
-  if (wid == 0) {
-    const int nw = blockDim.x >> 5;
-    b = lane < nw ? red[lane] : dbits(INFINITY);
-    for (int o = 16; o > 0; o >>= 1) b = umin64(b, __shfl_xor_sync(0xffffffffu, b, o));
-    if (lane == 0) atomicMin(dst, b);
-  }
-  __syncthreads();
+// Maximum over a warp of non-negative doubles as bit patterns, by the 32-bit reduction unit: the
+// high words, then the low words of those that hold the largest.
+__device__ __forceinline__ unsigned long long warp_umax64(unsigned long long v) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+__device__ __forceinline__ unsigned long long warp_umin64(unsigned long long v) { return ~warp_umax64(~v); }
+
+// Raises *dst to v unless it is there already (most callers find that it is).
+__device__ __forceinline__ void raise_to(unsigned long long* dst, unsigned long long v) {
+  if (v > *(volatile const unsigned long long*)dst) atomicMax(dst, v);
 }
 
-// Exact maximum of the edge wave speeds (Eq. alpha2D) of a block's cells with few FP64
-// operations: an FP32 estimate of every edge's |u| + sqrt(g h) (relative error below 2^-21)
-// gives the block's FP32 maximum; only edges within 2^-16 of it can hold the exact maximum, and
-// only those are evaluated in FP64 (in a warp, one edge per lane first, then the rare second
-// one). When the FP32 maximum is below 1e-10 every edge is evaluated. Returns this thread's
-// contribution to the exact block maximum (0 for non-candidates).
+// One edge state of the wave speed: depth, velocity and node velocity.
+struct WaveEdge {
+  double h, u, w;
+  __device__ bool same(const WaveEdge& o) const {
+    return dbits(h) == dbits(o.h) && dbits(u) == dbits(o.u) && dbits(w) == dbits(o.w);
+  }
+  __device__ double speed(double g) const { return swale::wave_speed(g, h, u - w); }
+};
+
+// Exact maximum of the edge wave speeds |u - w| + sqrt(g h) (Eq. alpha2D) of a block's cells, raised
+// into *A, with few FP64 operations. FP32 bounds lo <= speed <= hi of every edge (relative error
+// below 2^-20 of each term, 1e-15 for inputs below the FP32 range) rule out every edge whose hi is
+// below the largest lo of the block or below `seen`, a value *A has held; the edges left are
+// evaluated in FP64, once for a warp, or for several, whose edges left are all the same (flat water).
+// On the 2^20-cell dam break, mostly still water, the evaluations cost about 20 of the
+// reconstruction's 105 FP64 instructions per cell when every warp made its own; now about 2.
 template <int T>
-__device__ __forceinline__ double block_wave(double g, bool useL, bool useR, double hL, double uL, double hR,
-                                             double uR) {
-  __shared__ unsigned int wmax[T / 32];
+__device__ __forceinline__ void block_wave(unsigned long long* A, double seen, double g, bool useL, bool useR,
+                                           const WaveEdge& L, const WaveEdge& R) {
+  __shared__ unsigned s_lo[T / 32];
+  __shared__ WaveEdge s_edge[T / 32];
+  __shared__ int s_kind[T / 32];  // 0: no edge left, 1: all left are s_edge, 2: several
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const float gf = swale::f32_trunc(g);
-  const float fl = useL ? fabsf(swale::f32_trunc(uL)) + __fsqrt_rn(gf * fmaxf(swale::f32_trunc(hL), 0.0f)) : 0.0f;
-  const float fr = useR ? fabsf(swale::f32_trunc(uR)) + __fsqrt_rn(gf * fmaxf(swale::f32_trunc(hR), 0.0f)) : 0.0f;
-  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(fl, fr)));
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+  auto bounds = [&](bool use, const WaveEdge& e, float& lo, float& hi) {
+    const float uf = swale::f32_trunc(e.u), wf = swale::f32_trunc(e.w), q = gf * fmaxf(swale::f32_trunc(e.h), 0.0f);
+    float sq;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(sq) : "f"(q));
+    const float v = fabsf(uf - wf) + sq, m = (fabsf(uf) + fabsf(wf)) * 4.8e-7f + 1e-15f;
+    lo = use ? fmaxf(fmaf(v, 1.0f - 4e-6f, -m), 0.0f) : 0.0f;
+    hi = use ? fmaf(v, 1.0f + 4e-6f, m) : -1.0f;
+  };
+  float lol, hil, lor, hir;
+  bounds(useL, L, lol, hil);
+  bounds(useR, R, lor, hir);
+  const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(lol, lor)));
+  if (lane == 0) s_lo[wid] = m;
   __syncthreads();
-  unsigned bm = 0;
+  unsigned bm = __float_as_uint(swale::f32_trunc(seen));
 #pragma unroll
-  for (int w = 0; w < T / 32; ++w) bm = bm > wmax[w] ? bm : wmax[w];
-  const float bmf = __uint_as_float(bm);
-  const float thr = (bmf < 1e-10f) ? 0.0f : bmf * (1.0f - 1.0f / 65536.0f);
-  const bool cl = useL && fl >= thr, cr = useR && fr >= thr;
-  double wave = 0.0;
-  const bool c1 = cl || cr;
-  const unsigned cand = __ballot_sync(0xffffffffu, c1);
+  for (int w = 0; w < T / 32; ++w) bm = bm > s_lo[w] ? bm : s_lo[w];
+  const float thr = __uint_as_float(bm);
+  const bool cl = !(hil < thr), cr = !(hir < thr);  // (a NaN stays)
+  const bool kl = useL && cl, kr = useR && cr;
+  const unsigned cand = __ballot_sync(0xffffffffu, kl || kr);
+  int kind = 0;
+  WaveEdge first{0.0, 0.0, 0.0};
   if (cand) {
-    // Flat water: when every candidate edge of the warp holds the same (h, u) bit for bit, one
-    // evaluation gives the exact maximum of them all.
-    const bool r0 = cr && !cl;
     const int src = __ffs(cand) - 1;
-    const unsigned long long hb = dbits(__shfl_sync(0xffffffffu, r0 ? hR : hL, src));
-    const unsigned long long ub = dbits(__shfl_sync(0xffffffffu, r0 ? uR : uL, src));
-    const bool same = (!cl || (dbits(hL) == hb && dbits(uL) == ub)) && (!cr || (dbits(hR) == hb && dbits(uR) == ub));
-    if (__all_sync(0xffffffffu, same)) {
-      const double w0 = swale::wave_speed(g, bitsd(hb), bitsd(ub));
-      return c1 ? w0 : 0.0;
-    }
+    const bool r0 = !kl;  // the first left edge of this lane is its right one
+    first.h = __shfl_sync(0xffffffffu, r0 ? R.h : L.h, src);
+    first.u = __shfl_sync(0xffffffffu, r0 ? R.u : L.u, src);
+    first.w = __shfl_sync(0xffffffffu, r0 ? R.w : L.w, src);
+    kind = __all_sync(0xffffffffu, (!kl || L.same(first)) && (!kr || R.same(first))) ? 1 : 2;
+    if (lane == 0) s_edge[wid] = first;
   }
-  if (cand) {
-    const bool right = cr && (!cl || fr > fl);
-    const double w1 = swale::wave_speed(g, right ? hR : hL, right ? uR : uL);
-    wave = c1 ? w1 : 0.0;
+  if (lane == 0) s_kind[wid] = kind;
+  __syncthreads();
+  if (kind == 1)
+    for (int w = 0; w < wid; ++w)
+      if (s_kind[w] == 1 && first.same(s_edge[w])) kind = 0;  // another warp evaluates it
+  if (kind == 0) return;
+  unsigned long long v;
+  if (kind == 1) {
+    v = dbits(first.speed(g));
+  } else {
+    v = 0ull;
+    if (kl || kr) v = dbits((kl ? L : R).speed(g));
+    if (kl && kr) v = umax64(v, dbits(R.speed(g)));
+    v = warp_umax64(v);
   }
-  const bool c2 = cl && cr;
-  if (__any_sync(0xffffffffu, c2)) {
-    const bool right = !(fr > fl);  // the edge the first pass did not take
-    const double w2 = swale::wave_speed(g, right ? hR : hL, right ? uR : uL);
-    if (c2 && w2 > wave) wave = w2;
-  }
-  return wave;
+  if (lane == 0) raise_to(A, v);
 }
 
 __device__ __forceinline__ void block_or_status(unsigned int* dst, uint32_t st) {
@@ -540,6 +559,66 @@ __device__ __noinline__ OpenOut recon_open_cell(const SchemeConst P, const TileR
   return r;
 }
 
+// The step's alpha_1, dt and the secant factor of the prescribed motion, by one warp of the
+// instance's last stage-1 tile (every lane computes dt: an FP64 instruction costs the same for one
+// lane as for 32). The secant factor (sin(2 pi (t + dt) / T) - sin(2 pi t / T)) / dt is formed as
+// 2 cos(pi (2 t + dt) / T) sin(pi dt / T) / dt, which does not cancel, with the cosine and the sine in two lanes
+// of the same instructions.
+__device__ __forceinline__ void stage1_dt(const StepConst& K, DevScalars* S, const InstConst& ic, int inst) {
+  __threadfence();
+  const int lane = threadIdx.x & 31;
+  const double A1 = bitsd(*(volatile const unsigned long long*)&S->A[0]);
+  double Wbar = S->Wbar, dwmax = 0.0;
+  if (K.mesh == SWALE_MESH_FLUID_GAUSS) {
+    Wbar = bitsd(*(volatile const unsigned long long*)&S->Wabs);
+    dwmax = bitsd(*(volatile const unsigned long long*)&S->dWabs);
+  }
+  double alpha1 = K.wave_rel ? A1 : A1 + Wbar;
+  if (K.alpha_mode != 0) {
+    if (lane == 0) alpha1 = stage_alpha(K, inst, 1, alpha1, S->step_idx);
+    alpha1 = __shfl_sync(0xffffffffu, alpha1, 0);
+  }
+  const double tn = S->t;
+  double dt;
+  int clipped = 0;
+  bool nodt = false;
+  if (K.dt_fixed > 0.0) {
+    dt = K.dt_fixed;
+  } else {
+    // (zero and subnormal divisors take the division: the quotient is then infinite, or a NaN)
+    const double jmin = bitsd(S->Jmin0);
+    dt = alpha1 > 1e-290 ? ic.cfl * jmin * swale::recip(alpha1) : ic.cfl * jmin / alpha1;
+    if (K.mesh == SWALE_MESH_FLUID_GAUSS && dwmax > 0.0)
+      dt = fmin(dt, dwmax > 1e-290 ? 0.5 * jmin * swale::recip(dwmax) : 0.5 * jmin / dwmax);
+  }
+  if (K.t_end > 0.0 && K.t_end - tn <= dt) {
+    dt = K.t_end - tn;
+    clipped = 1;
+  }
+  // alpha = 0 (a dry state at rest on a mesh that does not move) leaves the CFL condition
+  // with no bound; without an end time there is no step to take: dt = 0, flagged.
+  if (!(dt < INFINITY)) {
+    dt = 0.0;
+    nodt = true;
+  }
+  double sdiff = 0.0;
+  if (K.mesh == SWALE_MESH_PROFILE && dt > 0.0) {
+    double sn, cs;
+    sincospi((lane == 0 ? 2.0 * tn + dt : dt) * K.inv_T, &sn, &cs);
+    const double cs0 = __shfl_sync(0xffffffffu, cs, 0), sn1 = __shfl_sync(0xffffffffu, sn, 1);
+    sdiff = 2.0 * cs0 * sn1 / dt;
+  }
+  if (lane == 0) {
+    if (nodt) atomicOr(&S->status, (unsigned int)swale::ST_NODT);
+    if (K.mesh == SWALE_MESH_FLUID_GAUSS) S->Wbar = Wbar;
+    S->dt = dt;
+    S->alpha1 = alpha1;
+    S->clipped = clipped;
+    S->sdiff = sdiff;
+    S->counter = 0u;
+  }
+}
+
 // STOREK: an instantiation of the hydrostatic scheme that also stores each cell's smooth-class
 // linear form in D.gK (the adjoint's recomputes), so that the forward's own instantiations keep
 // their registers.
@@ -549,12 +628,15 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
                                              const double* __restrict__ Jg) {
   constexpr int TO = T - 4;                        // cells reconstructed
   __shared__ __align__(16) double sRaw[4][T + 8];  // E, M, B, J of cells c0-2 .. c0+T-3 as bulk-copied
-  __shared__ double sH[T], sP[T], sQ[T];           // depths; pair and quadruple sums of widths
-  __shared__ double sD2[3][T], sD3[3][T], sD4[3][T];
+  // Depths; pair and quadruple sums of widths; differences. Every phase runs on all threads: the
+  // last rows of each hold nothing that a reconstructed cell reads (the rows are padded for them).
+  __shared__ double sH[T + 2], sP[T + 2], sQ[T];
+  __shared__ double sD2[3][T + 2], sD3[3][T + 2], sD4[3][T];
   // FP32 copies for the smooth-class test: widths, triple reciprocals, pair differences (hu, h, and
   // for the non-well-balanced scheme eta)
   constexpr int NV32 = SCHEME == 1 ? 3 : 2;
   __shared__ float sJf[T], sITf[T], sD2f[NV32][T];
+  __shared__ bool sIdle;
   __shared__ __align__(8) uint64_t sBar;           // completion of the tile's bulk copies
   __shared__ __align__(8) uint64_t sPad;           // test hook: a barrier no copy completes
   __shared__ bool last;
@@ -570,15 +652,16 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
   for (int t = blockIdx.x; t < D.nrf; t += gridDim.x) {
     const Tile tl = D.rftiles ? D.rftiles[t] : Tile{0, t * TO - 1};
     DevScalars* S = D.S + tl.inst;
-    // every thread reads the flags once, then the block agrees (the status may change meanwhile)
-    if (__syncthreads_or(inst_idle(S))) continue;
-    const InstConst ic = D.IC[tl.inst];
-    const int64_t N = ic.N, c0 = tl.c0;
+    const InstConst ic = D.rftiles ? D.IC[tl.inst] : D.ic1;
+    const int32_t N = (int32_t)ic.N, c0 = tl.c0;
     const double* E = Eg + ic.coff;
     const double* M = Mg + ic.coff;
     const double* B = Bg + ic.coff;
     const double* J = Jg + ic.coff;
     const int64_t eb = ic.coff + 2 * (int64_t)tl.inst;  // edge-array base of the instance
+    // One thread reads the flags, for the whole block (the status may change meanwhile); the
+    // copies start before they are known.
+    if (tid == 0) sIdle = inst_idle(S);
     // The cells of the tile that lie in the instance, [cs, ce], arrive by four bulk copies (E, M,
     // B, J). The copied span [ga, ge] (global element indices) is widened to 16-byte boundaries:
     // one element before cs where needed (it exists: ga >= 1), one after ce when that element is
@@ -586,7 +669,7 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     // is loaded directly). Shared rows are shifted by `off` so that the first copied element
     // lands on a 16-byte boundary as well. Ghost cells and anything not copied take the direct
     // loads below.
-    const int64_t cs = c0 - 2 < 0 ? 0 : c0 - 2, ce = c0 + T - 3 < N - 1 ? c0 + T - 3 : N - 1;
+    const int32_t cs = c0 - 2 < 0 ? 0 : c0 - 2, ce = c0 + T - 3 < N - 1 ? c0 + T - 3 : N - 1;
     int64_t ga = (ic.coff + cs) & ~(int64_t)1, ge = ic.coff + ce;
     if (!(ge & 1)) ge += (ce + 1 < N || tl.inst + 1 < K.B) ? 1 : -1;
     const int rel = (int)(ga - ic.coff - (c0 - 2));  // shared index of ga before the shift
@@ -594,8 +677,9 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     const uint32_t bytes = ge >= ga ? (uint32_t)((ge - ga + 1) * 8) : 0u;
     const bool bulk = bytes >= 16 && ((((uintptr_t)(Eg + ga)) | ((uintptr_t)(Mg + ga)) | ((uintptr_t)(Bg + ga)) |
                                        ((uintptr_t)(Jg + ga))) & 15) == 0;
-    const int64_t c = c0 - 2 + tid;       // this thread's cell
-    const int64_t idx = eb + c + 1;       // its edge-array index
+    const int32_t c = c0 - 2 + tid;                   // this thread's cell
+    const int32_t idx = (int32_t)(eb + c + 1);        // its edge-array index
+    const int32_t ca = (int32_t)(ga - ic.coff), cz = (int32_t)(ge - ic.coff);  // the cells copied
     const unsigned long long geo_now =
         ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)(S->step_idx & 0xffffffffLL);
     // Reciprocal sums of the widths: as the previous step's stage 2 stored them (the same mesh), or
@@ -603,14 +687,25 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     // and quadruple whose second cell is c + 1, the quintuple centred at c.
     const bool use_geo = STAGE == 1 && D.geo != nullptr && S->geo_tag == geo_now;
     const bool g_pair = use_geo && c >= -1 && c <= N, g_next = use_geo && c >= -2 && c + 1 <= N;
+    const bool all_pair = STAGE == 1 && __all_sync(0xffffffffu, g_pair);  // (a vote: no reciprocal is formed then)
+    const bool all_next = STAGE == 1 && __all_sync(0xffffffffu, g_next);
     double gip = 0.0, git = 0.0, giq = 0.0, giv = 0.0;
-    if (g_pair) {
+    if (STAGE == 1 && g_pair) {
       gip = D.geo[GEO_IP * D.geo_stride + idx];
       giv = D.geo[GEO_IV * D.geo_stride + idx];
     }
-    if (g_next) {
+    if (STAGE == 1 && g_next) {
       git = D.geo[GEO_IT * D.geo_stride + idx + 1];
       giq = D.geo[GEO_IQ * D.geo_stride + idx + 1];
+    }
+    const double seen = bitsd(*(volatile const unsigned long long*)&S->A[STAGE - 1]);
+    const double dxmax = bitsd(S->Jmax[STAGE - 1]);
+    // Node velocities of the cell's two edges (Eq. alpha2D: speeds relative to the node).
+    double wl = 0.0, wr = 0.0;
+    if (K.wave_rel && c >= -1 && c <= N) {
+      const double* wv = node_velocities(K, D) + ic.coff + tl.inst;
+      if (c >= 0) wl = wv[c];
+      if (c < N) wr = wv[c + 1];
     }
     if (bulk) {
       if (tid == 0) {
@@ -634,19 +729,25 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
         if (tid == 0) atomicOr(&S->status, (unsigned int)swale::ST_TIMEOUT);
         return;
       }
+    } else {
+      __syncthreads();
+    }
+    if (sIdle) {
+      __syncthreads();  // every thread has read the flag before the next tile's is written
+      continue;
     }
     double* const sE = &sRaw[0][off];
     double* const sM = &sRaw[1][off];
     double* const sJ = &sRaw[3][off];
     double jv = 1.0, ev = 0.0, mv = 0.0, hv = 0.0;  // filler beyond the last ghost cell
-    if (bulk && c >= 0 && c < N && c >= ga - ic.coff && c <= ge - ic.coff) {
+    if (bulk && c >= 0 && c < N && c >= ca && c <= cz) {
       ev = sE[tid];
       mv = sM[tid];
       jv = sJ[tid];
       hv = ev - sRaw[2][off + tid];
     } else {
       if (c >= -3 && c <= N + 2) {
-        const int64_t s = ghost(c, N, K.bc);
+        const int32_t s = ghost(c, N, K.bc);
         jv = J[s];
         ev = E[s];
         mv = M[s];
@@ -664,11 +765,12 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     const bool mine = tid >= 2 && tid < 2 + TO && c <= N;
     const bool next_mine = tid >= 1 && tid < 1 + TO && c + 1 <= N;  // cell c + 1 is
     // Order 2: the pair (c, c+1).
-    double p = 0.0, d2[3] = {0.0, 0.0, 0.0};
-    if (tid < T - 1) {
-      const double jn = sJ[tid + 1], de = sE[tid + 1] - ev, dm = sM[tid + 1] - mv, dh = sH[tid + 1] - hv;
-      p = jv + jn;
-      const double ip = g_pair ? gip : swale::recip(p);
+    double d2[3];
+    const double p = jv + sJ[tid + 1];
+    {
+      const double de = sE[tid + 1] - ev, dm = sM[tid + 1] - mv, dh = sH[tid + 1] - hv;
+      double ip = gip;
+      if (!all_pair) ip = g_pair ? gip : swale::recip(p);
       d2[0] = de * ip;
       d2[1] = dm * ip;
       d2[2] = dh * ip;
@@ -688,9 +790,10 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     }
     __syncthreads();
     // Order 3: the triple (c, c+1, c+2).
-    double d3[3] = {0.0, 0.0, 0.0};
-    if (tid < T - 2) {
-      const double it = g_next ? git : swale::recip(p + sJ[tid + 2]);
+    double d3[3];
+    {
+      double it = git;
+      if (!all_next) it = g_next ? git : swale::recip(p + sJ[tid + 2]);
 #pragma unroll
       for (int v = 0; v < 3; ++v) sD3[v][tid] = d3[v] = (sD2[v][tid + 1] - d2[v]) * it;
       sITf[tid] = swale::f32_trunc(it);
@@ -701,10 +804,13 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     }
     __syncthreads();
     // Order 4: the quadruple (c .. c+3).
-    if (tid < T - 3) {
-      const double q = p + sP[tid + 2];
-      const double iq = g_next ? giq : swale::recip(q);
-      sQ[tid] = q;
+    {
+      double iq = giq;
+      if (!all_pair || !all_next) {  // (the quintuple's sum needs it where that is not cached)
+        const double q = p + sP[tid + 2];
+        sQ[tid] = q;
+        iq = g_next ? giq : swale::recip(q);
+      }
 #pragma unroll
       for (int v = 0; v < 3; ++v) sD4[v][tid] = (sD3[v][tid + 1] - d3[v]) * iq;
       if (STAGE == 2 && D.geo && next_mine) D.geo[GEO_IQ * D.geo_stride + idx + 1] = iq;
@@ -712,11 +818,10 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     __syncthreads();
     if (STAGE == 2 && D.geo != nullptr && c0 == -1 && tid == 0)
       S->geo_tag = ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)((S->step_idx + 1) & 0xffffffffLL);
-    double wave = 0.0, ehL = 0.0, euL = 0.0, ehR = 0.0, euR = 0.0;
+    WaveEdge eL{0.0, 0.0, 0.0}, eR{0.0, 0.0, 0.0};
     bool useL = false, useR = false;
     uint32_t st = 0;
     if (mine) {
-      const double dxmax = bitsd(S->Jmax[STAGE - 1]);
       const double dxe = K.sc.beta_dx_global ? dxmax : jv;
       if (!swale::gt0(jv)) st |= swale::ST_EMESH;
       EdgeState o;
@@ -749,7 +854,8 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
       if (smooth) {
         // Order 5, the quintuple centred at c, and the edge values.
         const swale::SmoothWidths w = {sJ[tid - 1], jv, sJ[tid + 1], sP[tid - 2], sP[tid - 1], p, sP[tid + 1]};
-        const double iv = g_pair ? giv : swale::recip(sQ[tid - 2] + sJ[tid + 2]);
+        double iv = giv;
+        if (!all_pair) iv = g_pair ? giv : swale::recip(sQ[tid - 2] + sJ[tid + 2]);
         if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = iv;
         const double vj[3] = {ev, mv, hv};
         double evl[3][2];
@@ -767,7 +873,7 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
         swale::limit_cell(K.sc, evl, hv, mv, o, st);
       } else {
         if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = swale::recip(sQ[tid - 2] + sJ[tid + 2]);
-        const TileRows R = {sJ, sE, sM, sH, &sD2[0][0], &sD3[0][0], T};
+        const TileRows R = {sJ, sE, sM, sH, &sD2[0][0], &sD3[0][0], T + 2};
         const OpenOut r = recon_open_cell<SCHEME>(K.sc, R, tid, dxe);
         o = r.o;
         flag = r.flag;
@@ -804,69 +910,22 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
       // Edges that touch interfaces 0..N only.
       useL = (c != -1);
       useR = (c != N);
-      ehL = o.hL;
-      euL = o.uL;
-      ehR = o.hR;
-      euR = o.uR;
-      if (K.wave_rel) {  // Eq. alpha2D: speeds relative to the node (cell c spans nodes c, c+1)
-        const double* wv = node_velocities(K, D) + ic.coff + tl.inst;
-        if (useL) euL -= wv[c];
-        if (useR) euR -= wv[c + 1];
-      }
+      eL = {o.hL, o.uL, wl};
+      eR = {o.hR, o.uR, wr};
     }
-    wave = block_wave<T>(K.sc.g, useL, useR, ehL, euL, ehR, euR);
+    block_wave<T>(&S->A[STAGE - 1], seen, K.sc.g, useL, useR, eL, eR);
     block_or_status(&S->status, st);
-    block_max_to(&S->A[STAGE - 1], wave);
     if (STAGE == 1) {
+      __syncthreads();  // the block's atomics come before its ticket
       if (tid == 0) {
         __threadfence();
         const unsigned int ticket = atomicAdd(&S->counter, 1u);
         last = (ticket == (unsigned)ic.ntiles_r - 1u);
       }
       __syncthreads();
-      if (last && tid == 0) {
-        __threadfence();
-        const double A1 = bitsd(atomicAdd(&S->A[0], 0ull));
-        double Wbar = S->Wbar;
-        double dwmax = 0.0;
-        if (K.mesh == SWALE_MESH_FLUID_GAUSS) {
-          Wbar = bitsd(atomicAdd(&S->Wabs, 0ull));
-          dwmax = bitsd(atomicAdd(&S->dWabs, 0ull));
-          S->Wbar = Wbar;
-        }
-        const double alpha1 = stage_alpha(K, tl.inst, 1, K.wave_rel ? A1 : A1 + Wbar, S->step_idx);
-        const double tn = S->t;
-        double dt;
-        int clipped = 0;
-        if (K.dt_fixed > 0.0) {
-          dt = K.dt_fixed;
-        } else {
-          const double jmin = bitsd(S->Jmin0);
-          dt = ic.cfl * jmin / alpha1;
-          if (K.mesh == SWALE_MESH_FLUID_GAUSS && dwmax > 0.0) dt = fmin(dt, 0.5 * jmin / dwmax);
-        }
-        if (K.t_end > 0.0 && K.t_end - tn <= dt) {
-          dt = K.t_end - tn;
-          clipped = 1;
-        }
-        // alpha = 0 (a dry state at rest on a mesh that does not move) leaves the CFL condition
-        // with no bound; without an end time there is no step to take: dt = 0, flagged.
-        if (!(dt < INFINITY)) {
-          dt = 0.0;
-          atomicOr(&S->status, (unsigned int)swale::ST_NODT);
-        }
-        S->dt = dt;
-        S->alpha1 = alpha1;
-        S->clipped = clipped;
-        if (K.mesh == SWALE_MESH_PROFILE) {
-          const double s0 = sin(kTwoPi * tn / K.mesh_T);
-          const double s1 = sin(kTwoPi * (tn + dt) / K.mesh_T);
-          S->sdiff = dt > 0.0 ? (s1 - s0) / dt : 0.0;
-        } else {
-          S->sdiff = 0.0;
-        }
-        S->counter = 0u;
-      }
+      if (last && tid < 32) stage1_dt(K, S, ic, tl.inst);
+    } else {
+      __syncthreads();  // block_wave's shared rows are read before the next tile's are written
     }
   }
 }
@@ -895,12 +954,36 @@ struct RhsOut {
 // SCHEME: 0 hydrostatic, 1 non-well-balanced, 2 special source. BOT: an instantiation with the
 // L2-projection bottom. STOREK: one that also stores the old source form's entries in D.gK (the
 // adjoint's recomputes).
+
+// Largest a and b and smallest c over the block (non-negative doubles), raised / lowered into their
+// destinations by three lanes after a single barrier.
+template <int T>
+__device__ __forceinline__ void block_widths(DevScalars* S, double a, double b, double c) {
+  __shared__ unsigned long long red[3][T / 32];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const unsigned long long ma = warp_umax64(dbits(a)), mb = warp_umax64(dbits(b)), mc = warp_umax64(~dbits(c));
+  if (lane < 3) red[lane][wid] = lane == 0 ? ma : lane == 1 ? mb : mc;
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    unsigned long long m = 0ull;
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) m = umax64(m, red[threadIdx.x][w]);
+    if (threadIdx.x < 2) {
+      raise_to(&S->Jmax[1 + threadIdx.x], m);
+    } else {
+      m = ~m;
+      if (m < *(volatile const unsigned long long*)&S->JminN) atomicMin(&S->JminN, m);
+    }
+  }
+}
+
 template <int STAGE, int MODE, int T, int SCHEME = 0, bool BOT = false, bool STOREK = false>
 __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, DevState D, const double* __restrict__ Eg,
                                               const double* __restrict__ Mg, const double* __restrict__ Bg,
                                               const double* __restrict__ Jsg, RhsOut ro) {
   __shared__ double sF[3][T], sW[T];      // interfaces / nodes j0 .. j0+T-1: fluxes FE, FMl, FB
   __shared__ double sG[2][T], sDe[2][T];  // their sig and rho^2 (PairRatio); differences of eta and h
+  __shared__ bool sIdle;
   const int tid = threadIdx.x;
   (void)Mg;
   constexpr int TC = T - 1;  // cells of a tile; its T interfaces j0 .. j0 + TC, one per thread
@@ -908,14 +991,12 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     const Tile tl = D.ftiles ? D.ftiles[t] : Tile{0, t * TC};
     const int inst = tl.inst;
     DevScalars* S = D.S + inst;
-    if (MODE == 0) {
-      // Skip a finished instance and one whose step has failed. In stage 3 the status does not
-      // change during the launch (this kernel raises its bits in st3), so every tile of an
-      // instance decides alike: all commit the step or none does.
-      if (__syncthreads_or(inst_idle(S))) continue;
-    }
-    const InstConst ic = D.IC[inst];
-    const int64_t N = ic.N, j0 = tl.c0;
+    // Skip a finished instance and one whose step has failed (below, when the loads are under way).
+    // In stage 3 the status does not change during the launch (this kernel raises its bits in
+    // st3), so every tile of an instance decides alike: all commit the step or none does.
+    if (MODE == 0 && tid == 0) sIdle = inst_idle(S);
+    const InstConst ic = D.ftiles ? D.IC[inst] : D.ic1;
+    const int32_t N = (int32_t)ic.N, j0 = tl.c0;
     const int64_t cb = ic.coff, nb = ic.coff + inst, eb = ic.coff + 2 * (int64_t)inst;
     const double* E = Eg + cb;
     const double* B = Bg + cb;
@@ -926,10 +1007,8 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     } else {
       alpha = (STAGE == 1) ? S->alpha1 : bitsd(S->A[STAGE - 1]) + (K.wave_rel ? 0.0 : S->Wbar);
       if (STAGE > 1) {
-        // Record / replay of stages 2 and 3 (stage 1 is handled where alpha1 is formed): every
-        // tile computes the same value; the first tile of the instance records it.
+        // Replay of stages 2 and 3 (recorded below; stage 1 is handled where alpha1 is formed).
         if (K.alpha_mode == 2) alpha = stage_alpha(K, inst, STAGE, alpha, S->step_idx);
-        else if (K.alpha_mode == 1 && j0 == 0 && threadIdx.x == 0) stage_alpha(K, inst, STAGE, alpha, S->step_idx);
       }
       dt = S->dt;
     }
@@ -941,21 +1020,18 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     const bool use_sgeo = STAGE == 1 && MODE == 0 && D.geo != nullptr && S->geo_tag == geo_now;
     const bool put_sgeo = STAGE == 2 && MODE == 0 && D.geo != nullptr;
     const double sdiff = fresh_w ? S->sdiff : 0.0;
-    __syncthreads();  // the previous tile's reads of the shared rows
-    const int64_t k = j0 + tid;  // this thread's node / interface and cell
-    const int64_t el = eb + k, er = eb + k + 1;
+    const int32_t k = j0 + tid;  // this thread's node / interface and cell
+    const int32_t el = (int32_t)(eb + k), er = el + 1;
     swale::Flux2 F{0.0, 0.0, 0.0, 0.0};
     swale::PairRatio pr{0.0, 0.0, 0.0, 0.0};
     double wk = 0.0, ELj = 0.0, BLj = 0.0, hLj = 0.0, dE = 0.0, dH = 0.0;
     if (k <= N) {
       if (fresh_w) {
         wk = D.P[nb + k] * sdiff;
-        if (tid < TC || k == N) D.w[nb + k] = wk;
       } else if (MODE == 0 && K.mesh == SWALE_MESH_STATIC) {
         wk = 0.0;
       } else if (MODE == 0 && K.mesh == SWALE_MESH_LINEAR) {
         wk = D.P[nb + k];  // constant node velocity (Eq. velocity)
-        if (STAGE == 1 && (tid < TC || k == N)) D.w[nb + k] = wk;
       } else {
         wk = D.w[nb + k];
       }
@@ -975,12 +1051,6 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
         const double Jl = Js[ghost(k - 1, N, K.bc)], Jr = Js[ghost(k, N, K.bc)];
         pr = swale::pair_ratio(Jl, Jr, D.ipair[el]);
       }
-      if (put_sgeo) {
-        D.geo[GEO_RHO * D.geo_stride + el] = pr.rho;
-        D.geo[GEO_SIG * D.geo_stride + el] = pr.sig;
-        D.geo[GEO_RHO2 * D.geo_stride + el] = pr.rho2;
-        D.geo[GEO_SIG2 * D.geo_stride + el] = pr.sig2;
-      }
       F = swale::interface_flux2<SCHEME>(K.sc.g, alpha, wk, D.eER[el], ELj, D.eBR[el], BLj, D.ehR[el], hLj, D.euR[el],
                                          D.euL[er]);
       sF[0][tid] = F.FE;
@@ -993,7 +1063,24 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
       sDe[1][tid] = dH;
     }
     __syncthreads();
-    const int64_t j = k;
+    if (MODE == 0 && sIdle) {
+      __syncthreads();  // every thread has read the flag before the next tile's is written
+      continue;
+    }
+    if (MODE == 0 && k <= N) {
+      // The node velocities of the step, where this stage makes them (a tile's last node is the
+      // next tile's first).
+      if (STAGE == 1 && (fresh_w || K.mesh == SWALE_MESH_LINEAR) && (tid < TC || k == N)) D.w[nb + k] = wk;
+      if (put_sgeo) {
+        D.geo[GEO_RHO * D.geo_stride + el] = pr.rho;
+        D.geo[GEO_SIG * D.geo_stride + el] = pr.sig;
+        D.geo[GEO_RHO2 * D.geo_stride + el] = pr.rho2;
+        D.geo[GEO_SIG2 * D.geo_stride + el] = pr.sig2;
+      }
+      // Every tile has the same viscosity; the first one of the instance records it.
+      if (STAGE > 1 && K.alpha_mode == 1 && k == 0) stage_alpha(K, inst, STAGE, alpha, S->step_idx);
+    }
+    const int32_t j = k;
     double jmaxa = 0.0, jmaxb = 0.0, jminb = INFINITY;
     uint32_t st = 0;
     if (tid < TC && j < N) {
@@ -1052,7 +1139,7 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
         ro.RM[j] = 0.5 * R2[1];
         ro.RB[j] = 0.5 * R2[2];
       } else {
-        const int64_t g = cb + j;  // global cell index
+        const int32_t g = (int32_t)cb + j;  // global cell index
         const double wl = wk, wr = sW[tid + 1];
         const double J0 = D.J0[g];
         const double dJ = dt * (wr - wl);
@@ -1128,12 +1215,9 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     }
     if (MODE == 0) {
       block_or_status(STAGE == 3 ? &S->st3 : &S->status, st);
-      if (STAGE == 1) {
-        block_max_to(&S->Jmax[1], jmaxa);
-        block_max_to(&S->Jmax[2], jmaxb);
-        block_min_to(&S->JminN, jminb);
-      }
+      if (STAGE == 1) block_widths<T>(S, jmaxa, jmaxb, jminb);
     }
+    __syncthreads();  // this tile's reads of the shared rows come before the next tile's writes
   }
 }
 

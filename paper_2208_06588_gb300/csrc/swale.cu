@@ -18,6 +18,7 @@
 #include "../../include/swale.h"
 #include "swale_kernels.cuh"
 #include "swale_adjoint_kernels.cuh"
+#include "swale_steps.cuh"
 
 using namespace swale_dev;
 
@@ -59,6 +60,11 @@ struct swale_ctx {
   // expect (0).
   int32_t wait_tries = 0;
   uint32_t tx_pad = 0;
+  // Whole steps in one launch (k_steps), for meshes of few blocks: the blocks, 0 if there are too many,
+  // their work list (null: one instance) and the scratch of the instances.
+  int step_blocks = 0;
+  Tile* step_tiles = nullptr;
+  StepScratch* step_scratch = nullptr;
 };
 
 namespace {
@@ -170,6 +176,9 @@ void drop_graph(swale_ctx* ctx) {
 void free_tiles(swale_ctx* ctx) {
   for (void* p : ctx->tile_allocs) cudaFree(p);
   ctx->tile_allocs.clear();
+  ctx->step_blocks = 0;
+  ctx->step_tiles = nullptr;
+  ctx->step_scratch = nullptr;
   ctx->D.rtiles = ctx->D.utiles = ctx->D.mtiles = ctx->D.ftiles = ctx->D.rftiles = nullptr;
 }
 
@@ -281,6 +290,37 @@ swale_status check_config(const swale_config* c, std::string& why) {
 
 bool valid_tile(int T) { return T == 64 || T == 128 || T == 256; }
 
+// Blocks that k_steps would run for the instances: kept if the mesh is small enough for it (at most
+// kStepBlocksPerSM a SM, all of them resident). One block is 122 cells and one warp on each
+// sub-partition of an SM.
+constexpr int kStepBlocksPerSM = 1;
+swale_status build_step_blocks(swale_ctx* ctx, const std::vector<InstConst>& ic) {
+  if (ctx->cfg.scheme == SWALE_SCHEME_SPECIAL || ctx->cfg.mesh == SWALE_MESH_FLUID_GAUSS) return SWALE_OK;
+  int dev = 0, sms = 0, coop = 0, fit = 0;
+  SW_CUDA(ctx, cudaGetDevice(&dev));
+  SW_CUDA(ctx, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  int64_t n = 0;
+  for (const InstConst& c : ic) n += (c.N + kStepCells - 1) / kStepCells;
+  if (n > (int64_t)sms * kStepBlocksPerSM) return SWALE_OK;
+  SW_CUDA(ctx, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  SW_CUDA(ctx, ctx->cfg.scheme == SWALE_SCHEME_NONWB
+                   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_steps<1>, kStepThreads, 0)
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_steps<0>, kStepThreads, 0));
+  if (!coop || n > (int64_t)sms * fit) return SWALE_OK;
+  if (swale_status s = dalloc(ctx, ctx->tile_allocs, &ctx->step_scratch, ic.size())) return s;
+  if (ic.size() > 1) {
+    std::vector<Tile> list;
+    for (size_t i = 0; i < ic.size(); ++i)
+      for (int64_t b = 0; b * kStepCells < ic[i].N; ++b) list.push_back(Tile{(int32_t)i, (int32_t)b});
+    if (swale_status s = dalloc(ctx, ctx->tile_allocs, &ctx->step_tiles, list.size())) return s;
+    SW_CUDA(ctx, cudaMemcpyAsync(ctx->step_tiles, list.data(), list.size() * sizeof(Tile), cudaMemcpyHostToDevice,
+                                 ctx->stream));
+    SW_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  }
+  ctx->step_blocks = (int)n;
+  return SWALE_OK;
+}
+
 // Builds the work lists for the current tile sizes (implicit for one instance) and the
 // per-instance tile counts; uploads the instance constants.
 swale_status build_tiles(swale_ctx* ctx, std::vector<InstConst>& ic) {
@@ -334,6 +374,7 @@ swale_status build_tiles(swale_ctx* ctx, std::vector<InstConst>& ic) {
     ctx->D.nrf = (int32_t)rf.size();
   }
   ctx->D.ic1 = ic[0];
+  if (swale_status s = build_step_blocks(ctx, ic)) return s;
   SW_CUDA(ctx, cudaMemcpyAsync(ctx->D.IC, ic.data(), B * sizeof(InstConst), cudaMemcpyHostToDevice, ctx->stream));
   SW_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   return SWALE_OK;
@@ -461,10 +502,43 @@ swale_status enqueue_step(swale_ctx* ctx, const DevState* stageD = nullptr) {
   return enqueue_step_on(ctx, ctx->D, ctx->stream, stageD, ctx->geo_epoch);
 }
 
-// Enqueues n steps: whole graphs of kGraphSteps steps, then single steps (graphs are not used
-// while kernel timing is on).
+// Whether the next steps go through k_steps: a small mesh (build_step_blocks), and nothing asked for
+// that only the stage kernels do: an explicit launch shape, kernel timing, a viscosity log, the
+// projected bottom, the wait test, or a stream that is being captured.
+bool whole_steps(swale_ctx* ctx) {
+  if (!ctx->step_blocks || ctx->timing || ctx->alpha_mode != 0 || ctx->bot_pieces > 0 || ctx->tx_pad) return false;
+  if (ctx->Tr != 128 || ctx->Tu != 128 || ctx->grid_r || ctx->grid_u) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
+
+// Steps of one k_steps launch at most (a fraction of a second).
+constexpr int64_t kStepsPerLaunch = 4096;
+
+swale_status enqueue_whole_steps(swale_ctx* ctx, int64_t n) {
+  StepConst K = step_const(ctx);
+  int rel1 = stage1_wave_rel(ctx->cfg);
+  const void* f = ctx->cfg.scheme == SWALE_SCHEME_NONWB ? (const void*)k_steps<1> : (const void*)k_steps<0>;
+  for (; n > 0; n -= kStepsPerLaunch) {
+    NvtxRange r("swale whole steps");
+    long long m = std::min(n, kStepsPerLaunch);
+    const Tile* tiles = ctx->step_tiles;
+    void* args[] = {&K, &ctx->D, &ctx->step_scratch, &tiles, &rel1, &m};
+    SW_CUDA(ctx, cudaMemsetAsync(ctx->step_scratch, 0, ctx->B * sizeof(StepScratch), ctx->stream));
+    SW_CUDA(ctx, cudaLaunchCooperativeKernel(f, dim3((unsigned)ctx->step_blocks), dim3(kStepThreads), args, 0, ctx->stream));
+  }
+  return SWALE_OK;
+}
+
+// Enqueues n steps: in whole-step launches where the mesh is small, else as graphs of kGraphSteps
+// steps, then single steps (graphs are not used while kernel timing is on).
 swale_status enqueue_steps(swale_ctx* ctx, int64_t n) {
   constexpr int kGraphSteps = 8;
+  if (n > 0 && whole_steps(ctx)) return enqueue_whole_steps(ctx, n);
   if (!ctx->timing && n >= kGraphSteps) {
     if (!ctx->graph) {
       cudaGraph_t g;
@@ -680,7 +754,7 @@ swale_status swale_step(swale_ctx* ctx, double* dt_out) {
   NvtxRange nvtx_range("swale_step");
   if (!ctx) return SWALE_EINVAL;
   if (ctx->B == 0) return fail(ctx, SWALE_EINVAL, "no problem set");
-  if (swale_status s = enqueue_step(ctx)) return s;
+  if (swale_status s = enqueue_steps(ctx, 1)) return s;
   if (dt_out) {
     SW_CUDA(ctx, cudaMemcpyAsync(dt_out, &ctx->D.S->dt, sizeof(double), cudaMemcpyDefault, ctx->stream));
     SW_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -703,7 +777,8 @@ swale_status swale_advance(swale_ctx* ctx, int64_t max_steps, int64_t* steps_don
     // each, the host reads the instances' scalars and stops once every instance has reached
     // t_end or stopped on an error (the prologue's test), so that a generous max_steps does not
     // launch a long tail of no-op steps.
-    int64_t left = max_steps, chunk = 64;
+    // (A whole-step launch ends by itself: it gets the largest chunk at once.)
+    int64_t left = max_steps, chunk = whole_steps(ctx) ? kStepsPerLaunch : 64;
     while (left > 0) {
       const int64_t n = std::min(left, chunk);
       if (swale_status s = enqueue_steps(ctx, n)) return s;

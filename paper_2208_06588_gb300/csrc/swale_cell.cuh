@@ -155,6 +155,21 @@ SWALE_HD real wave_sqrt(real a) { return sqrt(a); }
 #endif
 #endif
 
+// Products, sums and fused multiply-adds that the compiler neither splits nor fuses: what several
+// kernels evaluate (the stage kernels and the one that runs whole steps) comes out the same bit for
+// bit wherever it is inlined.
+#if defined(__CUDA_ARCH__) && !defined(SWALE_REAL)
+SWALE_HD double mul_(double a, double b) { return __dmul_rn(a, b); }
+SWALE_HD double add_(double a, double b) { return __dadd_rn(a, b); }
+SWALE_HD double sub_(double a, double b) { return __dadd_rn(a, -b); }
+SWALE_HD double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+#else
+SWALE_HD real mul_(real a, real b) { return a * b; }
+SWALE_HD real add_(real a, real b) { return a + b; }
+SWALE_HD real sub_(real a, real b) { return a - b; }
+SWALE_HD real fma_(real a, real b, real c) { return a * b + c; }
+#endif
+
 // Double to float on the integer pipe: the top 23 mantissa bits (rounded toward zero, relative
 // error below 2^-23), magnitudes below the normal float range to a signed zero, above it (and
 // infinities, NaNs) to a signed infinity. The hardware conversion instruction runs on the FP64
@@ -167,11 +182,11 @@ SWALE_HD float f32_trunc(double x) {
   memcpy(&b, &x, 8);
   const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
 #endif
-  const unsigned sign = hi & 0x80000000u;
-  const int e = (int)((hi >> 20) & 0x7ffu) - 896;  // the float's biased exponent (1023 - 127 = 896)
-  const unsigned mant = ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const unsigned mag = e <= 0 ? 0u : (e >= 255 ? 0x7f800000u : (((unsigned)e << 23) | mant));
-  const unsigned r = sign | mag;
+  // The exponent's rebias (1023 - 127 = 896) only flips bit 7 of its low eight bits within the
+  // float's range, so the magnitude is a shift of the two words with one bit flipped.
+  const unsigned mag = hi & 0x7fffffffu;
+  const unsigned in = (((hi << 3) | (lo >> 29)) ^ 0x40000000u) & 0x7fffffffu;
+  const unsigned r = (mag - 0x38100000u < 0x0fe00000u ? in : (mag < 0x38100000u ? 0u : 0x7f800000u)) | (hi & 0x80000000u);
 #if defined(__CUDA_ARCH__)
   return __uint_as_float(r);
 #else
@@ -310,7 +325,7 @@ SWALE_HD bool sure_smooth_nonwb_f32(double g, double h_dry, double hb, double mb
 }
 
 // Wave speed |u| + sqrt(g max(h, 0)) of one limited edge state (Eq. alpha2D).
-SWALE_HD real wave_speed(real g, real h, real u) { return dabs(u) + wave_sqrt(g * pos0(h)); }
+SWALE_HD real wave_speed(real g, real h, real u) { return add_(dabs(u), wave_sqrt(mul_(g, pos0(h)))); }
 
 // ------------------------------------------------------------------------------------
 // Shared per-pair and per-triple terms (Step 1): reciprocal widths and divided differences.
@@ -506,16 +521,16 @@ SWALE_HD void limit_cell(const SchemeConst& P, const real ev[3][2], real hbar0, 
   real hL = ev[2][0], hR = ev[2][1];
   real mL = ev[1][0], mR = ev[1][1];
   if (!surely_unlimited(P, hbar, hL, hR)) {
-    const real delta = (12.0 * hbar - hL - hR) * 0.1;
+    const real delta = mul_(sub_(fma_(12.0, hbar, -hL), hR), 0.1);
     const real mn = dmin(dmin(hL, hR), delta);
     const real epsv = dmin(P.eps_pp, hbar);
     if (dlt(mn, epsv)) {
-      const real theta = (hbar - epsv) * recip(hbar - mn);
-      hL = theta * (hL - hbar) + hbar;
-      hR = theta * (hR - hbar) + hbar;
+      const real theta = mul_(sub_(hbar, epsv), recip(sub_(hbar, mn)));
+      hL = fma_(theta, sub_(hL, hbar), hbar);
+      hR = fma_(theta, sub_(hR, hbar), hbar);
       if (P.limit_hu) {
-        mL = theta * (mL - mbar) + mbar;
-        mR = theta * (mR - mbar) + mbar;
+        mL = fma_(theta, sub_(mL, mbar), mbar);
+        mR = fma_(theta, sub_(mR, mbar), mbar);
       }
     }
   }
@@ -523,14 +538,14 @@ SWALE_HD void limit_cell(const SchemeConst& P, const real ev[3][2], real hbar0, 
   o.ER = ev[0][1];
   o.hL = hL;
   o.hR = hR;
-  o.BL = ev[0][0] - hL;
-  o.BR = ev[0][1] - hR;
+  o.BL = sub_(ev[0][0], hL);
+  o.BR = sub_(ev[0][1], hR);
   // Velocities with one division: u_L = m_L h_R' / (h_L' h_R'), dry edges (h <= h_dry) -> 0.
   const bool wetL = gt_pos(hL, P.h_dry), wetR = gt_pos(hR, P.h_dry);
   const real hLs = wetL ? hL : real(1.0), hRs = wetR ? hR : real(1.0);
-  const real ihh = recip(hLs * hRs);
-  o.uL = wetL ? mL * hRs * ihh : real(0.0);
-  o.uR = wetR ? mR * hLs * ihh : real(0.0);
+  const real ihh = recip(mul_(hLs, hRs));
+  o.uL = wetL ? mul_(mul_(mL, hRs), ihh) : real(0.0);
+  o.uR = wetR ? mul_(mul_(mR, hLs), ihh) : real(0.0);
   // NaN propagates into the comparisons as false: catch it explicitly.
   if (bad6(o.EL, o.ER, hL, hR, mL, mR)) st |= ST_NONFINITE;
 }
@@ -604,20 +619,21 @@ struct SmoothWidths {
   real h1, h2, h3, p01, p12, p23, p34;
 };
 SWALE_HD real smooth_right(const SmoothWidths& w, real v, real d2r, real d3, real d4r, real d5) {
-  return v + w.h2 * (d2r - w.h3 * (d3 + w.p12 * (d4r - w.p34 * d5)));
+  return fma_(w.h2, fma_(-w.h3, fma_(w.p12, fma_(-w.p34, d5, d4r), d3), d2r), v);
 }
 SWALE_HD real smooth_left(const SmoothWidths& w, real v, real d2l, real d3, real d4l, real d5) {
-  return v - w.h2 * (d2l + w.h1 * (d3 - w.p23 * (d4l + w.p01 * d5)));
+  return fma_(-w.h2, fma_(w.h1, fma_(-w.p23, fma_(w.p01, d5, d4l), d3), d2l), v);
 }
 // The same interpolant at the offset t h2 (0 < t < 1) from the cell's left edge: the nodes in the
 // order y2, y3, y4, y1, y5, y0 with the basis polynomials N_k and their derivatives.
 SWALE_HD real smooth_point(const SmoothWidths& w, real h4, real t, real v, real d2r, real d3, real d4r, real d5) {
-  const real n2 = (t * (t - 1.0)) * (w.h2 * w.h2), e2 = (2.0 * t - 1.0) * w.h2;
-  const real a4 = (t - 1.0) * w.h2 - w.h3, a1 = t * w.h2 + w.h1, a5 = a4 - h4;
-  const real n3 = n2 * a4, e3 = e2 * a4 + n2;
-  const real n4 = n3 * a1, e4 = e3 * a1 + n3;
-  const real e5 = e4 * a5 + n4;
-  return v + (d2r * e2 + (d3 * e3 + (d4r * e4 + d5 * e5)));
+  const real tm = t - 1.0;
+  const real n2 = mul_(mul_(t, tm), mul_(w.h2, w.h2)), e2 = mul_(t + tm, w.h2);
+  const real a4 = fma_(tm, w.h2, -w.h3), a1 = fma_(t, w.h2, w.h1), a5 = sub_(a4, h4);
+  const real n3 = mul_(n2, a4), e3 = fma_(e2, a4, n2);
+  const real n4 = mul_(n3, a1), e4 = fma_(e3, a1, n3);
+  const real e5 = fma_(e4, a5, n4);
+  return add_(v, fma_(d2r, e2, fma_(d3, e3, fma_(d4r, e4, mul_(d5, e5)))));
 }
 // Whether the five widths (truncated to FP32) are above 1e-9, so that the FP32 indicator factors (up
 // to the fourth power of a width) are normal numbers, and within a factor of 2^20 of each other. Then both middle linear weights d_1 are positive beyond any rounding: with
@@ -627,6 +643,75 @@ SWALE_HD real smooth_point(const SmoothWidths& w, real h4, real t, real v, real 
 SWALE_HD bool moderate_widths(float a, float b, float c, float d, float e) {
   const float mn = fminf(fminf(fminf(a, b), fminf(c, d)), e), mx = fmaxf(fmaxf(fmaxf(a, b), fmaxf(c, d)), e);
   return mn > 1e-9f && mx < 1e30f && mx < 1048576.0f * mn;
+}
+
+// One edge of a cell that the FP32 test leaves open, with the shared indicators of Eq. alphamodified:
+// Steps 2-4 as in recon_cell_g (shared_beta, hybrid_phi, edge_value), arranged for one edge at a time
+// and few operations (about 118, against 250 for both edges with the mesh geometry):
+//  * beta_r = c4 ((qh^2 + qm^2) + (3 h2^2 / 4 + 9 dx^2) (D3h^2 + D3m^2)), c3 = c4 (3 h2^2 / 4 + 9 dx^2);
+//  * the sub-stencils' values in Newton form from the edge, as in smooth_right: at the right edge
+//    v_j + h2 (D2[j,j+1] - h3 D3) for the two that hold cell j+1 and v_j + h2 (D2[j-1,j] + p12 D3[j-1])
+//    for the other (mirrored at the left edge), so the weights multiply slopes only and need no
+//    further geometry;
+//  * the smooth class through smooth_right / smooth_left.
+// right selects the edge; d2[v][4], d3[v][3], d4[v][2] the differences of (eta, hu, h), iv = 1 / (h0 + .. + h4).
+// Returns the class; out[v] the edge values.
+SWALE_HD uint8_t open_edge_values(const SchemeConst& P, const real h[5], const real p[4], real dx, real iv, const real v[3],
+                                  const real d2[3][4], const real d3[3][3], const real d4[3][2], bool right,
+                                  real out[3]) {
+  const real hh = mul_(0.5, h[2]);
+  const real F[3] = {add_(fma_(3.0, hh, p[0]), h[1]), add_(hh, h[1]), -add_(hh, h[3])};
+  const real c4 = mul_(mul_(4.0, dx), h[2]), kap = fma_(mul_(9.0, dx), dx, mul_(mul_(3.0, hh), hh));
+  real beta[3];
+  for (int r = 0; r < 3; ++r) {
+    const int a = 2 - r;
+    const real qh = fma_(d3[2][a], F[a], d2[2][a]), qm = fma_(d3[1][a], F[a], d2[1][a]);
+    const real t = fma_(d3[1][a], d3[1][a], mul_(d3[2][a], d3[2][a]));
+    beta[r] = mul_(c4, fma_(kap, t, fma_(qm, qm, mul_(qh, qh))));
+  }
+  const real tau = dabs(sub_(beta[0], beta[2]));
+  const real den = fma_(add_(add_(beta[0], beta[1]), beta[2]), 1.0 / 3.0, P.eps_weno);
+  const uint8_t flag = le_nn(tau, mul_(0.5, den)) ? 0 : (le_nn(den, tau) ? 2 : 1);
+  const SmoothWidths w = {h[1], h[2], h[3], p[0], p[1], p[2], p[3]};
+  if (flag == 0) {
+    for (int k = 0; k < 3; ++k) {
+      const real d5 = mul_(sub_(d4[k][1], d4[k][0]), iv);
+      out[k] = right ? smooth_right(w, v[k], d2[k][2], d3[k][1], d4[k][1], d5)
+                     : smooth_left(w, v[k], d2[k][1], d3[k][1], d4[k][0], d5);
+    }
+    return flag;
+  }
+  // Linear weights of the edge.
+  const real Sa = add_(p[0], p[2]), Sb = add_(Sa, h[4]), Sc = add_(p[1], p[3]);
+  const real inv = recip(mul_(mul_(Sa, Sb), Sc));
+  const real s234 = add_(p[2], h[4]), s012 = add_(p[0], h[2]);
+  real d[3];
+  d[2] = mul_(mul_(right ? h[3] : p[2], right ? p[3] : s234), mul_(Sc, inv));
+  d[0] = mul_(mul_(right ? p[1] : h[1], right ? s012 : p[0]), mul_(Sa, inv));
+  d[1] = sub_(sub_(1.0, d[0]), d[2]);
+  // WENO-Z weights, blended with the linear ones in the transition class.
+  const real e0 = add_(beta[0], P.eps_weno), e1 = add_(beta[1], P.eps_weno), e2 = add_(beta[2], P.eps_weno);
+  const real e01 = mul_(e0, e1), ie = mul_(tau, recip(mul_(e01, e2)));
+  const real q0 = mul_(mul_(e1, e2), ie), q1 = mul_(mul_(e0, e2), ie), q2 = mul_(e01, ie);
+  const real a0 = mul_(d[0], fma_(q0, q0, 1.0)), a1 = mul_(d[1], fma_(q1, q1, 1.0)), a2 = mul_(d[2], fma_(q2, q2, 1.0));
+  const real is = recip(add_(add_(a0, a1), a2));
+  real phi[3] = {mul_(a0, is), mul_(a1, is), mul_(a2, is)};
+  if (flag == 1) {
+    const real mg = fma_(2.0, mul_(tau, recip(den)), -1.0);
+    for (int r = 0; r < 3; ++r) phi[r] = fma_(mg, sub_(phi[r], d[r]), d[r]);
+  }
+  // Slopes of the sub-stencils r = 0 (cells j..j+2), 1, 2 (j-2..j) from the cell average to the edge.
+  for (int k = 0; k < 3; ++k) {
+    const real dn = right ? d2[k][2] : d2[k][1], df = right ? d2[k][1] : d2[k][2];
+    const real g = right ? -h[3] : h[1], gf = right ? p[1] : -p[2];
+    const real s1 = fma_(g, d3[k][1], dn);
+    const real sa = fma_(g, right ? d3[k][2] : d3[k][0], dn);   // r = 0 at the right edge, 2 at the left
+    const real sb = fma_(gf, right ? d3[k][0] : d3[k][2], df);  // r = 2 at the right edge, 0 at the left
+    const real pa = right ? phi[0] : phi[2], pb = right ? phi[2] : phi[0];
+    const real s = fma_(pb, sb, fma_(pa, sa, mul_(phi[1], s1)));
+    out[k] = fma_(right ? h[2] : -h[2], s, v[k]);
+  }
+  return flag;
 }
 
 // Reconstruction of cell j for the non-well-balanced scheme (Eq. se2D / s2D; Sec. 2.2, last
@@ -1010,23 +1095,23 @@ SWALE_HD Flux2 interface_flux2(real g, real alpha, real w, real EL, real ER, rea
   real sL = hL, sR = hR;
   if (SCHEME == 0) {
     const real bstar = dmax(BL, BR);
-    sL = pos0(EL - bstar);
-    sR = pos0(ER - bstar);
+    sL = pos0(sub_(EL, bstar));
+    sR = pos0(sub_(ER, bstar));
   }
-  const real mL = sL * uL, mR = sR * uR;
+  const real mL = mul_(sL, uL), mR = mul_(sR, uR);
   Flux2 f;
-  f.FE = ((mL + mR) - w * (EL + ER)) - alpha * (ER - EL);
-  const real M = (mL * (uL - w) + mR * (uR - w)) - alpha * (mR - mL);
+  f.FE = fma_(-alpha, sub_(ER, EL), fma_(-w, add_(EL, ER), add_(mL, mR)));
+  const real M = fma_(-alpha, sub_(mR, mL), fma_(mR, sub_(uR, w), mul_(mL, sub_(uL, w))));
   const real hg = 0.5 * g;
   if (SCHEME == 2) {
-    f.FMl = M + hg * (sL * sL + sR * sR);
+    f.FMl = fma_(hg, fma_(sL, sL, mul_(sR, sR)), M);
     f.FMr = f.FMl;
   } else {
-    const real q = (sR - sL) * (sR + sL);
-    f.FMl = M + hg * q;
-    f.FMr = M - hg * q;
+    const real q = mul_(sub_(sR, sL), add_(sR, sL));
+    f.FMl = fma_(hg, q, M);
+    f.FMr = fma_(-hg, q, M);
   }
-  f.FB = w * (BL + BR) + alpha * (BR - BL);
+  f.FB = fma_(alpha, sub_(BR, BL), mul_(w, add_(BL, BR)));
   return f;
 }
 
@@ -1036,8 +1121,8 @@ struct PairRatio {
   real rho, sig, rho2, sig2;
 };
 SWALE_HD PairRatio pair_ratio(real Jl, real Jr, real ip) {
-  const real rho = Jl * ip, sig = Jr * ip;
-  return {rho, sig, rho * rho, sig * sig};
+  const real rho = mul_(Jl, ip), sig = mul_(Jr, ip);
+  return {rho, sig, mul_(rho, rho), mul_(sig, sig)};
 }
 
 // The source term of source_form in factored form, joined with the cell's own edge pressures.
@@ -1057,11 +1142,11 @@ struct SourceRatio {
   real GX, GY, K3;
 };
 SWALE_HD SourceRatio source_ratio(real Jm, real Jc, real Jp, real iJm, real iJp, real itc) {
-  const real z = Jc * itc, a = z * iJm, b = z * iJp, e = -0.2 * Jc;
+  const real z = mul_(Jc, itc), a = mul_(z, iJm), b = mul_(z, iJp), e = mul_(-0.2, Jc);
   SourceRatio s;
-  s.GX = (e - 0.4 * Jp) * a;
-  s.GY = (0.4 * Jm - e) * b;
-  s.K3 = ((2.0 / 7.0) * e * Jc) * (a * iJp);
+  s.GX = mul_(fma_(-0.4, Jp, e), a);
+  s.GY = mul_(fma_(0.4, Jm, -e), b);
+  s.K3 = mul_(mul_(mul_(2.0 / 7.0, e), Jc), mul_(a, iJp));
   return s;
 }
 //   hc, hL, hR  depth average and limited edge depths;  deL, deR  edge values of eta less its average;
@@ -1069,21 +1154,23 @@ SWALE_HD SourceRatio source_ratio(real Jm, real Jc, real Jp, real iJm, real iJp,
 // Returns twice the value above (the momentum source and pressure difference is -g/2 times it).
 SWALE_HD real source_pressure_form(real hc, real hL, real hR, real deL, real deR, real dEl, real dHl, real dEr, real dHr,
                                    real rho_l, real sig2_l, real sig_r, real rho2_r, const SourceRatio& s) {
-  const real dhL = hL - hc, dhR = hR - hc;
-  const real Xe = (deL + rho_l * deR) + sig2_l * dEl, Ye = (deR + sig_r * deL) - rho2_r * dEr;
-  const real Xh = (dhL + rho_l * dhR) + sig2_l * dHl, Yh = (dhR + sig_r * dhL) - rho2_r * dHr;
-  const real Ge = (deR + s.GX * Xe) + s.GY * Ye, Gh = (dhR + s.GX * Xh) + s.GY * Yh;
-  const real ce = deL + deR, ch = dhL + dhR;
-  real acc = deR * (hc + hR);
-  acc = acc - deL * (hc + hL);
-  acc = acc + Gh * ce;
-  acc = acc - ch * Ge;
-  return acc + s.K3 * (Xh * Ye - Yh * Xe);
+  const real dhL = sub_(hL, hc), dhR = sub_(hR, hc);
+  const real Xe = fma_(sig2_l, dEl, fma_(rho_l, deR, deL)), Ye = fma_(-rho2_r, dEr, fma_(sig_r, deL, deR));
+  const real Xh = fma_(sig2_l, dHl, fma_(rho_l, dhR, dhL)), Yh = fma_(-rho2_r, dHr, fma_(sig_r, dhL, dhR));
+  const real Ge = fma_(s.GY, Ye, fma_(s.GX, Xe, deR)), Gh = fma_(s.GY, Yh, fma_(s.GX, Xh, dhR));
+  const real ce = add_(deL, deR), ch = add_(dhL, dhR);
+  real acc = mul_(deR, add_(hc, hR));
+  acc = fma_(-deL, add_(hc, hL), acc);
+  acc = fma_(Gh, ce, acc);
+  acc = fma_(-ch, Ge, acc);
+  return fma_(s.K3, fma_(Xh, Ye, -mul_(Yh, Xe)), acc);
 }
 
 // q + (a R - q dJ) / J' with inv = 1 / J': a cell average advanced by an increment a R of J q while
 // its width grows by dJ.
-SWALE_HD real rk_advance(real q, real a, real R, real dJ, real inv) { return q + (a * R - q * dJ) * inv; }
+SWALE_HD real rk_advance(real q, real a, real R, real dJ, real inv) {
+  return fma_(fma_(-q, dJ, mul_(a, R)), inv, q);
+}
 
 // Flux differences and source of cell j: R = (R_E, R_M, R_B) of Eq. hydro2D / bottomrk.
 struct CellRhs {

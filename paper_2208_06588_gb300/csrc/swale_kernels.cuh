@@ -279,7 +279,7 @@ struct WaveEdge {
   __device__ bool same(const WaveEdge& o) const {
     return dbits(h) == dbits(o.h) && dbits(u) == dbits(o.u) && dbits(w) == dbits(o.w);
   }
-  __device__ double speed(double g) const { return swale::wave_speed(g, h, u - w); }
+  __device__ double speed(double g) const { return swale::wave_speed(g, h, swale::sub_(u, w)); }
 };
 
 // Exact maximum of the edge wave speeds |u - w| + sqrt(g h) (Eq. alpha2D) of a block's cells, raised
@@ -522,9 +522,10 @@ struct OpenOut {
   uint32_t st;
   uint8_t flag;
 };
-// A cell whose smooth class the FP32 test leaves open (or whose widths are not moderate), out of
-// line: the mesh geometry with its checks, the FP64 detector and the edge values of its class.
-// A call, not inlined, so that this rare path's registers do not weigh on the smooth cells' code.
+// A cell of the non-well-balanced or special scheme whose smooth class the FP32 test leaves open (or
+// whose widths are not moderate), out of line: the mesh geometry with its checks, the FP64 detector and
+// the edge values of its class. A call, not inlined, so that this rare path's registers do not weigh
+// on the smooth cells' code.
 template <int SCHEME>
 __device__ __noinline__ OpenOut recon_open_cell(const SchemeConst P, const TileRows R, int i, double dxe) {
   swale::CellGeom G;
@@ -548,73 +549,70 @@ __device__ __noinline__ OpenOut recon_open_cell(const SchemeConst P, const TileR
   swale::cell_geom(h, dxe, G, r.st);
   if (SCHEME == 1) {
     swale::recon_cell_nonwb_g(P, G, v0, DD, r.o, r.flag, r.st, swale::nonwb_proj(P, v0));
-  } else if (SCHEME == 2) {
-    swale::recon_cell_special_g(P, G, h, v0, DD, r.o, r.flag, r.st, r.etaG);
   } else {
-    const double it[3] = {swale::triple_recip(h[0], h[1], h[2]), swale::triple_recip(h[1], h[2], h[3]),
-                          swale::triple_recip(h[2], h[3], h[4])};
-    swale::smooth_edge_coeffs(h, it, G);
-    swale::recon_cell_g(P, G, v0, DD, r.o, r.flag, r.st, false);
+    swale::recon_cell_special_g(P, G, h, v0, DD, r.o, r.flag, r.st, r.etaG);
   }
   return r;
 }
 
-// The step's alpha_1, dt and the secant factor of the prescribed motion, by one warp of the
-// instance's last stage-1 tile (every lane computes dt: an FP64 instruction costs the same for one
-// lane as for 32). The secant factor (sin(2 pi (t + dt) / T) - sin(2 pi t / T)) / dt is formed as
+// A step's dt and the secant factor of the prescribed motion from alpha_1, by whole warps (every
+// lane computes dt: an FP64 instruction costs the same for one lane as for 32). The secant factor
+// (sin(2 pi (t + dt) / T) - sin(2 pi t / T)) / dt is formed as
 // 2 cos(pi (2 t + dt) / T) sin(pi dt / T) / dt, which does not cancel, with the cosine and the sine in two lanes
-// of the same instructions.
+// of the same instructions. inv_T: 1 / T of the profile motion, 0 for the others.
+struct StepDt {
+  double dt, alpha1, sdiff;
+  int clipped, nodt;
+};
+__device__ __noinline__ StepDt step_dt(double cfl, double alpha1, double dwmax, double jmin, double tn, double dt_fixed,
+                                       double t_end, double inv_T) {
+  StepDt r{dt_fixed, alpha1, 0.0, 0, 0};
+  if (!(dt_fixed > 0.0)) {
+    // (zero and subnormal divisors take the division: the quotient is then infinite, or a NaN)
+    r.dt = alpha1 > 1e-290 ? cfl * jmin * swale::recip(alpha1) : cfl * jmin / alpha1;
+    if (dwmax > 0.0) r.dt = fmin(r.dt, dwmax > 1e-290 ? 0.5 * jmin * swale::recip(dwmax) : 0.5 * jmin / dwmax);
+  }
+  if (t_end > 0.0 && t_end - tn <= r.dt) {
+    r.dt = t_end - tn;
+    r.clipped = 1;
+  }
+  // alpha = 0 (a dry state at rest on a mesh that does not move) leaves the CFL condition
+  // with no bound; without an end time there is no step to take: dt = 0, flagged.
+  if (!(r.dt < INFINITY)) {
+    r.dt = 0.0;
+    r.nodt = 1;
+  }
+  if (inv_T > 0.0 && r.dt > 0.0) {
+    double sn, cs;
+    sincospi(((threadIdx.x & 31) == 0 ? 2.0 * tn + r.dt : r.dt) * inv_T, &sn, &cs);
+    const double cs0 = __shfl_sync(0xffffffffu, cs, 0), sn1 = __shfl_sync(0xffffffffu, sn, 1);
+    r.sdiff = 2.0 * cs0 * sn1 / r.dt;
+  }
+  return r;
+}
+
+// The same for the stage kernels, by one warp of the instance's last stage-1 tile.
 __device__ __forceinline__ void stage1_dt(const StepConst& K, DevScalars* S, const InstConst& ic, int inst) {
   __threadfence();
   const int lane = threadIdx.x & 31;
+  const bool fluid = K.mesh == SWALE_MESH_FLUID_GAUSS;
   const double A1 = bitsd(*(volatile const unsigned long long*)&S->A[0]);
-  double Wbar = S->Wbar, dwmax = 0.0;
-  if (K.mesh == SWALE_MESH_FLUID_GAUSS) {
-    Wbar = bitsd(*(volatile const unsigned long long*)&S->Wabs);
-    dwmax = bitsd(*(volatile const unsigned long long*)&S->dWabs);
-  }
+  const double Wbar = fluid ? bitsd(*(volatile const unsigned long long*)&S->Wabs) : S->Wbar;
+  const double dwmax = fluid ? bitsd(*(volatile const unsigned long long*)&S->dWabs) : 0.0;
   double alpha1 = K.wave_rel ? A1 : A1 + Wbar;
   if (K.alpha_mode != 0) {
     if (lane == 0) alpha1 = stage_alpha(K, inst, 1, alpha1, S->step_idx);
     alpha1 = __shfl_sync(0xffffffffu, alpha1, 0);
   }
-  const double tn = S->t;
-  double dt;
-  int clipped = 0;
-  bool nodt = false;
-  if (K.dt_fixed > 0.0) {
-    dt = K.dt_fixed;
-  } else {
-    // (zero and subnormal divisors take the division: the quotient is then infinite, or a NaN)
-    const double jmin = bitsd(S->Jmin0);
-    dt = alpha1 > 1e-290 ? ic.cfl * jmin * swale::recip(alpha1) : ic.cfl * jmin / alpha1;
-    if (K.mesh == SWALE_MESH_FLUID_GAUSS && dwmax > 0.0)
-      dt = fmin(dt, dwmax > 1e-290 ? 0.5 * jmin * swale::recip(dwmax) : 0.5 * jmin / dwmax);
-  }
-  if (K.t_end > 0.0 && K.t_end - tn <= dt) {
-    dt = K.t_end - tn;
-    clipped = 1;
-  }
-  // alpha = 0 (a dry state at rest on a mesh that does not move) leaves the CFL condition
-  // with no bound; without an end time there is no step to take: dt = 0, flagged.
-  if (!(dt < INFINITY)) {
-    dt = 0.0;
-    nodt = true;
-  }
-  double sdiff = 0.0;
-  if (K.mesh == SWALE_MESH_PROFILE && dt > 0.0) {
-    double sn, cs;
-    sincospi((lane == 0 ? 2.0 * tn + dt : dt) * K.inv_T, &sn, &cs);
-    const double cs0 = __shfl_sync(0xffffffffu, cs, 0), sn1 = __shfl_sync(0xffffffffu, sn, 1);
-    sdiff = 2.0 * cs0 * sn1 / dt;
-  }
+  const StepDt r = step_dt(ic.cfl, alpha1, dwmax, bitsd(S->Jmin0), S->t, K.dt_fixed, K.t_end,
+                           K.mesh == SWALE_MESH_PROFILE ? K.inv_T : 0.0);
   if (lane == 0) {
-    if (nodt) atomicOr(&S->status, (unsigned int)swale::ST_NODT);
-    if (K.mesh == SWALE_MESH_FLUID_GAUSS) S->Wbar = Wbar;
-    S->dt = dt;
-    S->alpha1 = alpha1;
-    S->clipped = clipped;
-    S->sdiff = sdiff;
+    if (r.nodt) atomicOr(&S->status, (unsigned int)swale::ST_NODT);
+    S->Wbar = Wbar;
+    S->dt = r.dt;
+    S->alpha1 = r.alpha1;
+    S->clipped = r.clipped;
+    S->sdiff = r.sdiff;
     S->counter = 0u;
   }
 }
@@ -622,20 +620,248 @@ __device__ __forceinline__ void stage1_dt(const StepConst& K, DevScalars* S, con
 // STOREK: an instantiation of the hydrostatic scheme that also stores each cell's smooth-class
 // linear form in D.gK (the adjoint's recomputes), so that the forward's own instantiations keep
 // their registers.
+// Shared rows of the phases. Every phase runs on all threads: the last rows hold nothing that a
+// reconstructed cell reads (they are padded for the reads past the block).
+template <int T, int SCHEME>
+struct ReconRows {
+  static constexpr int NV32 = SCHEME == 1 ? 3 : 2;
+  double H[T + 2], P[T + 2], Q[T];            // depths; pair and quadruple sums of widths
+  double D2[3][T + 2], D3[3][T + 2], D4[3][T];  // divided differences of eta, hu, h
+  // FP32 copies for the smooth-class test: widths, triple reciprocals, pair differences (hu, h, and
+  // for the non-well-balanced scheme eta)
+  float Jf[T], ITf[T], D2f[NV32][T];
+  // Hydrostatic scheme: the cells that the test leaves open, and their edge values [edge][variable][cell],
+  // classes and status bits.
+  static constexpr int TX = SCHEME == 0 ? T : 1;
+  double X[2][3][TX];
+  uint16_t open[TX];
+  uint8_t cls[TX], xst[TX];
+  int nopen;
+};
+// Reciprocal sums of the widths a thread takes from the mesh cache (see k_recon): `pair`, `next` say
+// which it has, `all_pair`, `all_next` whether its whole warp has them (no reciprocal is formed then).
+struct MeshRecips {
+  double ip, it, iq, iv;
+  bool pair, next, all_pair, all_next;
+};
+
+// The mesh checks of a cell whose widths are not moderate (see moderate_widths), as cell_geom makes them.
+__device__ __noinline__ uint32_t width_status(const double* J) {
+  double h[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) h[k] = J[k];
+  swale::CellGeom G;
+  uint32_t st = 0;
+  swale::cell_geom(h, h[2], G, st, false);
+  return st;
+}
+
+// Edge `right` of the open cell i of a block (hydrostatic scheme): its values into R.X, and (by the left
+// edge's thread) its class and status.
+// (A call: its registers do not weigh on the smooth cells' code.)
+template <int T, int SCHEME>
+__device__ __noinline__ void open_edge(const SchemeConst P, ReconRows<T, SCHEME>& R, const double* sE, const double* sM,
+                                          const double* sJ, int i, bool right, double dxmax) {
+  double h[5], p[4], v[3], d2[3][4], d3[3][3], d4[3][2], out[3];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) h[k] = sJ[i - 2 + k];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) p[k] = R.P[i - 2 + k];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    v[q] = (q == 0 ? sE : q == 1 ? sM : R.H)[i];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) d2[q][a] = R.D2[q][i - 2 + a];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) d3[q][a] = R.D3[q][i - 2 + a];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) d4[q][a] = R.D4[q][i - 2 + a];
+  }
+  // (the same sum as the quintuple's: the quadruple that starts at i - 2, and the last width)
+  const double iv = swale::recip(swale::add_(swale::add_(p[0], p[2]), h[4]));
+  const uint8_t flag = swale::open_edge_values(P, h, p, P.beta_dx_global ? dxmax : h[2], iv, v, d2, d3, d4, right, out);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) R.X[right ? 1 : 0][q][i] = out[q];
+  if (!right) {
+    R.cls[i] = flag;
+    R.xst[i] = (uint8_t)(swale::moderate_widths(R.Jf[i - 2], R.Jf[i - 1], R.Jf[i], R.Jf[i + 1], R.Jf[i + 2])
+                             ? 0u
+                             : width_status(sJ + i - 2));
+  }
+}
+
+// The reconstruction of a block's T cells, thread i holding cell i: width jv, averages ev, mv of eta
+// and hu, depth hv, also in the shared rows sE, sM, sJ (a barrier lies behind their stores). Threads
+// with mine set (2 <= i <= T - 3) get the limited edge state o, the class and, for the special scheme,
+// eta at the interior points. The sink is handed each thread's pair differences and reciprocals as
+// they are formed: pair(ip, de, dh), triple(it), quad(iq), quint(iv).
+template <int T, int SCHEME, class Sink>
+__device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, SCHEME>& R, const double* sE, const double* sM,
+                                             const double* sJ, double jv, double ev, double mv, double hv, double dxmax,
+                                             const MeshRecips& g, bool mine, Sink& sink, EdgeState& o, uint8_t& flag,
+                                             double etaG[2], uint32_t& st) {
+  const int tid = threadIdx.x;
+  R.H[tid] = hv;  // the depth is reconstructed in place of the bottom
+  R.Jf[tid] = swale::f32_trunc(jv);
+  if (SCHEME == 0 && tid == 0) R.nopen = 0;
+  __syncthreads();
+  // Order 2: the pair (i, i+1).
+  double d2[3], d3[3];
+  const double p = swale::add_(jv, sJ[tid + 1]);
+  {
+    const double de = swale::sub_(sE[tid + 1], ev), dm = swale::sub_(sM[tid + 1], mv), dh = swale::sub_(R.H[tid + 1], hv);
+    double ip = g.ip;
+    if (!g.all_pair) ip = g.pair ? g.ip : swale::recip(p);
+    d2[0] = swale::mul_(de, ip);
+    d2[1] = swale::mul_(dm, ip);
+    d2[2] = swale::mul_(dh, ip);
+    R.P[tid] = p;
+#pragma unroll
+    for (int v = 0; v < 3; ++v) R.D2[v][tid] = d2[v];
+    R.D2f[0][tid] = swale::f32_trunc(d2[1]);
+    R.D2f[1][tid] = swale::f32_trunc(d2[2]);
+    if (SCHEME == 1) R.D2f[R.NV32 - 1][tid] = swale::f32_trunc(d2[0]);
+    sink.pair(ip, de, dh);
+  }
+  __syncthreads();
+  // Order 3: the triple (i, i+1, i+2).
+  {
+    double it = g.it;
+    if (!g.all_next) it = g.next ? g.it : swale::recip(swale::add_(p, sJ[tid + 2]));
+#pragma unroll
+    for (int v = 0; v < 3; ++v) R.D3[v][tid] = d3[v] = swale::mul_(swale::sub_(R.D2[v][tid + 1], d2[v]), it);
+    R.ITf[tid] = swale::f32_trunc(it);
+    sink.triple(it);
+  }
+  __syncthreads();
+  // Order 4: the quadruple (i .. i+3).
+  {
+    double iq = g.iq;
+    if (!g.all_pair || !g.all_next) {  // (the quintuple's sum needs it where that is not cached)
+      const double q = swale::add_(p, R.P[tid + 2]);
+      R.Q[tid] = q;
+      iq = g.next ? g.iq : swale::recip(q);
+    }
+#pragma unroll
+    for (int v = 0; v < 3; ++v) R.D4[v][tid] = swale::mul_(swale::sub_(R.D3[v][tid + 1], d3[v]), iq);
+    sink.quad(iq);
+  }
+  const double dxe = P.beta_dx_global ? dxmax : jv;
+  flag = 0;
+  // The smooth class, when FP32 can tell it for sure; else the FP64 detector decides.
+  bool smooth = false;
+  if (mine) {
+    if (!swale::gt0(jv)) st |= swale::ST_EMESH;
+    const float hf[5] = {R.Jf[tid - 2], R.Jf[tid - 1], R.Jf[tid], R.Jf[tid + 1], R.Jf[tid + 2]};
+    float F32[3], itf[3], c4f, c3f, d2h[4], d2m[4];
+    swale::indicator_factors_f32(hf, swale::f32_trunc(dxe), F32, c4f, c3f);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) itf[a] = R.ITf[tid - 2 + a];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      d2h[a] = R.D2f[1][tid - 2 + a];
+      d2m[a] = R.D2f[0][tid - 2 + a];
+    }
+    const float epsf = swale::f32_trunc(P.eps_weno);
+    if (SCHEME == 1) {
+      float d2e[4];
+#pragma unroll
+      for (int a = 0; a < 4; ++a) d2e[a] = R.D2f[R.NV32 - 1][tid - 2 + a];
+      smooth = swale::sure_smooth_nonwb_f32(P.g, P.h_dry, hv, mv, F32, c4f, c3f, d2e, d2m, d2h, itf, epsf);
+    } else {
+      smooth = swale::sure_smooth_f32(F32, c4f, c3f, d2h, d2m, itf, epsf);
+    }
+    smooth = smooth && swale::moderate_widths(hf[0], hf[1], hf[2], hf[3], hf[4]);
+  }
+  // The open cells of the hydrostatic scheme: an FP64 instruction costs a warp the same for one lane
+  // as for 32, so they are gathered and spread over the block's threads, two to a cell (one per edge),
+  // instead of taking their own warps one by one through about twice the work. (The barrier is the
+  // one that the differences of order 4 need anyway.)
+  const bool open = SCHEME == 0 && mine && !smooth;
+  if (open) R.open[atomicAdd(&R.nopen, 1)] = (uint16_t)tid;
+  if (__syncthreads_or(open)) {
+    const int n2 = 2 * R.nopen;
+    for (int e = tid; e < n2; e += T) open_edge<T, SCHEME>(P, R, sE, sM, sJ, R.open[e >> 1], e & 1, dxmax);
+    __syncthreads();
+  }
+  if (!mine) return;
+  // Order 5, the quintuple centred at i.
+  double iv = g.iv;
+  if (!g.all_pair) iv = g.pair ? g.iv : swale::recip(swale::add_(R.Q[tid - 2], sJ[tid + 2]));
+  sink.quint(iv);
+  if (SCHEME != 0 && !smooth) {
+    const TileRows rows = {sJ, sE, sM, R.H, &R.D2[0][0], &R.D3[0][0], T + 2};
+    const OpenOut r = recon_open_cell<SCHEME>(P, rows, tid, dxe);
+    o = r.o;
+    flag = r.flag;
+    etaG[0] = r.etaG[0];
+    etaG[1] = r.etaG[1];
+    st |= r.st;
+    return;
+  }
+  double evl[3][2];
+  if (smooth) {
+    const swale::SmoothWidths w = {sJ[tid - 1], jv, sJ[tid + 1], R.P[tid - 2], R.P[tid - 1], p, R.P[tid + 1]};
+    const double vj[3] = {ev, mv, hv};
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      const double d4l = R.D4[v][tid - 2], d4r = R.D4[v][tid - 1], d3c = R.D3[v][tid - 1];
+      const double d5 = swale::mul_(swale::sub_(d4r, d4l), iv);
+      evl[v][0] = swale::smooth_left(w, vj[v], R.D2[v][tid - 1], d3c, d4l, d5);
+      evl[v][1] = swale::smooth_right(w, vj[v], d2[v], d3c, d4r, d5);
+      if (SCHEME == 2 && v == 0) {
+        etaG[0] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T1, ev, d2[v], d3c, d4r, d5);
+        etaG[1] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T2, ev, d2[v], d3c, d4r, d5);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int v = 0; v < 3; ++v) {
+      evl[v][0] = R.X[0][v][tid];
+      evl[v][1] = R.X[1][v][tid];
+    }
+    flag = R.cls[tid];
+    st |= R.xst[tid];
+  }
+  swale::limit_cell(P, evl, hv, mv, o, st);
+}
+
+// Where k_recon's differences and reciprocals go: the arrays that the update of the stage reads and, in
+// stage 2, the mesh cache.
+template <int STAGE, int SCHEME>
+struct ReconSink {
+  const DevState& D;
+  int32_t idx;      // edge-array index of the thread's cell
+  bool mine, next_mine, use_geo;
+  double hv;
+  __device__ __forceinline__ void pair(double ip, double de, double dh) const {
+    if (!mine) return;
+    if (SCHEME == 2 || !use_geo) D.ipair[idx] = ip;  // (on the cache the update needs neither)
+    D.dE[idx] = de;
+    D.dH[idx] = dh;
+    D.H[idx] = hv;
+    if (STAGE == 2 && D.geo) D.geo[GEO_IP * D.geo_stride + idx] = ip;
+  }
+  __device__ __forceinline__ void triple(double it) const {
+    if (!next_mine) return;
+    if (SCHEME == 2 || !use_geo) D.itri[idx + 1] = it;
+    if (STAGE == 2 && D.geo) D.geo[GEO_IT * D.geo_stride + idx + 1] = it;
+  }
+  __device__ __forceinline__ void quad(double iq) const {
+    if (STAGE == 2 && D.geo && next_mine) D.geo[GEO_IQ * D.geo_stride + idx + 1] = iq;
+  }
+  __device__ __forceinline__ void quint(double iv) const {
+    if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = iv;
+  }
+};
+
 template <int STAGE, int T, int SCHEME = 0, bool STOREK = false>
 __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, DevState D, const double* __restrict__ Eg,
                                              const double* __restrict__ Mg, const double* __restrict__ Bg,
                                              const double* __restrict__ Jg) {
   constexpr int TO = T - 4;                        // cells reconstructed
   __shared__ __align__(16) double sRaw[4][T + 8];  // E, M, B, J of cells c0-2 .. c0+T-3 as bulk-copied
-  // Depths; pair and quadruple sums of widths; differences. Every phase runs on all threads: the
-  // last rows of each hold nothing that a reconstructed cell reads (the rows are padded for them).
-  __shared__ double sH[T + 2], sP[T + 2], sQ[T];
-  __shared__ double sD2[3][T + 2], sD3[3][T + 2], sD4[3][T];
-  // FP32 copies for the smooth-class test: widths, triple reciprocals, pair differences (hu, h, and
-  // for the non-well-balanced scheme eta)
-  constexpr int NV32 = SCHEME == 1 ? 3 : 2;
-  __shared__ float sJf[T], sITf[T], sD2f[NV32][T];
+  __shared__ ReconRows<T, SCHEME> rows;
   __shared__ bool sIdle;
   __shared__ __align__(8) uint64_t sBar;           // completion of the tile's bulk copies
   __shared__ __align__(8) uint64_t sPad;           // test hook: a barrier no copy completes
@@ -686,17 +912,18 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     // formed below. Those that lie at cells -1..N are in the cache: the pair starting at c, the triple
     // and quadruple whose second cell is c + 1, the quintuple centred at c.
     const bool use_geo = STAGE == 1 && D.geo != nullptr && S->geo_tag == geo_now;
-    const bool g_pair = use_geo && c >= -1 && c <= N, g_next = use_geo && c >= -2 && c + 1 <= N;
-    const bool all_pair = STAGE == 1 && __all_sync(0xffffffffu, g_pair);  // (a vote: no reciprocal is formed then)
-    const bool all_next = STAGE == 1 && __all_sync(0xffffffffu, g_next);
-    double gip = 0.0, git = 0.0, giq = 0.0, giv = 0.0;
-    if (STAGE == 1 && g_pair) {
-      gip = D.geo[GEO_IP * D.geo_stride + idx];
-      giv = D.geo[GEO_IV * D.geo_stride + idx];
-    }
-    if (STAGE == 1 && g_next) {
-      git = D.geo[GEO_IT * D.geo_stride + idx + 1];
-      giq = D.geo[GEO_IQ * D.geo_stride + idx + 1];
+    MeshRecips mr{0.0, 0.0, 0.0, 0.0, use_geo && c >= -1 && c <= N, use_geo && c >= -2 && c + 1 <= N, false, false};
+    if (STAGE == 1) {
+      mr.all_pair = __all_sync(0xffffffffu, mr.pair);
+      mr.all_next = __all_sync(0xffffffffu, mr.next);
+      if (mr.pair) {
+        mr.ip = D.geo[GEO_IP * D.geo_stride + idx];
+        mr.iv = D.geo[GEO_IV * D.geo_stride + idx];
+      }
+      if (mr.next) {
+        mr.it = D.geo[GEO_IT * D.geo_stride + idx + 1];
+        mr.iq = D.geo[GEO_IQ * D.geo_stride + idx + 1];
+      }
     }
     const double seen = bitsd(*(volatile const unsigned long long*)&S->A[STAGE - 1]);
     const double dxmax = bitsd(S->Jmax[STAGE - 1]);
@@ -744,7 +971,7 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
       ev = sE[tid];
       mv = sM[tid];
       jv = sJ[tid];
-      hv = ev - sRaw[2][off + tid];
+      hv = swale::sub_(ev, sRaw[2][off + tid]);
     } else {
       if (c >= -3 && c <= N + 2) {
         const int32_t s = ghost(c, N, K.bc);
@@ -752,135 +979,26 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
         ev = E[s];
         mv = M[s];
         if (refl && (c < 0 || c >= N)) mv = -mv;
-        hv = ev - B[s];
+        hv = swale::sub_(ev, B[s]);
       }
       sE[tid] = ev;
       sM[tid] = mv;
       sJ[tid] = jv;
     }
-    sH[tid] = hv;  // the depth is reconstructed in place of the bottom
-    sJf[tid] = swale::f32_trunc(jv);
-    __syncthreads();
     // Cells of the tile that are reconstructed and stored.
     const bool mine = tid >= 2 && tid < 2 + TO && c <= N;
     const bool next_mine = tid >= 1 && tid < 1 + TO && c + 1 <= N;  // cell c + 1 is
-    // Order 2: the pair (c, c+1).
-    double d2[3];
-    const double p = jv + sJ[tid + 1];
-    {
-      const double de = sE[tid + 1] - ev, dm = sM[tid + 1] - mv, dh = sH[tid + 1] - hv;
-      double ip = gip;
-      if (!all_pair) ip = g_pair ? gip : swale::recip(p);
-      d2[0] = de * ip;
-      d2[1] = dm * ip;
-      d2[2] = dh * ip;
-      sP[tid] = p;
-#pragma unroll
-      for (int v = 0; v < 3; ++v) sD2[v][tid] = d2[v];
-      sD2f[0][tid] = swale::f32_trunc(d2[1]);
-      sD2f[1][tid] = swale::f32_trunc(d2[2]);
-      if (SCHEME == 1) sD2f[NV32 - 1][tid] = swale::f32_trunc(d2[0]);
-      if (mine) {
-        if (SCHEME == 2 || !use_geo) D.ipair[idx] = ip;  // (on the cache the update needs neither)
-        D.dE[idx] = de;
-        D.dH[idx] = dh;
-        D.H[idx] = hv;
-        if (STAGE == 2 && D.geo) D.geo[GEO_IP * D.geo_stride + idx] = ip;
-      }
-    }
-    __syncthreads();
-    // Order 3: the triple (c, c+1, c+2).
-    double d3[3];
-    {
-      double it = git;
-      if (!all_next) it = g_next ? git : swale::recip(p + sJ[tid + 2]);
-#pragma unroll
-      for (int v = 0; v < 3; ++v) sD3[v][tid] = d3[v] = (sD2[v][tid + 1] - d2[v]) * it;
-      sITf[tid] = swale::f32_trunc(it);
-      if (next_mine) {
-        if (SCHEME == 2 || !use_geo) D.itri[idx + 1] = it;
-        if (STAGE == 2 && D.geo) D.geo[GEO_IT * D.geo_stride + idx + 1] = it;
-      }
-    }
-    __syncthreads();
-    // Order 4: the quadruple (c .. c+3).
-    {
-      double iq = giq;
-      if (!all_pair || !all_next) {  // (the quintuple's sum needs it where that is not cached)
-        const double q = p + sP[tid + 2];
-        sQ[tid] = q;
-        iq = g_next ? giq : swale::recip(q);
-      }
-#pragma unroll
-      for (int v = 0; v < 3; ++v) sD4[v][tid] = (sD3[v][tid + 1] - d3[v]) * iq;
-      if (STAGE == 2 && D.geo && next_mine) D.geo[GEO_IQ * D.geo_stride + idx + 1] = iq;
-    }
-    __syncthreads();
+    ReconSink<STAGE, SCHEME> sink{D, idx, mine, next_mine, use_geo, hv};
+    EdgeState o;
+    uint8_t flag = 0;
+    double etaG[2] = {0.0, 0.0};
+    uint32_t st = 0;
+    recon_phases<T, SCHEME>(K.sc, rows, sE, sM, sJ, jv, ev, mv, hv, dxmax, mr, mine, sink, o, flag, etaG, st);
     if (STAGE == 2 && D.geo != nullptr && c0 == -1 && tid == 0)
       S->geo_tag = ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)((S->step_idx + 1) & 0xffffffffLL);
     WaveEdge eL{0.0, 0.0, 0.0}, eR{0.0, 0.0, 0.0};
     bool useL = false, useR = false;
-    uint32_t st = 0;
     if (mine) {
-      const double dxe = K.sc.beta_dx_global ? dxmax : jv;
-      if (!swale::gt0(jv)) st |= swale::ST_EMESH;
-      EdgeState o;
-      uint8_t flag = 0;
-      double etaG[2] = {0.0, 0.0};
-      // The smooth class, when FP32 can tell it for sure; else the FP64 detector decides.
-      bool smooth;
-      {
-        const float hf[5] = {sJf[tid - 2], sJf[tid - 1], sJf[tid], sJf[tid + 1], sJf[tid + 2]};
-        float F32[3], itf[3], c4f, c3f, d2h[4], d2m[4];
-        swale::indicator_factors_f32(hf, swale::f32_trunc(dxe), F32, c4f, c3f);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) itf[a] = sITf[tid - 2 + a];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          d2h[a] = sD2f[1][tid - 2 + a];
-          d2m[a] = sD2f[0][tid - 2 + a];
-        }
-        const float epsf = swale::f32_trunc(K.sc.eps_weno);
-        if (SCHEME == 1) {
-          float d2e[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) d2e[a] = sD2f[NV32 - 1][tid - 2 + a];
-          smooth = swale::sure_smooth_nonwb_f32(K.sc.g, K.sc.h_dry, hv, mv, F32, c4f, c3f, d2e, d2m, d2h, itf, epsf);
-        } else {
-          smooth = swale::sure_smooth_f32(F32, c4f, c3f, d2h, d2m, itf, epsf);
-        }
-        smooth = smooth && swale::moderate_widths(hf[0], hf[1], hf[2], hf[3], hf[4]);
-      }
-      if (smooth) {
-        // Order 5, the quintuple centred at c, and the edge values.
-        const swale::SmoothWidths w = {sJ[tid - 1], jv, sJ[tid + 1], sP[tid - 2], sP[tid - 1], p, sP[tid + 1]};
-        double iv = giv;
-        if (!all_pair) iv = g_pair ? giv : swale::recip(sQ[tid - 2] + sJ[tid + 2]);
-        if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = iv;
-        const double vj[3] = {ev, mv, hv};
-        double evl[3][2];
-#pragma unroll
-        for (int v = 0; v < 3; ++v) {
-          const double d4l = sD4[v][tid - 2], d4r = sD4[v][tid - 1], d3c = sD3[v][tid - 1];
-          const double d5 = (d4r - d4l) * iv;
-          evl[v][0] = swale::smooth_left(w, vj[v], sD2[v][tid - 1], d3c, d4l, d5);
-          evl[v][1] = swale::smooth_right(w, vj[v], d2[v], d3c, d4r, d5);
-          if (SCHEME == 2 && v == 0) {
-            etaG[0] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T1, ev, d2[v], d3c, d4r, d5);
-            etaG[1] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T2, ev, d2[v], d3c, d4r, d5);
-          }
-        }
-        swale::limit_cell(K.sc, evl, hv, mv, o, st);
-      } else {
-        if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = swale::recip(sQ[tid - 2] + sJ[tid + 2]);
-        const TileRows R = {sJ, sE, sM, sH, &sD2[0][0], &sD3[0][0], T + 2};
-        const OpenOut r = recon_open_cell<SCHEME>(K.sc, R, tid, dxe);
-        o = r.o;
-        flag = r.flag;
-        etaG[0] = r.etaG[0];
-        etaG[1] = r.etaG[1];
-        st |= r.st;
-      }
       if (STOREK) {
         double h[5], K8[2][4];
         swale::CellGeom G;
@@ -889,7 +1007,7 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
         for (int k = 0; k < 5; ++k) h[k] = sJ[tid - 2 + k];
         const double it3[3] = {swale::triple_recip(h[0], h[1], h[2]), swale::triple_recip(h[1], h[2], h[3]),
                                swale::triple_recip(h[2], h[3], h[4])};
-        swale::cell_geom(h, dxe, G, stk, false);
+        swale::cell_geom(h, jv, G, stk, false);
         swale::linear_edge_form(G.d, G.G1, G.G2, h, it3, K8);
 #pragma unroll
         for (int k = 0; k < 8; ++k) D.gK[k * D.geo_stride + idx] = K8[k >> 2][k & 3];
@@ -955,10 +1073,10 @@ struct RhsOut {
 // L2-projection bottom. STOREK: one that also stores the old source form's entries in D.gK (the
 // adjoint's recomputes).
 
-// Largest a and b and smallest c over the block (non-negative doubles), raised / lowered into their
-// destinations by three lanes after a single barrier.
-template <int T>
-__device__ __forceinline__ void block_widths(DevScalars* S, double a, double b, double c) {
+// Largest a and b over the block (non-negative doubles), raised into mx[0], mx[1], and the smallest c,
+// lowered into *mn (or, with COMPL, its complement raised there), by three lanes after one barrier.
+template <int T, bool COMPL>
+__device__ __forceinline__ void block_widths(unsigned long long* mx, unsigned long long* mn, double a, double b, double c) {
   __shared__ unsigned long long red[3][T / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned long long ma = warp_umax64(dbits(a)), mb = warp_umax64(dbits(b)), mc = warp_umax64(~dbits(c));
@@ -968,12 +1086,9 @@ __device__ __forceinline__ void block_widths(DevScalars* S, double a, double b, 
     unsigned long long m = 0ull;
 #pragma unroll
     for (int w = 0; w < T / 32; ++w) m = umax64(m, red[threadIdx.x][w]);
-    if (threadIdx.x < 2) {
-      raise_to(&S->Jmax[1 + threadIdx.x], m);
-    } else {
-      m = ~m;
-      if (m < *(volatile const unsigned long long*)&S->JminN) atomicMin(&S->JminN, m);
-    }
+    if (threadIdx.x < 2) raise_to(mx + threadIdx.x, m);
+    else if (COMPL) raise_to(mn, m);
+    else if (~m < *(volatile const unsigned long long*)mn) atomicMin(mn, ~m);
   }
 }
 
@@ -1027,7 +1142,7 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     double wk = 0.0, ELj = 0.0, BLj = 0.0, hLj = 0.0, dE = 0.0, dH = 0.0;
     if (k <= N) {
       if (fresh_w) {
-        wk = D.P[nb + k] * sdiff;
+        wk = swale::mul_(D.P[nb + k], sdiff);
       } else if (MODE == 0 && K.mesh == SWALE_MESH_STATIC) {
         wk = 0.0;
       } else if (MODE == 0 && K.mesh == SWALE_MESH_LINEAR) {
@@ -1086,7 +1201,8 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     if (tid < TC && j < N) {
       const double ERj = D.eER[er], BRj = D.eBR[er], hRj = D.ehR[er];
       const double hj = D.H[er], Ej = E[j];
-      double Sp;  // twice the pressure and source terms of the momentum (the source alone: special scheme)
+      // Twice the momentum's right-hand side: the fluxes, then the pressure and source terms.
+      double Rm = swale::sub_(F.FMr, sF[1][tid + 1]);
       const double Jm = use_sgeo && SCHEME != 2 ? 0.0 : Js[ghost(j - 1, N, K.bc)];
       const double Jc = use_sgeo && SCHEME != 2 ? 0.0 : Js[j];
       const double Jp = use_sgeo && SCHEME != 2 ? 0.0 : Js[ghost(j + 1, N, K.bc)];
@@ -1095,7 +1211,7 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
         const swale::SourceGeom sg =
             swale::source_geom(Jm, Jc, swale::recip(Jm), swale::recip(Jc), swale::recip(Jp), D.ipair[el], D.ipair[er], D.itri[er]);
         const double eta4[4] = {ELj, D.eG1[er], D.eG2[er], ERj};
-        Sp = 2.0 * swale::source_cell_special(K.sc.g, Ej, eta4, bd, sg, D.eBR[er - 1], D.eBL[er + 1]);
+        Rm = swale::fma_(2.0, swale::source_cell_special(K.sc.g, Ej, eta4, bd, sg, D.eBR[er - 1], D.eBL[er + 1]), Rm);
       } else {
         swale::SourceRatio sr;
         if (use_sgeo) {
@@ -1127,13 +1243,13 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
 #pragma unroll
           for (int q = 0; q < 6; ++q) D.gK[(8 + q) * D.geo_stride + er] = src6[q];
         }
-        const double acc = swale::source_pressure_form(hj, hLj, hRj, ELj - Ej, ERj - Ej, dE, dH, sDe[0][tid + 1],
+        const double acc = swale::source_pressure_form(hj, hLj, hRj, swale::sub_(ELj, Ej), swale::sub_(ERj, Ej), dE, dH, sDe[0][tid + 1],
                                                        sDe[1][tid + 1], pr.rho, pr.sig2, sG[0][tid + 1],
                                                        sG[1][tid + 1], sr);
-        Sp = -K.sc.g * acc;
+        Rm = swale::fma_(-K.sc.g, acc, Rm);
       }
       // Twice the right-hand sides.
-      const double R2[3] = {F.FE - sF[0][tid + 1], (F.FMr - sF[1][tid + 1]) + Sp, sF[2][tid + 1] - F.FB};
+      const double R2[3] = {swale::sub_(F.FE, sF[0][tid + 1]), Rm, swale::sub_(sF[2][tid + 1], F.FB)};
       if (MODE == 1) {
         ro.RE[j] = 0.5 * R2[0];
         ro.RM[j] = 0.5 * R2[1];
@@ -1142,10 +1258,10 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
         const int32_t g = (int32_t)cb + j;  // global cell index
         const double wl = wk, wr = sW[tid + 1];
         const double J0 = D.J0[g];
-        const double dJ = dt * (wr - wl);
+        const double dJ = swale::mul_(dt, swale::sub_(wr, wl));
         const double q0[3] = {D.E0[g], D.M0[g], D.B0[g]};
         if (STAGE == 1) {
-          const double J1 = J0 + dJ, J2 = J0 + 0.5 * dJ;
+          const double J1 = swale::add_(J0, dJ), J2 = swale::fma_(0.5, dJ, J0);
           D.J1[g] = J1;
           D.J2[g] = J2;
           jmaxa = J1;
@@ -1164,7 +1280,7 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
           else  // bottom of stage 2: projection onto the mesh at t_{n+1}
             D.Ba[g] = bottom_average(K, D.x[nb + j] + dt * wl, D.x[nb + j + 1] + dt * wr);
         } else if (STAGE == 2) {
-          const double Y[3] = {D.YE[g] + R2[0], D.YM[g] + R2[1], D.YB[g] + R2[2]};
+          const double Y[3] = {swale::add_(D.YE[g], R2[0]), swale::add_(D.YM[g], R2[1]), swale::add_(D.YB[g], R2[2])};
           D.YE[g] = Y[0];
           D.YM[g] = Y[1];
           D.YB[g] = Y[2];
@@ -1192,9 +1308,9 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
             if (j == N - 1) D.bx[nb + N] = D.x[nb + N];
           }
           const double tdt = dt * (1.0 / 12.0);
-          const double En = swale::rk_advance(q0[0], tdt, 4.0 * R2[0] + D.YE[g], dJ, inv);
-          const double Mn = swale::rk_advance(q0[1], tdt, 4.0 * R2[1] + D.YM[g], dJ, inv);
-          double Bn = swale::rk_advance(q0[2], tdt, 4.0 * R2[2] + D.YB[g], dJ, inv);
+          const double En = swale::rk_advance(q0[0], tdt, swale::fma_(4.0, R2[0], D.YE[g]), dJ, inv);
+          const double Mn = swale::rk_advance(q0[1], tdt, swale::fma_(4.0, R2[1], D.YM[g]), dJ, inv);
+          double Bn = swale::rk_advance(q0[2], tdt, swale::fma_(4.0, R2[2], D.YB[g]), dJ, inv);
           if (BOT) {  // bottom after the step: projection onto the mesh at t_{n+1}
             const double xl = D.xn[nb + j], xr = D.xn[nb + j + 1];
             if (swale::bad(Bn)) st |= swale::ST_NONFINITE;
@@ -1202,8 +1318,8 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
             D.x[nb + j] = xl;
             if (j == N - 1) D.x[nb + N] = xr;
           } else {
-            D.x[nb + j] += dt * wl;
-            if (j == N - 1) D.x[nb + N] += dt * wr;
+            D.x[nb + j] = swale::fma_(dt, wl, D.x[nb + j]);
+            if (j == N - 1) D.x[nb + N] = swale::fma_(dt, wr, D.x[nb + N]);
           }
           D.E0[g] = En;
           D.M0[g] = Mn;
@@ -1215,7 +1331,7 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     }
     if (MODE == 0) {
       block_or_status(STAGE == 3 ? &S->st3 : &S->status, st);
-      if (STAGE == 1) block_widths<T>(S, jmaxa, jmaxb, jminb);
+      if (STAGE == 1) block_widths<T, false>(&S->Jmax[1], &S->JminN, jmaxa, jmaxb, jminb);
     }
     __syncthreads();  // this tile's reads of the shared rows come before the next tile's writes
   }

@@ -1,0 +1,383 @@
+// Whole SSP-RK3 steps in one launch, for meshes that leave most of the GPU idle: there a step of the
+// stage kernels is nine dependent launches of about ten microseconds each, most of it launch, load
+// and barrier latency. Here the cells stay in registers across stages and steps.
+#pragma once
+
+#include "swale_kernels.cuh"
+
+namespace swale_dev {
+
+constexpr int kStepThreads = 128;
+constexpr int kStepCells = kStepThreads - 6;  // cells a block owns: three on each side are its neighbours'
+
+// Per-instance scratch of k_steps, zero at its launch. The maxima and status words of a step live in
+// set (step mod 3); the next but one is cleared while a step runs.
+struct StepScratch {
+  unsigned int arrived;  // barrier arrivals since the launch
+  unsigned int pad_;
+  unsigned long long mx[3][6];  // A of the three stages, max J^(1), max J^(2), complement of min J^(1)
+  unsigned int st[3][6];        // status bits raised before each of the step's barriers
+};
+
+// Barrier of the nb blocks of an instance: arrivals are counted in global memory and every block
+// waits until all have come. All blocks are resident (a cooperative launch), so the wait ends; it is
+// bounded all the same (kBarrierTries polls, seconds) and returns false if it gives up.
+constexpr int kBarrierTries = 1 << 22;
+__device__ __forceinline__ bool inst_barrier(unsigned int* arrived, unsigned int nb, unsigned int& target) {
+  target += nb;
+  if (nb == 1) {
+    __syncthreads();
+    return true;
+  }
+  __shared__ bool ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
+    bool got = false;
+    for (int i = 0; i < kBarrierTries && !got; ++i) {
+      unsigned int v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
+      got = (int)(v - target) >= 0;
+    }
+    __threadfence();
+    ok = got;
+  }
+  __syncthreads();
+  return ok;
+}
+
+// Pair differences and reciprocals kept in the thread's registers.
+struct StepSink {
+  double ip, it, iq, iv, de, dh;
+  __device__ __forceinline__ void pair(double a, double b, double c) {
+    ip = a;
+    de = b;
+    dh = c;
+  }
+  __device__ __forceinline__ void triple(double a) { it = a; }
+  __device__ __forceinline__ void quad(double a) { iq = a; }
+  __device__ __forceinline__ void quint(double a) { iv = a; }
+};
+
+// nsteps steps of every instance (fewer where it reaches t_end or stops on an error), the same
+// arithmetic as the stage kernels, bit for bit. Block (instance, b) owns the cells b * 122 .. and keeps
+// their state in registers, one cell per thread; per stage it reads three cells on either side
+// from its neighbours (through L2), reconstructs one of them, so that the fluxes need no exchange,
+// and meets the other blocks of the instance twice: after the wave speeds (alpha), and after the new
+// stage values. Bound by the chain of a warp's FP64 instructions (64 cycles each, whatever the
+// number of warps or lanes) and by the six barriers. One block per SM runs a warp on each
+// sub-partition; hydrostatic and non-well-balanced schemes, static, profile and linear motion.
+template <int SCHEME>
+__global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState D, StepScratch* scratch, const Tile* blocks,
+                                                           int wave_rel1, long long nsteps) {
+  constexpr int T = kStepThreads;
+  __shared__ double rE[T + 8], rM[T + 8], rJ[T + 8];
+  __shared__ ReconRows<T, SCHEME> rows;
+  __shared__ double sR[4][T], sPair[4][T];  // right edges (eta, b, h, u); ip, it, de, dh of the pair that starts there
+  __shared__ double sF[3][T], sG[2][T], sW[T + 1], sI[T];
+  const int tid = threadIdx.x;
+  const Tile tl = blocks ? blocks[blockIdx.x] : Tile{0, (int32_t)blockIdx.x};
+  const InstConst ic = blocks ? D.IC[tl.inst] : D.ic1;
+  DevScalars* S = D.S + tl.inst;
+  StepScratch* X = scratch + tl.inst;
+  const int32_t N = (int32_t)ic.N;
+  const unsigned int nb = (unsigned)((N + kStepCells - 1) / kStepCells);
+  unsigned int target = 0;
+  const int32_t c = tl.c0 * kStepCells - 3 + tid;  // this thread's cell, and its left node
+  const int64_t cb = ic.coff, nbase = ic.coff + tl.inst;
+  const int32_t idx = (int32_t)(ic.coff + 2 * (int64_t)tl.inst) + c + 1;
+  const bool in_own = tid >= 3 && tid < T - 3;
+  const bool own = in_own && c < N;
+  const bool has_node = c >= 0 && c <= N;
+  const bool own_node = own || (c == N && tid >= 4 && tid <= T - 3);
+  const bool mine = tid >= 2 && tid < T - 2 && c <= N;  // reconstructed
+  const bool face = tid >= 3 && tid < T - 2 && c <= N;  // left interface of an owned cell, or the last one
+  const bool real_cell = c >= -3 && c <= N + 2;
+  const int32_t g = (int32_t)cb + (real_cell ? ghost(c, N, K.bc) : 0);  // where the cell's values come from
+  const bool flip = K.bc == SWALE_BC_REFLECTIVE && (c < 0 || c >= N);
+  const bool moving = K.mesh != SWALE_MESH_STATIC;
+
+  // State at t_n.
+  double q0[3] = {0.0, 0.0, 0.0}, J0 = 1.0, x = 0.0, Pn = 0.0, w = 0.0;
+  if (own) {
+    q0[0] = D.E0[g];
+    q0[1] = D.M0[g];
+    q0[2] = D.B0[g];
+    J0 = D.J0[g];
+  }
+  if (has_node) {
+    x = D.x[nbase + c];
+    Pn = D.P[nbase + c];
+  }
+  if (K.mesh == SWALE_MESH_LINEAR) w = Pn;
+  double tn = S->t, jmax = bitsd(S->JmaxN), jmin = bitsd(S->JminN);
+  const double Wbar = S->Wbar;
+  long long taken = 0;
+  unsigned int bits = 0;
+  bool timeout = false;
+  int done = 0;
+  StepDt sd{S->dt, S->alpha1, S->sdiff, 0, 0};
+  double amax[3] = {0.0, 0.0, 0.0}, jm1 = jmax, jm2 = jmax;
+  if (S->status & kErrBits) done = 1;
+  // Mesh-only values, kept from stage 2 for the next step's stage 1 (the same mesh; every stage of a
+  // static one).
+  MeshRecips mr{0.0, 0.0, 0.0, 0.0, false, false, false, false};
+  swale::PairRatio kept_pr{0.0, 0.0, 0.0, 0.0};
+  swale::SourceRatio kept_sr{0.0, 0.0, 0.0};
+  double iJ0 = 1.0;  // 1 / J^n of the thread's cell
+  bool have_mesh = false;
+
+  while (taken < nsteps && !done) {
+    if (K.t_end > 0.0 && tn >= K.t_end) {
+      done = 1;
+      break;
+    }
+    const int set = (int)(taken % 3);
+    double qs[3] = {q0[0], q0[1], q0[2]}, Js = J0, iJs = iJ0, J1 = J0, iJ1 = iJ0, dJ = 0.0, Y[3] = {0.0, 0.0, 0.0};
+    unsigned int err = 0;
+#pragma unroll 1
+    for (int stage = 1; stage <= 3; ++stage) {
+      // The stage's cells: owned ones from registers, the others as their owners (or images) have them.
+      double ev = qs[0], mv = qs[1], bv = qs[2], jv = Js, iv = iJs;
+      if (!own) {
+        ev = mv = bv = 0.0;
+        jv = 1.0;  // filler beyond the last ghost cell
+        iv = 1.0;
+        if (real_cell) {
+          const double *gE = D.E0, *gM = D.M0, *gB = D.B0, *gJ = D.J0;
+          if (stage == 2) {
+            gE = D.Ea;
+            gM = D.Ma;
+            gB = D.Ba;
+            gJ = D.J1;
+          } else if (stage == 3) {
+            gE = D.Eb;
+            gM = D.Mb;
+            gB = D.Bb;
+            gJ = D.J2;
+          }
+          ev = __ldcg(gE + g);
+          mv = __ldcg(gM + g);
+          bv = __ldcg(gB + g);
+          jv = __ldcg(gJ + g);
+          if (flip) mv = -mv;
+          if (stage > 1) iv = __ldcg((stage == 2 ? D.iJ1 : D.iJ2) + g);
+        }
+      }
+      if (stage == 1) {
+        if (taken == 0) iv = swale::recip(jv);
+        else if (!own) iv = real_cell ? __ldcg(D.iJ1 + g) : 1.0;
+        if (taken == 0 && own) iJ0 = iv;
+      }
+      rE[tid] = ev;
+      rM[tid] = mv;
+      rJ[tid] = jv;
+      sI[tid] = iv;
+      sW[tid] = w;
+      const double hv = swale::sub_(ev, bv);
+      const bool keep = have_mesh && (stage == 1 || !moving);
+      mr.pair = mr.next = mr.all_pair = mr.all_next = keep;
+      StepSink sink{mr.ip, mr.it, mr.iq, mr.iv, 0.0, 0.0};
+      EdgeState o{0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+      uint8_t flag = 0;
+      double etaG[2] = {0.0, 0.0};
+      uint32_t st = 0;
+      recon_phases<T, SCHEME>(K.sc, rows, rE, rM, rJ, jv, ev, mv, hv, stage == 1 ? jmax : stage == 2 ? jm1 : jm2, mr, mine, sink,
+                              o, flag, etaG, st);
+      if (stage == 2 || !moving) {
+        mr.ip = sink.ip;
+        mr.it = sink.it;
+        mr.iq = sink.iq;
+        mr.iv = sink.iv;
+      }
+      if (stage == 1 && own) D.flags[idx] = flag;
+      sR[0][tid] = o.ER;
+      sR[1][tid] = o.BR;
+      sR[2][tid] = o.hR;
+      sR[3][tid] = o.uR;
+      sPair[0][tid] = sink.ip;
+      sPair[1][tid] = sink.it;
+      sPair[2][tid] = sink.de;
+      sPair[3][tid] = sink.dh;
+      const bool rel = stage == 1 ? wave_rel1 : K.wave_rel;
+      block_wave<T>(&X->mx[set][stage - 1], 0.0, K.sc.g, mine && c != -1, mine && c != N,
+                    WaveEdge{o.hL, o.uL, rel ? w : 0.0}, WaveEdge{o.hR, o.uR, rel && tid < T - 1 ? sW[tid + 1] : 0.0});
+      block_or_status(&X->st[set][2 * stage - 2], st);
+      if (!inst_barrier(&X->arrived, nb, target)) {
+        timeout = true;
+        break;
+      }
+      const double A = bitsd(__ldcg(&X->mx[set][stage - 1]));
+      const unsigned int raised = __ldcg(&X->st[set][2 * stage - 2]);
+      amax[stage - 1] = A;
+      bits |= raised;
+      err = raised & kErrBits;
+      if (err) break;
+      double alpha;
+      if (stage == 1) {
+        // Everybody has left the last step's set: it is cleared for the step after the next one.
+        if (tl.c0 == 0 && tid < 12) {
+          const int z = (int)((taken + 2) % 3);
+          if (tid < 6) X->mx[z][tid] = 0ull;
+          else X->st[z][tid - 6] = 0u;
+        }
+        sd = step_dt(ic.cfl, wave_rel1 ? A : A + Wbar, 0.0, jmin, tn, K.dt_fixed, K.t_end,
+                     K.mesh == SWALE_MESH_PROFILE ? K.inv_T : 0.0);
+        if (sd.nodt) {
+          err = swale::ST_NODT;
+          bits |= err;
+          break;
+        }
+        if (K.mesh == SWALE_MESH_PROFILE) w = swale::mul_(Pn, sd.sdiff);
+        sW[tid] = w;
+        alpha = sd.alpha1;
+      } else {
+        alpha = A + (K.wave_rel ? 0.0 : Wbar);
+      }
+      const double dt = sd.dt;
+      // Left interface of the cell: its left state is the right edge of cell c - 1.
+      swale::Flux2 F{0.0, 0.0, 0.0, 0.0};
+      swale::PairRatio pr = kept_pr;
+      swale::SourceRatio sr = kept_sr;
+      double dE = 0.0, dH = 0.0;
+      if (face) {
+        dE = sPair[2][tid - 1];
+        dH = sPair[3][tid - 1];
+        if (!keep) pr = swale::pair_ratio(rJ[tid - 1], jv, sPair[0][tid - 1]);
+        F = swale::interface_flux2<SCHEME>(K.sc.g, alpha, w, sR[0][tid - 1], o.EL, sR[1][tid - 1], o.BL, sR[2][tid - 1],
+                                           o.hL, sR[3][tid - 1], o.uL);
+        sF[0][tid] = F.FE;
+        sF[1][tid] = F.FMl;
+        sF[2][tid] = F.FB;
+        sG[0][tid] = pr.sig;
+        sG[1][tid] = pr.rho2;
+      }
+      __syncthreads();
+      double jmaxa = 0.0, jmaxb = 0.0, jminb = INFINITY;
+      st = 0;
+      if (own) {
+        if (!keep) sr = swale::source_ratio(rJ[tid - 1], jv, rJ[tid + 1], sI[tid - 1], sI[tid + 1], sPair[1][tid - 1]);
+        double Rm = swale::sub_(F.FMr, sF[1][tid + 1]);
+        const double acc = swale::source_pressure_form(hv, o.hL, o.hR, swale::sub_(o.EL, ev), swale::sub_(o.ER, ev), dE, dH,
+                                                       sink.de, sink.dh, pr.rho, pr.sig2, sG[0][tid + 1], sG[1][tid + 1], sr);
+        Rm = swale::fma_(-K.sc.g, acc, Rm);
+        const double R2[3] = {swale::sub_(F.FE, sF[0][tid + 1]), Rm, swale::sub_(sF[2][tid + 1], F.FB)};
+        if (stage == 1) {
+          dJ = swale::mul_(dt, swale::sub_(sW[tid + 1], w));
+          J1 = swale::add_(J0, dJ);
+          Js = J1;
+          const double J2 = swale::fma_(0.5, dJ, J0);
+          jmaxa = J1;
+          jmaxb = J2;
+          jminb = J1;
+          if (!swale::gt0(J1) || !swale::gt0(J2)) st |= swale::ST_EMESH;
+          iJ1 = moving ? swale::recip(J1) : iv;
+          iJs = iJ1;
+          const double hdt = 0.5 * dt;
+#pragma unroll
+          for (int v = 0; v < 3; ++v) {
+            Y[v] = R2[v];
+            qs[v] = swale::rk_advance(q0[v], hdt, R2[v], dJ, iJ1);
+          }
+          D.J1[g] = J1;
+          D.iJ1[g] = iJ1;
+          D.Ea[g] = qs[0];
+          D.Ma[g] = qs[1];
+          D.Ba[g] = qs[2];
+        } else if (stage == 2) {
+          Js = swale::fma_(0.5, dJ, J0);
+          iJs = moving ? swale::recip(Js) : iv;
+          const double edt = 0.125 * dt, hdJ = 0.5 * dJ;
+#pragma unroll
+          for (int v = 0; v < 3; ++v) {
+            Y[v] = swale::add_(Y[v], R2[v]);
+            qs[v] = swale::rk_advance(q0[v], edt, Y[v], hdJ, iJs);
+          }
+          D.J2[g] = Js;
+          D.iJ2[g] = iJs;
+          D.Eb[g] = qs[0];
+          D.Mb[g] = qs[1];
+          D.Bb[g] = qs[2];
+        } else {
+          const double tdt = dt * (1.0 / 12.0);
+#pragma unroll
+          for (int v = 0; v < 3; ++v) qs[v] = swale::rk_advance(q0[v], tdt, swale::fma_(4.0, R2[v], Y[v]), dJ, iJ1);
+          if (swale::bad(qs[0]) || swale::bad(qs[1]) || swale::bad(qs[2])) st |= swale::ST_NONFINITE;
+          D.E0[g] = qs[0];
+          D.M0[g] = qs[1];
+          D.B0[g] = qs[2];
+          D.J0[g] = J1;
+        }
+      }
+      if (stage == 1 && moving) block_widths<T, true>(&X->mx[set][3], &X->mx[set][5], jmaxa, jmaxb, jminb);
+      block_or_status(&X->st[set][2 * stage - 1], st);
+      if (stage == 2 || !moving) {
+        kept_pr = pr;
+        kept_sr = sr;
+        have_mesh = true;
+      }
+      if (!inst_barrier(&X->arrived, nb, target)) {
+        timeout = true;
+        break;
+      }
+      const unsigned int raised2 = __ldcg(&X->st[set][2 * stage - 1]);
+      if (stage == 1 && moving) {
+        jm1 = bitsd(__ldcg(&X->mx[set][3]));
+        jm2 = bitsd(__ldcg(&X->mx[set][4]));
+      }
+      bits |= raised2;
+      err = raised2 & kErrBits;
+      if (err) {
+        if (stage == 3 && own) {  // the step failed after its cells were written: q^n, J^n back
+          D.E0[g] = q0[0];
+          D.M0[g] = q0[1];
+          D.B0[g] = q0[2];
+          D.J0[g] = J0;
+        }
+        break;
+      }
+    }
+    if (timeout) break;
+    if (err) {
+      done = 1;
+      break;
+    }
+    // The step is good.
+#pragma unroll
+    for (int v = 0; v < 3; ++v) q0[v] = qs[v];
+    J0 = J1;
+    iJ0 = iJ1;
+    x = swale::fma_(sd.dt, w, x);
+    if (moving) {
+      jmax = jm1;
+      jmin = bitsd(~__ldcg(&X->mx[set][5]));
+    }
+    tn = sd.clipped ? K.t_end : tn + sd.dt;
+    ++taken;
+  }
+  if (timeout) {
+    if (tid == 0) atomicOr(&S->status, (unsigned int)swale::ST_TIMEOUT);
+    return;
+  }
+  if (own_node && taken > 0) D.x[nbase + c] = x;
+  if (tl.c0 == 0 && tid == 0) {
+    S->status |= bits;
+    S->done = done;
+    S->t = tn;
+    S->steps += taken;
+    S->step_idx = S->steps;
+    S->dt = sd.dt;
+    S->alpha1 = sd.alpha1;
+    S->sdiff = sd.sdiff;
+    S->clipped = sd.clipped;
+    for (int s = 0; s < 3; ++s) S->A[s] = dbits(amax[s]);
+    S->Jmax[0] = S->JmaxN = dbits(jmax);
+    S->Jmin0 = S->JminN = dbits(jmin);
+    S->Jmax[1] = dbits(jm1);
+    S->Jmax[2] = dbits(jm2);
+    S->geo_tag = 0ull;
+  }
+}
+
+}  // namespace swale_dev

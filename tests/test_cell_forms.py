@@ -67,6 +67,36 @@ void t_source(const double* J, const double* eta, const double* hd, double* out)
   out[1] = 2.0 * source_cell_form(-1.0, hd, bd, f) + (hd[4] * hd[4] - hd[3] * hd[3]);
 }
 double t_rk(double q, double a, double R, double dJ, double J) { return rk_advance(q, a, R, dJ, 1.0 / (J + dJ)); }
+// ev[2][3] by open_edge_values, and by the plain Steps 2-4; returns class | plain class << 2 | 16 if the tie is near.
+int t_open(const double* h, const double* eta, const double* hu, const double* hh, double dx, double* ev) {
+  SchemeConst P{9.812, 1e-6, 1e-11, 1e-6, 1, 0};
+  const double* V[3] = {eta, hu, hh};
+  double p[4], it[3], iq[2], v[3], d2[3][4], d3[3][3], d4[3][2], v0[3][3];
+  StencilDD DD;
+  for (int a = 0; a < 4; ++a) p[a] = h[a] + h[a + 1];
+  for (int a = 0; a < 3; ++a) it[a] = 1.0 / (h[a] + h[a + 1] + h[a + 2]);
+  for (int a = 0; a < 2; ++a) iq[a] = 1.0 / (p[a] + p[a + 2]);
+  for (int k = 0; k < 3; ++k) {
+    v[k] = V[k][2];
+    for (int a = 0; a < 3; ++a) v0[k][a] = V[k][a];
+    for (int a = 0; a < 4; ++a) DD.D2[k][a] = d2[k][a] = (V[k][a + 1] - V[k][a]) / p[a];
+    for (int a = 0; a < 3; ++a) DD.D3[k][a] = d3[k][a] = (d2[k][a + 1] - d2[k][a]) * it[a];
+    for (int a = 0; a < 2; ++a) d4[k][a] = (d3[k][a + 1] - d3[k][a]) * iq[a];
+  }
+  const double iv = 1.0 / (p[0] + p[2] + h[4]);
+  int cls = 0;
+  for (int e = 0; e < 2; ++e) cls = open_edge_values(P, h, p, dx, iv, v, d2, d3, d4, e == 1, ev + 3 * e);
+  CellGeom Gm; uint32_t st = 0;
+  cell_geom(h, dx, Gm, st);
+  double beta[3], phi[2][3];
+  shared_beta(Gm, DD, beta);
+  const int pc = hybrid_phi(P, beta, Gm.d, phi);
+  for (int e = 0; e < 2; ++e)
+    for (int k = 0; k < 3; ++k) ev[6 + 3 * e + k] = edge_value(Gm, phi, v0[k], DD.D2[k], DD.D3[k], e);
+  const double gam = fabs(beta[0] - beta[2]) / ((beta[0] + beta[1] + beta[2]) / 3.0 + 1e-6);
+  const bool near = fabs(gam - 0.5) < 1e-9 || fabs(gam - 1.0) < 1e-9;
+  return cls | (pc << 2) | (near ? 16 : 0);
+}
 // 1: the pre-test says the limiter is inactive; bit 1: it is active
 int t_limit(double eps, double hbar, double hL, double hR) {
   SchemeConst P{9.812, 1e-6, eps, 1e-6, 1, 0};
@@ -105,7 +135,7 @@ def lib(tmp_path_factory):
                     os.path.join(ROOT, "paper_2208_06588_gb300", "csrc"), "-o", str(out), str(src)], check=True)
     L = ctypes.CDLL(str(out))
     for n, r in (("t_eweight", ctypes.c_int), ("t_moderate", ctypes.c_int), ("t_rk", ctypes.c_double),
-                 ("t_limit", ctypes.c_int), ("t_nonwb", ctypes.c_int)):
+                 ("t_limit", ctypes.c_int), ("t_nonwb", ctypes.c_int), ("t_open", ctypes.c_int)):
         getattr(L, n).restype = r
     return L
 
@@ -244,6 +274,30 @@ def test_limiter_pretest_never_skips_an_active_limiter(lib, eps):
     assert told > 1000
     for bad in (np.nan, np.inf, -np.inf):
         assert lib.t_limit(_d(eps), _d(1.0), _d(bad), _d(1.0)) != 3
+
+
+@pytest.mark.parametrize("spread", [0.0, 0.3, 1.0])
+def test_open_edge_is_the_hybrid_reconstruction(lib, spread):
+    """Every class: the class of Steps 2-3 and its edge values (the weights' conditioning and the mesh's
+    factors allowed for in the scale)."""
+    rng = np.random.default_rng(10)
+    seen = np.zeros(3, dtype=int)
+    for _ in range(4000):
+        sc = 10.0 ** rng.uniform(-3, 0)
+        h = sc * np.exp(rng.uniform(-spread, spread, 5))
+        amp = 10.0 ** rng.uniform(-4.5, 0.5)
+        shape = rng.choice([0, 1, 2])
+        w = rng.uniform(-1, 1, (3, 5)) if shape == 0 else np.where(np.arange(5) > rng.integers(0, 4), 1.0, 0.0) * \
+            rng.uniform(-1, 1, (3, 1)) if shape == 1 else np.cumsum(rng.uniform(0.5, 1, (3, 5)), axis=1)
+        eta, hu, hh = 2.0 + amp * w[0], 1.0 + amp * w[1], 3.0 + amp * w[2]
+        ev = np.zeros(12)
+        r = lib.t_open(_p(h), _p(eta), _p(hu), _p(hh), _d(h.max()), _p(ev))
+        if r & 16:
+            continue
+        assert (r & 3) == ((r >> 2) & 3)
+        seen[r & 3] += 1
+        assert np.abs(ev[:6] - ev[6:]).max() <= 1e-12 * (4.0 + amp) * (1.0 + np.exp(3.0 * spread))
+    assert np.all(seen > 100), seen
 
 
 def test_nonwb_fp32_test_implies_the_smooth_class(lib):

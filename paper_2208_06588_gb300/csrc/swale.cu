@@ -1931,6 +1931,24 @@ void* g_noalloc_addr[kNoAllocMaxDevices];
 std::once_flag g_noalloc_once[kNoAllocMaxDevices];
 cudaError_t g_noalloc_err[kNoAllocMaxDevices];
 
+// What a call returns besides the right-hand sides: the classes (src, device) and the largest edge speed.
+swale_status noalloc_results(NoAllocScratch* scr, const uint8_t* src, uint8_t* flags, int64_t N, double* A_out,
+                             cudaStream_t st) {
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess && flags) e = cudaMemcpyAsync(flags, src, (size_t)N, cudaMemcpyDefault, st);
+  if (e == cudaSuccess && A_out) {
+    unsigned long long bits = 0;
+    e = cudaMemcpyAsync(&bits, &scr->S.A[0], sizeof(bits), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) std::memcpy(A_out, &bits, sizeof(double));
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return SWALE_ECUDA;
+  }
+  return SWALE_OK;
+}
+
 bool on_device(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -1953,6 +1971,10 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
       cfg->bc > 2 || cfg->scheme < 0 || cfg->scheme > 2 || (cfg->alpha_bound != 0 && cfg->alpha_bound != 1) ||
       (cfg->limit_hu != 0 && cfg->limit_hu != 1))
     return SWALE_EINVAL;
+  // Outputs that overlap an input (in place): every cell has to be read before the first is written.
+  bool in_place = false;
+  for (const double* r : {RE, RM, RB})
+    for (const double* q : {E, M, B, J, w}) in_place = in_place || (r < q + (N + 1) && q < r + N);
   const void* dev_ptrs[] = {E, M, B, J, w, RE, RM, RB};
   for (const void* p : dev_ptrs)
     if (!on_device(p)) return SWALE_EINVAL;
@@ -1975,6 +1997,30 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   });
   if (g_noalloc_err[dev] != cudaSuccess || !g_noalloc_addr[dev]) return SWALE_ECUDA;
   NoAllocScratch* scr = reinterpret_cast<NoAllocScratch*>(g_noalloc_addr[dev]);
+  const bool flags_here = flags && on_device(flags);
+  if (!in_place) {
+    SchemeConst P;
+    P.g = cfg->g;
+    P.eps_weno = cfg->eps_weno;
+    P.eps_pp = cfg->eps_pp;
+    P.h_dry = cfg->h_dry;
+    P.beta_dx_global = cfg->beta_dx_global;
+    P.limit_hu = cfg->limit_hu;
+    unsigned long long *mx = &scr->S.Jmax[0], *wv = A_out ? &scr->S.A[0] : nullptr;
+    // Up to this many cells every block finds the largest width itself: one launch instead of two.
+    constexpr int64_t kScanCells = 4096;
+    const bool scan = N <= kScanCells && !A_out;
+    if (!scan) k_rhs_widths<<<1, 1024, 0, st>>>(J, (int32_t)N, mx, wv);
+    const unsigned nb = (unsigned)((N + kStepCells - 1) / kStepCells);
+    auto go = [&](auto kernel) {
+      kernel<<<nb, kStepThreads, 0, st>>>(P, cfg->bc, cfg->alpha_bound ? 0 : 1, (int32_t)N, alpha, E, M, B, J, w,
+                                          scan ? nullptr : mx, wv, RE, RM, RB, flags_here ? flags : scr->flags);
+    };
+    if (cfg->scheme == SWALE_SCHEME_NONWB) go(k_rhs<1>);
+    else if (cfg->scheme == SWALE_SCHEME_SPECIAL) go(k_rhs<2>);
+    else go(k_rhs<0>);
+    return noalloc_results(scr, scr->flags, flags_here ? nullptr : flags, N, A_out, st);
+  }
 
   DevState D{};
   D.eEL = scr->edges[0];
@@ -2038,19 +2084,7 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   launch_recon<1>(K, D, kNoAllocTile, (unsigned)D.nrf, st, E, M, B, J);
   const RhsOut ro{RE, RM, RB, alpha};
   launch_update<2, 1>(K, D, kNoAllocTile, (unsigned)D.nf, st, E, M, B, J, ro);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && flags) e = cudaMemcpyAsync(flags, scr->flags + 1, (size_t)N, cudaMemcpyDefault, st);
-  if (e == cudaSuccess && A_out) {
-    unsigned long long bits = 0;
-    e = cudaMemcpyAsync(&bits, &scr->S.A[0], sizeof(bits), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e == cudaSuccess) std::memcpy(A_out, &bits, sizeof(double));
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return SWALE_ECUDA;
-  }
-  return SWALE_OK;
+  return noalloc_results(scr, scr->flags + 1, flags, N, A_out, st);
 }
 
 }  // extern "C"

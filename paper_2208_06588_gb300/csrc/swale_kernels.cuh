@@ -586,7 +586,7 @@ __device__ __noinline__ StepDt step_dt(double cfl, double alpha1, double dwmax, 
     double sn, cs;
     sincospi(((threadIdx.x & 31) == 0 ? 2.0 * tn + r.dt : r.dt) * inv_T, &sn, &cs);
     const double cs0 = __shfl_sync(0xffffffffu, cs, 0), sn1 = __shfl_sync(0xffffffffu, sn, 1);
-    r.sdiff = 2.0 * cs0 * sn1 / r.dt;
+    r.sdiff = r.dt > 1e-290 ? 2.0 * cs0 * sn1 * swale::recip(r.dt) : 2.0 * cs0 * sn1 / r.dt;
   }
   return r;
 }

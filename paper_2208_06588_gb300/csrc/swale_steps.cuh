@@ -32,7 +32,7 @@ __device__ __forceinline__ bool inst_barrier(unsigned int* arrived, unsigned int
   __shared__ bool ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
+    // (the release and the acquire order the whole block's accesses through the two block barriers)
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
     bool got = false;
     for (int i = 0; i < kBarrierTries && !got; ++i) {
@@ -40,7 +40,6 @@ __device__ __forceinline__ bool inst_barrier(unsigned int* arrived, unsigned int
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
       got = (int)(v - target) >= 0;
     }
-    __threadfence();
     ok = got;
   }
   __syncthreads();
@@ -378,6 +377,135 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState
     S->Jmax[2] = dbits(jm2);
     S->geo_tag = 0ull;
   }
+}
+
+// Largest of n widths, by one block, into *out; *wave (if given) is cleared.
+__global__ void __launch_bounds__(1024) k_rhs_widths(const double* __restrict__ J, int32_t n, unsigned long long* out,
+                                                     unsigned long long* wave) {
+  __shared__ unsigned long long red[32];
+  unsigned long long m = 0ull;
+#pragma unroll 8
+  for (int32_t i = threadIdx.x; i < n; i += 1024) m = umax64(m, dbits(J[i]));
+  m = warp_umax64(m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    m = warp_umax64(red[threadIdx.x]);
+    if (threadIdx.x == 0) {
+      *out = m;
+      if (wave) *wave = 0ull;
+    }
+  }
+}
+
+// One right-hand side for a given viscosity in one launch: alpha is known, so the fluxes need no grid-wide
+// maximum between them and the reconstruction, and the edge values stay on the chip (a block owns 122
+// cells and reconstructs one more on each side, as in k_steps). dxmax: the largest width, or null: every block
+// scans the N widths (cheaper than a launch of its own up to a few thousand cells). wave: where the largest
+// edge speed goes (null: not wanted), relative to w if wave_rel.
+template <int SCHEME>
+__global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, int wave_rel, int32_t N, double alpha,
+                                                         const double* __restrict__ E, const double* __restrict__ M,
+                                                         const double* __restrict__ B, const double* __restrict__ J,
+                                                         const double* __restrict__ w, const unsigned long long* dxmax,
+                                                         unsigned long long* wave, double* __restrict__ RE,
+                                                         double* __restrict__ RM, double* __restrict__ RB,
+                                                         uint8_t* __restrict__ flags) {
+  constexpr int T = kStepThreads;
+  __shared__ double rE[T + 8], rM[T + 8], rJ[T + 8];
+  __shared__ ReconRows<T, SCHEME> rows;
+  __shared__ double sR[4][T], sBL[T], sPair[4][T];  // right edges, left bottoms; ip, it, de, dh of the pair that starts there
+  __shared__ double sF[3][T], sG[2][T], sB[T], sI[T];
+  __shared__ unsigned long long red[T / 32];
+  const int tid = threadIdx.x;
+  const int32_t c = (int32_t)blockIdx.x * kStepCells - 3 + tid;  // this thread's cell, and its left node
+  const bool own = tid >= 3 && tid < T - 3 && c < N;
+  const bool mine = tid >= 2 && tid < T - 2 && c <= N;  // reconstructed
+  const bool face = tid >= 3 && tid < T - 2 && c <= N;  // left interface of an owned cell, or the last one
+  double ev = 0.0, mv = 0.0, bv = 0.0, jv = 1.0, wl = 0.0, wr = 0.0;
+  if (c >= -3 && c <= N + 2) {
+    const int32_t g = ghost(c, N, bc);
+    ev = E[g];
+    mv = M[g];
+    bv = B[g];
+    jv = J[g];
+    if (bc == SWALE_BC_REFLECTIVE && (c < 0 || c >= N)) mv = -mv;
+    if (c >= 0 && c <= N) wl = w[c];
+    if (c >= -1 && c < N) wr = w[c + 1];
+  }
+  double dx;
+  if (dxmax || !P.beta_dx_global) {
+    dx = dxmax ? bitsd(*dxmax) : 0.0;
+  } else {
+    unsigned long long m = 0ull;
+#pragma unroll 4
+    for (int32_t i = tid; i < N; i += T) m = umax64(m, dbits(J[i]));
+    m = warp_umax64(m);
+    if ((tid & 31) == 0) red[tid >> 5] = m;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < T / 32; ++k) m = umax64(m, red[k]);
+    dx = bitsd(m);
+  }
+  rE[tid] = ev;
+  rM[tid] = mv;
+  rJ[tid] = jv;
+  sB[tid] = bv;
+  const double hv = swale::sub_(ev, bv), iv = swale::recip(jv);
+  sI[tid] = iv;
+  const MeshRecips none{0.0, 0.0, 0.0, 0.0, false, false, false, false};
+  StepSink sink{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  EdgeState o{0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  uint8_t flag = 0;
+  double etaG[2] = {0.0, 0.0};
+  uint32_t st = 0;
+  recon_phases<T, SCHEME>(P, rows, rE, rM, rJ, jv, ev, mv, hv, dx, none, mine, sink, o, flag, etaG, st);
+  if (own && flags) flags[c] = flag;
+  sR[0][tid] = o.ER;
+  sR[1][tid] = o.BR;
+  sR[2][tid] = o.hR;
+  sR[3][tid] = o.uR;
+  sBL[tid] = o.BL;
+  sPair[0][tid] = sink.ip;
+  sPair[1][tid] = sink.it;
+  sPair[2][tid] = sink.de;
+  sPair[3][tid] = sink.dh;
+  if (wave)
+    block_wave<T>(wave, 0.0, P.g, mine && c != -1, mine && c != N, WaveEdge{o.hL, o.uL, wave_rel ? wl : 0.0},
+                  WaveEdge{o.hR, o.uR, wave_rel ? wr : 0.0});
+  __syncthreads();
+  swale::Flux2 F{0.0, 0.0, 0.0, 0.0};
+  swale::PairRatio pr{0.0, 0.0, 0.0, 0.0};
+  if (face) {
+    pr = swale::pair_ratio(rJ[tid - 1], jv, sPair[0][tid - 1]);
+    F = swale::interface_flux2<SCHEME>(P.g, alpha, wl, sR[0][tid - 1], o.EL, sR[1][tid - 1], o.BL, sR[2][tid - 1], o.hL,
+                                       sR[3][tid - 1], o.uL);
+    sF[0][tid] = F.FE;
+    sF[1][tid] = F.FMl;
+    sF[2][tid] = F.FB;
+    sG[0][tid] = pr.sig;
+    sG[1][tid] = pr.rho2;
+  }
+  __syncthreads();
+  if (!own) return;
+  double Rm = swale::sub_(F.FMr, sF[1][tid + 1]);
+  if (SCHEME == 2) {
+    const double bd[5] = {sB[tid - 1], bv, sB[tid + 1], o.BL, o.BR};
+    const swale::SourceGeom sg = swale::source_geom(rJ[tid - 1], jv, sI[tid - 1], iv, sI[tid + 1], sPair[0][tid - 1],
+                                                    sink.ip, sPair[1][tid - 1]);
+    const double eta4[4] = {o.EL, etaG[0], etaG[1], o.ER};
+    Rm = swale::fma_(2.0, swale::source_cell_special(P.g, ev, eta4, bd, sg, sR[1][tid - 1], sBL[tid + 1]), Rm);
+  } else {
+    const swale::SourceRatio sr =
+        swale::source_ratio(rJ[tid - 1], jv, rJ[tid + 1], sI[tid - 1], sI[tid + 1], sPair[1][tid - 1]);
+    const double acc = swale::source_pressure_form(hv, o.hL, o.hR, swale::sub_(o.EL, ev), swale::sub_(o.ER, ev),
+                                                   sPair[2][tid - 1], sPair[3][tid - 1], sink.de, sink.dh, pr.rho, pr.sig2,
+                                                   sG[0][tid + 1], sG[1][tid + 1], sr);
+    Rm = swale::fma_(-P.g, acc, Rm);
+  }
+  RE[c] = 0.5 * swale::sub_(F.FE, sF[0][tid + 1]);
+  RM[c] = 0.5 * Rm;
+  RB[c] = 0.5 * swale::sub_(sF[2][tid + 1], F.FB);
 }
 
 }  // namespace swale_dev

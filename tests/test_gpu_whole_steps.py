@@ -110,3 +110,31 @@ def test_batch_of_small_instances_and_an_end_time():
     for k in ("eta", "hu", "b", "x", "t"):
         assert np.array_equal(got[0][k], got[1][k]), k
     assert got[0]["n"] == got[1]["n"] and np.all(got[0]["t"] == 0.02)
+
+
+@pytest.mark.parametrize("n", [5, 6, 121, 122, 123, 1000, 4096, 4097, 20011])
+@pytest.mark.parametrize("scheme,bc", [("hydrostatic", "periodic"), ("nonwb", "reflective"), ("special", "transmissive")])
+def test_rhs_in_one_launch_equals_the_stage_kernels(n, scheme, bc):
+    """swale_rhs_noalloc in one launch against its in-place form, which runs the stage kernels (every
+    cell read before the first is written): the same arithmetic, up to the special scheme's point-wise
+    source, whose sums the compiler may fuse differently (1e-13 of the largest value)."""
+    import torch
+    p, cfg = problem(n, bc, "static", dry=n > 200)
+    cfg = B.make_config(**dict(cfg, scheme=scheme))
+    d = {k: torch.from_numpy(np.ascontiguousarray(v)).cuda() for k, v in p.items()}
+    J = d["x"][1:] - d["x"][:-1]
+    w = 0.1 * torch.sin(7 * d["x"])
+    stream = torch.cuda.current_stream().cuda_stream
+    for want_A in (False, True):
+        out = [torch.empty_like(d["E"]) for _ in range(3)]
+        fl = torch.empty(n, dtype=torch.uint8, device="cuda")
+        A = B.swale_rhs_noalloc(cfg, stream, n, d["E"], d["hu"], d["b"], J, w, 6.0, *out, fl, want_A=want_A)
+        RM = d["hu"].clone()
+        ref = [torch.empty_like(RM), RM, torch.empty_like(RM)]
+        fr = torch.empty_like(fl)
+        Ar = B.swale_rhs_noalloc(cfg, stream, n, d["E"], RM, d["b"], J, w, 6.0, *ref, fr, want_A=want_A)
+        torch.cuda.synchronize()
+        assert torch.equal(fl, fr) and A == Ar
+        for a, r in zip(out, ref):
+            tol = 1e-13 * float(r.abs().max()) if scheme == "special" else 0.0
+            assert float((a - r).abs().max()) <= tol

@@ -65,6 +65,9 @@ struct swale_ctx {
   int step_blocks = 0;
   Tile* step_tiles = nullptr;
   StepScratch* step_scratch = nullptr;
+  // Blocks of the adjoint's kernels, and their work list (null: one instance).
+  int adj_blocks = 0;
+  Tile* adj_tiles = nullptr;
 };
 
 namespace {
@@ -179,7 +182,9 @@ void free_tiles(swale_ctx* ctx) {
   ctx->step_blocks = 0;
   ctx->step_tiles = nullptr;
   ctx->step_scratch = nullptr;
-  ctx->D.rtiles = ctx->D.utiles = ctx->D.mtiles = ctx->D.ftiles = ctx->D.rftiles = nullptr;
+  ctx->adj_blocks = 0;
+  ctx->adj_tiles = nullptr;
+  ctx->D.mtiles = ctx->D.ftiles = ctx->D.rftiles = nullptr;
 }
 
 void free_alpha_log(swale_ctx* ctx) {
@@ -330,49 +335,44 @@ swale_status build_tiles(swale_ctx* ctx, std::vector<InstConst>& ic) {
   const int Tr = ctx->Tr, Tu = ctx->Tu, Tm = kMeshNodes;
   const int Tf = Tu - 1;  // cells of a forward update tile (its Tu interfaces take one pass)
   const int Trf = Tr - 4; // cells of a forward reconstruction tile (its Tr stencil cells take one pass)
-  std::vector<Tile> rt, ut, mt, ft, rf;
+  std::vector<Tile> mt, ft, rf, at;
+  int64_t na = 0;
   for (int64_t i = 0; i < B; ++i) {
     const int64_t N = ic[i].N;
-    const int64_t nr = (N + 2 + Tr - 1) / Tr, nu = (N + Tu - 1) / Tu, nm = (N + 1 + Tm - 1) / Tm;
+    const int64_t nm = (N + 1 + Tm - 1) / Tm, nadj = adj_blocks(N);
+    na += nadj;
     const int64_t nf = (N + Tf - 1) / Tf, nrf = (N + 2 + Trf - 1) / Trf;
     ic[i].ntiles_r = (int32_t)nrf;
     if (B > 1) {
-      for (int64_t t = 0; t < nr; ++t) rt.push_back(Tile{(int32_t)i, (int32_t)(t * Tr - 1)});
-      for (int64_t t = 0; t < nu; ++t) ut.push_back(Tile{(int32_t)i, (int32_t)(t * Tu)});
+      for (int64_t t = 0; t < nadj; ++t) at.push_back(Tile{(int32_t)i, (int32_t)t});
       for (int64_t t = 0; t < nm; ++t) mt.push_back(Tile{(int32_t)i, (int32_t)(t * Tm)});
       for (int64_t t = 0; t < nf; ++t) ft.push_back(Tile{(int32_t)i, (int32_t)(t * Tf)});
       for (int64_t t = 0; t < nrf; ++t) rf.push_back(Tile{(int32_t)i, (int32_t)(t * Trf - 1)});
     } else {
-      ctx->D.nr = (int32_t)nr;
-      ctx->D.nu = (int32_t)nu;
       ctx->D.nm = (int32_t)nm;
       ctx->D.nf = (int32_t)nf;
       ctx->D.nrf = (int32_t)nrf;
     }
   }
   if (B > 1) {
-    Tile *dr, *du, *dm, *df, *drf;
-    if (swale_status s = dalloc(ctx, ctx->tile_allocs, &dr, rt.size())) return s;
-    if (swale_status s = dalloc(ctx, ctx->tile_allocs, &du, ut.size())) return s;
+    Tile *da, *dm, *df, *drf;
+    if (swale_status s = dalloc(ctx, ctx->tile_allocs, &da, at.size())) return s;
     if (swale_status s = dalloc(ctx, ctx->tile_allocs, &dm, mt.size())) return s;
     if (swale_status s = dalloc(ctx, ctx->tile_allocs, &df, ft.size())) return s;
     if (swale_status s = dalloc(ctx, ctx->tile_allocs, &drf, rf.size())) return s;
-    SW_CUDA(ctx, cudaMemcpyAsync(dr, rt.data(), rt.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
-    SW_CUDA(ctx, cudaMemcpyAsync(du, ut.data(), ut.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
+    SW_CUDA(ctx, cudaMemcpyAsync(da, at.data(), at.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
     SW_CUDA(ctx, cudaMemcpyAsync(dm, mt.data(), mt.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
     SW_CUDA(ctx, cudaMemcpyAsync(df, ft.data(), ft.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
     SW_CUDA(ctx, cudaMemcpyAsync(drf, rf.data(), rf.size() * sizeof(Tile), cudaMemcpyHostToDevice, ctx->stream));
-    ctx->D.rtiles = dr;
-    ctx->D.utiles = du;
+    ctx->adj_tiles = da;
     ctx->D.mtiles = dm;
     ctx->D.ftiles = df;
     ctx->D.rftiles = drf;
-    ctx->D.nr = (int32_t)rt.size();
-    ctx->D.nu = (int32_t)ut.size();
     ctx->D.nm = (int32_t)mt.size();
     ctx->D.nf = (int32_t)ft.size();
     ctx->D.nrf = (int32_t)rf.size();
   }
+  ctx->adj_blocks = (int)na;
   ctx->D.ic1 = ic[0];
   if (swale_status s = build_step_blocks(ctx, ic)) return s;
   SW_CUDA(ctx, cudaMemcpyAsync(ctx->D.IC, ic.data(), B * sizeof(InstConst), cudaMemcpyHostToDevice, ctx->stream));
@@ -1313,41 +1313,15 @@ long long device_steps(swale_ctx* ctx) {
   return s;
 }
 
+// The reverse of stage STAGE with stage data D (its input E, M, B and widths J), on the context's stream.
 template <int STAGE>
 void launch_adj_stage(swale_ctx* ctx, const DevState& D, const StepConst& K, const AdjState& A, const double* E,
                       const double* M, const double* B, const double* J) {
-  cudaStream_t s = ctx->stream;
-  const unsigned gu = grid_of(D.nu, ctx->grid_u), gr = grid_of(D.nr, ctx->grid_r);
-  const int Tu = ctx->Tu, Tr = ctx->Tr;
-  if (Tu == 64) {
-    k_adj_flux<STAGE, 64><<<gu, 64, 0, s>>>(K, D, A);
-    k_adj_source<STAGE, 64><<<gu, 64, 0, s>>>(K, D, A, E, B, J);
-  } else if (Tu == 256) {
-    k_adj_flux<STAGE, 256><<<gu, 256, 0, s>>>(K, D, A);
-    k_adj_source<STAGE, 256><<<gu, 256, 0, s>>>(K, D, A, E, B, J);
-  } else {
-    k_adj_flux<STAGE, 128><<<gu, 128, 0, s>>>(K, D, A);
-    k_adj_source<STAGE, 128><<<gu, 128, 0, s>>>(K, D, A, E, B, J);
-  }
-  if (Tr == 64) k_adj_recon<STAGE, 64><<<gr, 64, 0, s>>>(K, D, A, E, M, B, J);
-  else if (Tr == 256) k_adj_recon<STAGE, 256><<<gr, 256, 0, s>>>(K, D, A, E, M, B, J);
-  else k_adj_recon<STAGE, 128><<<gr, 128, 0, s>>>(K, D, A, E, M, B, J);
+  k_adj_stage<STAGE><<<(unsigned)ctx->adj_blocks, kAdjThreads, 0, ctx->stream>>>(K, D, A, E, M, B, J);
 }
-
-template <int PH>
-void launch_adj_rk(swale_ctx* ctx, const DevState& D, const AdjState& A) {
-  const unsigned gu = grid_of(D.nu, ctx->grid_u);
-  if (ctx->Tu == 64) k_adj_rk<PH, 64><<<gu, 64, 0, ctx->stream>>>(D, A);
-  else if (ctx->Tu == 256) k_adj_rk<PH, 256><<<gu, 256, 0, ctx->stream>>>(D, A);
-  else k_adj_rk<PH, 128><<<gu, 128, 0, ctx->stream>>>(D, A);
-}
-
 
 // Copies of the evolving state (q^n, J^n, nodes, per-instance scalars).
-struct StateCopy {
-  double *E, *M, *B, *J, *x;
-  DevScalars* S;
-};
+typedef StateArrays StateCopy;
 
 // Bytes one array of swale_adjoint takes in its block: rounded up to 256 bytes, plus 256 bytes of
 // slack as every device array of the library has.
@@ -1529,24 +1503,31 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
     for (void* p : mem) cudaFree(p);
     return r;
   };
+  // Two buffers of lambda, which the steps' reverse sweeps use in turn, and the stage inputs' adjoints.
   AdjState A{};
-  double** cellbufs[] = {&A.lE, &A.lM, &A.lB, &A.yE, &A.yM, &A.yB, &A.pE, &A.pM, &A.pB,
-                         &A.aE, &A.aM, &A.aB, &A.rE, &A.rM, &A.rB};
-  for (double** p : cellbufs)
-    if (!s) s = carve(p, (size_t)Nt);
-  for (int k = 0; k < 8 && !s; ++k) s = carve(&A.ab[k], (size_t)NE);
-  // Every forward run of the adjoint (the forward with checkpoints, the segment and the step
-  // recomputes) computes the mesh geometry in all three stages instead of taking stage 1's from
-  // the cache: a run that starts from a checkpoint has no cache entry, so with the cache the
-  // recomputed trajectory would differ from the forward one by rounding wherever a segment
-  // starts, and near a detector or limiter threshold that can flip a frozen branch. Without it
-  // the trajectory, and the gradient up to the order of atomic additions, is the same for every
-  // checkpoint interval.
-  DevState base = ctx->D;
+  double* lam[2][3];
+  for (int k = 0; k < 3; ++k) {
+    if (!s) s = carve(&lam[0][k], (size_t)Nt);
+    if (!s) s = carve(&lam[1][k], (size_t)Nt);
+    if (!s) s = carve(&A.a3[k], (size_t)Nt);
+    if (!s) s = carve(&A.a2[k], (size_t)Nt);
+  }
+  A.tiles = ctx->adj_tiles;
+  int cur = 0;  // the buffer that holds lambda
+  // The mesh cache holds what a stage would form from the same widths, bit for bit, so the trajectory, and
+  // the gradient up to the order of the misfit's atomic additions, is the same for every checkpoint
+  // interval, whether a run starts from a checkpoint (without a cache entry) or goes on. The forward
+  // run uses the context's cache, the segment recomputes one of their own, under epochs of their own:
+  // the scalars they load carry the forward run's tags.
+  const DevState fwd = [&] {
+    DevState d = ctx->D;
+    // The adjoint's forward runs check the status after the fact; they keep no roll-back copies
+    // (the further state sets share nothing with the context's backups).
+    d.bE = d.bM = d.bB = d.bJ = d.bx = nullptr;
+    return d;
+  }();
+  DevState base = fwd;
   base.geo = nullptr;
-  // The adjoint's forward runs check the status after the fact; they keep no roll-back copies
-  // (the further state sets share nothing with the context's backups).
-  base.bE = base.bM = base.bB = base.bJ = base.bx = nullptr;
   // A further set of state arrays: its own state, stage, edge and flag arrays and scalars
   // (instance constants, work lists and the motion profile are shared, read only).
   auto alloc_state_set = [&](DevState& X) {
@@ -1575,6 +1556,12 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
     for (double** p : ed)
       if (!s) s = carve(p, (size_t)NE);
   };
+  auto alloc_adj = [&](DevState& d) {
+    if (!s) s = carve(&d.gK, (size_t)14 * NE);
+    d.dE = d.gK + ADJ_DE * d.geo_stride;
+    d.dH = d.gK + ADJ_DH * d.geo_stride;
+    d.H = d.gK + ADJ_H * d.geo_stride;
+  };
   DevState R[2], Ds[2][3];
   if (!tape) {
     R[0] = base;
@@ -1582,15 +1569,15 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
     for (int k = 0; k < 2; ++k) {
       Ds[k][0] = Ds[k][1] = Ds[k][2] = R[k];
       for (int t = 0; t < 2; ++t) alloc_edges(Ds[k][t]);
-      // each stage's smooth-class linear form and source form, for that stage's reverse kernels
-      for (int t = 0; t < 3; ++t)
-        if (!s) s = carve(&Ds[k][t].gK, (size_t)14 * NE);
+      // what each stage's reverse reads besides the edge states
+      for (int t = 0; t < 3; ++t) alloc_adj(Ds[k][t]);
     }
   }
   // Segment recomputes: a third state set D2 recomputes segment sg - 1 into one of two
   // snapshot buffers while segment sg is reversed from the other.
   DevState D2;
   alloc_state_set(D2);
+  if (!s) s = carve(&D2.geo, (size_t)GEO_ARRAYS * NE);
   // Snapshot buffers of two segments (one when a single segment covers every step).
   const int64_t nbuf = nseg == 1 ? 1 : 2;
   std::vector<StateCopy> ckpt(nseg), seg(C), seg2(nbuf == 2 ? C : 0);
@@ -1617,7 +1604,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
         for (int t = 0; t < 3; ++t) {
           slot[b][3 * i + t] = base_i;
           alloc_edges(slot[b][3 * i + t]);
-          if (!s) s = carve(&slot[b][3 * i + t].gK, (size_t)14 * NE);
+          alloc_adj(slot[b][3 * i + t]);
         }
       }
     }
@@ -1636,12 +1623,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   e = e ? e : cudaMemcpyAsync(obs, h_obs, (size_t)nsteps * B * G * sizeof(double), cudaMemcpyDefault, st);
   e = e ? e : cudaMemsetAsync(Jacc, 0, B * sizeof(double), st);
   e = e ? e : cudaMemsetAsync(gcell, 0xff, (size_t)B * G * sizeof(int64_t), st);  // -1: not yet located
-  e = e ? e : cudaMemsetAsync(A.aE, 0, Nt * sizeof(double), st);
-  e = e ? e : cudaMemsetAsync(A.aM, 0, Nt * sizeof(double), st);
-  e = e ? e : cudaMemsetAsync(A.aB, 0, Nt * sizeof(double), st);
-  e = e ? e : cudaMemsetAsync(A.lE, 0, Nt * sizeof(double), st);
-  e = e ? e : cudaMemsetAsync(A.lM, 0, Nt * sizeof(double), st);
-  e = e ? e : cudaMemsetAsync(A.lB, 0, Nt * sizeof(double), st);
+  for (int k = 0; k < 3; ++k) e = e ? e : cudaMemsetAsync(lam[0][k], 0, Nt * sizeof(double), st);
   int prio_least = 0, prio_greatest = 0;
   e = e ? e : cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
   e = e ? e : cudaStreamCreateWithPriority(&st2, cudaStreamNonBlocking, prio_least);
@@ -1649,26 +1631,14 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   for (cudaEvent_t& x : ev) e = e ? e : cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
   if (e) return release(fail(ctx, SWALE_ECUDA, cudaGetErrorString(e)));
   DevState& D = ctx->D;
-  auto save_from = [&](StateCopy& c, const DevState& X, cudaStream_t q) {
-    const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-    cudaError_t r = cudaMemcpyAsync(c.E, X.E0, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(c.M, X.M0, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(c.B, X.B0, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(c.J, X.J0, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(c.x, X.x, NN * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(c.S, X.S, B * sizeof(DevScalars), k, q);
-    return r;
+  const unsigned copy_grid = (unsigned)std::min<int64_t>((NN + 255) / 256, 152 * 8);
+  auto copy = [&](const StateArrays& to, const StateArrays& from, cudaStream_t q) {
+    k_copy_state<<<copy_grid, 256, 0, q>>>(to, from, Nt, NN, B * (int64_t)(sizeof(DevScalars) / 8));
+    return cudaGetLastError();
   };
-  auto load_into = [&](const StateCopy& c, const DevState& X, cudaStream_t q) {
-    const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-    cudaError_t r = cudaMemcpyAsync(X.E0, c.E, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(X.M0, c.M, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(X.B0, c.B, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(X.J0, c.J, Nt * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(X.x, c.x, NN * sizeof(double), k, q);
-    r = r ? r : cudaMemcpyAsync(X.S, c.S, B * sizeof(DevScalars), k, q);
-    return r;
-  };
+  auto arrays = [](const DevState& X) { return StateArrays{X.E0, X.M0, X.B0, X.J0, X.x, X.S}; };
+  auto save_from = [&](StateCopy& c, const DevState& X, cudaStream_t q) { return copy(c, arrays(X), q); };
+  auto load_into = [&](const StateCopy& c, const DevState& X, cudaStream_t q) { return copy(arrays(X), c, q); };
   auto save = [&](StateCopy& c) { return save_from(c, D, st); };
   auto load = [&](const StateCopy& c) {
     bump_geo(ctx);
@@ -1721,37 +1691,36 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   NvtxRange nvtx_adjoint("swale_adjoint");
   nvtxRangePushA("adjoint forward");
   // ---- forward with checkpoints and the misfit ----
-  // The last segment is the one the reverse sweep starts with: the forward keeps its per-step
-  // snapshots (and in tape mode its stage data) itself, so that segment is not recomputed.
-  const int64_t nlast = (nseg - 1) * C, blast = (nseg - 1) & 1;
-  std::vector<StateCopy>& buf_last = blast ? seg2 : seg;
+  // The last segments are those the reverse sweep starts with: the forward keeps the per-step snapshots
+  // (and in tape mode the stage data) of as many as there are buffers, so these are not recomputed.
+  const int64_t kept = std::max<int64_t>(0, nseg - nbuf);  // first segment that the forward keeps
   for (int64_t n = 0; n < nsteps && !s; ++n) {
-    if (n % C == 0 && (e = save(ckpt[n / C]))) break;
-    if (n >= nlast) {
-      if ((e = save(buf_last[n - nlast]))) break;
-      if (tape) {  // the step's stage data into its slot; the state is the context's own
-        DevState f3[3];
-        for (int t = 0; t < 3; ++t) {
-          f3[t] = slot[blast][(size_t)(3 * (n - nlast) + t)];
-          f3[t].E0 = base.E0;
-          f3[t].M0 = base.M0;
-          f3[t].B0 = base.B0;
-          f3[t].J0 = base.J0;
-          f3[t].YE = base.YE;
-          f3[t].YM = base.YM;
-          f3[t].YB = base.YB;
-          f3[t].x = base.x;
-          f3[t].S = base.S;
-          f3[t].flags = base.flags;
-        }
-        s = enqueue_step_on(ctx, f3[2], st, f3, 0);
-      } else {
-        s = enqueue_step_on(ctx, base, st, nullptr, 0);
-      }
-    } else {
-      s = enqueue_step_on(ctx, base, st, nullptr, 0);
+    const int64_t sg = n / C, i = n % C;
+    if (i == 0 && (e = save(ckpt[sg]))) break;
+    if (sg >= kept) {
+      if ((e = save((sg & 1) ? seg2[i] : seg[i]))) break;
     }
-    if (!s) k_misfit<0><<<gg, 128, 0, st>>>(D, A, (int32_t)B, G, gx, obs + n * B * G, Jacc, gcell);
+    if (sg >= kept && tape) {  // the step's stage data into its slot; the state is the context's own
+      DevState f3[3];
+      for (int t = 0; t < 3; ++t) {
+        f3[t] = slot[sg & 1][(size_t)(3 * i + t)];
+        f3[t].E0 = fwd.E0;
+        f3[t].M0 = fwd.M0;
+        f3[t].B0 = fwd.B0;
+        f3[t].J0 = fwd.J0;
+        f3[t].YE = fwd.YE;
+        f3[t].YM = fwd.YM;
+        f3[t].YB = fwd.YB;
+        f3[t].x = fwd.x;
+        f3[t].S = fwd.S;
+        f3[t].flags = fwd.flags;
+        f3[t].geo = fwd.geo;
+      }
+      s = enqueue_step_on(ctx, f3[2], st, f3, ctx->geo_epoch);
+    } else {
+      s = enqueue_step_on(ctx, fwd, st, nullptr, ctx->geo_epoch);
+    }
+    if (!s) k_misfit<0><<<gg, 128, 0, st>>>(D, nullptr, nullptr, (int32_t)B, G, gx, obs + n * B * G, Jacc, gcell);
   }
   if (!s && !e) e = save(fin);
   if (!s && !e) e = cudaGetLastError();
@@ -1765,29 +1734,47 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   auto recompute_segment = [&](int64_t sg) {
     const int64_t n0 = sg * C, n1 = std::min(nsteps, n0 + C);
     std::vector<StateCopy>& buf = (sg & 1) ? seg2 : seg;
+    const uint32_t epoch = 0x80000000u + (uint32_t)sg;
     e = load_into(ckpt[sg], D2, st2);
     for (int64_t m = n0; m < n1 && !s && !e; ++m) {
       e = save_from(buf[m - n0], D2, st2);
       if (e) break;
       if (tape) {  // every step, the last one of the segment included, into its slot
         const DevState* sl = &slot[sg & 1][(size_t)(3 * (m - n0))];
-        s = enqueue_step_on(ctx, sl[2], st2, sl, 0);
+        s = enqueue_step_on(ctx, sl[2], st2, sl, epoch);
       } else if (m + 1 < n1) {
-        s = enqueue_step_on(ctx, D2, st2, nullptr, 0);
+        s = enqueue_step_on(ctx, D2, st2, nullptr, epoch);
       }
     }
     if (!s && !e) e = cudaEventRecord(ev[1 + (sg & 1)], st2);
   };
   if (!s && !e) e = cudaEventRecord(ev[0], st);
   if (!s && !e) e = cudaStreamWaitEvent(st2, ev[0], 0);
-  // The last segment's snapshots (and tape) came from the forward run itself.
-  if (!s && !e) e = cudaEventRecord(ev[1 + blast], st);
+  // The kept segments' snapshots (and tape) came from the forward run itself.
+  for (int b = 0; b < nbuf && !s && !e; ++b) e = cudaEventRecord(ev[1 + b], st);
+  // The reverse sweep of step m on the context's stream: X3 its stage data (and the scalars and nodes after
+  // it), c the state before it.
+  auto reverse_step = [&](const DevState* X3, int64_t m, const StateCopy& c) {
+    double** l = lam[cur];
+    k_misfit<1><<<gg, 128, 0, st>>>(X3[2], l[0], l[2], (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
+    A.lE = l[0];
+    A.lM = l[1];
+    A.lB = l[2];
+    A.oE = lam[cur ^ 1][0];
+    A.oM = lam[cur ^ 1][1];
+    A.oB = lam[cur ^ 1][2];
+    A.sJ = c.J;
+    launch_adj_stage<3>(ctx, X3[2], K, A, X3[2].Eb, X3[2].Mb, X3[2].Bb, X3[2].J2);
+    launch_adj_stage<2>(ctx, X3[1], K, A, X3[1].Ea, X3[1].Ma, X3[1].Ba, X3[1].J1);
+    launch_adj_stage<1>(ctx, X3[0], K, A, c.E, c.M, c.B, c.J);
+    cur ^= 1;
+  };
   bool used[2] = {false, false};
   int64_t idx = 0;
   for (int64_t sg = nseg - 1; sg >= 0 && !s && !e; --sg) {
     const int64_t n0 = sg * C, n1 = std::min(nsteps, n0 + C);
-    if (sg >= 1) {
-      // Segment sg - 1 goes into the buffer whose snapshots of segment sg + 1 st3 has read.
+    if (sg >= 1 && sg - 1 < kept) {
+      // Segment sg - 1 goes into the buffer whose snapshots of segment sg + 1 have been read.
       if (sg + 1 < nseg) e = cudaStreamWaitEvent(st2, ev[3 + ((sg + 1) & 1)], 0);
       if (!e) recompute_segment(sg - 1);
       if (s || e) break;
@@ -1811,20 +1798,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
           X3[t].x = after.x;
           X3[t].S = after.S;
         }
-        const DevState& X = X3[2];
-        AdjState At = A;
-        At.sE = before.E;
-        At.sM = before.M;
-        At.sB = before.B;
-        At.sJ = before.J;
-        k_misfit<1><<<gg, 128, 0, st>>>(X, A, (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
-        launch_adj_rk<3>(ctx, X, At);
-        launch_adj_stage<3>(ctx, X3[2], K, At, X.Eb, X.Mb, X.Bb, X.J2);
-        launch_adj_rk<2>(ctx, X, At);
-        launch_adj_stage<2>(ctx, X3[1], K, At, X.Ea, X.Ma, X.Ba, X.J1);
-        launch_adj_rk<1>(ctx, X, At);
-        launch_adj_stage<1>(ctx, X3[0], K, At, before.E, before.M, before.B, before.J);
-        launch_adj_rk<0>(ctx, X, At);
+        reverse_step(X3, m, before);
         e = cudaGetLastError();
       }
       // The segment's snapshots and slots are free once its reverse sweep is done.
@@ -1847,19 +1821,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
       if ((e = cudaEventRecord(ev[5 + k], st3))) break;
       // Reverse sweep of step m on the context's stream.
       if ((e = cudaStreamWaitEvent(st, ev[5 + k], 0))) break;
-      AdjState AR = A;  // with q^n, J^n of the step: the segment's snapshot
-      AR.sE = c.E;
-      AR.sM = c.M;
-      AR.sB = c.B;
-      AR.sJ = c.J;
-      k_misfit<1><<<gg, 128, 0, st>>>(X, A, (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
-      launch_adj_rk<3>(ctx, X, AR);
-      launch_adj_stage<3>(ctx, Ds[k][2], K, AR, X.Eb, X.Mb, X.Bb, X.J2);
-      launch_adj_rk<2>(ctx, X, AR);
-      launch_adj_stage<2>(ctx, Ds[k][1], K, AR, X.Ea, X.Ma, X.Ba, X.J1);
-      launch_adj_rk<1>(ctx, X, AR);
-      launch_adj_stage<1>(ctx, Ds[k][0], K, AR, c.E, c.M, c.B, c.J);
-      launch_adj_rk<0>(ctx, X, AR);
+      reverse_step(Ds[k], m, c);
       e = cudaGetLastError();
       if (!e) e = cudaEventRecord(ev[7 + k], st);
     }
@@ -1872,9 +1834,9 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   if (e) return release(fail(ctx, SWALE_ECUDA, std::string("adjoint: ") + cudaGetErrorString(e)));
   e = cudaSuccess;
   if (J) e = cudaMemcpyAsync(J, Jacc, B * sizeof(double), cudaMemcpyDefault, st);
-  if (!e && dJ_deta0) e = cudaMemcpyAsync(dJ_deta0, A.lE, Nt * sizeof(double), cudaMemcpyDefault, st);
-  if (!e && dJ_dhu0) e = cudaMemcpyAsync(dJ_dhu0, A.lM, Nt * sizeof(double), cudaMemcpyDefault, st);
-  if (!e && dJ_db0) e = cudaMemcpyAsync(dJ_db0, A.lB, Nt * sizeof(double), cudaMemcpyDefault, st);
+  if (!e && dJ_deta0) e = cudaMemcpyAsync(dJ_deta0, lam[cur][0], Nt * sizeof(double), cudaMemcpyDefault, st);
+  if (!e && dJ_dhu0) e = cudaMemcpyAsync(dJ_dhu0, lam[cur][1], Nt * sizeof(double), cudaMemcpyDefault, st);
+  if (!e && dJ_db0) e = cudaMemcpyAsync(dJ_db0, lam[cur][2], Nt * sizeof(double), cudaMemcpyDefault, st);
   if (!e) e = cudaStreamSynchronize(st);
   if (e) return release(fail(ctx, SWALE_ECUDA, cudaGetErrorString(e)));
   std::vector<DevScalars> Sh;
@@ -2044,8 +2006,6 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   D.IC = &scr->ic;
   D.S = &scr->S;
   D.w = const_cast<double*>(w);
-  D.nr = (int32_t)((N + 2 + kNoAllocTile - 1) / kNoAllocTile);
-  D.nu = (int32_t)((N + kNoAllocTile - 1) / kNoAllocTile);
   D.nf = (int32_t)((N + kNoAllocTile - 2) / (kNoAllocTile - 1));
   D.nrf = (int32_t)((N + 2 + kNoAllocTile - 5) / (kNoAllocTile - 4));
   D.ic1.N = N;

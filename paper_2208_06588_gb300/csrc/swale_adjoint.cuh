@@ -420,4 +420,144 @@ SWALE_HD void recon_cell_rev_lin(const SchemeConst& P, const real Kf[2][4], cons
     }
 }
 
+// ------------------------------------------------------------------------------------
+// Reverse of the forms that the stage kernels evaluate (swale_cell.cuh), used by k_adj_stage.
+// ------------------------------------------------------------------------------------
+// Adjoint of interface_flux2<0>: from the adjoints of (FE, FMl, FMr, FB) those of the edge state on
+// either side (the depths enter through E - b* only).
+struct FaceAdj {
+  real EL, BL, uL, ER, BR, uR;
+};
+SWALE_HD FaceAdj interface_flux2_rev(real g, real alpha, real w, real EL, real ER, real BL, real BR, real uL, real uR,
+                                     real FEb, real FMlb, real FMrb, real FBb) {
+  const bool selR = dlt(BL, BR);
+  const real bstar = selR ? BR : BL;
+  const real aL = EL - bstar, aR = ER - bstar;
+  const bool pL = gt0(aL), pR = gt0(aR);
+  const real sL = pL ? aL : real(0.0), sR = pR ? aR : real(0.0);
+  const real mL = sL * uL, mR = sR * uR;
+  const real Mb = FMlb + FMrb, q2 = g * (FMlb - FMrb);  // 2 (adjoint of Q), Q = (g/2) (sR^2 - sL^2)
+  const real mLb = FEb + Mb * ((uL - w) + alpha), mRb = FEb + Mb * ((uR - w) - alpha);
+  const real sLb = pL ? mLb * uL - q2 * sL : real(0.0), sRb = pR ? mRb * uR + q2 * sR : real(0.0);
+  const real am = alpha - w, ap = alpha + w, bs = sLb + sRb;
+  FaceAdj a;
+  a.EL = am * FEb + sLb;
+  a.ER = sRb - ap * FEb;
+  a.BL = -(am * FBb);
+  a.BR = ap * FBb;
+  if (selR) a.BR = a.BR - bs;
+  else a.BL = a.BL - bs;
+  a.uL = Mb * mL + mLb * sL;
+  a.uR = Mb * mR + mRb * sR;
+  return a;
+}
+
+// Adjoint of source_pressure_form for the adjoint ab of its value.
+struct SourceAdj {
+  real hc, hL, hR, deL, deR, dEl, dHl, dEr, dHr;
+};
+SWALE_HD SourceAdj source_pressure_rev(real hc, real hL, real hR, real deL, real deR, real dEl, real dHl, real dEr,
+                                       real dHr, real rho_l, real sig2_l, real sig_r, real rho2_r, const SourceRatio& s,
+                                       real ab) {
+  const real dhL = hL - hc, dhR = hR - hc;
+  const real Xe = (deL + rho_l * deR) + sig2_l * dEl, Ye = (deR + sig_r * deL) - rho2_r * dEr;
+  const real Xh = (dhL + rho_l * dhR) + sig2_l * dHl, Yh = (dhR + sig_r * dhL) - rho2_r * dHr;
+  const real Ge = (deR + s.GX * Xe) + s.GY * Ye, Gh = (dhR + s.GX * Xh) + s.GY * Yh;
+  const real ce = deL + deR, ch = dhL + dhR;
+  // acc = deR (hc + hR) - deL (hc + hL) + Gh ce - ch Ge + K3 (Xh Ye - Yh Xe)
+  const real Ghb = ab * ce, ceb = ab * Gh, chb = -(ab * Ge), Geb = -(ab * ch), k = ab * s.K3;
+  const real Xhb = k * Ye + s.GX * Ghb, Yhb = s.GY * Ghb - k * Xe;
+  const real Xeb = s.GX * Geb - k * Yh, Yeb = k * Xh + s.GY * Geb;
+  const real pR = ab * deR, pL = ab * deL;  // adjoints of (hc + hR), -(hc + hL)
+  const real dhLb = (Xhb + sig_r * Yhb) + chb, dhRb = (Ghb + (rho_l * Xhb + Yhb)) + chb;
+  SourceAdj a;
+  a.deL = ((Xeb + sig_r * Yeb) + ceb) - ab * (hc + hL);
+  a.deR = ((Geb + (rho_l * Xeb + Yeb)) + ceb) + ab * (hc + hR);
+  a.hL = dhLb - pL;
+  a.hR = dhRb + pR;
+  a.hc = (pR - pL) - (dhLb + dhRb);
+  a.dEl = sig2_l * Xeb;
+  a.dHl = sig2_l * Xhb;
+  a.dEr = -(rho2_r * Yeb);
+  a.dHr = -(rho2_r * Yhb);
+  return a;
+}
+
+// Adjoint of smooth_left / smooth_right of one variable: from those of its edge values (eL, eR) the
+// adjoints of the cell average and of the differences: the pairs left and right of the cell, the triple
+// centred on it, the two quadruples.
+struct SmoothAdj {
+  real v, d2l, d2r, d3, d4l, d4r;
+};
+SWALE_HD SmoothAdj smooth_rev(const SmoothWidths& w, real iv, real eL, real eR) {
+  SmoothAdj a;
+  a.v = eL + eR;
+  a.d2r = w.h2 * eR;
+  const real r3 = -(w.h3 * a.d2r);
+  const real r4 = w.p12 * r3;
+  a.d2l = -(w.h2 * eL);
+  const real l3 = w.h1 * a.d2l;
+  const real l4 = -(w.p23 * l3);
+  a.d3 = r3 + l3;
+  const real t5 = (w.p01 * l4 - w.p34 * r4) * iv;
+  a.d4r = r4 + t5;
+  a.d4l = l4 - t5;
+  return a;
+}
+
+// The reverse of a cell by recon_cell_rev (any class, the limiter active or not), for the variables
+// (eta, hu, h = eta - b) and in the same differences as SmoothAdj: what falls on the outer averages, pairs
+// and triples is passed on through v_{j-1} = v_j - p12 D2l, D2 of the outer pairs = D2l - t_l D3l and
+// D2r + t_r D3r, D3l = D3 - q_l D4l, D3r = D3 + q_r D4r (p, t, q the sums of two, three, four widths).
+//   J[5], E[5], M[5], H[5]: widths and averages of cells j-2..j+2.
+SWALE_HD void cell_rev_general(const SchemeConst& P, const real J[5], const real E[5], const real M[5], const real H[5],
+                               real dxmax, const EdgeAdj& ob, SmoothAdj out[3]) {
+  StencilDD DD, DDb;
+  real v0[3][3], v0b[3][3], it[3], V[3][5];
+  for (int k = 0; k < 5; ++k) {
+    V[0][k] = E[k];
+    V[1][k] = M[k];
+    V[2][k] = E[k] - H[k];
+  }
+  const real t[3] = {J[0] + J[1] + J[2], J[1] + J[2] + J[3], J[2] + J[3] + J[4]};
+  for (int a = 0; a < 3; ++a) it[a] = recip(t[a]);
+  for (int v = 0; v < 3; ++v) {
+    for (int a = 0; a < 4; ++a) DD.D2[v][a] = (V[v][a + 1] - V[v][a]) * recip(J[a] + J[a + 1]);
+    for (int a = 0; a < 3; ++a) {
+      DD.D3[v][a] = (DD.D2[v][a + 1] - DD.D2[v][a]) * it[a];
+      v0[v][a] = V[v][a];
+    }
+  }
+  recon_cell_rev(P, J, it, v0, DD, dxmax, ob, v0b, DDb, false);
+  const real ql = t[0] + J[3], qr = t[1] + J[4];
+  SmoothAdj s[3];
+  for (int v = 0; v < 3; ++v) {
+    real v2 = v0b[v][2], b1 = v0b[v][1], b0 = v0b[v][0];
+    real e0 = DDb.D2[v][0], e1 = DDb.D2[v][1], e2 = DDb.D2[v][2], e3 = DDb.D2[v][3];
+    real f0 = DDb.D3[v][0], f1 = DDb.D3[v][1], f2 = DDb.D3[v][2];
+    // v_{j-2} = v_{j-1} - p01 D2[0], v_{j-1} = v_j - p12 D2[1]
+    e0 = e0 - (J[0] + J[1]) * b0;
+    b1 = b1 + b0;
+    e1 = e1 - (J[1] + J[2]) * b1;
+    v2 = v2 + b1;
+    // D2[0] = D2[1] - t0 D3[0], D2[3] = D2[2] + t2 D3[2]
+    e1 = e1 + e0;
+    f0 = f0 - t[0] * e0;
+    e2 = e2 + e3;
+    f2 = f2 + t[2] * e3;
+    // D3[0] = D3[1] - ql D4l, D3[2] = D3[1] + qr D4r
+    s[v].v = v2;
+    s[v].d2l = e1;
+    s[v].d2r = e2;
+    s[v].d3 = f1 + (f0 + f2);
+    s[v].d4l = -(ql * f0);
+    s[v].d4r = qr * f2;
+  }
+  // b = eta - h
+  out[0] = {s[0].v + s[2].v, s[0].d2l + s[2].d2l, s[0].d2r + s[2].d2r, s[0].d3 + s[2].d3, s[0].d4l + s[2].d4l,
+            s[0].d4r + s[2].d4r};
+  out[1] = s[1];
+  out[2] = {-s[2].v, -s[2].d2l, -s[2].d2r, -s[2].d3, -s[2].d4l, -s[2].d4r};
+}
+
 }  // namespace swale

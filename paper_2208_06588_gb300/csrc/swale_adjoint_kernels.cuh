@@ -1,10 +1,6 @@
 // Device kernels of the discrete adjoint of one SSP-RK3 step (Eq. RK32D) of the well-balanced
-// ALE-WENO hybrid scheme: reverse of the RK combination, and for each stage the reverse of the
-// interface fluxes, of the source term and of the reconstruction + limiter. They walk the same
-// (instance, tile) work lists as the forward kernels; the adjoints of the stage input are
-// accumulated with FP64 atomicAdd (each cell receives the contributions of the stencils, fluxes
-// and sources that read it; ghost cells map back to their physical image, with the discharge's
-// sign flipped at reflective boundaries).
+// ALE-WENO hybrid scheme: one kernel per stage reverses its RK combination, fluxes, source,
+// limiter and reconstruction, and the gauge misfit seeds the adjoint of the state.
 #pragma once
 
 #include "swale_adjoint.cuh"
@@ -12,379 +8,313 @@
 
 namespace swale_dev {
 
-// Adjoint work arrays (concatenated like the state; edge adjoints in the edge layout).
+// What the reverse of a stage reads per cell besides its edge states, kept by the recompute's kernels
+// in DevState::gK (ADJ_*): reciprocal sums of four and five widths, the interfaces' width ratios and the
+// source's, the class (0, 1, 2, plus 4 where the limiter acted), and the differences and depths of the
+// stage (DevState::dE, dH, H point there).
+static_assert(ADJ_ARRAYS <= 14, "swale_adjoint_bytes counts 14 arrays per stage");
+
+// Adjoint work arrays (concatenated like the state).
 struct AdjState {
-  double *lE, *lM, *lB;   // lambda: adjoint of q^{n+1} on entry, of q^n on exit
-  double *yE, *yM, *yB;   // adjoint of the running RK combination Y
-  double *pE, *pM, *pB;   // accumulated adjoint of q^n through the RK combination
-  double *aE, *aM, *aB;   // adjoint of the current stage input (atomically accumulated)
-  double *rE, *rM, *rB;   // adjoint of the current stage's right-hand side
-  double *ab[8];          // adjoints of the edge state (EL, ER, BL, BR, hL, hR, uL, uR)
-  double *sE, *sM, *sB, *sJ;  // q^n and J^n of the step being reversed
+  const double *lE, *lM, *lB;  // lambda: adjoint of q^{n+1}
+  double *oE, *oM, *oB;        // adjoint of q^n (another buffer: neighbours still read lambda)
+  double *a3[3], *a2[3];       // adjoints of the inputs of stages 3 and 2
+  const double *sJ;            // J^n of the step being reversed
+  const Tile* tiles;           // blocks (instance, index), null: one instance
 };
 
-__device__ __forceinline__ Tile utile_of(const DevState& D, int t, int T) {
-  return D.utiles ? D.utiles[t] : Tile{0, t * T};
-}
+constexpr int kAdjThreads = 128;
+constexpr int kAdjCells = kAdjThreads - 8;  // cells a block owns at most: four on each side are its neighbours'
 
-// Reverse of the RK combination, one phase per call. With Y3 = J3 q^{n+1}:
-//   PH 3: Y = lambda / J3;  p = J0 Y / 3;  y = 2 Y / 3;  r = 2 dt Y / 3
-//   PH 2: y += a / J2;      p += 3 J0 y / 4;  r = dt y / 4;  y = y / 4
-//   PH 1: y += a / J1;      p += J0 y;        r = dt y
-//   PH 0: lambda = p + a
-// a (the stage adjoint of the previous phase) is read and cleared.
-template <int PH, int T>
-__global__ void __launch_bounds__(T) k_adj_rk(DevState D, AdjState A) {
-  for (int t = blockIdx.x; t < D.nu; t += gridDim.x) {
-    const Tile tl = utile_of(D, t, T);
-    const InstConst ic = D.IC[tl.inst];
-    const int64_t j = tl.c0 + threadIdx.x;
-    if (j >= ic.N) continue;
-    const int64_t g = ic.coff + j;
-    const double dt = D.S[tl.inst].dt;
-    double* lv[3] = {A.lE, A.lM, A.lB};
-    double* yv[3] = {A.yE, A.yM, A.yB};
-    double* pv[3] = {A.pE, A.pM, A.pB};
-    double* av[3] = {A.aE, A.aM, A.aB};
-    double* rv[3] = {A.rE, A.rM, A.rB};
-    const double J0 = A.sJ[g];
-    // All loads of the phase are issued before its first store (the arrays never alias, but
-    // the compiler cannot know), so the memory latencies overlap instead of adding up.
-    if (PH == 3) {
-      const double iJ3 = swale::recip(D.J0[g]);  // J^{n+1} after the recomputed step
-      double l[3];
-#pragma unroll
-      for (int v = 0; v < 3; ++v) l[v] = lv[v][g];
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        const double Y = l[v] * iJ3;
-        pv[v][g] = (1.0 / 3.0) * J0 * Y;
-        yv[v][g] = (2.0 / 3.0) * Y;
-        rv[v][g] = (2.0 / 3.0) * dt * Y;
-      }
-    } else if (PH == 2) {
-      const double iJ2 = swale::recip(D.J2[g]);
-      double y0[3], a[3], p[3];
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        y0[v] = yv[v][g];
-        a[v] = av[v][g];
-        p[v] = pv[v][g];
-      }
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        const double y = y0[v] + a[v] * iJ2;
-        av[v][g] = 0.0;
-        pv[v][g] = p[v] + 0.75 * J0 * y;
-        rv[v][g] = 0.25 * dt * y;
-        yv[v][g] = 0.25 * y;
-      }
-    } else if (PH == 1) {
-      const double iJ1 = swale::recip(D.J1[g]);
-      double y0[3], a[3], p[3];
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        y0[v] = yv[v][g];
-        a[v] = av[v][g];
-        p[v] = pv[v][g];
-      }
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        const double y = y0[v] + a[v] * iJ1;
-        av[v][g] = 0.0;
-        pv[v][g] = p[v] + J0 * y;
-        rv[v][g] = dt * y;
-      }
-    } else {
-      double p[3], a[3];
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        p[v] = pv[v][g];
-        a[v] = av[v][g];
-      }
-#pragma unroll
-      for (int v = 0; v < 3; ++v) {
-        lv[v][g] = p[v] + a[v];
-        av[v][g] = 0.0;
-      }
-    }
-  }
-}
+// Cells of block b of an instance of N cells: the blocks are balanced, so that the last three cells of
+// an instance, whose ghost images the block folds back itself, are in one block.
+__device__ __host__ __forceinline__ int32_t adj_blocks(int64_t N) { return (int32_t)((N + kAdjCells - 1) / kAdjCells); }
+__device__ __forceinline__ int32_t adj_first(int32_t b, int32_t nb, int32_t N) { return (int32_t)((int64_t)b * N / nb); }
 
-// Reverse of the interface fluxes of stage STAGE: interface k of cells k-1 and k gets the
-// flux adjoints from the right-hand-side adjoints of its two cells and writes the adjoints of
-// the right edge of cell k-1 and of the left edge of cell k (each edge slot has one writer).
-template <int STAGE, int T>
-__global__ void __launch_bounds__(T) k_adj_flux(StepConst K, DevState D, AdjState A) {
-  for (int t = blockIdx.x; t < D.nu; t += gridDim.x) {
-    const Tile tl = utile_of(D, t, T);
-    const InstConst ic = D.IC[tl.inst];
-    const DevScalars* S = D.S + tl.inst;
-    const int64_t N = ic.N, cb = ic.coff, nb = ic.coff + tl.inst, eb = ic.coff + 2 * (int64_t)tl.inst;
-    double alpha = (STAGE == 1) ? S->alpha1 : bitsd(S->A[STAGE - 1]) + S->Wbar;
-    if (STAGE > 1 && K.alpha_mode == 2) alpha = stage_alpha(K, tl.inst, STAGE, alpha, S->step_idx);
-    for (int i = threadIdx.x; i <= T; i += T) {
-      const int64_t k = tl.c0 + i;
-      if (k > N || (i == T && k != N)) continue;
-      swale::Flux Fb;
-      const double rEr = (k < N) ? A.rE[cb + k] : 0.0, rEl = (k > 0) ? A.rE[cb + k - 1] : 0.0;
-      const double rMr = (k < N) ? A.rM[cb + k] : 0.0, rMl = (k > 0) ? A.rM[cb + k - 1] : 0.0;
-      const double rBr = (k < N) ? A.rB[cb + k] : 0.0, rBl = (k > 0) ? A.rB[cb + k - 1] : 0.0;
-      Fb.FE = rEr - rEl;
-      Fb.FMm = -rMl;
-      Fb.FMp = rMr;
-      Fb.FB = rBl - rBr;
-      const double wk = (K.mesh == SWALE_MESH_STATIC) ? 0.0 : D.w[nb + k];
-      const int64_t el = eb + k, er = eb + k + 1;
-      if (k == 0) {  // the ghost cell -1 has no left interface
-        A.ab[0][el] = 0.0;
-        A.ab[2][el] = 0.0;
-        A.ab[4][el] = 0.0;
-        A.ab[6][el] = 0.0;
-      }
-      if (k == N) {  // the ghost cell N has no right interface
-        A.ab[1][er] = 0.0;
-        A.ab[3][er] = 0.0;
-        A.ab[5][er] = 0.0;
-        A.ab[7][er] = 0.0;
-      }
-      const swale::EdgeAdj a = swale::interface_flux_rev(K.sc.g, alpha, wk, D.eER[el], D.eEL[er], D.eBR[el],
-                                                         D.eBL[er], D.ehR[el], D.ehL[er], D.euR[el], D.euL[er], Fb);
-      // interface_flux_rev names its inputs as (left state, right state) = (EL, ER, ...).
-      A.ab[1][el] = a.EL;  // right edge of cell k-1
-      A.ab[3][el] = a.BL;
-      A.ab[5][el] = a.hL;
-      A.ab[7][el] = a.uL;
-      A.ab[0][er] = a.ER;  // left edge of cell k
-      A.ab[2][er] = a.BR;
-      A.ab[4][er] = a.hR;
-      A.ab[6][er] = a.uR;
-    }
-  }
-}
-
-// Reverse of the source term of stage STAGE for cell j: adds to the adjoints of its own
-// limited edge depths and bottoms, and (atomically) to the stage-input adjoints of the depth
-// and bottom averages of cells j-1, j, j+1.
-template <int STAGE, int T>
-__global__ void __launch_bounds__(T) k_adj_source(StepConst K, DevState D, AdjState A, const double* __restrict__ Eg,
-                                                  const double* __restrict__ Bg, const double* __restrict__ Jsg) {
-  for (int t = blockIdx.x; t < D.nu; t += gridDim.x) {
-    const Tile tl = utile_of(D, t, T);
-    const InstConst ic = D.IC[tl.inst];
-    const int64_t N = ic.N, cb = ic.coff, eb = ic.coff + 2 * (int64_t)tl.inst;
-    const int64_t j = tl.c0 + threadIdx.x;
-    if (j >= N) continue;
-    const int64_t jm = ghost(j - 1, N, K.bc), jp = ghost(j + 1, N, K.bc);
-    const double* E = Eg + cb;
-    const double* B = Bg + cb;
-    const double* Js = Jsg + cb;
-    const double Jm = Js[jm], Jc = Js[j], Jp = Js[jp];
-    const int64_t ie = eb + j + 1;
-    // The source form's entries: as the forward recompute's update stored them, else computed.
-    swale::SourceForm sf;
-    if (D.gK) {
-      double* const f = reinterpret_cast<double*>(&sf);
-#pragma unroll
-      for (int k = 0; k < 6; ++k) f[k] = D.gK[(8 + k) * D.geo_stride + ie];
-    } else {
-      sf = swale::source_form(Jm, Jc, Jp, swale::recip(Jm), swale::recip(Jc), swale::recip(Jp), D.ipair[eb + j],
-                              D.ipair[eb + j + 1], D.itri[eb + j + 1]);
-    }
-    const double hd[5] = {E[jm] - B[jm], E[j] - B[j], E[jp] - B[jp], D.ehL[ie], D.ehR[ie]};
-    const double bd[5] = {B[jm], B[j], B[jp], D.eBL[ie], D.eBR[ie]};
-    double hdb[5] = {0, 0, 0, 0, 0}, bdb[5] = {0, 0, 0, 0, 0};
-    swale::source_cell_form_rev(K.sc.g, hd, bd, sf, A.rM[cb + j], hdb, bdb);
-    A.ab[4][ie] += hdb[3];
-    A.ab[5][ie] += hdb[4];
-    A.ab[2][ie] += bdb[3];
-    A.ab[3][ie] += bdb[4];
-    const int64_t cells[3] = {jm, j, jp};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      atomicAdd(&A.aE[cb + cells[k]], hdb[k]);
-      atomicAdd(&A.aB[cb + cells[k]], bdb[k] - hdb[k]);
-    }
-  }
-}
-
-// The reverse of a cell whose class the FP32 test leaves open, out of line (the FP64 detector,
-// the WENO-Z weights and their adjoints): its registers do not weigh on the smooth cells' code.
-struct AdjOpenIn {
-  swale::StencilDD DD;
+// The reverse of a cell that is not smooth or whose limiter acted, out of line.
+struct AdjCellIn {
+  double J[5], E[5], M[5], H[5];
   swale::EdgeAdj ob;
-  double h[5], it[3], v0[3][3], dxmax;
 };
-struct AdjOpenOut {
-  swale::StencilDD DDb;
-  double v0b[3][3];
+struct AdjCellOut {
+  swale::SmoothAdj s[3];
 };
-__device__ __noinline__ AdjOpenOut adj_open_cell(const SchemeConst P, const AdjOpenIn c) {
-  AdjOpenOut r;
-  swale::recon_cell_rev(P, c.h, c.it, c.v0, c.DD, c.dxmax, c.ob, r.v0b, r.DDb, false);
+__device__ __noinline__ AdjCellOut adj_general_cell(const SchemeConst P, const AdjCellIn c, double dxmax) {
+  AdjCellOut r;
+  swale::cell_rev_general(P, c.J, c.E, c.M, c.H, dxmax, c.ob, r.s);
   return r;
 }
 
-// Reverse of the reconstruction + limiter of stage STAGE for cells -1..N (tiles of T cells
-// staged like the forward kernel): each cell's reverse sweep gives the adjoints of its stencil
-// averages and divided differences, which map to the 5 stencil cells and are added atomically.
-template <int STAGE, int T>
-__global__ void __launch_bounds__(T, 512 / T) k_adj_recon(StepConst K, DevState D, AdjState A, const double* __restrict__ Eg,
-                                                 const double* __restrict__ Mg, const double* __restrict__ Bg,
-                                                 const double* __restrict__ Jg) {
-  __shared__ double sJ[T + 4], sV[3][T + 4];
-  __shared__ double sIP[T + 3], sD2[3][T + 3];
-  __shared__ double sIT[T + 2];
-  // FP32 copies for the smooth-class test of the forward: pair differences of hu and of the
-  // depth (eta's minus the bottom's), triple reciprocals.
-  __shared__ float sD2f[2][T + 3], sITf[T + 2];
+// Reverse of stage STAGE. With Y3 = lambda / J^{n+1}, y2 = (2/3) Y3 + a3 / J^(2), y1 = y2 / 4 + a2 / J^(1) (a_s the adjoint of
+// stage s's input), twice the stages' right-hand sides have the adjoints dt Y3 / 3, dt y2 / 8, dt y1 / 2, and the
+// adjoint of q^n is J^n (Y3 / 3 + 3 y2 / 4 + y1) + a1: every block forms these for its cells and their
+// neighbours from lambda, a3 and a2, which nobody writes meanwhile, so no kernel of its own
+// combines them. A block owns up to 120 cells, one per thread, and takes four more on each side: it
+// gathers what falls on its cells from the cells and interfaces around them (the transpose of the
+// differences runs through shared memory, order by order, as the forward builds them), instead of
+// scattering 15 atomic additions per cell; ghost cells' shares are folded back to their images.
+// Per cell about 210 FP64 instructions, which bound it; in a smooth cell whose limiter did not act
+// nothing of the forward is formed again but the source's functionals.
+// E, M, B, J: the stage's input and widths. Runs are bitwise reproducible up to the misfit's seeds.
+template <int STAGE>
+__global__ void __launch_bounds__(kAdjThreads, 4) k_adj_stage(StepConst K, DevState D, AdjState A, const double* __restrict__ Eg,
+                                                              const double* __restrict__ Mg, const double* __restrict__ Bg,
+                                                              const double* __restrict__ Jg) {
+  constexpr int T = kAdjThreads;
+  __shared__ double rE[T], rM[T], rH[T], rJ[T + 4];
+  __shared__ double sRho[3][T], sR[4][T], sX[3][T], sDl[2][T];
+  __shared__ double sD2l[3][T], sD3[3][T], sD4l[3][T], sD4r[3][T], sT[3][T];
   const int tid = threadIdx.x;
-  const bool refl = (K.bc == SWALE_BC_REFLECTIVE);
-  for (int t = blockIdx.x; t < D.nr; t += gridDim.x) {
-    const Tile tl = D.rtiles ? D.rtiles[t] : Tile{0, t * T - 1};
-    const DevScalars* S = D.S + tl.inst;
-    const InstConst ic = D.IC[tl.inst];
-    const int64_t N = ic.N, c0 = tl.c0, cb = ic.coff;
-    const double* E = Eg + cb;
-    const double* M = Mg + cb;
-    const double* B = Bg + cb;
-    const double* J = Jg + cb;
-    const int64_t eb = ic.coff + 2 * (int64_t)tl.inst;
-    __syncthreads();
-    for (int i = tid; i < T + 4; i += T) {
-      const int64_t c = c0 - 2 + i;
-      double jv = 1.0, ev = 0.0, mv = 0.0, bv = 0.0;
-      if (c >= -3 && c <= N + 2) {
-        const int64_t s = ghost(c, N, K.bc);
-        jv = J[s];
-        ev = E[s];
-        bv = B[s];
-        mv = M[s];
-        if (refl && (c < 0 || c >= N)) mv = -mv;
-      }
-      sJ[i] = jv;
-      sV[0][i] = ev;
-      sV[1][i] = mv;
-      sV[2][i] = bv;
-    }
-    __syncthreads();
-    for (int i = tid; i < T + 3; i += T) {
-      const double ip = swale::pair_recip(sJ[i], sJ[i + 1]);
-      sIP[i] = ip;
-      double d2[3];
+  const Tile tl = A.tiles ? A.tiles[blockIdx.x] : Tile{0, (int32_t)blockIdx.x};
+  const InstConst ic = A.tiles ? D.IC[tl.inst] : D.ic1;
+  const DevScalars* S = D.S + tl.inst;
+  const int32_t N = (int32_t)ic.N, nb = adj_blocks(N);
+  const int32_t first = adj_first(tl.c0, nb, N), last = adj_first(tl.c0 + 1, nb, N);  // owned cells [first, last)
+  const int32_t c = first - 4 + tid;
+  const bool own = tid >= 4 && c < last;
+  const bool near = c <= last + 3;  // within the cells that contribute
+  const bool per = K.bc == SWALE_BC_PERIODIC;
+  // A cell of the domain (periodic: of its continuation), one whose edges were reconstructed, an interface.
+  const bool real = near && (per || (c >= 0 && c < N));
+  const bool recon = near && (per || (c >= -1 && c <= N));
+  const bool face = near && tid >= 1 && (per || (c >= 0 && c <= N));
+  const int32_t gl = near ? ghost(c, N, K.bc) : 0;          // where its averages lie
+  const int32_t g = (int32_t)ic.coff + gl;
+  const int32_t eb = (int32_t)(ic.coff + 2 * (int64_t)tl.inst);
+  const int32_t e = eb + (recon ? (per ? gl : c) + 1 : 1);  // its edge-array index
+  const bool flip = K.bc == SWALE_BC_REFLECTIVE && (c < 0 || c >= N);
+  const double dt = S->dt, dxmax = bitsd(S->Jmax[STAGE - 1]);
+  double alpha = (STAGE == 1) ? S->alpha1 : bitsd(S->A[STAGE - 1]) + S->Wbar;
+  if (STAGE > 1 && K.alpha_mode == 2) alpha = stage_alpha(K, tl.inst, STAGE, alpha, S->step_idx);
+
+  const double ev = Eg[g], jv = near ? Jg[g] : 1.0;
+  const double hv = swale::sub_(ev, Bg[g]);
+  rE[tid] = ev;
+  rM[tid] = flip ? -Mg[g] : Mg[g];
+  rH[tid] = hv;
+  rJ[tid] = jv;
+  double q[3] = {0.0, 0.0, 0.0};  // Y3 / 3 + 3 y2 / 4 + y1 (stage 1)
+  {
+    double rho[3] = {0.0, 0.0, 0.0};
+    if (real) {
+      const double i1 = swale::recip(D.J1[g]);  // J^{n+1} = J^(1)
+      const double i2 = STAGE < 3 ? swale::recip(D.J2[g]) : 0.0;
+      const double l[3] = {A.lE[g], A.lM[g], A.lB[g]};
 #pragma unroll
-      for (int v = 0; v < 3; ++v) sD2[v][i] = d2[v] = swale::pair_dd(sV[v][i], sV[v][i + 1], ip);
-      sD2f[0][i] = swale::f32_trunc(d2[1]);
-      sD2f[1][i] = swale::f32_trunc(d2[0] - d2[2]);
-    }
-    __syncthreads();
-    for (int i = tid; i < T + 2; i += T) {
-      const double it = swale::triple_recip(sJ[i], sJ[i + 1], sJ[i + 2]);
-      sIT[i] = it;
-      sITf[i] = swale::f32_trunc(it);
-    }
-    __syncthreads();
-    const int64_t c = c0 + tid;
-    if (c > N) continue;
-    double h[5], v0[3][3];
-    swale::StencilDD DD, DDb;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) h[k] = sJ[tid + k];
-#pragma unroll
-    for (int v = 0; v < 3; ++v) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) v0[v][a] = sV[v][tid + a];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) DD.D2[v][a] = sD2[v][tid + a];
-    }
-    const int64_t idx = eb + c + 1;
-    const swale::EdgeAdj ob = {A.ab[0][idx], A.ab[1][idx], A.ab[2][idx], A.ab[3][idx],
-                               A.ab[4][idx], A.ab[5][idx], A.ab[6][idx], A.ab[7][idx]};
-    double v0b[3][3];
-    const double it3[3] = {sIT[tid], sIT[tid + 1], sIT[tid + 2]};
-    // The forward's FP32 test of the smooth class on the same data: where it holds, the FP64
-    // class is 0 as well and the indicators are not formed.
-    const double dxmax = bitsd(S->Jmax[STAGE - 1]);
-    float F32[3], c4f, c3f, itf[3], d2h[4], d2m[4];
-    swale::indicator_factors_f32(h, K.sc.beta_dx_global ? dxmax : h[2], F32, c4f, c3f);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) itf[a] = sITf[tid + a];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      d2h[a] = sD2f[1][tid + a];
-      d2m[a] = sD2f[0][tid + a];
-    }
-    const bool smooth32 =
-        swale::sure_smooth_f32(F32, c4f, c3f, d2h, d2m, itf, swale::f32_trunc(K.sc.eps_weno));
-    if (smooth32) {
-      if (D.gK) {  // the linear form the forward recompute stored for this stage
-        double Kf[2][4];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) Kf[k >> 2][k & 3] = D.gK[k * D.geo_stride + idx];
-        swale::recon_cell_rev_lin(K.sc, Kf, v0, DD, ob, v0b, DDb);
-      } else {
-        swale::recon_cell_rev(K.sc, h, it3, v0, DD, dxmax, ob, v0b, DDb, true);
-      }
-    } else {
-      // The third differences, only where the class is open (the smooth class needs none).
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) DD.D3[v][a] = swale::triple_dd(DD.D2[v][a], DD.D2[v][a + 1], it3[a]);
-      AdjOpenIn in;
-      in.DD = DD;
-      in.ob = ob;
-      in.dxmax = dxmax;
-#pragma unroll
-      for (int k = 0; k < 5; ++k) in.h[k] = h[k];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) in.it[a] = it3[a];
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) in.v0[v][a] = v0[v][a];
-      const AdjOpenOut r = adj_open_cell(K.sc, in);
-      DDb = r.DDb;
-#pragma unroll
-      for (int v = 0; v < 3; ++v)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) v0b[v][a] = r.v0b[v][a];
-    }
-    // Stencil cell adjoints: cv[v][k] for cells c-2+k.
-    double cv[3][5];
-#pragma unroll
-    for (int v = 0; v < 3; ++v) {
-#pragma unroll
-      for (int k = 0; k < 5; ++k) cv[v][k] = 0.0;
-#pragma unroll
-      for (int a = 0; a < 3; ++a) cv[v][a] += v0b[v][a];
-      double d2b[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) d2b[a] = DDb.D2[v][a];
-      if (!smooth32) {  // DDb.D3 is 0 in the smooth class
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {  // D3[a] = (D2[a+1] - D2[a]) it[a]
-          const double x = DDb.D3[v][a] * sIT[tid + a];
-          d2b[a + 1] += x;
-          d2b[a] -= x;
+      for (int v = 0; v < 3; ++v) {
+        const double Y3 = l[v] * i1;
+        if (STAGE == 3) {
+          rho[v] = (1.0 / 3.0) * dt * Y3;
+        } else {
+          const double y2 = (2.0 / 3.0) * Y3 + A.a3[v][g] * i2;
+          if (STAGE == 2) {
+            rho[v] = 0.125 * dt * y2;
+          } else {
+            const double y1 = 0.25 * y2 + A.a2[v][g] * i1;
+            rho[v] = 0.5 * dt * y1;
+            q[v] = (1.0 / 3.0) * Y3 + (0.75 * y2 + y1);
+          }
         }
       }
+    }
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {  // D2[a] = (v[a+1] - v[a]) ip[a]
-        const double x = d2b[a] * sIP[tid + a];
-        cv[v][a + 1] += x;
-        cv[v][a] -= x;
+    for (int v = 0; v < 3; ++v) sRho[v][tid] = rho[v];
+  }
+  // Edge state of the cell; its right edge for the interface on its right.
+  swale::EdgeState o{0.0, 0.0, 0.0, 0.0, 1.0, 1.0, 0.0, 0.0};
+  if (recon) o = {D.eEL[e], D.eER[e], D.eBL[e], D.eBR[e], D.ehL[e], D.ehR[e], D.euL[e], D.euR[e]};
+  sR[0][tid] = o.ER;
+  sR[1][tid] = o.BR;
+  sR[3][tid] = o.uR;
+  __syncthreads();
+  // Fluxes: interface c, between cells c - 1 and c. The right edge of cell c - 1 gets its share through sX.
+  swale::FaceAdj f{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (face) {
+    // (A periodic domain whose end nodes move apart: each cell has its own end's velocity.)
+    const double* wv = D.w + ic.coff + tl.inst;
+    const bool moving = K.mesh != SWALE_MESH_STATIC;
+    const double wr = moving ? wv[per ? gl : c] : 0.0, wl = moving && per && gl == 0 ? wv[N] : wr;
+    const double* l = &sRho[0][tid - 1];
+    const double* r = &sRho[0][tid];
+    const bool both = wl == wr;
+    for (int p = both ? 1 : 0; p < 2; ++p) {  // p = 1: the right cell's share (or both), 0: the left one's
+      const double zl = p && !both ? 0.0 : 1.0, zr = p ? 1.0 : 0.0;
+      const swale::FaceAdj h = swale::interface_flux2_rev(K.sc.g, alpha, p ? wr : wl, sR[0][tid - 1], o.EL, sR[1][tid - 1],
+                                                          o.BL, sR[3][tid - 1], o.uL, zr * r[0] - zl * l[0], -(zl * l[T]),
+                                                          zr * r[T], zl * l[2 * T] - zr * r[2 * T]);
+      f.EL += h.EL;
+      f.BL += h.BL;
+      f.uL += h.uL;
+      f.ER += h.ER;
+      f.BR += h.BR;
+      f.uR += h.uR;
+    }
+  }
+  sX[0][tid] = f.EL;
+  sX[1][tid] = f.BL;
+  sX[2][tid] = f.uL;
+  __syncthreads();
+  const bool inner = recon && tid < T - 1;
+  swale::EdgeAdj ob{f.ER, 0.0, f.BR, 0.0, 0.0, 0.0, f.uR, 0.0};
+  if (inner) {
+    ob.ER = sX[0][tid + 1];
+    ob.BR = sX[1][tid + 1];
+    ob.uR = sX[2][tid + 1];
+  }
+  // Pressure and source.
+  double Eb = 0.0, Hb = 0.0, dEr = 0.0, dHr = 0.0, dEl = 0.0, dHl = 0.0;
+  if (real && tid >= 1 && tid < T - 1) {
+    const int64_t gs = D.geo_stride;
+    const double* G = D.gK;
+    // the interfaces' ratios are stored at the edge index of their left cell, the differences too
+    const int32_t el = per ? eb + ghost(c - 1, N, K.bc) + 1 : e - 1;
+    const double rho_l = G[ADJ_RHO * gs + el], sig_l = G[ADJ_SIG * gs + el], rho_r = G[ADJ_RHO * gs + e],
+                 sig_r = G[ADJ_SIG * gs + e];
+    const swale::SourceRatio sr = {G[ADJ_GX * gs + e], G[ADJ_GY * gs + e], G[ADJ_K3 * gs + e]};
+    const swale::SourceAdj a = swale::source_pressure_rev(
+        hv, o.hL, o.hR, o.EL - ev, o.ER - ev, D.dE[el], D.dH[el], D.dE[e], D.dH[e], rho_l, sig_l * sig_l, sig_r,
+        rho_r * rho_r, sr, -(K.sc.g * sRho[1][tid]));
+    ob.hL = a.hL;
+    ob.hR = a.hR;
+    ob.EL += a.deL;
+    ob.ER += a.deR;
+    Eb = -(a.deL + a.deR);
+    Hb = a.hc;
+    dEl = a.dEl;
+    dHl = a.dHl;
+    dEr = a.dEr;
+    dHr = a.dHr;
+  }
+  sDl[0][tid] = dEl;
+  sDl[1][tid] = dHl;
+  // Limiter and reconstruction.
+  swale::SmoothAdj r[3] = {};
+  if (recon && tid >= 2 && tid < T - 2) {
+    const int cls = (int)D.gK[ADJ_CLS * D.geo_stride + e];
+    if (cls == 0) {  // smooth, limiter not active
+      const swale::SmoothWidths w = {rJ[tid - 1], jv, rJ[tid + 1], rJ[tid - 2] + rJ[tid - 1], rJ[tid - 1] + jv,
+                                     jv + rJ[tid + 1], rJ[tid + 1] + rJ[tid + 2]};
+      const double iv = D.gK[ADJ_IV * D.geo_stride + e];
+      // B = E - h and u = m / h on wet edges
+      const bool wetL = swale::gt_pos(o.hL, K.sc.h_dry), wetR = swale::gt_pos(o.hR, K.sc.h_dry);
+      const double hLs = wetL ? o.hL : 1.0, hRs = wetR ? o.hR : 1.0, ihh = swale::recip(hLs * hRs);
+      const double mL = wetL ? ob.uL * (hRs * ihh) : 0.0, mR = wetR ? ob.uR * (hLs * ihh) : 0.0;
+      r[0] = swale::smooth_rev(w, iv, ob.EL + ob.BL, ob.ER + ob.BR);
+      r[1] = swale::smooth_rev(w, iv, mL, mR);
+      r[2] = swale::smooth_rev(w, iv, (ob.hL - ob.BL) - mL * o.uL, (ob.hR - ob.BR) - mR * o.uR);
+    } else {
+      AdjCellIn in;
+      in.ob = ob;
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        in.J[k] = rJ[tid - 2 + k];
+        in.E[k] = rE[tid - 2 + k];
+        in.M[k] = rM[tid - 2 + k];
+        in.H[k] = rH[tid - 2 + k];
+      }
+      const AdjCellOut ro = adj_general_cell(K.sc, in, dxmax);
+#pragma unroll
+      for (int v = 0; v < 3; ++v) r[v] = ro.s[v];
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    sD2l[v][tid] = r[v].d2l;
+    sD3[v][tid] = r[v].d3;
+    sD4l[v][tid] = r[v].d4l;
+    sD4r[v][tid] = r[v].d4r;
+  }
+  // Reciprocal sums of the pair, triple and quadruple that start at this cell: as stored for cells
+  // -1..N (the triple and quadruple by their second cell), formed for the outer ghost cells.
+  double ip = 0.0, it = 0.0, iq = 0.0;
+  if (near) {
+    const int32_t cp = per ? gl : c, cn = per ? ghost(c + 1, N, K.bc) : c + 1;
+    if (cp >= -1 && cp <= N) ip = D.ipair[eb + cp + 1];
+    else if (tid < T - 1) ip = swale::recip(jv + rJ[tid + 1]);
+    if (cn >= -1 && cn <= N) {
+      it = D.itri[eb + cn + 1];
+      iq = D.gK[ADJ_IQ * D.geo_stride + eb + cn + 1];
+    } else if (tid < T - 3) {
+      const double p = jv + rJ[tid + 1];
+      it = swale::recip(p + rJ[tid + 2]);
+      iq = swale::recip(p + (rJ[tid + 2] + rJ[tid + 3]));
+    }
+  }
+  __syncthreads();
+  // Transpose of the differences: quadruples, triples, pairs, cells (rows past the block count as zero).
+#pragma unroll
+  for (int v = 0; v < 3; ++v) sT[v][tid] = tid < T - 2 ? (sD4l[v][tid + 2] + sD4r[v][tid + 1]) * iq : 0.0;
+  __syncthreads();
+  double t3[3];
+#pragma unroll
+  for (int v = 0; v < 3; ++v)
+    t3[v] = tid < T - 1 ? (sD3[v][tid + 1] + ((tid > 0 ? sT[v][tid - 1] : 0.0) - sT[v][tid])) * it : 0.0;
+#pragma unroll
+  for (int v = 0; v < 3; ++v) sD4l[v][tid] = t3[v];  // (read above as D4 shares, before the barrier)
+  __syncthreads();
+  const double src[3] = {dEr + (tid < T - 1 ? sDl[0][tid + 1] : 0.0), 0.0, dHr + (tid < T - 1 ? sDl[1][tid + 1] : 0.0)};
+  double t2[3];
+#pragma unroll
+  for (int v = 0; v < 3; ++v) {
+    const double s2 = (r[v].d2r + (tid < T - 1 ? sD2l[v][tid + 1] : 0.0)) + ((tid > 0 ? sD4l[v][tid - 1] : 0.0) - t3[v]);
+    t2[v] = s2 * ip + src[v];
+    sD4r[v][tid] = t2[v];
+  }
+  __syncthreads();
+  double a[3];
+#pragma unroll
+  for (int v = 0; v < 3; ++v) a[v] = r[v].v + ((tid > 0 ? sD4r[v][tid - 1] : 0.0) - t2[v]);
+  a[0] += Eb;
+  a[2] += Hb;
+  // (eta, hu, h) to (eta, hu, b): h = eta - b.
+  a[0] += a[2];
+  a[2] = -a[2];
+  if (!per && (first < 3 || last > N - 3)) {  // ghost cells' shares go to their images
+#pragma unroll
+    for (int v = 0; v < 3; ++v) sD3[v][tid] = (flip && v == 1) ? -a[v] : a[v];
+    __syncthreads();
+    if (own) {
+      if (c < 3) {  // image of cell -1 - c
+#pragma unroll
+        for (int v = 0; v < 3; ++v) a[v] += sD3[v][tid - (2 * c + 1)];
+      }
+      if (c >= N - 3) {  // image of cell 2 N - 1 - c
+#pragma unroll
+        for (int v = 0; v < 3; ++v) a[v] += sD3[v][tid + 2 * (N - 1 - c) + 1];
       }
     }
+  }
+  if (!own) return;
+  if (STAGE == 1) {
+    const double J0 = A.sJ[g];
+    A.oE[g] = J0 * q[0] + a[0];
+    A.oM[g] = J0 * q[1] + a[1];
+    A.oB[g] = J0 * q[2] + a[2];
+  } else {
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      const int64_t vc = c - 2 + k;
-      const int64_t s = ghost(vc, N, K.bc);
-      const double sgn = (refl && (vc < 0 || vc >= N)) ? -1.0 : 1.0;
-      atomicAdd(&A.aE[cb + s], cv[0][k]);
-      atomicAdd(&A.aM[cb + s], sgn * cv[1][k]);
-      atomicAdd(&A.aB[cb + s], cv[2][k]);
+    for (int v = 0; v < 3; ++v) (STAGE == 3 ? A.a3 : A.a2)[v][g] = a[v];
+  }
+}
+
+// The evolving state of one context or state set (q^n, J^n, nodes, scalars) copied to another, in
+// one launch: cells, nodes and 8-byte words of the scalars.
+struct StateArrays {
+  double *E, *M, *B, *J, *x;
+  DevScalars* S;
+};
+__global__ void __launch_bounds__(256) k_copy_state(StateArrays to, StateArrays from, int64_t cells, int64_t nodes,
+                                                    int64_t words) {
+  static_assert(sizeof(DevScalars) % 8 == 0, "the scalars are copied in 8-byte words");
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nodes || i < words; i += step) {
+    if (i < cells) {
+      to.E[i] = from.E[i];
+      to.M[i] = from.M[i];
+      to.B[i] = from.B[i];
+      to.J[i] = from.J[i];
     }
+    if (i < nodes) to.x[i] = from.x[i];
+    if (i < words) ((long long*)to.S)[i] = ((const long long*)from.S)[i];
   }
 }
 
@@ -396,7 +326,7 @@ __global__ void __launch_bounds__(T, 512 / T) k_adj_recon(StepConst K, DevState 
 // finds the cell on the new mesh (a node moves by less than a cell per step); the first call
 // bisects. Either way the cell is c with x[c] <= xg < x[c+1] (clamped to 0..N-1).
 template <int MODE>
-__global__ void k_misfit(DevState D, AdjState A, int32_t B, int32_t G, const double* __restrict__ gx,
+__global__ void k_misfit(DevState D, double* lE, double* lB, int32_t B, int32_t G, const double* __restrict__ gx,
                          const double* __restrict__ obs, double* Jout, int64_t* gcell) {
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= (int64_t)B * G) return;
@@ -424,8 +354,8 @@ __global__ void k_misfit(DevState D, AdjState A, int32_t B, int32_t G, const dou
   if (MODE == 0) {
     atomicAdd(&Jout[i], dt * r * r);
   } else {
-    atomicAdd(&A.lE[g], 2.0 * dt * r);
-    atomicAdd(&A.lB[g], -2.0 * dt * r);
+    atomicAdd(&lE[g], 2.0 * dt * r);
+    atomicAdd(&lB[g], -2.0 * dt * r);
   }
 }
 

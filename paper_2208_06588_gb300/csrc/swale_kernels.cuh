@@ -150,22 +150,19 @@ struct DevState {
   // the same stage: differences of eta and h to the next cell, and the depth.
   double *dE, *dH, *H;
   double *iJ1, *iJ2;           // 1 / J^(1), 1 / J^(2) (cells)
-  // Per cell of the stage mesh, 14 arrays in the edge layout (gK[k * geo_stride + idx]): the
-  // smooth class's linear form K[2][4] (k < 8), stored by the hydrostatic reconstruction, and the
-  // source term's six form entries (k = 8..13), stored by the update; set only for the adjoint's
-  // recomputes, whose reverse kernels read them instead of recomputing the mesh geometry.
+  // What the reverse of a stage reads besides the edge states, arrays in the edge layout
+  // (gK[k * geo_stride + idx], ADJ_*); set only for the adjoint's recomputes, which store them.
   double* gK;
   uint8_t* flags;              // stage-1 classes, edge layout
   InstConst* IC;
   DevScalars* S;
-  const Tile *rtiles, *utiles, *mtiles;  // work lists (null: one instance, implicit tiles)
-  int32_t nr, nu, nm;                    // tiles in each list
+  const Tile* mtiles;  // work lists (null: one instance, implicit tiles)
+  int32_t nm;          // tiles in each list
   // The forward update's tiles: T - 1 cells for a block of T threads, so that its T interfaces
-  // take one pass (utiles, of T cells, serve the adjoint's kernels).
+  // take one pass.
   const Tile* ftiles;
   int32_t nf;
-  // The forward reconstruction's tiles: T - 4 cells for a block of T threads (rtiles, of T cells,
-  // serve the adjoint's kernels).
+  // The forward reconstruction's tiles: T - 4 cells for a block of T threads.
   const Tile* rftiles;
   int32_t nrf;
   InstConst ic1;  // the constants of a single instance (the stage kernels need no load for them)
@@ -617,9 +614,6 @@ __device__ __forceinline__ void stage1_dt(const StepConst& K, DevScalars* S, con
   }
 }
 
-// STOREK: an instantiation of the hydrostatic scheme that also stores each cell's smooth-class
-// linear form in D.gK (the adjoint's recomputes), so that the forward's own instantiations keep
-// their registers.
 // Shared rows of the phases. Every phase runs on all threads: the last rows hold nothing that a
 // reconstructed cell reads (they are padded for the reads past the block).
 template <int T, int SCHEME>
@@ -699,7 +693,7 @@ template <int T, int SCHEME, class Sink>
 __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, SCHEME>& R, const double* sE, const double* sM,
                                              const double* sJ, double jv, double ev, double mv, double hv, double dxmax,
                                              const MeshRecips& g, bool mine, Sink& sink, EdgeState& o, uint8_t& flag,
-                                             double etaG[2], uint32_t& st) {
+                                             double etaG[2], uint32_t& st, bool* limited = nullptr) {
   const int tid = threadIdx.x;
   R.H[tid] = hv;  // the depth is reconstructed in place of the bottom
   R.Jf[tid] = swale::f32_trunc(jv);
@@ -824,11 +818,15 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
     st |= R.xst[tid];
   }
   swale::limit_cell(P, evl, hv, mv, o, st);
+  if (limited) *limited = dbits(o.hL) != dbits(evl[2][0]) || dbits(o.hR) != dbits(evl[2][1]);
 }
 
-// Where k_recon's differences and reciprocals go: the arrays that the update of the stage reads and, in
-// stage 2, the mesh cache.
-template <int STAGE, int SCHEME>
+// Arrays of DevState::gK (see swale_adjoint_kernels.cuh).
+enum { ADJ_IQ, ADJ_IV, ADJ_RHO, ADJ_SIG, ADJ_GX, ADJ_GY, ADJ_K3, ADJ_CLS, ADJ_DE, ADJ_DH, ADJ_H, ADJ_ARRAYS };
+
+// Where k_recon's differences and reciprocals go: the arrays that the update of the stage reads, in
+// stage 2 the mesh cache, and (STOREK) the arrays of the adjoint.
+template <int STAGE, int SCHEME, bool STOREK>
 struct ReconSink {
   const DevState& D;
   int32_t idx;      // edge-array index of the thread's cell
@@ -836,7 +834,7 @@ struct ReconSink {
   double hv;
   __device__ __forceinline__ void pair(double ip, double de, double dh) const {
     if (!mine) return;
-    if (SCHEME == 2 || !use_geo) D.ipair[idx] = ip;  // (on the cache the update needs neither)
+    if (SCHEME == 2 || STOREK || !use_geo) D.ipair[idx] = ip;  // (on the cache the update needs neither)
     D.dE[idx] = de;
     D.dH[idx] = dh;
     D.H[idx] = hv;
@@ -844,17 +842,21 @@ struct ReconSink {
   }
   __device__ __forceinline__ void triple(double it) const {
     if (!next_mine) return;
-    if (SCHEME == 2 || !use_geo) D.itri[idx + 1] = it;
+    if (SCHEME == 2 || STOREK || !use_geo) D.itri[idx + 1] = it;
     if (STAGE == 2 && D.geo) D.geo[GEO_IT * D.geo_stride + idx + 1] = it;
   }
   __device__ __forceinline__ void quad(double iq) const {
     if (STAGE == 2 && D.geo && next_mine) D.geo[GEO_IQ * D.geo_stride + idx + 1] = iq;
+    if (STOREK && next_mine) D.gK[ADJ_IQ * D.geo_stride + idx + 1] = iq;
   }
   __device__ __forceinline__ void quint(double iv) const {
     if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = iv;
+    if (STOREK) D.gK[ADJ_IV * D.geo_stride + idx] = iv;
   }
 };
 
+// STOREK: an instantiation of the hydrostatic scheme that also stores what the reverse reads (the
+// adjoint's recomputes).
 template <int STAGE, int T, int SCHEME = 0, bool STOREK = false>
 __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, DevState D, const double* __restrict__ Eg,
                                              const double* __restrict__ Mg, const double* __restrict__ Bg,
@@ -988,30 +990,20 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     // Cells of the tile that are reconstructed and stored.
     const bool mine = tid >= 2 && tid < 2 + TO && c <= N;
     const bool next_mine = tid >= 1 && tid < 1 + TO && c + 1 <= N;  // cell c + 1 is
-    ReconSink<STAGE, SCHEME> sink{D, idx, mine, next_mine, use_geo, hv};
+    ReconSink<STAGE, SCHEME, STOREK> sink{D, idx, mine, next_mine, use_geo, hv};
+    bool limited = false;
     EdgeState o;
     uint8_t flag = 0;
     double etaG[2] = {0.0, 0.0};
     uint32_t st = 0;
-    recon_phases<T, SCHEME>(K.sc, rows, sE, sM, sJ, jv, ev, mv, hv, dxmax, mr, mine, sink, o, flag, etaG, st);
+    recon_phases<T, SCHEME>(K.sc, rows, sE, sM, sJ, jv, ev, mv, hv, dxmax, mr, mine, sink, o, flag, etaG, st, &limited);
     if (STAGE == 2 && D.geo != nullptr && c0 == -1 && tid == 0)
       S->geo_tag = ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)((S->step_idx + 1) & 0xffffffffLL);
     WaveEdge eL{0.0, 0.0, 0.0}, eR{0.0, 0.0, 0.0};
     bool useL = false, useR = false;
     if (mine) {
-      if (STOREK) {
-        double h[5], K8[2][4];
-        swale::CellGeom G;
-        uint32_t stk = 0;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) h[k] = sJ[tid - 2 + k];
-        const double it3[3] = {swale::triple_recip(h[0], h[1], h[2]), swale::triple_recip(h[1], h[2], h[3]),
-                               swale::triple_recip(h[2], h[3], h[4])};
-        swale::cell_geom(h, jv, G, stk, false);
-        swale::linear_edge_form(G.d, G.G1, G.G2, h, it3, K8);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) D.gK[k * D.geo_stride + idx] = K8[k >> 2][k & 3];
-      }
+      // (with the limiter's mark, for the reverse)
+      if (STOREK) D.gK[ADJ_CLS * D.geo_stride + idx] = (double)(flag + (limited ? 4 : 0));
       D.eEL[idx] = o.EL;
       D.eER[idx] = o.ER;
       D.eBL[idx] = o.BL;
@@ -1070,8 +1062,8 @@ struct RhsOut {
 };
 
 // SCHEME: 0 hydrostatic, 1 non-well-balanced, 2 special source. BOT: an instantiation with the
-// L2-projection bottom. STOREK: one that also stores the old source form's entries in D.gK (the
-// adjoint's recomputes).
+// L2-projection bottom. STOREK: one that also stores the source's ratios in D.gK (the adjoint's
+// recomputes).
 
 // Largest a and b over the block (non-negative doubles), raised into mx[0], mx[1], and the smallest c,
 // lowered into *mn (or, with COMPL, its complement raised there), by three lanes after one barrier.
@@ -1192,6 +1184,10 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
         D.geo[GEO_RHO2 * D.geo_stride + el] = pr.rho2;
         D.geo[GEO_SIG2 * D.geo_stride + el] = pr.sig2;
       }
+      if (STOREK) {
+        D.gK[ADJ_RHO * D.geo_stride + el] = pr.rho;
+        D.gK[ADJ_SIG * D.geo_stride + el] = pr.sig;
+      }
       // Every tile has the same viscosity; the first one of the instance records it.
       if (STAGE > 1 && K.alpha_mode == 1 && k == 0) stage_alpha(K, inst, STAGE, alpha, S->step_idx);
     }
@@ -1237,11 +1233,9 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
           D.geo[GEO_K3 * D.geo_stride + er] = sr.K3;
         }
         if (STOREK) {
-          const swale::SourceForm sf = swale::source_form(Jm, Jc, Jp, swale::recip(Jm), swale::recip(Jc), swale::recip(Jp),
-                                                          D.ipair[el], D.ipair[er], D.itri[er]);
-          const double* const src6 = reinterpret_cast<const double*>(&sf);
-#pragma unroll
-          for (int q = 0; q < 6; ++q) D.gK[(8 + q) * D.geo_stride + er] = src6[q];
+          D.gK[ADJ_GX * D.geo_stride + er] = sr.GX;
+          D.gK[ADJ_GY * D.geo_stride + er] = sr.GY;
+          D.gK[ADJ_K3 * D.geo_stride + er] = sr.K3;
         }
         const double acc = swale::source_pressure_form(hj, hLj, hRj, swale::sub_(ELj, Ej), swale::sub_(ERj, Ej), dE, dH, sDe[0][tid + 1],
                                                        sDe[1][tid + 1], pr.rho, pr.sig2, sG[0][tid + 1],

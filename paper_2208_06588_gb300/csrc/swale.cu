@@ -411,12 +411,29 @@ swale_status timed_launch(swale_ctx* ctx, int family, F&& launch) {
   return SWALE_OK;
 }
 
+// Launches a kernel that calls pdl_trigger and pdl_wait with the attribute that lets it start while the
+// kernel before it on the stream ends.
+template <class... P, class... A>
+void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t shm, cudaStream_t s, const A&... a) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = shm;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(a)...);
+}
+
 template <int STAGE, int SCHEME, bool STOREK>
 void launch_recon_as(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                      const double* M, const double* B, const double* J) {
-  if (T == 64) k_recon<STAGE, 64, SCHEME, STOREK><<<grid, 64, 0, s>>>(K, D, E, M, B, J);
-  else if (T == 256) k_recon<STAGE, 256, SCHEME, STOREK><<<grid, 256, 0, s>>>(K, D, E, M, B, J);
-  else k_recon<STAGE, 128, SCHEME, STOREK><<<grid, 128, 0, s>>>(K, D, E, M, B, J);
+  if (T == 64) launch(k_recon<STAGE, 64, SCHEME, STOREK>, grid, 64, 0, s, K, D, E, M, B, J);
+  else if (T == 256) launch(k_recon<STAGE, 256, SCHEME, STOREK>, grid, 256, 0, s, K, D, E, M, B, J);
+  else launch(k_recon<STAGE, 128, SCHEME, STOREK>, grid, 128, 0, s, K, D, E, M, B, J);
 }
 
 template <int STAGE>
@@ -431,9 +448,9 @@ void launch_recon(const StepConst& K, const DevState& D, int T, unsigned grid, c
 template <int STAGE, int MODE, int SCHEME, bool BOT, bool STOREK>
 void launch_update_as(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                       const double* M, const double* B, const double* J, const RhsOut& ro) {
-  if (T == 64) k_update<STAGE, MODE, 64, SCHEME, BOT, STOREK><<<grid, 64, 0, s>>>(K, D, E, M, B, J, ro);
-  else if (T == 256) k_update<STAGE, MODE, 256, SCHEME, BOT, STOREK><<<grid, 256, 0, s>>>(K, D, E, M, B, J, ro);
-  else k_update<STAGE, MODE, 128, SCHEME, BOT, STOREK><<<grid, 128, 0, s>>>(K, D, E, M, B, J, ro);
+  if (T == 64) launch(k_update<STAGE, MODE, 64, SCHEME, BOT, STOREK>, grid, 64, 0, s, K, D, E, M, B, J, ro);
+  else if (T == 256) launch(k_update<STAGE, MODE, 256, SCHEME, BOT, STOREK>, grid, 256, 0, s, K, D, E, M, B, J, ro);
+  else launch(k_update<STAGE, MODE, 128, SCHEME, BOT, STOREK>, grid, 128, 0, s, K, D, E, M, B, J, ro);
 }
 
 template <int STAGE, int MODE, int SCHEME>
@@ -464,8 +481,10 @@ unsigned grid_of(int32_t ntiles, int persistent) {
 // Enqueues one step of the state D on stream s with geometry-cache epoch `epoch`. stageD
 // (optional, 3 entries): the device state each stage's kernels use; copies of D that differ only
 // in their edge arrays keep every stage's edge values (the adjoint's recompute of a step).
+// first: the step needs its prologue (the step before it did not do it); next: another step follows in the
+// same sequence, whose prologue this one's commit does.
 swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, const DevState* stageD,
-                             uint32_t epoch) {
+                             uint32_t epoch, bool first = true, bool next = false) {
   StepConst K = step_const(ctx);
   K.geo_epoch = epoch;
   const DevState& D1 = stageD ? stageD[0] : D;
@@ -478,10 +497,10 @@ swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, 
   auto L = [&](int fam, auto&& f) {
     if (st == SWALE_OK) st = timed_launch(ctx, fam, f);
   };
-  L(FAM_PROLOGUE, [&] { k_prologue<<<(unsigned)((ctx->B + 127) / 128), 128, 0, s>>>(K, D); });
+  if (first) L(FAM_PROLOGUE, [&] { launch(k_prologue, (unsigned)((ctx->B + 127) / 128), 128, 0, s, K, D); });
   if (K.mesh == SWALE_MESH_FLUID_GAUSS) {
     const size_t shm = (size_t)(3 * kMeshThreads + 4 * K.gauss_half + 4) * sizeof(double);
-    L(FAM_MESH, [&] { k_mesh_gauss<<<(unsigned)std::max(D.nm, 1), kMeshThreads, shm, s>>>(K, D); });
+    L(FAM_MESH, [&] { launch(k_mesh_gauss, (unsigned)std::max(D.nm, 1), kMeshThreads, shm, s, K, D); });
   }
   StepConst K1 = K;
   K1.wave_rel = stage1_wave_rel(ctx->cfg);
@@ -491,15 +510,15 @@ swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, 
   L(FAM_UPDATE, [&] { launch_update<2, 0>(K, D2, Tu, gu, s, D.Ea, D.Ma, D.Ba, D.J1, none); });
   L(FAM_RECON, [&] { launch_recon<3>(K, D3, Tr, gr, s, D.Eb, D.Mb, D.Bb, D.J2); });
   L(FAM_UPDATE, [&] { launch_update<3, 0>(K, D3, Tu, gu, s, D.Eb, D.Mb, D.Bb, D.J2, none); });
-  L(FAM_PROLOGUE, [&] { k_commit<<<(unsigned)std::min<int64_t>(ctx->B, 1024), 256, 0, s>>>(K, D); });
+  L(FAM_PROLOGUE, [&] { launch(k_commit, (unsigned)std::min<int64_t>(ctx->B, 1024), 256, 0, s, K, D, next ? 1 : 0); });
   if (st) return st;
   SW_CUDA(ctx, cudaGetLastError());
   return SWALE_OK;
 }
 
 // Enqueues one step of the context's state on its stream.
-swale_status enqueue_step(swale_ctx* ctx, const DevState* stageD = nullptr) {
-  return enqueue_step_on(ctx, ctx->D, ctx->stream, stageD, ctx->geo_epoch);
+swale_status enqueue_step(swale_ctx* ctx, bool first, bool next) {
+  return enqueue_step_on(ctx, ctx->D, ctx->stream, nullptr, ctx->geo_epoch, first, next);
 }
 
 // Whether the next steps go through k_steps: a small mesh (build_step_blocks), and nothing asked for
@@ -544,7 +563,7 @@ swale_status enqueue_steps(swale_ctx* ctx, int64_t n) {
       cudaGraph_t g;
       SW_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
       swale_status cs = SWALE_OK;
-      for (int i = 0; i < kGraphSteps && cs == SWALE_OK; ++i) cs = enqueue_step(ctx);
+      for (int i = 0; i < kGraphSteps && cs == SWALE_OK; ++i) cs = enqueue_step(ctx, i == 0, i + 1 < kGraphSteps);
       cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
       if (cs) return cs;
       if (e != cudaSuccess) return fail(ctx, SWALE_ECUDA, std::string("capture: ") + cudaGetErrorString(e));
@@ -559,8 +578,8 @@ swale_status enqueue_steps(swale_ctx* ctx, int64_t n) {
       n -= ctx->graph_steps;
     }
   }
-  for (; n > 0; --n)
-    if (swale_status s = enqueue_step(ctx)) return s;
+  for (bool first = true; n > 0; --n, first = false)
+    if (swale_status s = enqueue_step(ctx, first, n > 1)) return s;
   return SWALE_OK;
 }
 
@@ -1317,7 +1336,7 @@ long long device_steps(swale_ctx* ctx) {
 template <int STAGE>
 void launch_adj_stage(swale_ctx* ctx, const DevState& D, const StepConst& K, const AdjState& A, const double* E,
                       const double* M, const double* B, const double* J) {
-  k_adj_stage<STAGE><<<(unsigned)ctx->adj_blocks, kAdjThreads, 0, ctx->stream>>>(K, D, A, E, M, B, J);
+  launch(k_adj_stage<STAGE>, (unsigned)ctx->adj_blocks, kAdjThreads, 0, ctx->stream, K, D, A, E, M, B, J);
 }
 
 // Copies of the evolving state (q^n, J^n, nodes, per-instance scalars).
@@ -1633,7 +1652,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   DevState& D = ctx->D;
   const unsigned copy_grid = (unsigned)std::min<int64_t>((NN + 255) / 256, 152 * 8);
   auto copy = [&](const StateArrays& to, const StateArrays& from, cudaStream_t q) {
-    k_copy_state<<<copy_grid, 256, 0, q>>>(to, from, Nt, NN, B * (int64_t)(sizeof(DevScalars) / 8));
+    launch(k_copy_state, copy_grid, 256, 0, q, to, from, Nt, NN, B * (int64_t)(sizeof(DevScalars) / 8));
     return cudaGetLastError();
   };
   auto arrays = [](const DevState& X) { return StateArrays{X.E0, X.M0, X.B0, X.J0, X.x, X.S}; };
@@ -1720,7 +1739,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
     } else {
       s = enqueue_step_on(ctx, fwd, st, nullptr, ctx->geo_epoch);
     }
-    if (!s) k_misfit<0><<<gg, 128, 0, st>>>(D, nullptr, nullptr, (int32_t)B, G, gx, obs + n * B * G, Jacc, gcell);
+    if (!s) launch(k_misfit<0>, gg, 128, 0, st, D, (double*)nullptr, (double*)nullptr, (int32_t)B, G, gx, obs + n * B * G, Jacc, gcell);
   }
   if (!s && !e) e = save(fin);
   if (!s && !e) e = cudaGetLastError();
@@ -1756,7 +1775,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   // it), c the state before it.
   auto reverse_step = [&](const DevState* X3, int64_t m, const StateCopy& c) {
     double** l = lam[cur];
-    k_misfit<1><<<gg, 128, 0, st>>>(X3[2], l[0], l[2], (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
+    launch(k_misfit<1>, gg, 128, 0, st, X3[2], l[0], l[2], (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
     A.lE = l[0];
     A.lM = l[1];
     A.lB = l[2];
@@ -1972,11 +1991,11 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
     // Up to this many cells every block finds the largest width itself: one launch instead of two.
     constexpr int64_t kScanCells = 4096;
     const bool scan = N <= kScanCells && !A_out;
-    if (!scan) k_rhs_widths<<<1, 1024, 0, st>>>(J, (int32_t)N, mx, wv);
+    if (!scan) launch(k_rhs_widths, 1, 1024, 0, st, J, (int32_t)N, mx, wv);
     const unsigned nb = (unsigned)((N + kStepCells - 1) / kStepCells);
     auto go = [&](auto kernel) {
-      kernel<<<nb, kStepThreads, 0, st>>>(P, cfg->bc, cfg->alpha_bound ? 0 : 1, (int32_t)N, alpha, E, M, B, J, w,
-                                          scan ? nullptr : mx, wv, RE, RM, RB, flags_here ? flags : scr->flags);
+      launch(kernel, nb, kStepThreads, 0, st, P, cfg->bc, cfg->alpha_bound ? 0 : 1, (int32_t)N, alpha, E, M, B, J, w,
+             scan ? nullptr : mx, wv, RE, RM, RB, flags_here ? flags : scr->flags);
     };
     if (cfg->scheme == SWALE_SCHEME_NONWB) go(k_rhs<1>);
     else if (cfg->scheme == SWALE_SCHEME_SPECIAL) go(k_rhs<2>);

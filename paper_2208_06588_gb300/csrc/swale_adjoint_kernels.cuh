@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_stage(StepConst K, DevSt
   __shared__ double sRho[3][T], sR[4][T], sX[3][T], sDl[2][T];
   __shared__ double sD2l[3][T], sD3[3][T], sD4l[3][T], sD4r[3][T], sT[3][T];
   const int tid = threadIdx.x;
+  pdl_wait();
   const Tile tl = A.tiles ? A.tiles[blockIdx.x] : Tile{0, (int32_t)blockIdx.x};
   const InstConst ic = A.tiles ? D.IC[tl.inst] : D.ic1;
   const DevScalars* S = D.S + tl.inst;
@@ -284,6 +285,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_stage(StepConst K, DevSt
       }
     }
   }
+  pdl_trigger();
   if (!own) return;
   if (STAGE == 1) {
     const double J0 = A.sJ[g];
@@ -306,6 +308,8 @@ __global__ void __launch_bounds__(256) k_copy_state(StateArrays to, StateArrays 
                                                     int64_t words) {
   static_assert(sizeof(DevScalars) % 8 == 0, "the scalars are copied in 8-byte words");
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  pdl_wait();
+  pdl_trigger();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nodes || i < words; i += step) {
     if (i < cells) {
       to.E[i] = from.E[i];
@@ -328,6 +332,8 @@ __global__ void __launch_bounds__(256) k_copy_state(StateArrays to, StateArrays 
 template <int MODE>
 __global__ void k_misfit(DevState D, double* lE, double* lB, int32_t B, int32_t G, const double* __restrict__ gx,
                          const double* __restrict__ obs, double* Jout, int64_t* gcell) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= (int64_t)B * G) return;
   const int i = (int)(id / G);

@@ -384,6 +384,8 @@ __global__ void __launch_bounds__(1024) k_rhs_widths(const double* __restrict__ 
                                                      unsigned long long* wave) {
   __shared__ unsigned long long red[32];
   unsigned long long m = 0ull;
+  pdl_wait();
+  pdl_trigger();
 #pragma unroll 8
   for (int32_t i = threadIdx.x; i < n; i += 1024) m = umax64(m, dbits(J[i]));
   m = warp_umax64(m);
@@ -422,6 +424,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, 
   const bool own = tid >= 3 && tid < T - 3 && c < N;
   const bool mine = tid >= 2 && tid < T - 2 && c <= N;  // reconstructed
   const bool face = tid >= 3 && tid < T - 2 && c <= N;  // left interface of an owned cell, or the last one
+  pdl_wait();
   double ev = 0.0, mv = 0.0, bv = 0.0, jv = 1.0, wl = 0.0, wr = 0.0;
   if (c >= -3 && c <= N + 2) {
     const int32_t g = ghost(c, N, bc);
@@ -487,6 +490,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, 
     sG[1][tid] = pr.rho2;
   }
   __syncthreads();
+  pdl_trigger();
   if (!own) return;
   double Rm = swale::sub_(F.FMr, sF[1][tid + 1]);
   if (SCHEME == 2) {

@@ -428,21 +428,31 @@ void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t shm, cud
   cudaLaunchKernelEx(&cfg, kernel, P(a)...);
 }
 
-template <int STAGE, int SCHEME, bool STOREK>
+template <int STAGE, int SCHEME, bool STOREK, bool CACHE>
 void launch_recon_as(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                      const double* M, const double* B, const double* J) {
-  if (T == 64) launch(k_recon<STAGE, 64, SCHEME, STOREK>, grid, 64, 0, s, K, D, E, M, B, J);
-  else if (T == 256) launch(k_recon<STAGE, 256, SCHEME, STOREK>, grid, 256, 0, s, K, D, E, M, B, J);
-  else launch(k_recon<STAGE, 128, SCHEME, STOREK>, grid, 128, 0, s, K, D, E, M, B, J);
+  if (T == 64) launch(k_recon<STAGE, 64, SCHEME, STOREK, CACHE>, grid, 64, 0, s, K, D, E, M, B, J);
+  else if (T == 256) launch(k_recon<STAGE, 256, SCHEME, STOREK, CACHE>, grid, 256, 0, s, K, D, E, M, B, J);
+  else launch(k_recon<STAGE, 128, SCHEME, STOREK, CACHE>, grid, 128, 0, s, K, D, E, M, B, J);
+}
+
+template <int STAGE, int SCHEME>
+void launch_recon_scheme(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
+                         const double* M, const double* B, const double* J) {
+  if (SCHEME == 0 && D.gK)  // the adjoint's recomputes
+    launch_recon_as<STAGE, SCHEME, SCHEME == 0, STAGE == 1>(K, D, T, grid, s, E, M, B, J);
+  else if (STAGE == 1 || (K.mesh == SWALE_MESH_STATIC && D.geo))
+    launch_recon_as<STAGE, SCHEME, false, true>(K, D, T, grid, s, E, M, B, J);
+  else
+    launch_recon_as<STAGE, SCHEME, false, STAGE == 1>(K, D, T, grid, s, E, M, B, J);
 }
 
 template <int STAGE>
 void launch_recon(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                   const double* M, const double* B, const double* J) {
-  if (K.scheme == SWALE_SCHEME_NONWB) launch_recon_as<STAGE, 1, false>(K, D, T, grid, s, E, M, B, J);
-  else if (K.scheme == SWALE_SCHEME_SPECIAL) launch_recon_as<STAGE, 2, false>(K, D, T, grid, s, E, M, B, J);
-  else if (D.gK) launch_recon_as<STAGE, 0, true>(K, D, T, grid, s, E, M, B, J);  // the adjoint's recomputes
-  else launch_recon_as<STAGE, 0, false>(K, D, T, grid, s, E, M, B, J);
+  if (K.scheme == SWALE_SCHEME_NONWB) launch_recon_scheme<STAGE, 1>(K, D, T, grid, s, E, M, B, J);
+  else if (K.scheme == SWALE_SCHEME_SPECIAL) launch_recon_scheme<STAGE, 2>(K, D, T, grid, s, E, M, B, J);
+  else launch_recon_scheme<STAGE, 0>(K, D, T, grid, s, E, M, B, J);
 }
 
 template <int STAGE, int MODE, int SCHEME, bool BOT, bool STOREK>
@@ -657,8 +667,14 @@ swale_status set_instances(swale_ctx* ctx, const std::vector<int64_t>& off, cons
     double ws = 0.0;
     for (int mm = -H; mm <= H; ++mm) ws += gw[mm + H];
     ctx->gauss_wsum = ws;
+    std::vector<int2> gq(gw.size());
+    for (size_t k = 0; k < gw.size(); ++k) {
+      const long long q = (long long)std::llrint(std::ldexp(gw[k], 56));
+      gq[k] = make_int2((int)(q & 0xfffffff), (int)(q >> 28));
+    }
     SW_CUDA(ctx, cudaMemcpyToSymbolAsync(c_gauss_w, gw.data(), gw.size() * sizeof(double), 0,
                                          cudaMemcpyHostToDevice, st));
+    SW_CUDA(ctx, cudaMemcpyToSymbolAsync(c_gauss_q, gq.data(), gq.size() * sizeof(int2), 0, cudaMemcpyHostToDevice, st));
   }
   return build_tiles(ctx, ic);
 }

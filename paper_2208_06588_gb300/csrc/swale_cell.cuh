@@ -1051,34 +1051,46 @@ SWALE_HD real source_cell_form(real g, const real hd[5], const real bd[5], const
 // the Gauss-Lobatto points t = 0, (1 -+ 1/sqrt 5)/2, 1 (weights 1/12, 5/12, 5/12, 1/12).
 //   eta4: eta at the four points;  bd: bottom data as in source_cell_form;  bLm: right-edge bottom of
 //   cell j-1, bRp: left-edge bottom of cell j+1.
+// Twice the value, arranged for few operations (about 58 instead of 90): with c_k the Newton coefficients of
+// the bottom's primitive and e_q = eta_q - etabar, b_h'(t) = sum_k c_k (2 m_k' + (t + r_m) m_k''), m_k = t, t^2, t^3 - t^2,
+// t^4 - 2 t^3 + t^2, so the sum over the points needs the four moments sum_q w_q e_q t_q^n only; and the edge terms
+// are products of differences, (b_R - b_L) (b_R + b_L - 2 etabar), of either side.
+SWALE_HD real source_special2(real g, real etabar, const real eta4[4], const real bd[5], const SourceGeom& sg, real bLm,
+                              real bRp) {
+  const real o2a = mul_(sub_(bd[3], bd[0]), sg.irm), o2b = sub_(bd[1], bd[3]), o2c = sub_(bd[4], bd[1]);
+  const real o2d = mul_(sub_(bd[2], bd[4]), sg.irp);
+  const real o3a = mul_(sub_(o2b, o2a), sg.i1m), o3b = sub_(o2c, o2b), o3c = mul_(sub_(o2d, o2c), sg.i1p);
+  const real o4a = mul_(sub_(o3b, o3a), sg.i1m), o4b = mul_(sub_(o3c, o3b), sg.i1p);
+  const real o5 = mul_(sub_(o4b, o4a), sg.i1mp);
+  const double t1 = SWALE_GLO_T1, t2 = SWALE_GLO_T2;
+  const real e0 = sub_(eta4[0], etabar), e1 = sub_(eta4[1], etabar), e2 = sub_(eta4[2], etabar), e3 = sub_(eta4[3], etabar);
+  // 12 times the moments of order 0..3 (weights 1, 5, 5, 1), times 2, 6, 12, 20
+  const real A = fma_(10.0, add_(e1, e2), mul_(2.0, add_(e0, e3)));
+  const real B = fma_(30.0 * t1, e1, fma_(30.0 * t2, e2, mul_(6.0, e3)));
+  const real C = fma_(60.0 * t1 * t1, e1, fma_(60.0 * t2 * t2, e2, mul_(12.0, e3)));
+  const real D = fma_(100.0 * t1 * t1 * t1, e1, fma_(100.0 * t2 * t2 * t2, e2, mul_(20.0, e3)));
+  const real BA = sub_(B, A), CB = sub_(C, B), DC = sub_(D, C);
+  const real p3 = fma_(sg.rm, A, B), p4 = fma_(sg.rm, BA, CB), p5 = fma_(sg.rm, sub_(CB, BA), sub_(DC, CB));
+  const real S12 = fma_(o5, p5, fma_(o4a, p4, fma_(o3a, p3, mul_(o2a, A))));  // 12 sum_q w_q e_q b_h'(t_q)
+  const real x = mul_(sub_(bd[4], bd[3]), fma_(-2.0, etabar, add_(bd[4], bd[3])));
+  const real y = fma_(sub_(bRp, bLm), fma_(-2.0, etabar, add_(bRp, bLm)), x);
+  return mul_(g, fma_(-1.0 / 6.0, S12, mul_(0.5, y)));
+}
 SWALE_HD real source_cell_special(real g, real etabar, const real eta4[4], const real bd[5], const SourceGeom& sg,
                                   real bLm, real bRp) {
-  const real* u = bd;
-  const real o2a = (u[3] - u[0]) * sg.irm;
-  const real o2b = u[1] - u[3];
-  const real o2c = u[4] - u[1];
-  const real o2d = (u[2] - u[4]) * sg.irp;
-  const real o3a = (o2b - o2a) * sg.i1m;
-  const real o3b = o2c - o2b;
-  const real o3c = (o2d - o2c) * sg.i1p;
-  const real o4a = (o3b - o3a) * sg.i1m;
-  const real o4b = (o3c - o3b) * sg.i1p;
-  const real o5 = (o4b - o4a) * sg.i1mp;
-  const real cb[6] = {0.0, u[0], o2a, o3a, o4a, o5};
-  const double tq[4] = {0.0, SWALE_GLO_T1, SWALE_GLO_T2, 1.0};
-  const double wq[4] = {1.0 / 12.0, 5.0 / 12.0, 5.0 / 12.0, 1.0 / 12.0};
-  real S2 = 0.0;
-  for (int q = 0; q < 4; ++q) {
-    const double t = tq[q], t2 = t * t;
-    const double md[6] = {0, 0, 1.0, 2.0 * t, 3.0 * t2 - 2.0 * t, 4.0 * t2 * t - 6.0 * t2 + 2.0 * t};
-    const double mdd[6] = {0, 0, 0.0, 2.0, 6.0 * t - 2.0, 12.0 * t2 - 12.0 * t + 2.0};
-    real bdv = 0.0;
-    for (int k = 2; k <= 5; ++k) bdv += cb[k] * ((2.0 * md[k] + t * mdd[k]) + sg.rm * mdd[k]);
-    S2 += wq[q] * (eta4[q] - etabar) * bdv;
-  }
-  const real bL = 0.5 * (bLm + u[3]), bR = 0.5 * (u[4] + bRp);
-  const real b2L = 0.5 * (bLm * bLm + u[3] * u[3]), b2R = 0.5 * (u[4] * u[4] + bRp * bRp);
-  return (0.5 * g) * (b2R - b2L) - g * etabar * (bR - bL) - g * S2;
+  return 0.5 * source_special2(g, etabar, eta4, bd, sg, bLm, bRp);
+}
+
+// Flux differences and source of cell j: R = (R_E, R_M, R_B) of Eq. hydro2D / bottomrk.
+struct CellRhs {
+  real RE, RM, RB;
+};
+SWALE_HD CellRhs cell_rhs(const Flux& Fl, const Flux& Fr, real S) {
+  CellRhs o;
+  o.RE = -(Fr.FE - Fl.FE);
+  o.RM = -(Fr.FMm - Fl.FMp) + S;
+  o.RB = Fr.FB - Fl.FB;
+  return o;
 }
 
 // The interface fluxes at twice their value, with each side's own edge pressure left out of the
@@ -1170,18 +1182,6 @@ SWALE_HD real source_pressure_form(real hc, real hL, real hR, real deL, real deR
 // its width grows by dJ.
 SWALE_HD real rk_advance(real q, real a, real R, real dJ, real inv) {
   return fma_(fma_(-q, dJ, mul_(a, R)), inv, q);
-}
-
-// Flux differences and source of cell j: R = (R_E, R_M, R_B) of Eq. hydro2D / bottomrk.
-struct CellRhs {
-  real RE, RM, RB;
-};
-SWALE_HD CellRhs cell_rhs(const Flux& Fl, const Flux& Fr, real S) {
-  CellRhs o;
-  o.RE = -(Fr.FE - Fl.FE);
-  o.RM = -(Fr.FMm - Fl.FMp) + S;
-  o.RB = Fr.FB - Fl.FB;
-  return o;
 }
 
 }  // namespace swale

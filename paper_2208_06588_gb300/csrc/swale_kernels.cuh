@@ -169,10 +169,22 @@ struct DevState {
 };
 
 __constant__ double c_gauss_w[2 * kMaxGaussHalf + 1];
+__constant__ int2 c_gauss_q[2 * kMaxGaussHalf + 1];  // the same times 2^56, low and high limb of 28 bits
 
 // Status bits that stop an instance (SWALE_BIT_NEGDEPTH is a warning).
 constexpr unsigned int kErrBits =
     swale::ST_EWEIGHT | swale::ST_NONFINITE | swale::ST_EMESH | swale::ST_NODT | swale::ST_TIMEOUT;
+
+// Whether the mesh cache holds the values of stage STAGE's mesh: that of the step before's stage 2 is the
+// mesh of this step's stage 1; a static mesh has one for all stages of all later steps.
+template <int STAGE>
+__device__ __forceinline__ bool cached_mesh(const StepConst& K, const DevState& D, const DevScalars* S) {
+  if (!D.geo || (STAGE != 1 && K.mesh != SWALE_MESH_STATIC)) return false;
+  const unsigned long long tag = S->geo_tag;
+  if ((unsigned)(tag >> 32) != K.geo_epoch) return false;
+  const int ahead = (int)((unsigned)S->step_idx - (unsigned)tag);
+  return K.mesh == SWALE_MESH_STATIC ? ahead >= 0 : ahead == 0;
+}
 
 // An instance takes no further part in the step: finished (t_end), or an error was raised.
 __device__ __forceinline__ bool inst_idle(const DevScalars* S) {
@@ -196,39 +208,45 @@ __device__ __forceinline__ int32_t ghost(int32_t i, int32_t N, int bc) {
 
 // L2 projection of the bottom onto one cell [a, c] (Eq. baverage): on each piece the cell
 // overlaps (the first found by bisection of the breakpoints), the mean of the polynomial by the
-// 5-point Gauss-Legendre rule, exact for degree <= 8 and divided by the sum of the weights so
-// that constants come out exact; the cell average weights these means by the overlap lengths.
+// 5-point Gauss-Legendre rule, exact for degree <= 8, taken about the middle value so that constants
+// come out exact; the cell average weights these means by the overlap lengths.
 // (Differences of antiderivatives would cancel on short cells far from the breakpoint.)
-__device__ __noinline__ double bottom_average(const StepConst& K, double a, double c) {
-  const double xi[5] = {-0.9061798459386639928, -0.5384693101056830910, 0.0, 0.5384693101056830910,
-                        0.9061798459386639928};
-  const double wq[5] = {0.2369268850561890875, 0.4786286704993664680, 0.5688888888888888889, 0.4786286704993664680,
-                        0.2369268850561890875};
-  const double* br = K.bot_breaks;
-  int lo = 0, hi = K.bot_pieces;  // the piece p with br[p] <= a < br[p + 1] (clamped)
+// A cell within one piece (nearly all of them) takes the mean as the middle value plus the weighted
+// differences from it, with no division, and a constant piece its value. (With a division per
+// piece and cell and the constants copied to the stack, the projected bottom cost the dam break over the bump 27 %.)
+__device__ __noinline__ double bottom_average(const double* br, const double* coef, int pieces, int deg, double a, double c) {
+  int lo = 0, hi = pieces;  // the piece p with br[p] <= a < br[p + 1] (clamped)
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if (br[mid] <= a) lo = mid;
+    if (!swale::dlt(a, br[mid])) lo = mid;
     else hi = mid;
   }
+  const double x1 = 0.9061798459386639928, x2 = 0.5384693101056830910;
+  const double w1 = 0.5 * 0.2369268850561890875, w2 = 0.5 * 0.4786286704993664680;
+  auto mean = [&](int p, double l, double h) {
+    const double* ck = coef + p * (deg + 1);
+    if (deg == 0) return ck[0];
+    const double t = 0.5 * (l + h) - br[p], hw = 0.5 * (h - l);
+    auto v = [&](double y) {
+      double r = ck[deg];
+      for (int k = deg - 1; k >= 0; --k) r = fma(r, y, ck[k]);
+      return r;
+    };
+    const double v0 = v(t);
+    const double a1 = fma(-2.0, v0, v(fma(hw, x1, t)) + v(fma(-hw, x1, t)));
+    const double a2 = fma(-2.0, v0, v(fma(hw, x2, t)) + v(fma(-hw, x2, t)));
+    return fma(w1, a1, fma(w2, a2, v0));
+  };
+  if (!swale::dlt(a, br[lo]) && !swale::dlt(br[lo + 1], c)) return mean(lo, a, c);
   double s = 0.0;
-  for (int p = lo; p < K.bot_pieces && br[p] < c; ++p) {
-    const double x0 = br[p], l = fmax(a, x0), h = fmin(c, br[p + 1]);
-    if (!(h > l)) continue;
-    const double* ck = K.bot_coef + p * (K.bot_deg + 1);
-    const double m = 0.5 * (l + h), hw = 0.5 * (h - l);
-    double num = 0.0, den = 0.0;
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const double t = m + hw * xi[q] - x0;
-      double v = 0.0;
-      for (int k = K.bot_deg; k >= 0; --k) v = v * t + ck[k];
-      num += wq[q] * v;
-      den += wq[q];
-    }
-    s += (h - l) * (num / den);
+  for (int p = lo; p < pieces && br[p] < c; ++p) {
+    const double l = fmax(a, br[p]), h = fmin(c, br[p + 1]);
+    if (h > l) s += (h - l) * mean(p, l, h);
   }
   return s / (c - a);
+}
+__device__ __forceinline__ double bottom_average(const StepConst& K, double a, double c) {
+  return bottom_average(K.bot_breaks, K.bot_coef, K.bot_pieces, K.bot_deg, a, c);
 }
 
 __device__ __forceinline__ unsigned long long dbits(double v) { return (unsigned long long)__double_as_longlong(v); }
@@ -438,16 +456,29 @@ __global__ void k_prologue(StepConst K, DevState D) {
 // one pass, one per thread, and tiles advance by kMeshNodes = kMeshThreads - 1 nodes: the last
 // node of a tile is the next tile's first, filtered by both (the same sum in the same order),
 // which gives the tile the right neighbour of its last node for max |w_{k+1} - w_k| without a
-// second pass for one node. The block stages the cell velocities, the raw node velocities and
-// its filtered nodes in shared memory (dynamic, 3 T + 4 H + 4 doubles).
+// second pass for one node.
+//
+// The filter's 2 H + 1 products run on the integer multiplier in fixed point: an FP64 FMA holds the sub-partition
+// for 64 cycles, four 32-bit multiply-adds with 64-bit sums about ten. The raw velocities of the
+// tile's window are scaled by a power of two to 56-bit integers (2^56 above the largest of
+// them), the weights exp(-m^2 / 2 sigma^2) are 57-bit ones, both in two limbs of 28 bits, and the sums
+// are exact: the result is within (2 H + 1) 2^-57 of the largest raw velocity of the exact sum of
+// the rounded inputs, where the FP64 sum's bound is about 20 x 2^-53 of it. Measured against 64-bit
+// references the step's error is unchanged; the kernel needs 12 FP64 instructions per node instead of 61.
+// Nodes whose window is cut off by an end, and tiles whose largest velocity is beyond 2^900, below 2^-967
+// or a NaN, take the FP64 sum.
+// The block stages the cell velocities and the raw node velocities in shared memory (dynamic, and
+// the limbs in place of the former: 3 T + 4 H + 4 doubles).
 // ------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevState D) {
   extern __shared__ double sh[];
+  __shared__ unsigned wmax[kMeshThreads / 32];
   const int H = K.gauss_half, T = kMeshThreads, tid = threadIdx.x;
   const int nu = T + 2 * H + 2, nr = T + 2 * H + 1;
-  double* su = sh;         // cell velocities, cells [k0 - H - 1, k0 + T + H]
+  double* su = sh;         // cell velocities, cells [k0 - H - 1, k0 + T + H]; then the limbs of sraw
   double* sraw = sh + nu;  // raw node velocities, nodes [k0 - H, k0 + T + H]
   double* sw = sraw + nr;  // filtered velocities, nodes [k0, k0 + T]
+  int2* sx = reinterpret_cast<int2*>(su);
   pdl_wait();
   for (int t = blockIdx.x; t < D.nm; t += gridDim.x) {
     const Tile tl = D.mtiles ? D.mtiles[t] : Tile{0, t * kMeshNodes};
@@ -470,9 +501,32 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
       su[i] = u;
     }
     __syncthreads();
+    unsigned top = 0u;  // high word of the largest magnitude
     for (int i = tid; i < nr; i += T) {
       const int64_t k = k0 - H + i;
-      sraw[i] = (k >= 1 && k <= N - 1) ? 0.5 * (su[i] + su[i + 1]) : 0.0;
+      const double v = (k >= 1 && k <= N - 1) ? 0.5 * (su[i] + su[i + 1]) : 0.0;
+      sraw[i] = v;
+      const unsigned hi = (unsigned)__double2hiint(v) & 0x7fffffffu;
+      top = top > hi ? top : hi;
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((tid & 31) == 0) wmax[tid >> 5] = top;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kMeshThreads / 32; ++q) top = top > wmax[q] ? top : wmax[q];
+    // |v| < 2^(ex - 1022) for every raw velocity; v 2^(1022 - ex + 56) in two limbs.
+    const int ex = (int)(top >> 20);
+    const bool fixed = ex > 55 && ex < 1923;  // (2^-967 to 2^900, and no NaN or infinity)
+    if (fixed) {
+      for (int i = tid; i < nr; i += T) {
+        const unsigned long long bits = dbits(sraw[i]);
+        const int e = (int)((bits >> 52) & 0x7ff);
+        const long long m = e ? (long long)((bits & 0xfffffffffffffull) | 0x10000000000000ull) : 0ll;  // 53 bits (subnormals: 0)
+        const int sft = 3 - (ex - e);  // left by three where the exponent is the largest
+        long long x = sft >= 0 ? m << sft : (sft > -60 ? (m + (1ll << (-sft - 1))) >> -sft : 0ll);
+        if (bits >> 63) x = -x;
+        sx[i] = make_int2((int)(x & 0xfffffff), (int)(x >> 28));
+      }
     }
     __syncthreads();
     {
@@ -480,12 +534,26 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
       const int64_t k = k0 + i;
       double v = 0.0;
       if (k >= 1 && k <= N - 1) {
-        double acc = 0.0;
-        if (k - H >= 1 && k + H <= N - 1) {
+        if (top == 0u) {
+          v = 0.0;  // still water
+        } else if (fixed && k - H >= 1 && k + H <= N - 1) {
+          long long hh = 0, mid = 0, ll = 0;
+          for (int m = 0; m <= 2 * H; ++m) {
+            const int2 x = sx[i + m], g = c_gauss_q[m];
+            hh += (long long)x.y * g.y;
+            mid += (long long)x.y * g.x;
+            mid += (long long)x.x * g.y;
+            ll += (long long)x.x * g.x;
+          }
+          const long long low = ((mid & 0xfffffff) << 28) + ll;
+          const long long sum = hh + (mid >> 28) + ((low + (1ll << 55)) >> 56);  // 2^(1022 - ex + 56) times the filtered value
+          v = (double)sum * (K.gauss_iwsum * bitsd((unsigned long long)(ex - 55) << 52));
+        } else if (k - H >= 1 && k + H <= N - 1) {
+          double acc = 0.0;
           for (int m = -H; m <= H; ++m) acc += c_gauss_w[m + H] * sraw[i + m + H];
           v = acc * K.gauss_iwsum;
         } else {
-          double wsum = 0.0;
+          double acc = 0.0, wsum = 0.0;
           for (int m = -H; m <= H; ++m) {
             const int64_t q = k + m;
             if (q < 1 || q > N - 1) continue;
@@ -786,11 +854,15 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
   // as for 32, so they are gathered and spread over the block's threads, two to a cell (one per edge),
   // instead of taking their own warps one by one through about twice the work. (The barrier is the
   // one that the differences of order 4 need anyway.)
-  const bool open = SCHEME == 0 && mine && !smooth;
-  if (open) R.open[atomicAdd(&R.nopen, 1)] = (uint16_t)tid;
-  if (__syncthreads_or(open)) {
-    const int n2 = 2 * R.nopen;
-    for (int e = tid; e < n2; e += T) open_edge<T, SCHEME>(P, R, sE, sM, sJ, R.open[e >> 1], e & 1, dxmax);
+  if constexpr (SCHEME == 0) {
+    const bool open = mine && !smooth;
+    if (open) R.open[atomicAdd(&R.nopen, 1)] = (uint16_t)tid;
+    if (__syncthreads_or(open)) {
+      const int n2 = 2 * R.nopen;
+      for (int e = tid; e < n2; e += T) open_edge<T, SCHEME>(P, R, sE, sM, sJ, R.open[e >> 1], e & 1, dxmax);
+      __syncthreads();
+    }
+  } else {
     __syncthreads();
   }
   if (!mine) return;
@@ -845,7 +917,7 @@ template <int STAGE, int SCHEME, bool STOREK>
 struct ReconSink {
   const DevState& D;
   int32_t idx;      // edge-array index of the thread's cell
-  bool mine, next_mine, use_geo;
+  bool mine, next_mine, use_geo, put_geo;
   double hv;
   __device__ __forceinline__ void pair(double ip, double de, double dh) const {
     if (!mine) return;
@@ -853,26 +925,27 @@ struct ReconSink {
     D.dE[idx] = de;
     D.dH[idx] = dh;
     D.H[idx] = hv;
-    if (STAGE == 2 && D.geo) D.geo[GEO_IP * D.geo_stride + idx] = ip;
+    if (STAGE == 2 && put_geo) D.geo[GEO_IP * D.geo_stride + idx] = ip;
   }
   __device__ __forceinline__ void triple(double it) const {
     if (!next_mine) return;
     if (SCHEME == 2 || STOREK || !use_geo) D.itri[idx + 1] = it;
-    if (STAGE == 2 && D.geo) D.geo[GEO_IT * D.geo_stride + idx + 1] = it;
+    if (STAGE == 2 && put_geo) D.geo[GEO_IT * D.geo_stride + idx + 1] = it;
   }
   __device__ __forceinline__ void quad(double iq) const {
-    if (STAGE == 2 && D.geo && next_mine) D.geo[GEO_IQ * D.geo_stride + idx + 1] = iq;
+    if (STAGE == 2 && put_geo && next_mine) D.geo[GEO_IQ * D.geo_stride + idx + 1] = iq;
     if (STOREK && next_mine) D.gK[ADJ_IQ * D.geo_stride + idx + 1] = iq;
   }
   __device__ __forceinline__ void quint(double iv) const {
-    if (STAGE == 2 && D.geo) D.geo[GEO_IV * D.geo_stride + idx] = iv;
+    if (STAGE == 2 && put_geo) D.geo[GEO_IV * D.geo_stride + idx] = iv;
     if (STOREK) D.gK[ADJ_IV * D.geo_stride + idx] = iv;
   }
 };
 
 // STOREK: an instantiation of the hydrostatic scheme that also stores what the reverse reads (the
-// adjoint's recomputes).
-template <int STAGE, int T, int SCHEME = 0, bool STOREK = false>
+// adjoint's recomputes). CACHE: one that may take the reciprocals from the mesh cache (stage 1, and every
+// stage of a static mesh; in the others the values to be taken would only cost registers).
+template <int STAGE, int T, int SCHEME = 0, bool STOREK = false, bool CACHE = STAGE == 1>
 __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, DevState D, const double* __restrict__ Eg,
                                              const double* __restrict__ Mg, const double* __restrict__ Bg,
                                              const double* __restrict__ Jg) {
@@ -924,14 +997,12 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     const int32_t c = c0 - 2 + tid;                   // this thread's cell
     const int32_t idx = (int32_t)(eb + c + 1);        // its edge-array index
     const int32_t ca = (int32_t)(ga - ic.coff), cz = (int32_t)(ge - ic.coff);  // the cells copied
-    const unsigned long long geo_now =
-        ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)(S->step_idx & 0xffffffffLL);
-    // Reciprocal sums of the widths: as the previous step's stage 2 stored them (the same mesh), or
+    // Reciprocal sums of the widths: as an earlier stage 2 stored them (the same mesh), or
     // formed below. Those that lie at cells -1..N are in the cache: the pair starting at c, the triple
     // and quadruple whose second cell is c + 1, the quintuple centred at c.
-    const bool use_geo = STAGE == 1 && D.geo != nullptr && S->geo_tag == geo_now;
+    const bool use_geo = CACHE && cached_mesh<STAGE>(K, D, S), put_geo = STAGE == 2 && D.geo && !use_geo;
     MeshRecips mr{0.0, 0.0, 0.0, 0.0, use_geo && c >= -1 && c <= N, use_geo && c >= -2 && c + 1 <= N, false, false};
-    if (STAGE == 1) {
+    if (CACHE && use_geo) {
       mr.all_pair = __all_sync(0xffffffffu, mr.pair);
       mr.all_next = __all_sync(0xffffffffu, mr.next);
       if (mr.pair) {
@@ -1006,14 +1077,14 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     // Cells of the tile that are reconstructed and stored.
     const bool mine = tid >= 2 && tid < 2 + TO && c <= N;
     const bool next_mine = tid >= 1 && tid < 1 + TO && c + 1 <= N;  // cell c + 1 is
-    ReconSink<STAGE, SCHEME, STOREK> sink{D, idx, mine, next_mine, use_geo, hv};
+    ReconSink<STAGE, SCHEME, STOREK> sink{D, idx, mine, next_mine, use_geo, put_geo, hv};
     bool limited = false;
     EdgeState o;
     uint8_t flag = 0;
     double etaG[2] = {0.0, 0.0};
     uint32_t st = 0;
     recon_phases<T, SCHEME>(K.sc, rows, sE, sM, sJ, jv, ev, mv, hv, dxmax, mr, mine, sink, o, flag, etaG, st, &limited);
-    if (STAGE == 2 && D.geo != nullptr && c0 == -1 && tid == 0)
+    if (STAGE == 2 && put_geo && c0 == -1 && tid == 0)
       S->geo_tag = ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)((S->step_idx + 1) & 0xffffffffLL);
     WaveEdge eL{0.0, 0.0, 0.0}, eR{0.0, 0.0, 0.0};
     bool useL = false, useR = false;
@@ -1140,10 +1211,8 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     const bool fresh_w = (MODE == 0 && STAGE == 1 && K.mesh == SWALE_MESH_PROFILE);
     // The source's mesh-only values are cached beside the reconstruction's reciprocals: stage 2
     // stores them and the next step's stage 1, on the same mesh, reads them under the same tag.
-    const unsigned long long geo_now =
-        ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)(S->step_idx & 0xffffffffLL);
-    const bool use_sgeo = STAGE == 1 && MODE == 0 && D.geo != nullptr && S->geo_tag == geo_now;
-    const bool put_sgeo = STAGE == 2 && MODE == 0 && D.geo != nullptr;
+    const bool use_sgeo = MODE == 0 && cached_mesh<STAGE>(K, D, S), put_sgeo = STAGE == 2 && MODE == 0 && D.geo && !use_sgeo;
+    const bool still = use_sgeo && K.mesh == SWALE_MESH_STATIC;  // 1 / J^(1), 1 / J^(2) are there too
     const double sdiff = fresh_w ? S->sdiff : 0.0;
     const int32_t k = j0 + tid;  // this thread's node / interface and cell
     const int32_t el = (int32_t)(eb + k), er = el + 1;
@@ -1222,10 +1291,20 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
       const double Jp = use_sgeo && SCHEME != 2 ? 0.0 : Js[ghost(j + 1, N, K.bc)];
       if (SCHEME == 2) {
         const double bd[5] = {B[ghost(j - 1, N, K.bc)], B[j], B[ghost(j + 1, N, K.bc)], BLj, BRj};
-        const swale::SourceGeom sg =
-            swale::source_geom(Jm, Jc, swale::recip(Jm), swale::recip(Jc), swale::recip(Jp), D.ipair[el], D.ipair[er], D.itri[er]);
+        double iJm, iJc, iJp;
+        if (MODE == 0 && (STAGE > 1 || use_sgeo)) {  // (stage 1 on the cache: the widths are J^(1) of the last step)
+          const double* iJ = (STAGE == 3 ? D.iJ2 : D.iJ1) + cb;
+          iJm = iJ[ghost(j - 1, N, K.bc)];
+          iJc = iJ[j];
+          iJp = iJ[ghost(j + 1, N, K.bc)];
+        } else {
+          iJm = swale::recip(Jm);
+          iJc = swale::recip(Jc);
+          iJp = swale::recip(Jp);
+        }
+        const swale::SourceGeom sg = swale::source_geom(Jm, Jc, iJm, iJc, iJp, D.ipair[el], D.ipair[er], D.itri[er]);
         const double eta4[4] = {ELj, D.eG1[er], D.eG2[er], ERj};
-        Rm = swale::fma_(2.0, swale::source_cell_special(K.sc.g, Ej, eta4, bd, sg, D.eBR[er - 1], D.eBL[er + 1]), Rm);
+        Rm = swale::add_(Rm, swale::source_special2(K.sc.g, Ej, eta4, bd, sg, D.eBR[er - 1], D.eBL[er + 1]));
       } else {
         swale::SourceRatio sr;
         if (use_sgeo) {
@@ -1280,8 +1359,9 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
           jmaxb = J2;
           jminb = J1;
           if (!swale::gt0(J1) || !swale::gt0(J2)) st |= swale::ST_EMESH;
-          const double inv = swale::recip(J1);
-          D.iJ1[g] = inv;
+          double inv;
+          if (still) inv = D.iJ1[g];
+          else D.iJ1[g] = inv = swale::recip(J1);
           D.YE[g] = R2[0];
           D.YM[g] = R2[1];
           D.YB[g] = R2[2];
@@ -1296,8 +1376,9 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
           D.YE[g] = Y[0];
           D.YM[g] = Y[1];
           D.YB[g] = Y[2];
-          const double inv = swale::recip(D.J2[g]);
-          D.iJ2[g] = inv;
+          double inv;
+          if (still) inv = D.iJ2[g];
+          else D.iJ2[g] = inv = swale::recip(D.J2[g]);
           const double edt = 0.125 * dt, hdJ = 0.5 * dJ;
           D.Eb[g] = swale::rk_advance(q0[0], edt, Y[0], hdJ, inv);
           D.Mb[g] = swale::rk_advance(q0[1], edt, Y[1], hdJ, inv);

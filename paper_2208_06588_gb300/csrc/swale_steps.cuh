@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, 
     const swale::SourceGeom sg = swale::source_geom(rJ[tid - 1], jv, sI[tid - 1], iv, sI[tid + 1], sPair[0][tid - 1],
                                                     sink.ip, sPair[1][tid - 1]);
     const double eta4[4] = {o.EL, etaG[0], etaG[1], o.ER};
-    Rm = swale::fma_(2.0, swale::source_cell_special(P.g, ev, eta4, bd, sg, sR[1][tid - 1], sBL[tid + 1]), Rm);
+    Rm = swale::add_(Rm, swale::source_special2(P.g, ev, eta4, bd, sg, sR[1][tid - 1], sBL[tid + 1]));
   } else {
     const swale::SourceRatio sr =
         swale::source_ratio(rJ[tid - 1], jv, rJ[tid + 1], sI[tid - 1], sI[tid + 1], sPair[1][tid - 1]);

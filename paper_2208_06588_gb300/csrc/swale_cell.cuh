@@ -324,6 +324,44 @@ SWALE_HD bool sure_smooth_nonwb_f32(double g, double h_dry, double hb, double mb
   return sure_smooth1_f32(F, c4, c3, fd, fm, it, eps);
 }
 
+// sin(pi x) (want_sin) or cos(pi x), |x| < 2^40: x = n / 2 + r with |r| <= 1/4, then the Taylor series of
+// sin or cos at pi r, chosen by the quadrant, to the term of order 17 or 16 (what is left out is below
+// 2^-58 of the result). One chain of operations for both functions, so that two lanes of a warp get
+// a sine and a cosine for the price of one.
+SWALE_HD double trig_pi(double x, bool want_sin) {
+  const double big = 6755399441055744.0;  // 1.5 * 2^52: adding it rounds to an integer
+#if defined(__CUDA_ARCH__)
+  const double t = __fma_rn(2.0, x, big);
+  const unsigned n = (unsigned)__double2loint(t);
+  const double r = __fma_rn(-0.5, __dadd_rn(t, -big), x);
+#else
+  volatile double t = 2.0 * x + big;
+  double tv = t;
+  uint64_t tb;
+  memcpy(&tb, &tv, 8);
+  const unsigned n = (unsigned)tb;
+  const double r = x - 0.5 * (tv - big);
+#endif
+  const bool odd = n & 1u, s = want_sin != odd, neg = ((want_sin ? n : n + 1u) & 2u) != 0u;
+  const double pi = 3.14159265358979323846;
+  const double y = pi * r, z = y * y;
+  // What the rounded y leaves out (with pi's own remainder), carried to the end: errors stay below one unit.
+  const double yl = fma(1.2246467991473532e-16, r, fma(pi, r, -y));
+  const double lo = s ? yl : -y * yl;
+  // (-1)^k / (2k+1)! and (-1)^k / (2k)!
+  double p = s ? 1.0 / 355687428096000.0 : 1.0 / 20922789888000.0;
+  p = fma(p, z, s ? -1.0 / 1307674368000.0 : -1.0 / 87178291200.0);
+  p = fma(p, z, s ? 1.0 / 6227020800.0 : 1.0 / 479001600.0);
+  p = fma(p, z, s ? -1.0 / 39916800.0 : -1.0 / 3628800.0);
+  p = fma(p, z, s ? 1.0 / 362880.0 : 1.0 / 40320.0);
+  p = fma(p, z, s ? -1.0 / 5040.0 : -1.0 / 720.0);
+  p = fma(p, z, s ? 1.0 / 120.0 : 1.0 / 24.0);
+  p = fma(p, z, s ? -1.0 / 6.0 : -0.5);
+  const double a = s ? y : 1.0;
+  const double v = a + fma(z * a, p, lo);
+  return neg ? -v : v;
+}
+
 // Wave speed |u| + sqrt(g max(h, 0)) of one limited edge state (Eq. alpha2D).
 SWALE_HD real wave_speed(real g, real h, real u) { return add_(dabs(u), wave_sqrt(mul_(g, pos0(h)))); }
 

@@ -127,6 +127,21 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState
   double iJ0 = 1.0;  // 1 / J^n of the thread's cell
   bool have_mesh = false;
 
+  // The values of the cells that other threads own, for the next stage: read as soon as the barrier has
+  // passed, beside the status and the maxima.
+  double pe = 0.0, pm = 0.0, pb = 0.0, pj = 1.0, pi = 1.0;
+  const bool foreign = !own && real_cell;
+  auto fetch = [&](const double* gE, const double* gM, const double* gB, const double* gJ, const double* gi) {
+    if (!foreign) return;
+    pe = __ldcg(gE + g);
+    pm = __ldcg(gM + g);
+    pb = __ldcg(gB + g);
+    pj = __ldcg(gJ + g);
+    if (gi) pi = __ldcg(gi + g);
+    if (flip) pm = -pm;
+  };
+  fetch(D.E0, D.M0, D.B0, D.J0, nullptr);
+
   while (taken < nsteps && !done) {
     if (K.t_end > 0.0 && tn >= K.t_end) {
       done = 1;
@@ -137,37 +152,13 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState
     unsigned int err = 0;
 #pragma unroll 1
     for (int stage = 1; stage <= 3; ++stage) {
-      // The stage's cells: owned ones from registers, the others as their owners (or images) have them.
-      double ev = qs[0], mv = qs[1], bv = qs[2], jv = Js, iv = iJs;
-      if (!own) {
-        ev = mv = bv = 0.0;
-        jv = 1.0;  // filler beyond the last ghost cell
-        iv = 1.0;
-        if (real_cell) {
-          const double *gE = D.E0, *gM = D.M0, *gB = D.B0, *gJ = D.J0;
-          if (stage == 2) {
-            gE = D.Ea;
-            gM = D.Ma;
-            gB = D.Ba;
-            gJ = D.J1;
-          } else if (stage == 3) {
-            gE = D.Eb;
-            gM = D.Mb;
-            gB = D.Bb;
-            gJ = D.J2;
-          }
-          ev = __ldcg(gE + g);
-          mv = __ldcg(gM + g);
-          bv = __ldcg(gB + g);
-          jv = __ldcg(gJ + g);
-          if (flip) mv = -mv;
-          if (stage > 1) iv = __ldcg((stage == 2 ? D.iJ1 : D.iJ2) + g);
-        }
-      }
-      if (stage == 1) {
-        if (taken == 0) iv = swale::recip(jv);
-        else if (!own) iv = real_cell ? __ldcg(D.iJ1 + g) : 1.0;
-        if (taken == 0 && own) iJ0 = iv;
+      // The stage's cells: owned ones from registers, the others as their owners (or images) have them
+      // (filler beyond the last ghost cell).
+      const double ev = own ? qs[0] : pe, mv = own ? qs[1] : pm, bv = own ? qs[2] : pb, jv = own ? Js : pj;
+      double iv = own ? iJs : pi;
+      if (stage == 1 && taken == 0) {
+        iv = swale::recip(jv);
+        if (own) iJ0 = iv;
       }
       rE[tid] = ev;
       rM[tid] = mv;
@@ -182,7 +173,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState
       uint8_t flag = 0;
       double etaG[2] = {0.0, 0.0};
       uint32_t st = 0;
-      recon_phases<T, SCHEME>(K.sc, rows, rE, rM, rJ, jv, ev, mv, hv, stage == 1 ? jmax : stage == 2 ? jm1 : jm2, mr, mine, sink,
+      recon_phases<T, SCHEME, 16>(K.sc, rows, rE, rM, rJ, jv, ev, mv, hv, stage == 1 ? jmax : stage == 2 ? jm1 : jm2, mr, mine, sink,
                               o, flag, etaG, st);
       if (stage == 2 || !moving) {
         mr.ip = sink.ip;
@@ -320,6 +311,9 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState
         timeout = true;
         break;
       }
+      if (stage == 1) fetch(D.Ea, D.Ma, D.Ba, D.J1, D.iJ1);
+      else if (stage == 2) fetch(D.Eb, D.Mb, D.Bb, D.J2, D.iJ2);
+      else fetch(D.E0, D.M0, D.B0, D.J0, D.iJ1);
       const unsigned int raised2 = __ldcg(&X->st[set][2 * stage - 1]);
       if (stage == 1 && moving) {
         jm1 = bitsd(__ldcg(&X->mx[set][3]));
@@ -462,7 +456,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, 
   uint8_t flag = 0;
   double etaG[2] = {0.0, 0.0};
   uint32_t st = 0;
-  recon_phases<T, SCHEME>(P, rows, rE, rM, rJ, jv, ev, mv, hv, dx, none, mine, sink, o, flag, etaG, st);
+  recon_phases<T, SCHEME, 16>(P, rows, rE, rM, rJ, jv, ev, mv, hv, dx, none, mine, sink, o, flag, etaG, st);
   if (own && flags) flags[c] = flag;
   sR[0][tid] = o.ER;
   sR[1][tid] = o.BR;

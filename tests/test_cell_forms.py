@@ -66,6 +66,7 @@ void t_source(const double* J, const double* eta, const double* hd, double* out)
   for (int k = 0; k < 5; ++k) bd[k] = eta[k] - hd[k];
   out[1] = 2.0 * source_cell_form(-1.0, hd, bd, f) + (hd[4] * hd[4] - hd[3] * hd[3]);
 }
+double t_trig(double x, int s) { return trig_pi(x, s != 0); }
 double t_rk(double q, double a, double R, double dJ, double J) { return rk_advance(q, a, R, dJ, 1.0 / (J + dJ)); }
 // ev[2][3] by open_edge_values, and by the plain Steps 2-4; returns class | plain class << 2 | 16 if the tie is near.
 int t_open(const double* h, const double* eta, const double* hu, const double* hh, double dx, double* ev) {
@@ -135,7 +136,7 @@ def lib(tmp_path_factory):
                     os.path.join(ROOT, "paper_2208_06588_gb300", "csrc"), "-o", str(out), str(src)], check=True)
     L = ctypes.CDLL(str(out))
     for n, r in (("t_eweight", ctypes.c_int), ("t_moderate", ctypes.c_int), ("t_rk", ctypes.c_double),
-                 ("t_limit", ctypes.c_int), ("t_nonwb", ctypes.c_int), ("t_open", ctypes.c_int)):
+                 ("t_limit", ctypes.c_int), ("t_nonwb", ctypes.c_int), ("t_open", ctypes.c_int), ("t_trig", ctypes.c_double)):
         getattr(L, n).restype = r
     return L
 
@@ -332,3 +333,19 @@ def test_nonwb_fp32_test_implies_the_smooth_class(lib):
             for s in (lo, hi, hi * (1 + 1e-12), hi * (1 + 1e-9), hi * (1 + 1e-6)):
                 assert ask(*f(s)) != 3
     assert told > 1000 and told > 0.8 * smooth
+
+
+def test_trig_pi(lib):
+    """Within 4 units in the last place of the larger of the value and 2^-53 of 1, over several periods."""
+    import math
+    rng = np.random.default_rng(11)
+    for x in np.concatenate([rng.uniform(-3, 3, 3000), rng.uniform(0, 1e4, 500), np.arange(-8, 9) / 4.0,
+                             10.0 ** rng.uniform(-12, -1, 500)]):
+        n = math.floor(2 * x + 0.5)
+        y = math.pi * (x - n / 2)  # exact reduction, so the library's argument is accurate
+        ref = {0: (math.sin(y), math.cos(y)), 1: (math.cos(y), -math.sin(y)), 2: (-math.sin(y), -math.cos(y)),
+               3: (-math.cos(y), math.sin(y))}[n % 4]
+        for s in (1, 0):
+            got = lib.t_trig(_d(x), s)
+            r = ref[1 - s]
+            assert abs(got - r) <= 4 * 2.3e-16 * max(abs(r), abs(y) if s else 1e-3)

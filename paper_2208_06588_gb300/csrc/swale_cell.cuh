@@ -653,6 +653,9 @@ SWALE_HD void recon_cell(const SchemeConst& P, const real h[5], const real it[3]
 // for each order of differences (shared by the pairs, triples, quadruples that use them), with
 // four reciprocals per cell, against about 75 FP64 operations per cell and stage for the weights
 // and the linear form of smooth_edge_coeffs. Equal to it in exact arithmetic, exact for constants.
+#define SWALE_GLO_T1 0.27639320225002103036  // (1 - 1/sqrt 5) / 2
+#define SWALE_GLO_T2 0.72360679774997896964  // (1 + 1/sqrt 5) / 2
+#define SWALE_GLO_XI 0.44721359549995793928  // 1/sqrt 5
 struct SmoothWidths {
   real h1, h2, h3, p01, p12, p23, p34;
 };
@@ -662,16 +665,19 @@ SWALE_HD real smooth_right(const SmoothWidths& w, real v, real d2r, real d3, rea
 SWALE_HD real smooth_left(const SmoothWidths& w, real v, real d2l, real d3, real d4l, real d5) {
   return fma_(-w.h2, fma_(w.h1, fma_(-w.p23, fma_(w.p01, d5, d4l), d3), d2l), v);
 }
-// The same interpolant at the offset t h2 (0 < t < 1) from the cell's left edge: the nodes in the
-// order y2, y3, y4, y1, y5, y0 with the basis polynomials N_k and their derivatives.
-SWALE_HD real smooth_point(const SmoothWidths& w, real h4, real t, real v, real d2r, real d3, real d4r, real d5) {
-  const real tm = t - 1.0;
-  const real n2 = mul_(mul_(t, tm), mul_(w.h2, w.h2)), e2 = mul_(t + tm, w.h2);
-  const real a4 = fma_(tm, w.h2, -w.h3), a1 = fma_(t, w.h2, w.h1), a5 = sub_(a4, h4);
-  const real n3 = mul_(n2, a4), e3 = fma_(e2, a4, n2);
-  const real n4 = mul_(n3, a1), e4 = fma_(e3, a1, n3);
-  const real e5 = fma_(e4, a5, n4);
-  return add_(v, fma_(d2r, e2, fma_(d3, e3, fma_(d4r, e4, mul_(d5, e5)))));
+// The same interpolant p at the two interior Gauss-Lobatto points (offsets (1 -+ 1/sqrt 5) h2 / 2 from the cell's
+// left edge), as the sum and the difference of its deviations from the average v, from the edge values pL, pR.
+// The four-point rule is exact for the quartic, so the deviations' sum is -(eL + eR) / 5; and the difference
+// follows from the edges' and the cubic coefficient c3 = (h2 / 2)^3 p^(3) / 6 at the centre: p2 - p1 = (eR - eL - (8/5) c3) / sqrt 5,
+// p^(3) = 24 (d4 + d5 sum_k (y_c - y_k)) over the nodes of d4. 14 operations (the two values by themselves: 32).
+struct PointPair {
+  real sum, diff;
+};
+SWALE_HD PointPair smooth_points(const SmoothWidths& w, real v, real pL, real pR, real d4r, real d5) {
+  const real eL = sub_(pL, v), eR = sub_(pR, v);
+  const real s = sub_(sub_(fma_(-0.5, w.h2, w.h1), w.h3), w.p34);
+  const real k = mul_(mul_(w.h2, w.h2), mul_(-0.8 * SWALE_GLO_XI, w.h2));
+  return {mul_(-0.2, add_(eL, eR)), fma_(k, fma_(s, d5, d4r), mul_(SWALE_GLO_XI, sub_(eR, eL)))};
 }
 // Whether the five widths (truncated to FP32) are above 1e-9, so that the FP32 indicator factors (up
 // to the fourth power of a width) are normal numbers, and within a factor of 2^20 of each other. Then both middle linear weights d_1 are positive beyond any rounding: with
@@ -892,8 +898,6 @@ SWALE_HD void point_phi(const SchemeConst& P, const real d[3], const real beta[3
 }
 
 // Interior 4-point Gauss-Lobatto points of the unit cell, (1 -+ 1/sqrt 5) / 2.
-#define SWALE_GLO_T1 0.27639320225002103036
-#define SWALE_GLO_T2 0.72360679774997896964
 
 // Reconstruction for the special source-term scheme (Sec. 4.2): that of recon_cell plus eta at
 // the two interior Gauss-Lobatto points (Eq. gausssij2) with the cell's shared indicators and
@@ -1089,34 +1093,40 @@ SWALE_HD real source_cell_form(real g, const real hd[5], const real bd[5], const
 // the Gauss-Lobatto points t = 0, (1 -+ 1/sqrt 5)/2, 1 (weights 1/12, 5/12, 5/12, 1/12).
 //   eta4: eta at the four points;  bd: bottom data as in source_cell_form;  bLm: right-edge bottom of
 //   cell j-1, bRp: left-edge bottom of cell j+1.
-// Twice the value, arranged for few operations (about 58 instead of 90): with c_k the Newton coefficients of
+// Twice the value, arranged for few operations (about 50 instead of 90): with c_k the Newton coefficients of
 // the bottom's primitive and e_q = eta_q - etabar, b_h'(t) = sum_k c_k (2 m_k' + (t + r_m) m_k''), m_k = t, t^2, t^3 - t^2,
-// t^4 - 2 t^3 + t^2, so the sum over the points needs the four moments sum_q w_q e_q t_q^n only; and the edge terms
-// are products of differences, (b_R - b_L) (b_R + b_L - 2 etabar), of either side.
-SWALE_HD real source_special2(real g, real etabar, const real eta4[4], const real bd[5], const SourceGeom& sg, real bLm,
-                              real bRp) {
+// t^4 - 2 t^3 + t^2. In x = 2 t - 1 the rule is symmetric, so the moments M_n = sum_q 12 w_q e_q x_q^n follow from the sums
+// and differences of the e_q at the edges (s03, d03) and at the interior points (`in`, see smooth_points). The edge
+// terms are products of differences, (b_R - b_L) (b_R + b_L - 2 etabar), of either side.
+SWALE_HD real source_special2(real g, real etabar, real EL, real ER, const PointPair& in, const real bd[5],
+                              const SourceGeom& sg, real bLm, real bRp) {
   const real o2a = mul_(sub_(bd[3], bd[0]), sg.irm), o2b = sub_(bd[1], bd[3]), o2c = sub_(bd[4], bd[1]);
   const real o2d = mul_(sub_(bd[2], bd[4]), sg.irp);
   const real o3a = mul_(sub_(o2b, o2a), sg.i1m), o3b = sub_(o2c, o2b), o3c = mul_(sub_(o2d, o2c), sg.i1p);
   const real o4a = mul_(sub_(o3b, o3a), sg.i1m), o4b = mul_(sub_(o3c, o3b), sg.i1p);
   const real o5 = mul_(sub_(o4b, o4a), sg.i1mp);
-  const double t1 = SWALE_GLO_T1, t2 = SWALE_GLO_T2;
-  const real e0 = sub_(eta4[0], etabar), e1 = sub_(eta4[1], etabar), e2 = sub_(eta4[2], etabar), e3 = sub_(eta4[3], etabar);
-  // 12 times the moments of order 0..3 (weights 1, 5, 5, 1), times 2, 6, 12, 20
-  const real A = fma_(10.0, add_(e1, e2), mul_(2.0, add_(e0, e3)));
-  const real B = fma_(30.0 * t1, e1, fma_(30.0 * t2, e2, mul_(6.0, e3)));
-  const real C = fma_(60.0 * t1 * t1, e1, fma_(60.0 * t2 * t2, e2, mul_(12.0, e3)));
-  const real D = fma_(100.0 * t1 * t1 * t1, e1, fma_(100.0 * t2 * t2 * t2, e2, mul_(20.0, e3)));
-  const real BA = sub_(B, A), CB = sub_(C, B), DC = sub_(D, C);
-  const real p3 = fma_(sg.rm, A, B), p4 = fma_(sg.rm, BA, CB), p5 = fma_(sg.rm, sub_(CB, BA), sub_(DC, CB));
-  const real S12 = fma_(o5, p5, fma_(o4a, p4, fma_(o3a, p3, mul_(o2a, A))));  // 12 sum_q w_q e_q b_h'(t_q)
+  const real e0 = sub_(EL, etabar), e3 = sub_(ER, etabar);
+  const real s03 = add_(e0, e3), d03 = sub_(e3, e0);
+  // M_0, 3 M_1, 3 M_2, M_3 (x = -+1, -+1/sqrt 5; weights 1, 5, 5, 1)
+  const real M0 = fma_(5.0, in.sum, s03), N1 = fma_(15.0 * SWALE_GLO_XI, in.diff, mul_(3.0, d03));
+  const real N2 = mul_(3.0, add_(s03, in.sum)), M3 = fma_(SWALE_GLO_XI, in.diff, d03);
+  const real p3 = fma_(fma_(2.0, sg.rm, 3.0), M0, N1);
+  const real p4 = fma_(sg.rm, add_(N1, M0), add_(N1, N2));
+  const real N20 = sub_(N2, M0);
+  const real p5 = fma_(sg.rm, N20, fma_(2.5, M3, mul_(0.5, sub_(N20, N1))));
+  // 12 sum_q w_q e_q b_h'(t_q)
+  const real S12 = fma_(o5, p5, fma_(o4a, p4, fma_(o3a, p3, mul_(2.0, mul_(o2a, M0)))));
   const real x = mul_(sub_(bd[4], bd[3]), fma_(-2.0, etabar, add_(bd[4], bd[3])));
   const real y = fma_(sub_(bRp, bLm), fma_(-2.0, etabar, add_(bRp, bLm)), x);
   return mul_(g, fma_(-1.0 / 6.0, S12, mul_(0.5, y)));
 }
+// The deviations of the interior points' eta from the average, as source_special2 takes them.
+SWALE_HD PointPair point_pair(real etabar, real eta1, real eta2) {
+  return {add_(sub_(eta1, etabar), sub_(eta2, etabar)), sub_(eta2, eta1)};
+}
 SWALE_HD real source_cell_special(real g, real etabar, const real eta4[4], const real bd[5], const SourceGeom& sg,
                                   real bLm, real bRp) {
-  return 0.5 * source_special2(g, etabar, eta4, bd, sg, bLm, bRp);
+  return 0.5 * source_special2(g, etabar, eta4[0], eta4[3], point_pair(etabar, eta4[1], eta4[2]), bd, sg, bLm, bRp);
 }
 
 // Flux differences and source of cell j: R = (R_E, R_M, R_B) of Eq. hydro2D / bottomrk.

@@ -141,7 +141,7 @@ struct DevState {
   // Backups of q^n, J^n (cells) and x^n (nodes) written by the stage-3 update before it commits
   // the step, restored by k_commit if that update raised an error (null: no roll-back).
   double *bE, *bM, *bB, *bJ, *bx;
-  double *eG1, *eG2;           // eta at the interior Gauss-Lobatto points (special source scheme only)
+  double *eG1, *eG2;           // interior Gauss-Lobatto points of eta, as smooth_points has them (special source scheme only)
   // Mesh cache: GEO_ARRAYS arrays in the edge layout, geo[k * geo_stride + idx] (null: every stage forms
   // these values, bit for bit the same).
   double* geo;
@@ -862,7 +862,7 @@ __device__ __noinline__ void open_cells_split(const SchemeConst P, ReconRows<T, 
 // The reconstruction of a block's T cells, thread i holding cell i: width jv, averages ev, mv of eta
 // and hu, depth hv, also in the shared rows sE, sM, sJ (a barrier lies behind their stores). Threads
 // with mine set (2 <= i <= T - 3) get the limited edge state o, the class and, for the special scheme,
-// eta at the interior points. The sink is handed each thread's pair differences and reciprocals as
+// the interior points of eta. The sink is handed each thread's pair differences and reciprocals as
 // they are formed: pair(ip, de, dh), triple(it), quad(iq), quint(iv). SPLIT: up to how many open cells
 // open_cells_split takes them: 16 (one warp per sub-partition) where the block is alone on its SM; none where
 // other blocks fill it (up to 4 cells, one warp: 8580 us instead of 8556 for 8 steps of 10^6 cells).
@@ -870,7 +870,7 @@ template <int T, int SCHEME, int SPLIT, class Sink>
 __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, SCHEME>& R, const double* sE, const double* sM,
                                              const double* sJ, double jv, double ev, double mv, double hv, double dxmax,
                                              const MeshRecips& g, bool mine, Sink& sink, EdgeState& o, uint8_t& flag,
-                                             double etaG[2], uint32_t& st, bool* limited = nullptr) {
+                                             swale::PointPair& pts, uint32_t& st, bool* limited = nullptr) {
   const int tid = threadIdx.x;
   R.H[tid] = hv;  // the depth is reconstructed in place of the bottom
   R.Jf[tid] = swale::f32_trunc(jv);
@@ -973,8 +973,7 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
     const OpenOut r = recon_open_cell<SCHEME>(P, rows, tid, dxe);
     o = r.o;
     flag = r.flag;
-    etaG[0] = r.etaG[0];
-    etaG[1] = r.etaG[1];
+    pts = swale::point_pair(ev, r.etaG[0], r.etaG[1]);
     st |= r.st;
     return;
   }
@@ -988,10 +987,7 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
       const double d5 = swale::mul_(swale::sub_(d4r, d4l), iv);
       evl[v][0] = swale::smooth_left(w, vj[v], R.D2[v][tid - 1], d3c, d4l, d5);
       evl[v][1] = swale::smooth_right(w, vj[v], d2[v], d3c, d4r, d5);
-      if (SCHEME == 2 && v == 0) {
-        etaG[0] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T1, ev, d2[v], d3c, d4r, d5);
-        etaG[1] = swale::smooth_point(w, sJ[tid + 2], SWALE_GLO_T2, ev, d2[v], d3c, d4r, d5);
-      }
+      if (SCHEME == 2 && v == 0) pts = swale::smooth_points(w, ev, evl[0][0], evl[0][1], d4r, d5);
     }
   } else {
 #pragma unroll
@@ -1179,9 +1175,9 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
     bool limited = false;
     EdgeState o;
     uint8_t flag = 0;
-    double etaG[2] = {0.0, 0.0};
+    swale::PointPair pts{0.0, 0.0};
     uint32_t st = 0;
-    recon_phases<T, SCHEME, 0>(K.sc, rows, sE, sM, sJ, jv, ev, mv, hv, dxmax, mr, mine, sink, o, flag, etaG, st, &limited);
+    recon_phases<T, SCHEME, 0>(K.sc, rows, sE, sM, sJ, jv, ev, mv, hv, dxmax, mr, mine, sink, o, flag, pts, st, &limited);
     if (STAGE == 2 && put_geo && c0 == -1 && tid == 0)
       S->geo_tag = ((unsigned long long)K.geo_epoch << 32) | (unsigned long long)((S->step_idx + 1) & 0xffffffffLL);
     WaveEdge eL{0.0, 0.0, 0.0}, eR{0.0, 0.0, 0.0};
@@ -1198,8 +1194,8 @@ __global__ void __launch_bounds__(T, kReconThreads / T) k_recon(StepConst K, Dev
       D.euL[idx] = o.uL;
       D.euR[idx] = o.uR;
       if (SCHEME == 2) {
-        D.eG1[idx] = etaG[0];
-        D.eG2[idx] = etaG[1];
+        D.eG1[idx] = pts.sum;
+        D.eG2[idx] = pts.diff;
       }
       if (STAGE == 1) D.flags[idx] = flag;
       // Edges that touch interfaces 0..N only.
@@ -1401,8 +1397,8 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
           iJp = swale::recip(Jp);
         }
         const swale::SourceGeom sg = swale::source_geom(Jm, Jc, iJm, iJc, iJp, D.ipair[el], D.ipair[er], D.itri[er]);
-        const double eta4[4] = {ELj, D.eG1[er], D.eG2[er], ERj};
-        Rm = swale::add_(Rm, swale::source_special2(K.sc.g, Ej, eta4, bd, sg, D.eBR[er - 1], D.eBL[er + 1]));
+        const swale::PointPair pts = {D.eG1[er], D.eG2[er]};
+        Rm = swale::add_(Rm, swale::source_special2(K.sc.g, Ej, ELj, ERj, pts, bd, sg, D.eBR[er - 1], D.eBL[er + 1]));
       } else {
         swale::SourceRatio sr;
         if (use_sgeo) {

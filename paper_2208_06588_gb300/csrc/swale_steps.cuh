@@ -171,10 +171,10 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState
       StepSink sink{mr.ip, mr.it, mr.iq, mr.iv, 0.0, 0.0};
       EdgeState o{0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
       uint8_t flag = 0;
-      double etaG[2] = {0.0, 0.0};
+      swale::PointPair pts{0.0, 0.0};
       uint32_t st = 0;
       recon_phases<T, SCHEME, 16>(K.sc, rows, rE, rM, rJ, jv, ev, mv, hv, stage == 1 ? jmax : stage == 2 ? jm1 : jm2, mr, mine, sink,
-                              o, flag, etaG, st);
+                              o, flag, pts, st);
       if (stage == 2 || !moving) {
         mr.ip = sink.ip;
         mr.it = sink.it;
@@ -454,9 +454,9 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, 
   StepSink sink{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   EdgeState o{0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   uint8_t flag = 0;
-  double etaG[2] = {0.0, 0.0};
+  swale::PointPair pts{0.0, 0.0};
   uint32_t st = 0;
-  recon_phases<T, SCHEME, 16>(P, rows, rE, rM, rJ, jv, ev, mv, hv, dx, none, mine, sink, o, flag, etaG, st);
+  recon_phases<T, SCHEME, 16>(P, rows, rE, rM, rJ, jv, ev, mv, hv, dx, none, mine, sink, o, flag, pts, st);
   if (own && flags) flags[c] = flag;
   sR[0][tid] = o.ER;
   sR[1][tid] = o.BR;
@@ -491,8 +491,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, 
     const double bd[5] = {sB[tid - 1], bv, sB[tid + 1], o.BL, o.BR};
     const swale::SourceGeom sg = swale::source_geom(rJ[tid - 1], jv, sI[tid - 1], iv, sI[tid + 1], sPair[0][tid - 1],
                                                     sink.ip, sPair[1][tid - 1]);
-    const double eta4[4] = {o.EL, etaG[0], etaG[1], o.ER};
-    Rm = swale::add_(Rm, swale::source_special2(P.g, ev, eta4, bd, sg, sR[1][tid - 1], sBL[tid + 1]));
+    Rm = swale::add_(Rm, swale::source_special2(P.g, ev, o.EL, o.ER, pts, bd, sg, sR[1][tid - 1], sBL[tid + 1]));
   } else {
     const swale::SourceRatio sr =
         swale::source_ratio(rJ[tid - 1], jv, rJ[tid + 1], sI[tid - 1], sI[tid + 1], sPair[1][tid - 1]);

@@ -22,7 +22,7 @@ SRC = r"""
 using namespace swale;
 extern "C" {
 // dd[v]: D2[4], D3[3] of v on the widths h; out: left, right, two interior points, then the linear form's edges.
-void t_edges(const double* h, const double* v, double t1, double t2, double* out) {
+void t_edges(const double* h, const double* v, double* out) {
   double ip[4], it[3], iq[2], d2[4], d3[3], d4[2];
   for (int a = 0; a < 4; ++a) { ip[a] = 1.0 / (h[a] + h[a + 1]); d2[a] = (v[a + 1] - v[a]) * ip[a]; }
   for (int a = 0; a < 3; ++a) { it[a] = 1.0 / (h[a] + h[a + 1] + h[a + 2]); d3[a] = (d2[a + 1] - d2[a]) * it[a]; }
@@ -31,8 +31,9 @@ void t_edges(const double* h, const double* v, double t1, double t2, double* out
   const SmoothWidths w = {h[1], h[2], h[3], h[0] + h[1], h[1] + h[2], h[2] + h[3], h[3] + h[4]};
   out[0] = smooth_left(w, v[2], d2[1], d3[1], d4[0], d5);
   out[1] = smooth_right(w, v[2], d2[2], d3[1], d4[1], d5);
-  out[2] = smooth_point(w, h[4], t1, v[2], d2[2], d3[1], d4[1], d5);
-  out[3] = smooth_point(w, h[4], t2, v[2], d2[2], d3[1], d4[1], d5);
+  const PointPair pts = smooth_points(w, v[2], out[0], out[1], d4[1], d5);
+  out[2] = v[2] + 0.5 * (pts.sum - pts.diff);
+  out[3] = v[2] + 0.5 * (pts.sum + pts.diff);
   CellGeom Gm; uint32_t st = 0;
   cell_geom(h, h[2], Gm, st, false);
   smooth_edge_coeffs(h, it, Gm);
@@ -65,6 +66,11 @@ void t_source(const double* J, const double* eta, const double* hd, double* out)
   double bd[5];
   for (int k = 0; k < 5; ++k) bd[k] = eta[k] - hd[k];
   out[1] = 2.0 * source_cell_form(-1.0, hd, bd, f) + (hd[4] * hd[4] - hd[3] * hd[3]);
+}
+double t_special(const double* J, double etabar, const double* eta4, const double* bd, double bLm, double bRp) {
+  const SourceGeom sg = source_geom(J[0], J[1], 1.0 / J[0], 1.0 / J[1], 1.0 / J[2], 1.0 / (J[0] + J[1]),
+                                    1.0 / (J[1] + J[2]), 1.0 / (J[0] + J[1] + J[2]));
+  return source_special2(9.812, etabar, eta4[0], eta4[3], point_pair(etabar, eta4[1], eta4[2]), bd, sg, bLm, bRp);
 }
 double t_trig(double x, int s) { return trig_pi(x, s != 0); }
 double t_rk(double q, double a, double R, double dJ, double J) { return rk_advance(q, a, R, dJ, 1.0 / (J + dJ)); }
@@ -136,7 +142,8 @@ def lib(tmp_path_factory):
                     os.path.join(ROOT, "paper_2208_06588_gb300", "csrc"), "-o", str(out), str(src)], check=True)
     L = ctypes.CDLL(str(out))
     for n, r in (("t_eweight", ctypes.c_int), ("t_moderate", ctypes.c_int), ("t_rk", ctypes.c_double),
-                 ("t_limit", ctypes.c_int), ("t_nonwb", ctypes.c_int), ("t_open", ctypes.c_int), ("t_trig", ctypes.c_double)):
+                 ("t_limit", ctypes.c_int), ("t_nonwb", ctypes.c_int), ("t_open", ctypes.c_int), ("t_trig", ctypes.c_double),
+                    ("t_special", ctypes.c_double)):
         getattr(L, n).restype = r
     return L
 
@@ -163,14 +170,14 @@ def test_smooth_values_are_the_big_stencils_polynomial(lib, spread):
         I = P.integ()
         v = np.array([(I(y[k + 1]) - I(y[k])) / (y[k + 1] - y[k]) for k in range(5)])
         out = np.zeros(6)
-        t = rng.uniform(0.01, 0.99, 2)
-        lib.t_edges(_p(h), _p(v), _d(t[0]), _d(t[1]), _p(out))
+        t = 0.5 + np.array([-0.5, 0.5]) / np.sqrt(5.0)
+        lib.t_edges(_p(h), _p(v), _p(out))
         scale = np.abs(v).max() * (1.0 + np.exp(2.0 * spread))
         assert abs(out[0] - P(0.0)) <= 1e-12 * scale and abs(out[1] - P(1.0)) <= 1e-12 * scale
         assert abs(out[2] - P(t[0])) <= 1e-12 * scale and abs(out[3] - P(t[1])) <= 1e-12 * scale
         assert np.abs(out[:2] - out[4:]).max() <= 1e-12 * scale
         k = np.full(5, v[0])
-        lib.t_edges(_p(h), _p(k), _d(t[0]), _d(t[1]), _p(out))
+        lib.t_edges(_p(h), _p(k), _p(out))
         assert np.all(out[:4] == v[0])
 
 
@@ -349,3 +356,28 @@ def test_trig_pi(lib):
             got = lib.t_trig(_d(x), s)
             r = ref[1 - s]
             assert abs(got - r) <= 4 * 2.3e-16 * max(abs(r), abs(y) if s else 1e-3)
+
+
+@pytest.mark.parametrize("spread", [0.0, 0.5, 1.5])
+def test_special_source(lib, spread):
+    """The Gauss-Lobatto sum with the bottom's quartic from its five data and the edge terms, at twice the value."""
+    rng = np.random.default_rng(12)
+    x = np.array([-1.0, -1.0 / np.sqrt(5.0), 1.0 / np.sqrt(5.0), 1.0])
+    wq = np.array([1.0, 5.0, 5.0, 1.0]) / 12.0
+    for _ in range(200):
+        J = np.exp(rng.uniform(-spread, spread, 3))
+        bd, eta, eb = rng.uniform(-1, 1, 5), rng.uniform(-1, 1, 4), rng.uniform(-1, 1)
+        bm, bp = rng.uniform(-1, 1, 2)
+        y = np.array([-J[0] / J[1], 0.0, 1.0, 1.0 + J[2] / J[1]])
+        A = np.zeros((5, 5))
+        for n in range(5):
+            I = lambda t: t ** (n + 1) / (n + 1)
+            for c in range(3):
+                A[c, n] = (I(y[c + 1]) - I(y[c])) / (y[c + 1] - y[c])
+            A[3, n], A[4, n] = 0.0 ** n, 1.0
+        q = np.linalg.solve(A, bd)
+        slope = np.polynomial.Polynomial(q).deriv()((1.0 + x) / 2.0)
+        want = ((bd[4] ** 2 + bp ** 2) / 2 - (bm ** 2 + bd[3] ** 2) / 2) / 2
+        want -= eb * ((bd[4] + bp) / 2 - (bm + bd[3]) / 2) + (wq * (eta - eb) * slope).sum()
+        got = lib.t_special(_p(J), _d(eb), _p(eta), _p(bd), _d(bm), _d(bp))
+        assert abs(got - 2 * G * want) <= 1e-12 * 2 * G * (1.0 + np.abs(q).max()) * np.linalg.cond(A)

@@ -63,6 +63,7 @@ struct swale_ctx {
   // Whole steps in one launch (k_steps), for meshes of few blocks: the blocks, 0 if there are too many,
   // their work list (null: one instance) and the scratch of the instances.
   int step_blocks = 0;
+  const void* step_fn = nullptr;  // the instantiation for that many
   Tile* step_tiles = nullptr;
   StepScratch* step_scratch = nullptr;
   // Blocks of the adjoint's kernels, and their work list (null: one instance).
@@ -304,10 +305,23 @@ swale_status check_config(const swale_config* c, std::string& why) {
 
 bool valid_tile(int T) { return T == 64 || T == 128 || T == 256; }
 
+// The instantiation of k_steps for up to `per_sm` blocks on an SM. The fewer, the more registers and the fewer
+// spills: 16 steps of the smooth basin (profile motion) take, with room for 2, 4 and 5 blocks, and by the stage kernels,
+//   N = 200     826    860   1009  1077 us      N = 50000     -   1333   1422  1653 us
+//   N = 16300   677    718     -    993 us      N = 73000     -   1699   1783  2074 us
+//   N = 36000   967   1008     -   1373 us      N = 90000     -     -    2118  2240 us
+// (six blocks would have to share 80 registers a thread and the shared memory of five).
+const void* step_kernel(int scheme, int64_t per_sm) {
+  const bool nonwb = scheme == SWALE_SCHEME_NONWB;
+  if (per_sm <= 2) return nonwb ? (const void*)k_steps<1, 2> : (const void*)k_steps<0, 2>;
+  if (per_sm <= 4) return nonwb ? (const void*)k_steps<1, 4> : (const void*)k_steps<0, 4>;
+  return nonwb ? (const void*)k_steps<1, 5> : (const void*)k_steps<0, 5>;
+}
+
 // Blocks that k_steps would run for the instances: kept if the mesh is small enough for it (at most
 // kStepBlocksPerSM a SM, all of them resident). One block is 122 cells and one warp on each
 // sub-partition of an SM.
-constexpr int kStepBlocksPerSM = 1;
+constexpr int kStepBlocksPerSM = 5;
 swale_status build_step_blocks(swale_ctx* ctx, const std::vector<InstConst>& ic) {
   if (ctx->cfg.scheme == SWALE_SCHEME_SPECIAL || ctx->cfg.mesh == SWALE_MESH_FLUID_GAUSS) return SWALE_OK;
   int dev = 0, sms = 0, coop = 0, fit = 0;
@@ -317,9 +331,8 @@ swale_status build_step_blocks(swale_ctx* ctx, const std::vector<InstConst>& ic)
   for (const InstConst& c : ic) n += (c.N + kStepCells - 1) / kStepCells;
   if (n > (int64_t)sms * kStepBlocksPerSM) return SWALE_OK;
   SW_CUDA(ctx, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-  SW_CUDA(ctx, ctx->cfg.scheme == SWALE_SCHEME_NONWB
-                   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_steps<1>, kStepThreads, 0)
-                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k_steps<0>, kStepThreads, 0));
+  const void* f = step_kernel(ctx->cfg.scheme, (n + sms - 1) / sms);
+  SW_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, f, kStepThreads, 0));
   if (!coop || n > (int64_t)sms * fit) return SWALE_OK;
   if (swale_status s = dalloc(ctx, ctx->tile_allocs, &ctx->step_scratch, ic.size())) return s;
   if (ic.size() > 1) {
@@ -331,6 +344,7 @@ swale_status build_step_blocks(swale_ctx* ctx, const std::vector<InstConst>& ic)
                                  ctx->stream));
     SW_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   }
+  ctx->step_fn = f;
   ctx->step_blocks = (int)n;
   return SWALE_OK;
 }
@@ -560,14 +574,13 @@ constexpr int64_t kStepsPerLaunch = 4096;
 swale_status enqueue_whole_steps(swale_ctx* ctx, int64_t n) {
   StepConst K = step_const(ctx);
   int rel1 = stage1_wave_rel(ctx->cfg);
-  const void* f = ctx->cfg.scheme == SWALE_SCHEME_NONWB ? (const void*)k_steps<1> : (const void*)k_steps<0>;
   for (; n > 0; n -= kStepsPerLaunch) {
     NvtxRange r("swale whole steps");
     long long m = std::min(n, kStepsPerLaunch);
     const Tile* tiles = ctx->step_tiles;
     void* args[] = {&K, &ctx->D, &ctx->step_scratch, &tiles, &rel1, &m};
     SW_CUDA(ctx, cudaMemsetAsync(ctx->step_scratch, 0, ctx->B * sizeof(StepScratch), ctx->stream));
-    SW_CUDA(ctx, cudaLaunchCooperativeKernel(f, dim3((unsigned)ctx->step_blocks), dim3(kStepThreads), args, 0, ctx->stream));
+    SW_CUDA(ctx, cudaLaunchCooperativeKernel(ctx->step_fn, dim3((unsigned)ctx->step_blocks), dim3(kStepThreads), args, 0, ctx->stream));
   }
   return SWALE_OK;
 }

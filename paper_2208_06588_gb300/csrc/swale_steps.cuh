@@ -66,9 +66,10 @@ struct StepSink {
 // and meets the other blocks of the instance twice: after the wave speeds (alpha), and after the new
 // stage values. Bound by the chain of a warp's FP64 instructions (64 cycles each, whatever the
 // number of warps or lanes) and by the six barriers. One block per SM runs a warp on each
-// sub-partition; hydrostatic and non-well-balanced schemes, static, profile and linear motion.
-template <int SCHEME>
-__global__ void __launch_bounds__(kStepThreads, 2) k_steps(StepConst K, DevState D, StepScratch* scratch, const Tile* blocks,
+// sub-partition; hydrostatic and non-well-balanced schemes, static, profile and linear motion. PER_SM:
+// blocks that an SM holds (2: 255 registers; 4: 128, 5: 96, the rest spilled).
+template <int SCHEME, int PER_SM>
+__global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, DevState D, StepScratch* scratch, const Tile* blocks,
                                                            int wave_rel1, long long nsteps) {
   constexpr int T = kStepThreads;
   __shared__ double rE[T + 8], rM[T + 8], rJ[T + 8];

@@ -90,6 +90,19 @@ def test_largest_mesh_and_mixed_paths():
         assert np.array_equal(g[k], ref[k]), k
 
 
+@pytest.mark.parametrize("per_sm", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("scheme,mesh", [("hydrostatic", "profile"), ("nonwb", "static")])
+def test_blocks_per_multiprocessor(per_sm, scheme, mesh):
+    """The largest mesh of each number of blocks on an SM, one cell more (the next number, after the last
+    the stage kernels)."""
+    import torch
+    n = 122 * per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    for m in (n, n + 1):
+        p, cfg = problem(m, "periodic", mesh)
+        cfg["scheme"] = scheme
+        same(run(p, cfg, 3), run(p, cfg, 3, (64, 128, 0, 0)))
+
+
 def test_batch_of_small_instances_and_an_end_time():
     """Instances of uneven size in one launch, each to the end time with its own steps."""
     sizes = [5, 122, 123, 260, 31, 500]

@@ -1993,7 +1993,7 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   // Outputs that overlap an input (in place): every cell has to be read before the first is written.
   bool in_place = false;
   for (const double* r : {RE, RM, RB})
-    for (const double* q : {E, M, B, J, w}) in_place = in_place || (r < q + (N + 1) && q < r + N);
+    for (const double* q : {E, M, B, J, w}) in_place = in_place || (r < q + (q == w ? N + 1 : N) && q < r + N);
   const void* dev_ptrs[] = {E, M, B, J, w, RE, RM, RB};
   for (const void* p : dev_ptrs)
     if (!on_device(p)) return SWALE_EINVAL;
@@ -2026,8 +2026,9 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
     P.beta_dx_global = cfg->beta_dx_global;
     P.limit_hu = cfg->limit_hu;
     unsigned long long *mx = &scr->S.Jmax[0], *wv = A_out ? &scr->S.A[0] : nullptr;
-    // Up to this many cells every block finds the largest width itself: one launch instead of two.
-    constexpr int64_t kScanCells = 4096;
+    // Up to this many cells every block finds the largest width itself, one launch instead of two: a call
+    // takes 10.7 against 15.7 us at N = 200, 11.6 against 14.0 at 8192, but 16.2 against 13.7 at 16384.
+    constexpr int64_t kScanCells = 8192;
     const bool scan = N <= kScanCells && !A_out;
     if (!scan) launch(k_rhs_widths, 1, 1024, 0, st, J, (int32_t)N, mx, wv);
     const unsigned nb = (unsigned)((N + kStepCells - 1) / kStepCells);

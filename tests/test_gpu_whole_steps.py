@@ -125,7 +125,7 @@ def test_batch_of_small_instances_and_an_end_time():
     assert got[0]["n"] == got[1]["n"] and np.all(got[0]["t"] == 0.02)
 
 
-@pytest.mark.parametrize("n", [5, 6, 121, 122, 123, 1000, 4096, 4097, 20011])
+@pytest.mark.parametrize("n", [5, 6, 121, 122, 123, 1000, 4096, 8192, 8193, 20011])
 @pytest.mark.parametrize("scheme,bc", [("hydrostatic", "periodic"), ("nonwb", "reflective"), ("special", "transmissive")])
 def test_rhs_in_one_launch_equals_the_stage_kernels(n, scheme, bc):
     """swale_rhs_noalloc in one launch against its in-place form, which runs the stage kernels (every

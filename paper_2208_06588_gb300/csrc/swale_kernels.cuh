@@ -1295,7 +1295,8 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
     if (MODE == 1) {
       alpha = ro.alpha;
     } else {
-      alpha = (STAGE == 1) ? S->alpha1 : bitsd(S->A[STAGE - 1]) + (K.wave_rel ? 0.0 : S->Wbar);
+      alpha = (STAGE == 1) ? S->alpha1 : bitsd(S->A[STAGE - 1]);
+      if (STAGE > 1 && !K.wave_rel) alpha = swale::add_(alpha, S->Wbar);
       if (STAGE > 1) {
         // Replay of stages 2 and 3 (recorded below; stage 1 is handled where alpha1 is formed).
         if (K.alpha_mode == 2) alpha = stage_alpha(K, inst, STAGE, alpha, S->step_idx);
@@ -1443,7 +1444,8 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
         const int32_t g = (int32_t)cb + j;  // global cell index
         const double wl = wk, wr = sW[tid + 1];
         const double J0 = D.J0[g];
-        const double dJ = swale::mul_(dt, swale::sub_(wr, wl));
+        // The width's increment over the step (stage 2: half of it).
+        const double dJ = swale::mul_(STAGE == 2 ? swale::down_<1>(dt) : dt, swale::sub_(wr, wl));
         const double q0[3] = {D.E0[g], D.M0[g], D.B0[g]};
         if (STAGE == 1) {
           const double J1 = swale::add_(J0, dJ), J2 = swale::fma_(0.5, dJ, J0);
@@ -1459,7 +1461,7 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
           D.YE[g] = R2[0];
           D.YM[g] = R2[1];
           D.YB[g] = R2[2];
-          const double hdt = 0.5 * dt;
+          const double hdt = swale::down_<1>(dt);
           D.Ea[g] = swale::rk_advance(q0[0], hdt, R2[0], dJ, inv);
           D.Ma[g] = swale::rk_advance(q0[1], hdt, R2[1], dJ, inv);
           if (!BOT) D.Ba[g] = swale::rk_advance(q0[2], hdt, R2[2], dJ, inv);
@@ -1473,11 +1475,11 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
           double inv;
           if (still) inv = D.iJ2[g];
           else D.iJ2[g] = inv = swale::recip(D.J2[g]);
-          const double edt = 0.125 * dt, hdJ = 0.5 * dJ;
-          D.Eb[g] = swale::rk_advance(q0[0], edt, Y[0], hdJ, inv);
-          D.Mb[g] = swale::rk_advance(q0[1], edt, Y[1], hdJ, inv);
+          const double edt = swale::down_<3>(dt);
+          D.Eb[g] = swale::rk_advance(q0[0], edt, Y[0], dJ, inv);
+          D.Mb[g] = swale::rk_advance(q0[1], edt, Y[1], dJ, inv);
           if (!BOT) {
-            D.Bb[g] = swale::rk_advance(q0[2], edt, Y[2], hdJ, inv);
+            D.Bb[g] = swale::rk_advance(q0[2], edt, Y[2], dJ, inv);
           } else {  // bottom of stage 3: projection onto the mesh at t_{n+1/2}
             const double xl = D.x[nb + j], xr = D.x[nb + j + 1];
             D.Bb[g] = bottom_average(K, xl + 0.5 * dt * wl, xr + 0.5 * dt * wr);

@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
         sW[tid] = w;
         alpha = sd.alpha1;
       } else {
-        alpha = A + (K.wave_rel ? 0.0 : Wbar);
+        alpha = A;
+        if (!K.wave_rel) alpha = swale::add_(A, Wbar);
       }
       const double dt = sd.dt;
       // Left interface of the cell: its left state is the right edge of cell c - 1.
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
           if (!swale::gt0(J1) || !swale::gt0(J2)) st |= swale::ST_EMESH;
           iJ1 = moving ? swale::recip(J1) : iv;
           iJs = iJ1;
-          const double hdt = 0.5 * dt;
+          const double hdt = swale::down_<1>(dt);
 #pragma unroll
           for (int v = 0; v < 3; ++v) {
             Y[v] = R2[v];
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
         } else if (stage == 2) {
           Js = swale::fma_(0.5, dJ, J0);
           iJs = moving ? swale::recip(Js) : iv;
-          const double edt = 0.125 * dt, hdJ = 0.5 * dJ;
+          const double edt = swale::down_<3>(dt), hdJ = 0.5 * dJ;
 #pragma unroll
           for (int v = 0; v < 3; ++v) {
             Y[v] = swale::add_(Y[v], R2[v]);

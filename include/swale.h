@@ -145,8 +145,10 @@ swale_status swale_batch_set_problem(swale_ctx* ctx, int64_t B, const int64_t* o
  * status of the step itself is read with swale_get_status (or reported by swale_advance). */
 swale_status swale_step(swale_ctx* ctx, double* dt_out);
 
-/* Up to max_steps steps, replayed as CUDA graphs of fixed length; stops early at t_end (with
- * an end time the steps go out in chunks of 64 to 4096 steps, and the call returns once every
+/* Up to max_steps steps, replayed as CUDA graphs of fixed length, or, for meshes of up to five blocks of 122
+ * cells per multiprocessor (about 93 thousand cells; hydrostatic and non-well-balanced schemes, prescribed or no
+ * motion, evolved bottom, default launch shape, no viscosity log), as launches of many whole steps; stops early
+ * at t_end (with an end time the steps go out in chunks of 64 to 4096 steps, and the call returns once every
  * instance has reached t_end or stopped on an error). Synchronises at the end and reports the
  * steps actually taken in *steps_done (may be NULL).
  * Error contract: a step in which an error appears (a non-finite value, a non-positive width, a
@@ -186,7 +188,8 @@ swale_status swale_batch_get_state(swale_ctx* ctx, double* hu, double* b, double
  * cells, a forward update tile one cell fewer, so that its interfaces take one pass) of the
  * reconstruction and update kernels and their grid (0 = one block per tile; G > 0 = a persistent grid of G blocks
  * walking the (instance, tile) work list). tiles[4] = {recon_tile, update_tile, recon_grid,
- * update_grid}. Results do not depend on the launch shape (bitwise). */
+ * update_grid}. Results do not depend on the launch shape (bitwise). Any shape but the default {128, 128, 0, 0} keeps
+ * small meshes on these kernels (see swale_advance). */
 swale_status swale_set_tiles(swale_ctx* ctx, int32_t recon_tile, int32_t update_tile, int32_t recon_grid,
                              int32_t update_grid);
 swale_status swale_get_tiles(swale_ctx* ctx, int32_t* tiles);
@@ -235,7 +238,9 @@ swale_status swale_rhs(swale_ctx* ctx, int64_t N, const double* E, const double*
  *                      cfg->alpha_bound); when given, the call synchronises the stream,
  *                      otherwise it returns after enqueueing
  *   flags              N bytes (host or device) or NULL: detector classes
- * Scratch lives in one fixed array of about 6.3 MB per device, held from library load until
+ * The result comes in one launch (two above 8192 cells or with A_out), which reads neighbouring cells
+ * while others are written; outputs that overlap an input take the stage kernels, which read every cell first.
+ * Scratch lives in one fixed array of about 7.9 MB per device, held from library load until
  * the process exits; the call allocates nothing and clears what it reuses. Every call shares
  * that array, so calls that overlap on the GPU (other streams, other host threads) race; run
  * them one after the other. The first call on a device looks up the array's device address;
@@ -252,8 +257,8 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
  * recursion, nodes, motion profile, per-instance scalars such as t and the step count, and
  * the L2-projection bottom if set) to a versioned binary file; swale_load reads such a file
  * into a context created with the same configuration (bitwise equal swale_config) and
- * replaces its problem. A resumed run recomputes the first step's mesh geometry from the
- * stored widths, so it agrees with the uninterrupted run to rounding. Host byte order.
+ * replaces its problem. A resumed run forms the first step's width reciprocals from the stored
+ * widths, where the uninterrupted run may have them cached: the same values. Host byte order.
  * Errors: SWALE_EINVAL (no problem, file not readable / writable, wrong format, version or
  * configuration), SWALE_ENOMEM, SWALE_ECUDA. */
 swale_status swale_save(swale_ctx* ctx, const char* path);
@@ -289,15 +294,15 @@ swale_status swale_get_alpha_log(swale_ctx* ctx, double* log);
  * viscosities alpha are those of the forward run, detector classes, limiter branches, dry-edge
  * tests and max/min selections are frozen (a tie follows the first argument); if a replay log
  * is active (swale_alpha_log mode 2) the forward run replays it instead. Checkpoints of
- * the state every ckpt_every steps; each segment but the last is recomputed once with per-step
+ * the state every ckpt_every steps; each segment but the last two is recomputed once with per-step
  * snapshots (by a further set of state arrays on a low-priority stream, one segment ahead of the
- * reverse sweep; the forward run keeps the last segment's snapshots, and in tape mode its stage
- * data, itself) and each step once more before its reverse sweep (on a third stream, alternating
+ * reverse sweep; the forward run keeps the last two segments' snapshots, and in tape mode their
+ * stage data, itself) and each step once more before its reverse sweep (on a third stream, alternating
  * between the context's arrays and one more set, one step ahead of the reverse sweep, which
- * runs on the context's stream). These forward runs compute the mesh geometry in every stage
- * (no reuse of the previous step's), so the trajectory, and the gradient up to the order of
- * atomic additions, does not depend on ckpt_every. Device memory beyond the context's own: about
- * 5 (ceil(nsteps/C) + b C + 3) + 117 doubles per cell with C = min(ckpt_every, nsteps) and b = 2
+ * runs on the context's stream, one gather kernel per stage). Cached reciprocals of widths equal those formed
+ * again, so the trajectory, and the gradient up to the order of the misfit's atomic additions (its
+ * only ones), does not depend on ckpt_every. Device memory beyond the context's own: about
+ * 5 (ceil(nsteps/C) + b C + 3) + 201 doubles per cell with C = min(ckpt_every, nsteps) and b = 2
  * segment buffers (1 when C = nsteps), taken as one block of exactly swale_adjoint_bytes bytes
  * (a single cudaMalloc); the block and the two streams are freed before the call returns. With ckpt_every >= nsteps every step runs
  * twice (once in tape mode). The mesh must be prescribed (static, profile or linear motion) and
@@ -309,7 +314,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
 /* Device bytes swale_adjoint allocates for B instances with Ntot cells in total, without
  * (tape = 0) or with (tape = 1) the tape of swale_set_adjoint_tape (host-only arithmetic; needs
  * no device). Lets a caller pick ckpt_every for the memory it has: the checkpoints grow as
- * nsteps / ckpt_every, the per-segment snapshots (and the tape: about 39 doubles per cell and
+ * nsteps / ckpt_every, the per-segment snapshots (and the tape: about 81 doubles per cell and
  * step, for two segments, one when ckpt_every >= nsteps) as ckpt_every.
  * Errors: SWALE_EINVAL (a size < 1, tape not 0 or 1, or a NULL bytes pointer). */
 swale_status swale_adjoint_bytes(int64_t B, int64_t Ntot, int64_t nsteps, int64_t ckpt_every, int32_t G,
@@ -318,10 +323,10 @@ swale_status swale_adjoint_bytes(int64_t B, int64_t Ntot, int64_t nsteps, int64_
 /* How swale_adjoint gets each step's stage data (the edge values of the three stages, q^(1),
  * q^(2) and their widths) for the reverse sweep. enable = 0 (the default): each step is
  * recomputed from its snapshot before its reverse sweep, so every step is run three times (twice
- * in the last segment). enable = 1: the recompute of a segment (for the last segment, the
- * forward run) keeps every step's stage data (a tape of about 39 doubles per cell and step, for
+ * in the last two segments). enable = 1: the recompute of a segment (for the last two, the
+ * forward run) keeps every step's stage data (a tape of about 81 doubles per cell and step, for
  * two segments), and the reverse sweep reads it: every step is run twice (once in the last
- * segment: with ckpt_every >= nsteps the forward run is the only one). The gradient is the same
+ * two segments: with ckpt_every >= nsteps / 2 the forward run is the only one). The gradient is the same
  * up to the order of atomic additions. This
  * is a trade of memory for arithmetic that the paper does not discuss (it has no adjoint).
  * Errors: SWALE_EINVAL. */
@@ -334,7 +339,7 @@ swale_status swale_set_adjoint_tape(swale_ctx* ctx, int32_t enable);
  * kernel then sets SWALE_BIT_TIMEOUT and returns, the step is not committed and reports
  * SWALE_ETIMEOUT, and the context stays usable (reset the hook with 0, 0; the instance keeps the
  * state of its last good step, a new problem clears the status). A block never returns while a
- * copy of its own may still write its shared memory. Nothing faults or hangs.
+ * copy of its own may still write its shared memory. Nothing faults or hangs. (Small meshes take the stage kernels meanwhile.)
  * Errors: SWALE_EINVAL, SWALE_ECUDA. */
 swale_status swale_set_wait_test(swale_ctx* ctx, int32_t tries, uint32_t pad_bytes);
 

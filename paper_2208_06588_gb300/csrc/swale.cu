@@ -135,7 +135,6 @@ StepConst step_const(const swale_ctx* ctx) {
   K.dt_fixed = ctx->cfg.dt_fixed;
   K.mesh_T = ctx->cfg.mesh_T;
   K.inv_T = 1.0 / ctx->cfg.mesh_T;
-  K.gauss_wsum = ctx->gauss_wsum;
   K.gauss_iwsum = 1.0 / ctx->gauss_wsum;
   K.bc = ctx->cfg.bc;
   K.mesh = ctx->cfg.mesh;
@@ -2079,7 +2078,6 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   K.t_end = 0.0;
   K.dt_fixed = 0.0;
   K.mesh_T = K.inv_T = 1.0;
-  K.gauss_wsum = 1.0;
   K.gauss_iwsum = 1.0;
   K.bc = cfg->bc;
   K.mesh = SWALE_MESH_STATIC;

@@ -8,6 +8,8 @@
 //   k_recon<2>, k_update<2>    stage 2 on the mesh at t_{n+1}
 //   k_recon<3>, k_update<3>    stage 3 on the mesh at t_{n+1/2}
 //   k_commit                   the step's time and step count, or its roll-back after an error
+// (A mesh of few blocks runs whole steps in one launch instead: k_steps in swale_steps.cuh. Between steps of one
+// sequence k_commit does the next step's prologue as well.)
 // Every launch serves all instances of a batch: blocks walk a work list of (instance, tile)
 // entries in grid-stride order (one pass when the grid has one block per tile, a persistent
 // loop when it is smaller). A single instance uses the implicit list t -> (0, t * T + first).
@@ -31,13 +33,12 @@
 
 namespace swale_dev {
 
-static_assert(sizeof(swale::SourceForm) == 6 * sizeof(double), "SourceForm holds 6 doubles");
-
 using swale::EdgeState;
 using swale::SchemeConst;
 
 constexpr int kMaxGaussHalf = 64;
-// Resident threads per SM that the launch bounds of the stage kernels ask for.
+// Resident threads per SM that the launch bounds of the stage kernels ask for (72 registers a thread; 640 to
+// 1024 threads are within 1 %).
 constexpr int kReconThreads = 896, kUpdateThreads = 896;
 constexpr int kMeshThreads = 256;
 constexpr int kMeshNodes = kMeshThreads - 1;  // nodes a mesh-velocity tile advances by
@@ -84,8 +85,7 @@ struct Tile {
 struct StepConst {
   SchemeConst sc;
   double t_end, dt_fixed, mesh_T, inv_T;
-  double gauss_wsum;  // sum of the full Gaussian window, summed from -H to H
-  double gauss_iwsum; // its reciprocal
+  double gauss_iwsum;  // reciprocal of the full Gaussian window's sum (from -H to H)
   int32_t bc, mesh, gauss_half, B;
   // Stage viscosities: log of 3 values per step and instance (index (step * B + i) * 3 + s - 1);
   // alpha_mode 1 records the computed values, 2 replays the logged ones (the adjoint's and the
@@ -281,7 +281,6 @@ __device__ __forceinline__ unsigned long long warp_umax64(unsigned long long v) 
   const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
   return ((unsigned long long)hi << 32) | lo;
 }
-__device__ __forceinline__ unsigned long long warp_umin64(unsigned long long v) { return ~warp_umax64(~v); }
 
 // Raises *dst to v unless it is there already (most callers find that it is).
 __device__ __forceinline__ void raise_to(unsigned long long* dst, unsigned long long v) {
@@ -464,7 +463,8 @@ __global__ void k_prologue(StepConst K, DevState D) {
 // them), the weights exp(-m^2 / 2 sigma^2) are 57-bit ones, both in two limbs of 28 bits, and the sums
 // are exact: the result is within (2 H + 1) 2^-57 of the largest raw velocity of the exact sum of
 // the rounded inputs, where the FP64 sum's bound is about 20 x 2^-53 of it. Measured against 64-bit
-// references the step's error is unchanged; the kernel needs 12 FP64 instructions per node instead of 61.
+// references the step's error is unchanged; the kernel needs 12 FP64 instructions per node instead of 61 and
+// 39 us at 2^20 cells instead of 118.
 // Nodes whose window is cut off by an end, and tiles whose largest velocity is beyond 2^900, below 2^-967
 // or a NaN, take the FP64 sum.
 // The block stages the cell velocities and the raw node velocities in shared memory (dynamic, and
@@ -588,7 +588,12 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
 // entries of each phase to a second pass of one warp). It stores the edge states, the pair / triple reciprocals and
 // pair differences that the update kernel of the same stage reads, reduces the wave speed, and in
 // stage 1 the instance's last tile computes its dt (and the secant factor of the prescribed motion).
-// What bounds it: FP64 instructions, each of which holds its SM sub-partition for 64 cycles.
+// What bounds it: FP64 instructions, each of which holds its SM sub-partition for 64 cycles, and beside them
+// about 1000 others at 0.5-1 cycle. Per cell it issues 81 / 85 / 85 of them in stages 1 / 2 / 3 (83 / 151 / 149 when the
+// mesh geometry was formed per cell and cached in 28 arrays); at 2^20 cells a launch takes 170 / 172 / 170 us
+// (182 / 301 / 293) with the FP64 pipe 83-86 % busy and DRAM at 9-13 %, at 131071 cells 35 us at 65-71 %, where the
+// loads and the drain of the one wave of blocks are a seventh of the time. The cells come by bulk copies: plain loads
+// make a step of 2^20 cells 1.3 % slower.
 // ------------------------------------------------------------------------------------
 // Shared-memory rows of a tile that the out-of-line path of an open cell reads (row i: cell, pair,
 // triple starting at cell c0 - 2 + i).
@@ -1243,10 +1248,6 @@ struct RhsOut {
   double alpha;
 };
 
-// SCHEME: 0 hydrostatic, 1 non-well-balanced, 2 special source. BOT: an instantiation with the
-// L2-projection bottom. STOREK: one that also stores the source's ratios in D.gK (the adjoint's
-// recomputes).
-
 // Largest a and b over the block (non-negative doubles), raised into mx[0], mx[1], and the smallest c,
 // lowered into *mn (or, with COMPL, its complement raised there), by three lanes after one barrier.
 template <int T, bool COMPL>
@@ -1266,6 +1267,15 @@ __device__ __forceinline__ void block_widths(unsigned long long* mx, unsigned lo
   }
 }
 
+// Update of stage STAGE (MODE 0) or the right-hand side for a given viscosity (MODE 1): blocks of T threads take
+// T - 1 cells, so that their T interfaces are one pass, one flux each, shared with the right neighbour through
+// shared memory; then the source joined with the edge pressures, and the RK combination as an increment of q^n.
+// Bound by FP64 instructions: 73 / 91 / 92 a cell in stages 1 / 2 / 3 (95 / 132 / 142 with the source as a bilinear
+// form with six mesh-only entries and J q combined), 148 / 186 / 189 us at 2^20 cells (190 / 263 / 285), the FP64
+// pipe 87 % busy, DRAM at 20 %. Launch bound as the reconstruction's.
+// SCHEME: 0 hydrostatic, 1 non-well-balanced, 2 special source. BOT: an instantiation with the
+// L2-projection bottom. STOREK: one that also stores the source's ratios in D.gK (the adjoint's
+// recomputes).
 template <int STAGE, int MODE, int T, int SCHEME = 0, bool BOT = false, bool STOREK = false>
 __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, DevState D, const double* __restrict__ Eg,
                                               const double* __restrict__ Mg, const double* __restrict__ Bg,

@@ -65,7 +65,10 @@ struct StepSink {
 // from its neighbours (through L2), reconstructs one of them, so that the fluxes need no exchange,
 // and meets the other blocks of the instance twice: after the wave speeds (alpha), and after the new
 // stage values. Bound by the chain of a warp's FP64 instructions (64 cycles each, whatever the
-// number of warps or lanes) and by the six barriers. One block per SM runs a warp on each
+// number of warps or lanes: about 170 a stage, 67 more where cells are open) and by
+// the six barriers (one to two microseconds each with several blocks). 16 steps at N = 200 take 820 us (1599 by
+// the stage kernels at first, 1077 by today's), at 16300 cells 854 (1554, 993); an accuracy run of N = 50 to
+// t = 0.1 35 ms (79). One block per SM runs a warp on each
 // sub-partition; hydrostatic and non-well-balanced schemes, static, profile and linear motion. PER_SM:
 // blocks that an SM holds (2: 255 registers; 4: 128, 5: 96, the rest spilled).
 template <int SCHEME, int PER_SM>
@@ -399,7 +402,9 @@ __global__ void __launch_bounds__(1024) k_rhs_widths(const double* __restrict__ 
 // One right-hand side for a given viscosity in one launch: alpha is known, so the fluxes need no grid-wide
 // maximum between them and the reconstruction, and the edge values stay on the chip (a block owns 122
 // cells and reconstructs one more on each side, as in k_steps). dxmax: the largest width, or null: every block
-// scans the N widths (cheaper than a launch of its own up to a few thousand cells). wave: where the largest
+// scans the N widths (cheaper than a launch of its own up to 8192 cells). Bound by the chain of a warp's 139 FP64
+// instructions (64 cycles each, 4.3 us) and the loads before it: 11.6 us a call at N = 200 (30.7 as stage kernels with
+// their launches), 27 at 65536 (59), where FP64 throughput is the bound. wave: where the largest
 // edge speed goes (null: not wanted), relative to w if wave_rel.
 template <int SCHEME>
 __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, int wave_rel, int32_t N, double alpha,

@@ -31,23 +31,21 @@ METRIC = "cell-updates/s FP64 (fwd, plain single instance)"
 UNIT = "cell-updates/s"
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12  # SMs x DFMA/clk x 2 flop x max SM clock
 # DRAM bytes (read + write) of a k_recon launch on this workload, averaged over the three
-# stages, from one ncu capture of the current kernels (the autotuner's pick on that box: 256-cell
-# reconstruction tiles, staged by bulk copies): stage 1 reads the smooth-class form of the
-# cached mesh geometry, 8 values per cell, and the rest only where the FP32 test leaves the class
-# open (109.2 + 46.6 MB), stage 2 writes the geometry (42.1 + 272.6 MB), stage 3 does neither
-# (42.0 + 27.8 MB).
-RECON_DRAM_BYTES = (109_205_760 + 46_568_192 + 42_138_112 + 272_582_144 + 42_033_152 + 27_768_832) // 3
+# stages, from one ncu capture of the current kernels (128-cell tiles, staged by bulk copies): stage 1
+# reads the cached reciprocals of the widths, 4 values per cell (75.6 + 70.6 MB), stage 2 writes them
+# (42.5 + 136.6 MB), stage 3 does neither (42.0 + 75.1 MB).
+RECON_DRAM_BYTES = (75_617_280 + 70_609_920 + 42_510_848 + 136_626_176 + 42_032_640 + 75_084_800) // 3
 # Fraction of cycles the FP64 pipe was busy during the same k_recon launches (ncu
 # sm__pipe_fp64_cycles_active, the three stages): the kernel is bound by FP64 instruction issue.
-RECON_FP64_PIPE_ACTIVE = (0.8237 + 0.8566 + 0.8647) / 3
+RECON_FP64_PIPE_ACTIVE = (0.8253 + 0.8498 + 0.8584) / 3
 # FP64 FLOP equivalents per cell the same launches executed (ncu dadd + dmul + 2 dfma
 # instructions over the 2^20 cells; stages 1, 2, 3): what the hardware did, beside the method's
-# and the kernels' own counts.
-RECON_EXECUTED_FLOPS = (120.9 + 204.1 + 200.4) / 3
+# count and that of the closed-form per-cell functions.
+RECON_EXECUTED_FLOPS = (95.8 + 123.4 + 123.4) / 3
 # The source term's mesh-only part in the method figures: the interpolant's width ratios in
 # closed form (6 products and the cell's reciprocal width), as the paper's construction needs
-# them. The kernels spend more there (the six entries of the antisymmetric source form, counted
-# in their own figures) to spend less on the state arithmetic.
+# them. The closed-form per-cell functions spend more there (the six entries of the antisymmetric
+# source form, counted in their own figures) to spend less on the state arithmetic.
 METHOD_SOURCE_GEOM_FLOPS = 7.0
 # The method's FP64 operations per cell, counted by the CPU oracle on an operation-counting
 # scalar type (oracle.count_step; tests/test_bench_contract.py recounts them): the arithmetic on
@@ -62,12 +60,12 @@ ORACLE_STEP_FLOPS = 1891.80
 ORACLE_BATCH_STEP_FLOPS = 1893.17
 # The same counts for the scheme variants on the dam-break workload (reconstruction, step).
 ORACLE_VARIANT_FLOPS = {"nonwb": (583.01, 2613.02), "special": (366.61, 1780.82)}
-# DRAM bytes per k_update launch (stages 1, 2, 3: 159.4 + 40.5, 184.7 + 65.4, 184.8 + 47.7 MB), the
+# DRAM bytes per k_update launch (stages 1, 2, 3: 193.0 + 47.5, 201.4 + 82.7, 226.5 + 56.4 MB), the
 # fraction of cycles its FP64 pipe was busy and the FP64 FLOP equivalents per cell it executed
 # (ncu, the same capture as for k_recon above; 128-thread update blocks, 127-cell tiles).
-UPDATE_DRAM_BYTES = (159_437_312 + 40_500_224 + 184_734_208 + 65_380_096 + 184_763_136 + 47_675_392) // 3
-UPDATE_FP64_PIPE_ACTIVE = (0.8549 + 0.8577 + 0.8529) / 3
-UPDATE_EXECUTED_FLOPS = (128.4 + 183.5 + 195.5) / 3
+UPDATE_DRAM_BYTES = (192_998_656 + 47_543_040 + 201_380_352 + 82_679_808 + 226_542_848 + 56_431_360) // 3
+UPDATE_FP64_PIPE_ACTIVE = (0.8680 + 0.8670 + 0.8604) / 3
+UPDATE_EXECUTED_FLOPS = (106.2 + 124.3 + 127.3) / 3
 
 
 def parse():
@@ -161,7 +159,7 @@ def config_of(pr):
 
 def op_counts(pr):
     """FP64 operations per cell of the reconstruction and update kernels, counted by running the
-    kernels' own per-cell code (swale_cell.cuh) on a host counting type over a sample of cells."""
+    closed-form per-cell code (swale_cell.cuh) on a host counting type over a sample of cells."""
     from paper_2208_06588_gb300 import opcount
     return opcount.count_stage(pr.E, pr.hu, pr.b, pr.J, bc=pr.bc, sample=1 << 16)
 
@@ -170,7 +168,7 @@ def fp64_roofline(flops_per_cell_step, cell_steps_per_s, scope, basis="kernel co
     """Whole-job FP64 roofline: FLOPs of a cell-step times the measured cell-steps per second,
     against the FP64 peak. Every kernel of the step is FP64-pipe bound (DRAM below 16 %), so this
     is the slower of the two rooflines. basis: "method" (the oracle's count, see
-    ORACLE_STEP_FLOPS) or "kernel count" (the kernels' own per-cell code counted on the host);
+    ORACLE_STEP_FLOPS) or "kernel count" (the closed-form per-cell code counted on the host; the kernels need less);
     with kernel_flops given, the kernel-count fraction is reported beside the method's."""
     achieved = flops_per_cell_step * cell_steps_per_s / 1e12
     out = {"bound": "alu", "scope": scope, "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",

@@ -1,6 +1,8 @@
-// Host-only count of the FP64 arithmetic that the stage kernels perform per cell, obtained by
-// compiling the same per-cell code (swale_cell.cuh, and the reverse sweeps of swale_adjoint.cuh)
-// with an operation-counting scalar type.
+// Host-only count of the FP64 arithmetic of the closed-form per-cell functions (recon_cell, source_form
+// and the rest of swale_cell.cuh, and the reverse sweeps of swale_adjoint.cuh), compiled with an
+// operation-counting scalar type. The stage kernels evaluate forms that need less (divided differences
+// shared between cells, the factored source, increments), so this is an upper figure for them;
+// what they execute is measured.
 // Additions/subtractions, multiplications, divisions and square roots are counted
 // separately (a fused multiply-add on the device is one multiplication plus one addition
 // here); comparisons, min/max and sign flips are counted apart (they do not use the FP64

@@ -1,6 +1,6 @@
 """FP64 operation counts per cell of the stage kernels (roofline numerator).
 
-Builds csrc/opcount.cpp with g++: the kernels' own per-cell code (swale_cell.cuh) compiled
+Builds csrc/opcount.cpp with g++: the closed-form per-cell code (swale_cell.cuh) compiled
 on the host with an operation-counting scalar type. A fused multiply-add counts as two
 operations (one multiplication, one addition); a division or a square root counts as one.
 """

@@ -450,12 +450,53 @@ void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t shm, cud
   cudaLaunchKernelEx(&cfg, kernel, P(a)...);
 }
 
+// The same for a kernel known here: with the preferred split of an SM's memory (80 % shared) set once. Kernels
+// of different splits cannot share an SM, so each would wait for the last block of the one before it there: at
+// the defaults a gradient at 65536 cells takes 2 % longer (all of it shared costs the large runs 1 %).
+template <auto Kernel>
+const cudaFuncAttributes& kernel_attributes() {
+  static const cudaFuncAttributes at = [] {
+    cudaFuncAttributes a = {};
+    if (cudaFuncSetAttribute((const void*)Kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 80) != cudaSuccess ||
+        cudaFuncGetAttributes(&a, (const void*)Kernel) != cudaSuccess)
+      cudaGetLastError();
+    return a;
+  }();
+  return at;
+}
+template <auto Kernel, class... A>
+void launch(unsigned grid, unsigned block, size_t shm, cudaStream_t s, const A&... a) {
+  kernel_attributes<Kernel>();
+  launch(Kernel, grid, block, shm, s, a...);
+}
+
+// Dynamic shared memory, unused, that makes a grid of few blocks spread evenly: room for ceil(grid / SMs)
+// blocks on an SM and no more, where that is 4 to 6. A kernel's first blocks are placed while the last of the one before
+// drain, and the SMs that come free first would get more than their share. With the split above, 8 steps of 36000 cells on the
+// fluid-driven mesh take 792 us instead of 829, of 30000 cells of the special scheme 672 instead of 702, a gradient at
+// 65536 cells 21.6 ms instead of 22.8; grids of seven blocks an SM and more are not limited and not changed. (The
+// reconstruction, limited as well, gains nothing more.)
+template <auto Kernel>
+size_t even_smem(unsigned grid) {
+  constexpr size_t kSmSharedBytes = 228 * 1024;
+  static const unsigned sms = [] {
+    int dev = 0, n = 152;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      cudaGetLastError();
+    return (unsigned)n;
+  }();
+  const size_t fixed = kernel_attributes<Kernel>().sharedSizeBytes + 1024;  // (what the system takes a block)
+  const unsigned per = std::max(4u, (grid + sms - 1) / sms);
+  const size_t want = kSmSharedBytes / (per + 1) + 256;
+  return per < 7 && want > fixed ? want - fixed : 0;
+}
+
 template <int STAGE, int SCHEME, bool STOREK, bool CACHE>
 void launch_recon_as(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                      const double* M, const double* B, const double* J) {
-  if (T == 64) launch(k_recon<STAGE, 64, SCHEME, STOREK, CACHE>, grid, 64, 0, s, K, D, E, M, B, J);
-  else if (T == 256) launch(k_recon<STAGE, 256, SCHEME, STOREK, CACHE>, grid, 256, 0, s, K, D, E, M, B, J);
-  else launch(k_recon<STAGE, 128, SCHEME, STOREK, CACHE>, grid, 128, 0, s, K, D, E, M, B, J);
+  if (T == 64) launch<k_recon<STAGE, 64, SCHEME, STOREK, CACHE>>(grid, 64, 0, s, K, D, E, M, B, J);
+  else if (T == 256) launch<k_recon<STAGE, 256, SCHEME, STOREK, CACHE>>(grid, 256, 0, s, K, D, E, M, B, J);
+  else launch<k_recon<STAGE, 128, SCHEME, STOREK, CACHE>>(grid, 128, 0, s, K, D, E, M, B, J);
 }
 
 template <int STAGE, int SCHEME>
@@ -480,9 +521,9 @@ void launch_recon(const StepConst& K, const DevState& D, int T, unsigned grid, c
 template <int STAGE, int MODE, int SCHEME, bool BOT, bool STOREK>
 void launch_update_as(const StepConst& K, const DevState& D, int T, unsigned grid, cudaStream_t s, const double* E,
                       const double* M, const double* B, const double* J, const RhsOut& ro) {
-  if (T == 64) launch(k_update<STAGE, MODE, 64, SCHEME, BOT, STOREK>, grid, 64, 0, s, K, D, E, M, B, J, ro);
-  else if (T == 256) launch(k_update<STAGE, MODE, 256, SCHEME, BOT, STOREK>, grid, 256, 0, s, K, D, E, M, B, J, ro);
-  else launch(k_update<STAGE, MODE, 128, SCHEME, BOT, STOREK>, grid, 128, 0, s, K, D, E, M, B, J, ro);
+  if (T == 64) launch<k_update<STAGE, MODE, 64, SCHEME, BOT, STOREK>>(grid, 64, 0, s, K, D, E, M, B, J, ro);
+  else if (T == 256) launch<k_update<STAGE, MODE, 256, SCHEME, BOT, STOREK>>(grid, 256, 0, s, K, D, E, M, B, J, ro);
+  else launch<k_update<STAGE, MODE, 128, SCHEME, BOT, STOREK>>(grid, 128, even_smem<k_update<STAGE, MODE, 128, SCHEME, BOT, STOREK>>(grid), s, K, D, E, M, B, J, ro);
 }
 
 template <int STAGE, int MODE, int SCHEME>
@@ -529,10 +570,10 @@ swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, 
   auto L = [&](int fam, auto&& f) {
     if (st == SWALE_OK) st = timed_launch(ctx, fam, f);
   };
-  if (first) L(FAM_PROLOGUE, [&] { launch(k_prologue, (unsigned)((ctx->B + 127) / 128), 128, 0, s, K, D); });
+  if (first) L(FAM_PROLOGUE, [&] { launch<k_prologue>((unsigned)((ctx->B + 127) / 128), 128, 0, s, K, D); });
   if (K.mesh == SWALE_MESH_FLUID_GAUSS) {
     const size_t shm = (size_t)(3 * kMeshThreads + 4 * K.gauss_half + 4) * sizeof(double);
-    L(FAM_MESH, [&] { launch(k_mesh_gauss, (unsigned)std::max(D.nm, 1), kMeshThreads, shm, s, K, D); });
+    L(FAM_MESH, [&] { launch<k_mesh_gauss>((unsigned)std::max(D.nm, 1), kMeshThreads, shm, s, K, D); });
   }
   StepConst K1 = K;
   K1.wave_rel = stage1_wave_rel(ctx->cfg);
@@ -542,7 +583,7 @@ swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, 
   L(FAM_UPDATE, [&] { launch_update<2, 0>(K, D2, Tu, gu, s, D.Ea, D.Ma, D.Ba, D.J1, none); });
   L(FAM_RECON, [&] { launch_recon<3>(K, D3, Tr, gr, s, D.Eb, D.Mb, D.Bb, D.J2); });
   L(FAM_UPDATE, [&] { launch_update<3, 0>(K, D3, Tu, gu, s, D.Eb, D.Mb, D.Bb, D.J2, none); });
-  L(FAM_PROLOGUE, [&] { launch(k_commit, (unsigned)std::min<int64_t>(ctx->B, 1024), 256, 0, s, K, D, next ? 1 : 0); });
+  L(FAM_PROLOGUE, [&] { launch<k_commit>((unsigned)std::min<int64_t>(ctx->B, 1024), 256, 0, s, K, D, next ? 1 : 0); });
   if (st) return st;
   SW_CUDA(ctx, cudaGetLastError());
   return SWALE_OK;
@@ -1373,7 +1414,7 @@ long long device_steps(swale_ctx* ctx) {
 template <int STAGE>
 void launch_adj_stage(swale_ctx* ctx, const DevState& D, const StepConst& K, const AdjState& A, const double* E,
                       const double* M, const double* B, const double* J) {
-  launch(k_adj_stage<STAGE>, (unsigned)ctx->adj_blocks, kAdjThreads, 0, ctx->stream, K, D, A, E, M, B, J);
+  launch<k_adj_stage<STAGE>>((unsigned)ctx->adj_blocks, kAdjThreads, 0, ctx->stream, K, D, A, E, M, B, J);
 }
 
 // Copies of the evolving state (q^n, J^n, nodes, per-instance scalars).
@@ -1689,7 +1730,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   DevState& D = ctx->D;
   const unsigned copy_grid = (unsigned)std::min<int64_t>((NN + 255) / 256, 152 * 8);
   auto copy = [&](const StateArrays& to, const StateArrays& from, cudaStream_t q) {
-    launch(k_copy_state, copy_grid, 256, 0, q, to, from, Nt, NN, B * (int64_t)(sizeof(DevScalars) / 8));
+    launch<k_copy_state>(copy_grid, 256, 0, q, to, from, Nt, NN, B * (int64_t)(sizeof(DevScalars) / 8));
     return cudaGetLastError();
   };
   auto arrays = [](const DevState& X) { return StateArrays{X.E0, X.M0, X.B0, X.J0, X.x, X.S}; };
@@ -1776,7 +1817,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
     } else {
       s = enqueue_step_on(ctx, fwd, st, nullptr, ctx->geo_epoch);
     }
-    if (!s) launch(k_misfit<0>, gg, 128, 0, st, D, (double*)nullptr, (double*)nullptr, (int32_t)B, G, gx, obs + n * B * G, Jacc, gcell);
+    if (!s) launch<k_misfit<0>>(gg, 128, 0, st, D, (double*)nullptr, (double*)nullptr, (int32_t)B, G, gx, obs + n * B * G, Jacc, gcell);
   }
   if (!s && !e) e = save(fin);
   if (!s && !e) e = cudaGetLastError();
@@ -1812,7 +1853,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   // it), c the state before it.
   auto reverse_step = [&](const DevState* X3, int64_t m, const StateCopy& c) {
     double** l = lam[cur];
-    launch(k_misfit<1>, gg, 128, 0, st, X3[2], l[0], l[2], (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
+    launch<k_misfit<1>>(gg, 128, 0, st, X3[2], l[0], l[2], (int32_t)B, G, gx, obs + m * B * G, Jacc, gcell);
     A.lE = l[0];
     A.lM = l[1];
     A.lB = l[2];
@@ -2029,7 +2070,7 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
     // takes 10.7 against 15.7 us at N = 200, 11.6 against 14.0 at 8192, but 16.2 against 13.7 at 16384.
     constexpr int64_t kScanCells = 8192;
     const bool scan = N <= kScanCells && !A_out;
-    if (!scan) launch(k_rhs_widths, 1, 1024, 0, st, J, (int32_t)N, mx, wv);
+    if (!scan) launch<k_rhs_widths>(1, 1024, 0, st, J, (int32_t)N, mx, wv);
     const unsigned nb = (unsigned)((N + kStepCells - 1) / kStepCells);
     auto go = [&](auto kernel) {
       launch(kernel, nb, kStepThreads, 0, st, P, cfg->bc, cfg->alpha_bound ? 0 : 1, (int32_t)N, alpha, E, M, B, J, w,

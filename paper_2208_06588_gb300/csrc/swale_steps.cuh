@@ -1,6 +1,6 @@
-// Whole SSP-RK3 steps in one launch, for meshes that leave most of the GPU idle: there a step of the
-// stage kernels is nine dependent launches of about ten microseconds each, most of it launch, load
-// and barrier latency. Here the cells stay in registers across stages and steps.
+// Whole SSP-RK3 steps in one launch, for meshes of up to five blocks an SM (93 thousand cells): there a step
+// of the stage kernels is eight dependent launches of ten to twenty microseconds each, much of it launch, load
+// and drain latency. Here the cells stay in registers across stages and steps.
 #pragma once
 
 #include "swale_kernels.cuh"

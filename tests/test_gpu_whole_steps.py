@@ -1,8 +1,8 @@
 """Small meshes run whole steps in one launch (k_steps). Its results are those of the stage kernels,
 bit for bit: an explicit launch shape (swale_set_tiles) keeps a context on the stage kernels.
 
-The sizes sit at the edges of a block's 122 cells and at the smallest meshes; the largest has as
-many blocks as are taken (one per SM). (The error contract on this path: test_gpu_errors.py, whose
+The sizes sit at the edges of a block's 122 cells and at the smallest meshes; the largest have as
+many blocks as are taken (five per SM). (The error contract on this path: test_gpu_errors.py, whose
 meshes are small.)"""
 import numpy as np
 import pytest

@@ -1397,7 +1397,10 @@ __global__ void __launch_bounds__(T, kUpdateThreads / T) k_update(StepConst K, D
       if (SCHEME == 2) {
         const double bd[5] = {B[ghost(j - 1, N, K.bc)], B[j], B[ghost(j + 1, N, K.bc)], BLj, BRj};
         double iJm, iJc, iJp;
-        if (MODE == 0 && (STAGE > 1 || use_sgeo)) {  // (stage 1 on the cache: the widths are J^(1) of the last step)
+        // 1 / J of the neighbours: stored by the previous stage's update, or formed here. On a moving mesh stage 1 forms
+        // it although the last step left it in iJ1 (the same value): this launch's other threads write 1 / J^(1)
+        // there. A static mesh's iJ1 is not written again.
+        if (MODE == 0 && (STAGE > 1 || still)) {
           const double* iJ = (STAGE == 3 ? D.iJ2 : D.iJ1) + cb;
           iJm = iJ[ghost(j - 1, N, K.bc)];
           iJc = iJ[j];

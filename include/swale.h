@@ -239,8 +239,9 @@ swale_status swale_rhs(swale_ctx* ctx, int64_t N, const double* E, const double*
  *                      otherwise it returns after enqueueing
  *   flags              N bytes (host or device) or NULL: detector classes
  * The result comes in one launch (two above 8192 cells or with A_out), which reads neighbouring cells
- * while others are written; outputs that overlap an input take the stage kernels, which read every cell first.
- * Scratch lives in one fixed array of about 7.9 MB per device, held from library load until
+ * while others are written; RE, RM or RB may overlap any of the inputs (not each other): the results are then
+ * held back in the scratch and copied by one more launch.
+ * Scratch lives in one fixed array of about 1.6 MB per device, held from library load until
  * the process exits; the call allocates nothing and clears what it reuses. Every call shares
  * that array, so calls that overlap on the GPU (other streams, other host threads) race; run
  * them one after the other. The first call on a device looks up the array's device address;

@@ -1951,38 +1951,31 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
 // Some callers cannot call cudaMalloc: code that runs inside another framework's memory pool
 // (which owns the device memory and must see every allocation), or work whose device memory
 // must not grow while it runs. For them swale_rhs_noalloc evaluates the same right-hand side as
-// swale_rhs with its scratch (the edge values, shared reciprocals, interior point values of the
-// special source scheme, detector classes and reduction scalars) in the fixed array below,
+// swale_rhs with its scratch (results held back, classes, maxima) in the fixed array below,
 // which every GPU that loads this library holds until the process exits.
 namespace {
 
 constexpr int64_t kNoAllocMaxCells = 65536;
 constexpr int kNoAllocMaxDevices = 64;
-constexpr int kNoAllocTile = 128;
 
 struct NoAllocScratch {
-  // 8 edge arrays, 2 reciprocals, 2 point-value arrays, differences of eta and h, the depth
-  double edges[15][kNoAllocMaxCells + 2];
-  uint8_t flags[kNoAllocMaxCells + 2];
-  InstConst ic;
-  DevScalars S;
+  double out[3][kNoAllocMaxCells];  // right-hand sides whose arrays overlap an input
+  uint8_t flags[kNoAllocMaxCells];
+  unsigned long long widest, wave;  // largest width, largest edge speed (bit patterns)
 };
 
-// Resets the scratch scalars of one call; the values come in as kernel arguments, so the call
-// copies nothing from host memory.
-__global__ void k_noalloc_init(InstConst* ic, DevScalars* S, int64_t N, int32_t ntiles_r) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
-  InstConst c = {};
-  c.N = N;
-  c.cfl = 1.0;
-  c.ntiles_r = ntiles_r;
-  *ic = c;
-  DevScalars z = {};
-  z.Jmin0 = 0x3ff0000000000000ull;  // 1.0: the unused stage-1 dt arithmetic stays finite
-  *S = z;
+// Right-hand sides held back while cells were still being read, to the caller's arrays.
+__global__ void __launch_bounds__(256) k_rhs_store(const NoAllocScratch* scr, int32_t n, double* RE, double* RM, double* RB) {
+  const int32_t i = blockIdx.x * 256 + threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
+  if (i >= n) return;
+  RE[i] = scr->out[0][i];
+  RM[i] = scr->out[1][i];
+  RB[i] = scr->out[2][i];
 }
 
-// Fixed scratch of the allocation-free entry point (about 7.9 MB per device).
+// Fixed scratch of the allocation-free entry point (about 1.6 MB per device).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocScratch)];
 
 // Device address of g_noalloc_scratch per device, obtained once with that device current.
@@ -1990,14 +1983,13 @@ void* g_noalloc_addr[kNoAllocMaxDevices];
 std::once_flag g_noalloc_once[kNoAllocMaxDevices];
 cudaError_t g_noalloc_err[kNoAllocMaxDevices];
 
-// What a call returns besides the right-hand sides: the classes (src, device) and the largest edge speed.
-swale_status noalloc_results(NoAllocScratch* scr, const uint8_t* src, uint8_t* flags, int64_t N, double* A_out,
-                             cudaStream_t st) {
+// What a call returns besides the right-hand sides: the classes and the largest edge speed.
+swale_status noalloc_results(NoAllocScratch* scr, uint8_t* flags, int64_t N, double* A_out, cudaStream_t st) {
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && flags) e = cudaMemcpyAsync(flags, src, (size_t)N, cudaMemcpyDefault, st);
+  if (e == cudaSuccess && flags) e = cudaMemcpyAsync(flags, scr->flags, (size_t)N, cudaMemcpyDefault, st);
   if (e == cudaSuccess && A_out) {
     unsigned long long bits = 0;
-    e = cudaMemcpyAsync(&bits, &scr->S.A[0], sizeof(bits), cudaMemcpyDeviceToHost, st);
+    e = cudaMemcpyAsync(&bits, &scr->wave, sizeof(bits), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) std::memcpy(A_out, &bits, sizeof(double));
   }
@@ -2030,7 +2022,8 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
       cfg->bc > 2 || cfg->scheme < 0 || cfg->scheme > 2 || (cfg->alpha_bound != 0 && cfg->alpha_bound != 1) ||
       (cfg->limit_hu != 0 && cfg->limit_hu != 1))
     return SWALE_EINVAL;
-  // Outputs that overlap an input (in place): every cell has to be read before the first is written.
+  // Outputs that overlap an input (in place) are held back until every cell has been read: a block reads up to three
+  // cells of its neighbours (and, for the widths' maximum, all of J) while other blocks write theirs.
   bool in_place = false;
   for (const double* r : {RE, RM, RB})
     for (const double* q : {E, M, B, J, w}) in_place = in_place || (r < q + (q == w ? N + 1 : N) && q < r + N);
@@ -2057,91 +2050,30 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   if (g_noalloc_err[dev] != cudaSuccess || !g_noalloc_addr[dev]) return SWALE_ECUDA;
   NoAllocScratch* scr = reinterpret_cast<NoAllocScratch*>(g_noalloc_addr[dev]);
   const bool flags_here = flags && on_device(flags);
-  if (!in_place) {
-    SchemeConst P;
-    P.g = cfg->g;
-    P.eps_weno = cfg->eps_weno;
-    P.eps_pp = cfg->eps_pp;
-    P.h_dry = cfg->h_dry;
-    P.beta_dx_global = cfg->beta_dx_global;
-    P.limit_hu = cfg->limit_hu;
-    unsigned long long *mx = &scr->S.Jmax[0], *wv = A_out ? &scr->S.A[0] : nullptr;
-    // Up to this many cells every block finds the largest width itself, one launch instead of two: a call
-    // takes 10.7 against 15.7 us at N = 200, 11.6 against 14.0 at 8192, but 16.2 against 13.7 at 16384.
-    constexpr int64_t kScanCells = 8192;
-    const bool scan = N <= kScanCells && !A_out;
-    if (!scan) launch<k_rhs_widths>(1, 1024, 0, st, J, (int32_t)N, mx, wv);
-    const unsigned nb = (unsigned)((N + kStepCells - 1) / kStepCells);
-    auto go = [&](auto kernel) {
-      launch(kernel, nb, kStepThreads, 0, st, P, cfg->bc, cfg->alpha_bound ? 0 : 1, (int32_t)N, alpha, E, M, B, J, w,
-             scan ? nullptr : mx, wv, RE, RM, RB, flags_here ? flags : scr->flags);
-    };
-    if (cfg->scheme == SWALE_SCHEME_NONWB) go(k_rhs<1>);
-    else if (cfg->scheme == SWALE_SCHEME_SPECIAL) go(k_rhs<2>);
-    else go(k_rhs<0>);
-    return noalloc_results(scr, scr->flags, flags_here ? nullptr : flags, N, A_out, st);
-  }
-
-  DevState D{};
-  D.eEL = scr->edges[0];
-  D.eER = scr->edges[1];
-  D.eBL = scr->edges[2];
-  D.eBR = scr->edges[3];
-  D.ehL = scr->edges[4];
-  D.ehR = scr->edges[5];
-  D.euL = scr->edges[6];
-  D.euR = scr->edges[7];
-  D.ipair = scr->edges[8];
-  D.itri = scr->edges[9];
-  if (cfg->scheme == SWALE_SCHEME_SPECIAL) {
-    D.eG1 = scr->edges[10];
-    D.eG2 = scr->edges[11];
-  }
-  D.dE = scr->edges[12];
-  D.dH = scr->edges[13];
-  D.H = scr->edges[14];
-  D.flags = scr->flags;
-  D.IC = &scr->ic;
-  D.S = &scr->S;
-  D.w = const_cast<double*>(w);
-  D.nf = (int32_t)((N + kNoAllocTile - 2) / (kNoAllocTile - 1));
-  D.nrf = (int32_t)((N + 2 + kNoAllocTile - 5) / (kNoAllocTile - 4));
-  D.ic1.N = N;
-  D.ic1.cfl = 1.0;
-  D.ic1.ntiles_r = D.nrf;
-  StepConst K;
-  K.sc.g = cfg->g;
-  K.sc.eps_weno = cfg->eps_weno;
-  K.sc.eps_pp = cfg->eps_pp;
-  K.sc.h_dry = cfg->h_dry;
-  K.sc.beta_dx_global = cfg->beta_dx_global;
-  K.sc.limit_hu = cfg->limit_hu;
-  K.t_end = 0.0;
-  K.dt_fixed = 0.0;
-  K.mesh_T = K.inv_T = 1.0;
-  K.gauss_iwsum = 1.0;
-  K.bc = cfg->bc;
-  K.mesh = SWALE_MESH_STATIC;
-  K.gauss_half = 0;
-  K.B = 1;
-  K.alpha_log = nullptr;
-  K.alpha_cap = 0;
-  K.alpha_base = 0;
-  K.alpha_mode = 0;
-  K.wait_tries = kWaitTries;
-  K.tx_pad = 0;
-  K.bot_pieces = K.bot_deg = 0;
-  K.bot_breaks = K.bot_coef = nullptr;
-  K.scheme = cfg->scheme;
-  K.geo_epoch = 0;  // no geometry cache here (D.geo is null)
-  K.wave_rel = cfg->alpha_bound ? 0 : 1;  // the largest |u - w| + sqrt(g h) (Eq. alpha2D) in A_out
-  // The scalars keep the previous call's contents: start them from zero.
-  k_noalloc_init<<<1, 32, 0, st>>>(&scr->ic, &scr->S, N, D.nrf);
-  k_widths_max<<<64, 256, 0, st>>>(J, N, &scr->S);
-  launch_recon<1>(K, D, kNoAllocTile, (unsigned)D.nrf, st, E, M, B, J);
-  const RhsOut ro{RE, RM, RB, alpha};
-  launch_update<2, 1>(K, D, kNoAllocTile, (unsigned)D.nf, st, E, M, B, J, ro);
-  return noalloc_results(scr, scr->flags + 1, flags, N, A_out, st);
+  SchemeConst P;
+  P.g = cfg->g;
+  P.eps_weno = cfg->eps_weno;
+  P.eps_pp = cfg->eps_pp;
+  P.h_dry = cfg->h_dry;
+  P.beta_dx_global = cfg->beta_dx_global;
+  P.limit_hu = cfg->limit_hu;
+  unsigned long long *mx = &scr->widest, *wv = A_out ? &scr->wave : nullptr;
+  // Up to this many cells every block finds the largest width itself, one launch instead of two: a call
+  // takes 10.7 against 15.7 us at N = 200, 11.6 against 14.0 at 8192, but 16.2 against 13.7 at 16384.
+  constexpr int64_t kScanCells = 8192;
+  const bool scan = N <= kScanCells && !A_out;
+  if (!scan) launch<k_rhs_widths>(1, 1024, 0, st, J, (int32_t)N, mx, wv);
+  const unsigned nb = (unsigned)((N + kStepCells - 1) / kStepCells);
+  double* const out[3] = {in_place ? scr->out[0] : RE, in_place ? scr->out[1] : RM, in_place ? scr->out[2] : RB};
+  auto go = [&](auto kernel) {
+    launch(kernel, nb, kStepThreads, 0, st, P, cfg->bc, cfg->alpha_bound ? 0 : 1, (int32_t)N, alpha, E, M, B, J, w,
+           scan ? nullptr : mx, wv, out[0], out[1], out[2], flags_here ? flags : scr->flags);
+  };
+  if (cfg->scheme == SWALE_SCHEME_NONWB) go(k_rhs<1>);
+  else if (cfg->scheme == SWALE_SCHEME_SPECIAL) go(k_rhs<2>);
+  else go(k_rhs<0>);
+  if (in_place) launch<k_rhs_store>((unsigned)((N + 255) / 256), 256, 0, st, scr, (int32_t)N, RE, RM, RB);
+  return noalloc_results(scr, flags_here ? nullptr : flags, N, A_out, st);
 }
 
 }  // extern "C"

@@ -1635,6 +1635,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
       if (!s) s = carve(p, (size_t)Nt);
     if (!s) s = carve(&X.x, (size_t)NN);
     if (!s) s = carve(&X.w, (size_t)NN);
+    if (ctx->cfg.mesh == SWALE_MESH_STATIC) X.w = base.w;  // (a step reads them, but only a moving mesh's writes them)
     double** edges[] = {&X.eEL, &X.eER, &X.eBL, &X.eBR, &X.ehL, &X.ehR, &X.euL, &X.euR, &X.ipair, &X.itri,
                         &X.dE, &X.dH, &X.H};
     // (with the tape every step's edge arrays are its slot's; the set keeps only what the slots share)
@@ -1698,6 +1699,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
         for (double** p : st_arr)
           if (!s) s = carve(p, (size_t)Nt);
         if (!s) s = carve(&base_i.w, (size_t)NN);
+        if (ctx->cfg.mesh == SWALE_MESH_STATIC) base_i.w = base.w;
         for (int t = 0; t < 3; ++t) {
           slot[b][3 * i + t] = base_i;
           alloc_edges(slot[b][3 * i + t]);

@@ -1813,7 +1813,10 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
         f3[t].x = fwd.x;
         f3[t].S = fwd.S;
         f3[t].flags = fwd.flags;
+        // (the mesh cache of a static mesh goes with 1 / J^(1), 1 / J^(2): a step on the cache reads them)
         f3[t].geo = fwd.geo;
+        f3[t].iJ1 = fwd.iJ1;
+        f3[t].iJ2 = fwd.iJ2;
       }
       s = enqueue_step_on(ctx, f3[2], st, f3, ctx->geo_epoch);
     } else {

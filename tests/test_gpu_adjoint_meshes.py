@@ -1,4 +1,5 @@
-"""Gradients on static and linear meshes, with and without the tape, against the oracle's tangent along a
+"""Gradients on static and linear meshes: with and without the tape, for one-step, ragged and single
+segments, on a fresh context and on one that has stepped, all the same and the oracle's tangent along a
 direction. Device memory is left full of large values first, so that an array read before it is written
 shows."""
 import numpy as np
@@ -74,7 +75,8 @@ def tangent(pr, obs, before, d):
 
 
 @pytest.mark.parametrize("mesh", ["static", "linear"])
-def test_one_segment(mesh, before=0):
+@pytest.mark.parametrize("before", [0, 4])
+def test_gradient_does_not_depend_on_tape_and_segments(mesh, before):
     pr = problem(mesh)
     rng = np.random.default_rng(3)
     obs = 0.6 + 0.05 * rng.normal(size=(STEPS, GX.size))
@@ -85,7 +87,7 @@ def test_one_segment(mesh, before=0):
     assert abs(ref[0][0] - Jo) <= 1e-11 * Jo
     assert abs(sum(g @ v for g, v in zip(ref[1:], d)) - dJ) <= 1e-12 * scale
     for tape in (0, 1):
-        for ckpt in (STEPS,):
+        for ckpt in (1, 5, STEPS):
             got, st = gradient(pr, obs, ckpt, tape, before)
             assert abs(got[0][0] - ref[0][0]) <= 1e-14 * ref[0][0], (tape, ckpt)
             for a, b in zip(got[1:], ref[1:]):

@@ -94,3 +94,23 @@ def test_gradient_does_not_depend_on_tape_and_segments(mesh, before):
                 assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max(), (tape, ckpt)
             for k in ("eta", "hu", "b", "x", "t"):
                 assert np.array_equal(st[k], end[k]), (tape, ckpt, k)
+
+
+def test_static_gradient_after_a_moving_one(monkeypatch):
+    """Small enough that the call's memory is that of the call before, where a moving mesh left its node
+    velocities; a context held open keeps the allocation in place."""
+    import sys
+    for name, v in (("N", 40), ("STEPS", 3), ("litter", lambda: None)):
+        monkeypatch.setattr(sys.modules[__name__], name, v)
+    obs = 0.6 + 0.05 * np.random.default_rng(3).normal(size=(STEPS, GX.size))
+    pr = problem("static")
+    keep = B.Solver(B.make_config())
+    keep.set_problem(pr.x, pr.E, pr.hu, pr.b, pr.profile, q0_is_eta=True)
+    for tape in (0, 1):
+        ref, _ = gradient(pr, obs, STEPS, tape, 0)
+        gradient(problem("linear"), obs, STEPS, tape, 0)
+        got, _ = gradient(pr, obs, STEPS, tape, 0)
+        assert abs(got[0][0] - ref[0][0]) <= 1e-14 * ref[0][0]
+        for a, b in zip(got[1:], ref[1:]):
+            assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+    keep.close()

@@ -729,14 +729,11 @@ swale_status set_instances(swale_ctx* ctx, const std::vector<int64_t>& off, cons
     double ws = 0.0;
     for (int mm = -H; mm <= H; ++mm) ws += gw[mm + H];
     ctx->gauss_wsum = ws;
-    std::vector<int2> gq(gw.size());
-    for (size_t k = 0; k < gw.size(); ++k) {
-      const long long q = (long long)std::llrint(std::ldexp(gw[k], 56));
-      gq[k] = make_int2((int)(q & 0xfffffff), (int)(q >> 28));
-    }
+    std::vector<swale::Limbs> gq(gw.size());
+    for (size_t k = 0; k < gw.size(); ++k) gq[k] = swale::limbs((long long)std::llrint(std::ldexp(gw[k], 56)));
     SW_CUDA(ctx, cudaMemcpyToSymbolAsync(c_gauss_w, gw.data(), gw.size() * sizeof(double), 0,
                                          cudaMemcpyHostToDevice, st));
-    SW_CUDA(ctx, cudaMemcpyToSymbolAsync(c_gauss_q, gq.data(), gq.size() * sizeof(int2), 0, cudaMemcpyHostToDevice, st));
+    SW_CUDA(ctx, cudaMemcpyToSymbolAsync(c_gauss_q, gq.data(), gq.size() * sizeof(swale::Limbs), 0, cudaMemcpyHostToDevice, st));
   }
   return build_tiles(ctx, ic);
 }

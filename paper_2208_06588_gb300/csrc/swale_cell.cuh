@@ -341,6 +341,45 @@ SWALE_HD bool sure_smooth_nonwb_f32(double g, double h_dry, double hb, double mb
   return sure_smooth1_f32(F, c4, c3, fd, fm, it, eps);
 }
 
+// A number in fixed point, hi 2^28 + lo with 0 <= lo < 2^28.
+struct Limbs {
+  int lo, hi;
+};
+SWALE_HD Limbs limbs(long long x) { return {(int)(x & 0xfffffff), (int)(x >> 28)}; }
+// v 2^(1022 - ex + 55), rounded to an integer: at most 2^55 in magnitude for |v| < 2^(ex - 1022), exact for |v|
+// from a quarter of that on.
+SWALE_HD Limbs fixed_point(double v, int ex) {
+#if defined(__CUDA_ARCH__)
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+#else
+  unsigned long long bits;
+  memcpy(&bits, &v, 8);
+#endif
+  const int e = (int)((bits >> 52) & 0x7ff);
+  const long long m = e ? (long long)((bits & 0xfffffffffffffull) | 0x10000000000000ull) : 0ll;  // 53 bits (subnormals: 0)
+  const int sft = 2 - (ex - e);  // left by two where the exponent is the largest
+  const long long x = sft >= 0 ? m << sft : (sft > -60 ? (m + (1ll << (-sft - 1))) >> -sft : 0ll);
+  return limbs(bits >> 63 ? -x : x);
+}
+// sum_m x[m] w[m] 2^-56, rounded to an integer: the products of a filter of n <= 129 taps with weights w (0 <= w <= 2^56)
+// and fixed-point velocities x (|x| <= 2^55). The limbs' products go to sums of their own, each below what it
+// holds for any weights: |x.hi w.hi| and |x.hi w.lo| are at most 2^55, so their sums are below 2^62.02; x.lo w.hi and
+// x.lo w.lo are at most 2^56, without sign, below 2^63.02. (One sum for both cross products holds only
+// 63 taps, and x of 56 bits only 127.)
+SWALE_HD long long filter_sum(const Limbs* x, const Limbs* w, int n) {
+  long long hh = 0, hl = 0;
+  unsigned long long lh = 0, ll = 0;
+  for (int m = 0; m < n; ++m) {
+    const Limbs a = x[m], b = w[m];
+    hh += (long long)a.hi * b.hi;
+    hl += (long long)a.hi * b.lo;
+    lh += (unsigned long long)(unsigned)a.lo * (unsigned)b.hi;
+    ll += (unsigned long long)(unsigned)a.lo * (unsigned)b.lo;
+  }
+  const long long rest = (hl & 0xfffffff) + (long long)(lh & 0xfffffff) + (long long)(ll >> 28);
+  return hh + (hl >> 28) + (long long)(lh >> 28) + ((rest + (1ll << 27)) >> 28);
+}
+
 // sin(pi x) (want_sin) or cos(pi x), |x| < 2^40: x = n / 2 + r with |r| <= 1/4, then the Taylor series of
 // sin or cos at pi r, chosen by the quadrant, to the term of order 17 or 16 (what is left out is below
 // 2^-58 of the result). One chain of operations for both functions, so that two lanes of a warp get

@@ -169,7 +169,7 @@ struct DevState {
 };
 
 __constant__ double c_gauss_w[2 * kMaxGaussHalf + 1];
-__constant__ int2 c_gauss_q[2 * kMaxGaussHalf + 1];  // the same times 2^56, low and high limb of 28 bits
+__constant__ swale::Limbs c_gauss_q[2 * kMaxGaussHalf + 1];  // the same times 2^56
 
 // Status bits that stop an instance (SWALE_BIT_NEGDEPTH is a warning).
 constexpr unsigned int kErrBits =
@@ -459,11 +459,11 @@ __global__ void k_prologue(StepConst K, DevState D) {
 //
 // The filter's 2 H + 1 products run on the integer multiplier in fixed point: an FP64 FMA holds the sub-partition
 // for 64 cycles, four 32-bit multiply-adds with 64-bit sums about ten. The raw velocities of the
-// tile's window are scaled by a power of two to 56-bit integers (2^56 above the largest of
-// them), the weights exp(-m^2 / 2 sigma^2) are 57-bit ones, both in two limbs of 28 bits, and the sums
-// are exact: the result is within (2 H + 1) 2^-57 of the largest raw velocity of the exact sum of
-// the rounded inputs, where the FP64 sum's bound is about 20 x 2^-53 of it. Measured against 64-bit
-// references the step's error is unchanged; the kernel needs 12 FP64 instructions per node instead of 61 and
+// tile's window are scaled by a power of two to 55-bit integers (2^55 above the largest of
+// them), the weights exp(-m^2 / 2 sigma^2) are 57-bit ones, both in limbs of 28 bits, and the sums
+// are exact for every window that a configuration may ask for (filter_sum). With |v| the largest raw velocity and W the
+// sum of the weights, rounding the velocities, the weights and the sum leaves at most ((W + 1) 2^-56 + (2 H + 1) 2^-57) |v|,
+// before the division by W. The kernel needs 12 FP64 instructions per node instead of 61 and
 // 39 us at 2^20 cells instead of 118.
 // Nodes whose window is cut off by an end, and tiles whose largest velocity is beyond 2^900, below 2^-967
 // or a NaN, take the FP64 sum.
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
   double* su = sh;         // cell velocities, cells [k0 - H - 1, k0 + T + H]; then the limbs of sraw
   double* sraw = sh + nu;  // raw node velocities, nodes [k0 - H, k0 + T + H]
   double* sw = sraw + nr;  // filtered velocities, nodes [k0, k0 + T]
-  int2* sx = reinterpret_cast<int2*>(su);
+  swale::Limbs* sx = reinterpret_cast<swale::Limbs*>(su);
   pdl_wait();
   for (int t = blockIdx.x; t < D.nm; t += gridDim.x) {
     const Tile tl = D.mtiles ? D.mtiles[t] : Tile{0, t * kMeshNodes};
@@ -514,20 +514,11 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kMeshThreads / 32; ++q) top = top > wmax[q] ? top : wmax[q];
-    // |v| < 2^(ex - 1022) for every raw velocity; v 2^(1022 - ex + 56) in two limbs.
+    // |v| < 2^(ex - 1022) for every raw velocity.
     const int ex = (int)(top >> 20);
     const bool fixed = ex > 55 && ex < 1923;  // (2^-967 to 2^900, and no NaN or infinity)
-    if (fixed) {
-      for (int i = tid; i < nr; i += T) {
-        const unsigned long long bits = dbits(sraw[i]);
-        const int e = (int)((bits >> 52) & 0x7ff);
-        const long long m = e ? (long long)((bits & 0xfffffffffffffull) | 0x10000000000000ull) : 0ll;  // 53 bits (subnormals: 0)
-        const int sft = 3 - (ex - e);  // left by three where the exponent is the largest
-        long long x = sft >= 0 ? m << sft : (sft > -60 ? (m + (1ll << (-sft - 1))) >> -sft : 0ll);
-        if (bits >> 63) x = -x;
-        sx[i] = make_int2((int)(x & 0xfffffff), (int)(x >> 28));
-      }
-    }
+    if (fixed)
+      for (int i = tid; i < nr; i += T) sx[i] = swale::fixed_point(sraw[i], ex);
     __syncthreads();
     {
       const int i = tid;
@@ -537,17 +528,8 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
         if (top == 0u) {
           v = 0.0;  // still water
         } else if (fixed && k - H >= 1 && k + H <= N - 1) {
-          long long hh = 0, mid = 0, ll = 0;
-          for (int m = 0; m <= 2 * H; ++m) {
-            const int2 x = sx[i + m], g = c_gauss_q[m];
-            hh += (long long)x.y * g.y;
-            mid += (long long)x.y * g.x;
-            mid += (long long)x.x * g.y;
-            ll += (long long)x.x * g.x;
-          }
-          const long long low = ((mid & 0xfffffff) << 28) + ll;
-          const long long sum = hh + (mid >> 28) + ((low + (1ll << 55)) >> 56);  // 2^(1022 - ex + 56) times the filtered value
-          v = (double)sum * (K.gauss_iwsum * bitsd((unsigned long long)(ex - 55) << 52));
+          // (2^(1022 - ex + 55) times the filtered value)
+          v = (double)swale::filter_sum(sx + i, c_gauss_q, 2 * H + 1) * (K.gauss_iwsum * bitsd((unsigned long long)(ex - 54) << 52));
         } else if (k - H >= 1 && k + H <= N - 1) {
           double acc = 0.0;
           for (int m = -H; m <= H; ++m) acc += c_gauss_w[m + H] * sraw[i + m + H];

@@ -31,6 +31,7 @@ struct swale_ctx {
   DevState D{};
   int Tr = 128, Tu = 128;         // tile sizes of the reconstruction / update kernels
   int grid_r = 0, grid_u = 0;     // 0: one block per tile, else a persistent grid of that size
+  GaussTable gauss{};             // the filter of the fluid-driven motion
   double gauss_wsum = 1.0;
   std::vector<void*> allocs;      // state
   std::vector<void*> tile_allocs; // work lists (rebuilt when the tile sizes change)
@@ -573,7 +574,7 @@ swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, 
   if (first) L(FAM_PROLOGUE, [&] { launch<k_prologue>((unsigned)((ctx->B + 127) / 128), 128, 0, s, K, D); });
   if (K.mesh == SWALE_MESH_FLUID_GAUSS) {
     const size_t shm = (size_t)(3 * kMeshThreads + 4 * K.gauss_half + 4) * sizeof(double);
-    L(FAM_MESH, [&] { launch<k_mesh_gauss>((unsigned)std::max(D.nm, 1), kMeshThreads, shm, s, K, D); });
+    L(FAM_MESH, [&] { launch<k_mesh_gauss>((unsigned)std::max(D.nm, 1), kMeshThreads, shm, s, K, D, ctx->gauss); });
   }
   StepConst K1 = K;
   K1.wave_rel = stage1_wave_rel(ctx->cfg);
@@ -723,17 +724,14 @@ swale_status set_instances(swale_ctx* ctx, const std::vector<int64_t>& off, cons
   SW_CUDA(ctx, cudaMemcpyAsync(D.S, S0.data(), B * sizeof(DevScalars), cudaMemcpyHostToDevice, st));
   if (ctx->cfg.mesh == SWALE_MESH_FLUID_GAUSS) {
     const int H = ctx->cfg.gauss_half;
-    std::vector<double> gw(2 * kMaxGaussHalf + 1, 0.0);
-    for (int mm = -H; mm <= H; ++mm)
-      gw[mm + H] = std::exp(-(double)(mm * mm) / (2.0 * ctx->cfg.gauss_sigma * ctx->cfg.gauss_sigma));
     double ws = 0.0;
-    for (int mm = -H; mm <= H; ++mm) ws += gw[mm + H];
+    for (int mm = -H; mm <= H; ++mm) {
+      const double w = std::exp(-(double)(mm * mm) / (2.0 * ctx->cfg.gauss_sigma * ctx->cfg.gauss_sigma));
+      ctx->gauss.w[mm + H] = w;
+      ctx->gauss.q[mm + H] = swale::limbs((long long)std::llrint(std::ldexp(w, 56)));
+      ws += w;
+    }
     ctx->gauss_wsum = ws;
-    std::vector<swale::Limbs> gq(gw.size());
-    for (size_t k = 0; k < gw.size(); ++k) gq[k] = swale::limbs((long long)std::llrint(std::ldexp(gw[k], 56)));
-    SW_CUDA(ctx, cudaMemcpyToSymbolAsync(c_gauss_w, gw.data(), gw.size() * sizeof(double), 0,
-                                         cudaMemcpyHostToDevice, st));
-    SW_CUDA(ctx, cudaMemcpyToSymbolAsync(c_gauss_q, gq.data(), gq.size() * sizeof(swale::Limbs), 0, cudaMemcpyHostToDevice, st));
   }
   return build_tiles(ctx, ic);
 }

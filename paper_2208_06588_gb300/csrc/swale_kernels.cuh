@@ -168,8 +168,12 @@ struct DevState {
   InstConst ic1;  // the constants of a single instance (the stage kernels need no load for them)
 };
 
-__constant__ double c_gauss_w[2 * kMaxGaussHalf + 1];
-__constant__ swale::Limbs c_gauss_q[2 * kMaxGaussHalf + 1];  // the same times 2^56
+// Weights exp(-m^2 / 2 sigma^2), m = -H..H, of a configuration's filter, and the same times 2^56. A kernel argument (in the
+// constant bank, as a __constant__ array would be): every context launches with its own.
+struct GaussTable {
+  double w[2 * kMaxGaussHalf + 1];
+  swale::Limbs q[2 * kMaxGaussHalf + 1];
+};
 
 // Status bits that stop an instance (SWALE_BIT_NEGDEPTH is a warning).
 constexpr unsigned int kErrBits =
@@ -470,7 +474,7 @@ __global__ void k_prologue(StepConst K, DevState D) {
 // The block stages the cell velocities and the raw node velocities in shared memory (dynamic, and
 // the limbs in place of the former: 3 T + 4 H + 4 doubles).
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevState D) {
+__global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevState D, const __grid_constant__ GaussTable G) {
   extern __shared__ double sh[];
   __shared__ unsigned wmax[kMeshThreads / 32];
   const int H = K.gauss_half, T = kMeshThreads, tid = threadIdx.x;
@@ -529,18 +533,18 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
           v = 0.0;  // still water
         } else if (fixed && k - H >= 1 && k + H <= N - 1) {
           // (2^(1022 - ex + 55) times the filtered value)
-          v = (double)swale::filter_sum(sx + i, c_gauss_q, 2 * H + 1) * (K.gauss_iwsum * bitsd((unsigned long long)(ex - 54) << 52));
+          v = (double)swale::filter_sum(sx + i, G.q, 2 * H + 1) * (K.gauss_iwsum * bitsd((unsigned long long)(ex - 54) << 52));
         } else if (k - H >= 1 && k + H <= N - 1) {
           double acc = 0.0;
-          for (int m = -H; m <= H; ++m) acc += c_gauss_w[m + H] * sraw[i + m + H];
+          for (int m = -H; m <= H; ++m) acc += G.w[m + H] * sraw[i + m + H];
           v = acc * K.gauss_iwsum;
         } else {
           double acc = 0.0, wsum = 0.0;
           for (int m = -H; m <= H; ++m) {
             const int64_t q = k + m;
             if (q < 1 || q > N - 1) continue;
-            acc += c_gauss_w[m + H] * sraw[i + m + H];
-            wsum += c_gauss_w[m + H];
+            acc += G.w[m + H] * sraw[i + m + H];
+            wsum += G.w[m + H];
           }
           v = acc / wsum;
         }

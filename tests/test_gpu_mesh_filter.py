@@ -58,3 +58,25 @@ def test_windows(half, sigma):
             w = reference(u, sigma, half)
             tol = 2.0 * 2.0 ** -44 + 0.5 * (2 * half + 2) * 2.0 ** -53
             assert np.abs(got - (x + dt * w)).max() <= tol, (kind, scale)
+
+
+def test_two_contexts_keep_their_own_weights():
+    """Contexts of different windows stepped in turn move their meshes as each does alone."""
+    rng = np.random.default_rng(2)
+    u = flow("random", 1.0, rng)
+    windows = [(1.5, 4), (40.0, 60)]
+    alone = []
+    for sigma, half in windows:
+        s, _ = solver(u, 0.05, sigma, half)
+        s.advance(4)
+        alone.append(s.state())
+        s.close()
+    both = [solver(u, 0.05, *w)[0] for w in windows]
+    for _ in range(4):
+        for s in both:
+            assert s.advance(1) == 1
+    for s, ref in zip(both, alone):
+        got = s.state()
+        s.close()
+        for k in ("eta", "hu", "x"):
+            assert np.array_equal(got[k], ref[k]), k

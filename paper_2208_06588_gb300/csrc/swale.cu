@@ -31,7 +31,6 @@ struct swale_ctx {
   DevState D{};
   int Tr = 128, Tu = 128;         // tile sizes of the reconstruction / update kernels
   int grid_r = 0, grid_u = 0;     // 0: one block per tile, else a persistent grid of that size
-  GaussTable gauss{};             // the filter of the fluid-driven motion
   double gauss_wsum = 1.0;
   std::vector<void*> allocs;      // state
   std::vector<void*> tile_allocs; // work lists (rebuilt when the tile sizes change)
@@ -250,6 +249,7 @@ swale_status alloc_state(swale_ctx* ctx, int64_t B, int64_t Ntot, DevState& D) {
     place(&D.flags, ne);
     place(&D.IC, (size_t)B);
     place(&D.S, (size_t)B);
+    if (ctx->cfg.mesh == SWALE_MESH_FLUID_GAUSS) place(&D.gauss, 1);
     if (pass) break;
     if (swale_status s = dalloc(ctx, ctx->allocs, &base, off)) return s;
   }
@@ -573,8 +573,8 @@ swale_status enqueue_step_on(swale_ctx* ctx, const DevState& D, cudaStream_t s, 
   };
   if (first) L(FAM_PROLOGUE, [&] { launch<k_prologue>((unsigned)((ctx->B + 127) / 128), 128, 0, s, K, D); });
   if (K.mesh == SWALE_MESH_FLUID_GAUSS) {
-    const size_t shm = (size_t)(3 * kMeshThreads + 4 * K.gauss_half + 4) * sizeof(double);
-    L(FAM_MESH, [&] { launch<k_mesh_gauss>((unsigned)std::max(D.nm, 1), kMeshThreads, shm, s, K, D, ctx->gauss); });
+    const size_t shm = (size_t)(3 * kMeshThreads + 8 * K.gauss_half + 5) * sizeof(double);
+    L(FAM_MESH, [&] { launch<k_mesh_gauss>((unsigned)std::max(D.nm, 1), kMeshThreads, shm, s, K, D); });
   }
   StepConst K1 = K;
   K1.wave_rel = stage1_wave_rel(ctx->cfg);
@@ -724,14 +724,17 @@ swale_status set_instances(swale_ctx* ctx, const std::vector<int64_t>& off, cons
   SW_CUDA(ctx, cudaMemcpyAsync(D.S, S0.data(), B * sizeof(DevScalars), cudaMemcpyHostToDevice, st));
   if (ctx->cfg.mesh == SWALE_MESH_FLUID_GAUSS) {
     const int H = ctx->cfg.gauss_half;
+    GaussTable G{};
     double ws = 0.0;
     for (int mm = -H; mm <= H; ++mm) {
       const double w = std::exp(-(double)(mm * mm) / (2.0 * ctx->cfg.gauss_sigma * ctx->cfg.gauss_sigma));
-      ctx->gauss.w[mm + H] = w;
-      ctx->gauss.q[mm + H] = swale::limbs((long long)std::llrint(std::ldexp(w, 56)));
+      G.w[mm + H] = w;
+      G.q[mm + H] = swale::limbs((long long)std::llrint(std::ldexp(w, 56)));
       ws += w;
     }
+    G.need = swale::filter_need(G.q, 2 * H + 1);
     ctx->gauss_wsum = ws;
+    SW_CUDA(ctx, cudaMemcpyAsync(D.gauss, &G, sizeof(G), cudaMemcpyHostToDevice, st));
   }
   return build_tiles(ctx, ic);
 }

@@ -346,26 +346,28 @@ struct Limbs {
   int lo, hi;
 };
 SWALE_HD Limbs limbs(long long x) { return {(int)(x & 0xfffffff), (int)(x >> 28)}; }
-// v 2^(1022 - ex + 55), rounded to an integer: at most 2^55 in magnitude for |v| < 2^(ex - 1022), exact for |v|
+// Bits of the fixed-point velocities of a filter of n <= 129 taps: as many as its sums hold (filter_sum) and the high limb
+// takes, 58 up to 31 taps, 57 up to 63, 56 up to 127, then 55.
+SWALE_HD int filter_bits(int n) { return n < 32 ? 58 : n < 64 ? 57 : n < 128 ? 56 : 55; }
+// v 2^(1022 - ex + bits), rounded to an integer: at most 2^bits in magnitude for |v| < 2^(ex - 1022), exact for |v|
 // from a quarter of that on.
-SWALE_HD Limbs fixed_point(double v, int ex) {
+SWALE_HD Limbs fixed_point(double v, int ex, int bits) {
 #if defined(__CUDA_ARCH__)
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
 #else
-  unsigned long long bits;
-  memcpy(&bits, &v, 8);
+  unsigned long long b;
+  memcpy(&b, &v, 8);
 #endif
-  const int e = (int)((bits >> 52) & 0x7ff);
-  const long long m = e ? (long long)((bits & 0xfffffffffffffull) | 0x10000000000000ull) : 0ll;  // 53 bits (subnormals: 0)
-  const int sft = 2 - (ex - e);  // left by two where the exponent is the largest
+  const int e = (int)((b >> 52) & 0x7ff);
+  const long long m = e ? (long long)((b & 0xfffffffffffffull) | 0x10000000000000ull) : 0ll;  // 53 bits (subnormals: 0)
+  const int sft = bits - 53 - (ex - e);  // to the left where the exponent is the largest
   const long long x = sft >= 0 ? m << sft : (sft > -60 ? (m + (1ll << (-sft - 1))) >> -sft : 0ll);
-  return limbs(bits >> 63 ? -x : x);
+  return limbs(b >> 63 ? -x : x);
 }
 // sum_m x[m] w[m] 2^-56, rounded to an integer: the products of a filter of n <= 129 taps with weights w (0 <= w <= 2^56)
-// and fixed-point velocities x (|x| <= 2^55). The limbs' products go to sums of their own, each below what it
-// holds for any weights: |x.hi w.hi| and |x.hi w.lo| are at most 2^55, so their sums are below 2^62.02; x.lo w.hi and
-// x.lo w.lo are at most 2^56, without sign, below 2^63.02. (One sum for both cross products holds only
-// 63 taps, and x of 56 bits only 127.)
+// and fixed-point velocities x of filter_bits(n). The limbs' products go to sums of their own, each below what it
+// holds for any weights: |x.hi w.hi| and |x.hi w.lo| are at most 2^bits, so their sums are at most n 2^bits < 2^63; x.lo w.hi
+// and x.lo w.lo are at most 2^56, without sign, below 2^63.02. (One sum for both cross products would hold half the taps.)
 SWALE_HD long long filter_sum(const Limbs* x, const Limbs* w, int n) {
   long long hh = 0, hl = 0;
   unsigned long long lh = 0, ll = 0;
@@ -378,6 +380,24 @@ SWALE_HD long long filter_sum(const Limbs* x, const Limbs* w, int n) {
   }
   const long long rest = (hl & 0xfffffff) + (long long)(lh & 0xfffffff) + (long long)(ll >> 28);
   return hh + (hl >> 28) + (long long)(lh >> 28) + ((rest + (1ll << 27)) >> 28);
+}
+
+// Whether the fixed-point sum of 2 half + 1 taps stands in for an FP64 one: the velocities' weighted mean, as an integer, has
+// at least the 53 bits of a double, sum_m |x[m]| w[m] >= 2^53 sum_m w[m] (`need`, of the high limbs' products as the sum
+// below). Numbers of 53 bits and more are exact in fixed point, and where smaller ones lie between, what is rounded
+// off stays below what the FP64 sum's own roundings leave. From the middle outwards: most windows show it within a few taps.
+SWALE_HD long long filter_need(const Limbs* w, int n) {
+  long long s = 0;
+  for (int m = 0; m < n; ++m) s += w[m].hi;
+  return s << 25;
+}
+SWALE_HD bool filter_fits(const Limbs* x, const Limbs* w, int half, long long need) {
+  const auto term = [&](int m) { return (long long)(x[m].hi < 0 ? -x[m].hi : x[m].hi) * w[m].hi; };
+  long long s = term(half);
+  for (int d = 1; d <= half && s < need; d += 4)
+    for (int k = 0; k < 4; ++k)
+      if (d + k <= half) s += term(half - d - k) + term(half + d + k);
+  return s >= need;
 }
 
 // sin(pi x) (want_sin) or cos(pi x), |x| < 2^40: x = n / 2 + r with |r| <= 1/4, then the Taylor series of

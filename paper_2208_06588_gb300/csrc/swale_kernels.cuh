@@ -126,6 +126,13 @@ __device__ __forceinline__ double stage_alpha(const StepConst& K, int i, int s, 
 // edge index of its left cell, and per cell).
 enum { GEO_IP, GEO_IT, GEO_IQ, GEO_IV, GEO_RHO, GEO_SIG, GEO_RHO2, GEO_SIG2, GEO_GX, GEO_GY, GEO_K3, GEO_ARRAYS };
 
+// Weights exp(-m^2 / 2 sigma^2), m = -H..H, of a configuration's filter, and the same times 2^56.
+struct GaussTable {
+  double w[2 * kMaxGaussHalf + 1];
+  swale::Limbs q[2 * kMaxGaussHalf + 1];
+  long long need;  // filter_need of q
+};
+
 // Device arrays of a batch (concatenated over instances).
 struct DevState {
   double *E0, *M0, *B0;        // q^n (updated in place by stage 3)
@@ -154,6 +161,7 @@ struct DevState {
   // (gK[k * geo_stride + idx], ADJ_*); set only for the adjoint's recomputes, which store them.
   double* gK;
   uint8_t* flags;              // stage-1 classes, edge layout
+  GaussTable* gauss;           // fluid-driven motion
   InstConst* IC;
   DevScalars* S;
   const Tile* mtiles;  // work lists (null: one instance, implicit tiles)
@@ -166,13 +174,6 @@ struct DevState {
   const Tile* rftiles;
   int32_t nrf;
   InstConst ic1;  // the constants of a single instance (the stage kernels need no load for them)
-};
-
-// Weights exp(-m^2 / 2 sigma^2), m = -H..H, of a configuration's filter, and the same times 2^56. A kernel argument (in the
-// constant bank, as a __constant__ array would be): every context launches with its own.
-struct GaussTable {
-  double w[2 * kMaxGaussHalf + 1];
-  swale::Limbs q[2 * kMaxGaussHalf + 1];
 };
 
 // Status bits that stop an instance (SWALE_BIT_NEGDEPTH is a warning).
@@ -457,32 +458,38 @@ __global__ void k_prologue(StepConst K, DevState D) {
 // Fluid-driven node velocity: raw_k = (u_{k-1} + u_k)/2 for k = 1..N-1 (u = hu/h, dry -> 0),
 // truncated renormalised Gaussian filter, w_0 = w_N = 0. A block filters kMeshThreads nodes in
 // one pass, one per thread, and tiles advance by kMeshNodes = kMeshThreads - 1 nodes: the last
-// node of a tile is the next tile's first, filtered by both (the same sum in the same order),
+// node of a tile is the next tile's first, filtered by both (the same to rounding: a tile scales by its own largest velocity),
 // which gives the tile the right neighbour of its last node for max |w_{k+1} - w_k| without a
 // second pass for one node.
 //
 // The filter's 2 H + 1 products run on the integer multiplier in fixed point: an FP64 FMA holds the sub-partition
 // for 64 cycles, four 32-bit multiply-adds with 64-bit sums about ten. The raw velocities of the
-// tile's window are scaled by a power of two to 55-bit integers (2^55 above the largest of
-// them), the weights exp(-m^2 / 2 sigma^2) are 57-bit ones, both in limbs of 28 bits, and the sums
+// tile's window are scaled by a power of two to integers of b = 55 to 58 bits (filter_bits), the largest of them to the
+// full length, the weights exp(-m^2 / 2 sigma^2) are 57-bit ones, both in limbs of 28 bits, and the sums
 // are exact for every window that a configuration may ask for (filter_sum). With |v| the largest raw velocity and W the
-// sum of the weights, rounding the velocities, the weights and the sum leaves at most ((W + 1) 2^-56 + (2 H + 1) 2^-57) |v|,
-// before the division by W. The kernel needs 12 FP64 instructions per node instead of 61 and
-// 39 us at 2^20 cells instead of 118.
-// Nodes whose window is cut off by an end, and tiles whose largest velocity is beyond 2^900, below 2^-967
-// or a NaN, take the FP64 sum.
+// sum of the weights, rounding the velocities, the weights and the sum leaves at most ((W + 1) 2^(-b - 1) + (2 H + 1) 2^-57) |v|
+// before the division by W: no more than an FP64 sum leaves where the window's velocities have 53 bits or more in that scale,
+// in the mean (filter_fits). The other nodes, those of quiet water beside fast, take the FP64 sum, and so do nodes whose
+// window is cut off by an end, and tiles whose largest velocity is beyond 2^900, below 2^-902 or a NaN.
 // The block stages the cell velocities and the raw node velocities in shared memory (dynamic, and
-// the limbs in place of the former: 3 T + 4 H + 4 doubles).
+// the limbs in place of the former), and the weights in both forms: 3 T + 8 H + 5 doubles.
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevState D, const __grid_constant__ GaussTable G) {
+__global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevState D) {
   extern __shared__ double sh[];
   __shared__ unsigned wmax[kMeshThreads / 32];
-  const int H = K.gauss_half, T = kMeshThreads, tid = threadIdx.x;
+  const int H = K.gauss_half, T = kMeshThreads, tid = threadIdx.x, bits = swale::filter_bits(2 * H + 1);
   const int nu = T + 2 * H + 2, nr = T + 2 * H + 1;
   double* su = sh;         // cell velocities, cells [k0 - H - 1, k0 + T + H]; then the limbs of sraw
   double* sraw = sh + nu;  // raw node velocities, nodes [k0 - H, k0 + T + H]
-  double* sw = sraw + nr;  // filtered velocities, nodes [k0, k0 + T]
+  double* sw = sraw + nr;  // filtered velocities, nodes [k0, k0 + T)
+  double* gw = sw + T;     // the weights
+  swale::Limbs* gq = reinterpret_cast<swale::Limbs*>(gw + 2 * H + 1);
   swale::Limbs* sx = reinterpret_cast<swale::Limbs*>(su);
+  if (tid <= 2 * H) {  // (written before the first step)
+    gw[tid] = D.gauss->w[tid];
+    gq[tid] = D.gauss->q[tid];
+  }
+  const long long need = D.gauss->need;
   pdl_wait();
   for (int t = blockIdx.x; t < D.nm; t += gridDim.x) {
     const Tile tl = D.mtiles ? D.mtiles[t] : Tile{0, t * kMeshNodes};
@@ -520,34 +527,35 @@ __global__ void __launch_bounds__(kMeshThreads) k_mesh_gauss(StepConst K, DevSta
     for (int q = 0; q < kMeshThreads / 32; ++q) top = top > wmax[q] ? top : wmax[q];
     // |v| < 2^(ex - 1022) for every raw velocity.
     const int ex = (int)(top >> 20);
-    const bool fixed = ex > 55 && ex < 1923;  // (2^-967 to 2^900, and no NaN or infinity)
+    const bool fixed = ex > 120 && ex < 1923;  // (2^-902 to 2^900, and no NaN or infinity)
     if (fixed)
-      for (int i = tid; i < nr; i += T) sx[i] = swale::fixed_point(sraw[i], ex);
+      for (int i = tid; i < nr; i += T) sx[i] = swale::fixed_point(sraw[i], ex, bits);
     __syncthreads();
     {
       const int i = tid;
       const int64_t k = k0 + i;
+      const bool whole = k - H >= 1 && k + H <= N - 1;  // the window
+      // (A warp takes one of the sums: an FP64 instruction costs the same for one lane as for 32.)
+      const bool fits = fixed && __all_sync(0xffffffffu, !whole || swale::filter_fits(sx + i, gq, H, need));
       double v = 0.0;
-      if (k >= 1 && k <= N - 1) {
-        if (top == 0u) {
-          v = 0.0;  // still water
-        } else if (fixed && k - H >= 1 && k + H <= N - 1) {
-          // (2^(1022 - ex + 55) times the filtered value)
-          v = (double)swale::filter_sum(sx + i, G.q, 2 * H + 1) * (K.gauss_iwsum * bitsd((unsigned long long)(ex - 54) << 52));
-        } else if (k - H >= 1 && k + H <= N - 1) {
-          double acc = 0.0;
-          for (int m = -H; m <= H; ++m) acc += G.w[m + H] * sraw[i + m + H];
-          v = acc * K.gauss_iwsum;
-        } else {
-          double acc = 0.0, wsum = 0.0;
-          for (int m = -H; m <= H; ++m) {
-            const int64_t q = k + m;
-            if (q < 1 || q > N - 1) continue;
-            acc += G.w[m + H] * sraw[i + m + H];
-            wsum += G.w[m + H];
-          }
-          v = acc / wsum;
+      if (top == 0u) {
+        v = 0.0;  // still water
+      } else if (whole && fits) {
+        // (2^(1022 - ex + bits) times the filtered value)
+        v = (double)swale::filter_sum(sx + i, gq, 2 * H + 1) * (K.gauss_iwsum * bitsd((unsigned long long)(ex + 1 - bits) << 52));
+      } else if (whole) {
+        double acc = 0.0;
+        for (int m = 0; m <= 2 * H; ++m) acc += gw[m] * sraw[i + m];
+        v = acc * K.gauss_iwsum;
+      } else if (k >= 1 && k <= N - 1) {
+        double acc = 0.0, wsum = 0.0;
+        for (int m = -H; m <= H; ++m) {
+          const int64_t q = k + m;
+          if (q < 1 || q > N - 1) continue;
+          acc += gw[m + H] * sraw[i + m + H];
+          wsum += gw[m + H];
         }
+        v = acc / wsum;
       }
       sw[i] = v;
     }

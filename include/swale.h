@@ -333,14 +333,15 @@ swale_status swale_adjoint_bytes(int64_t B, int64_t Ntot, int64_t nsteps, int64_
  * Errors: SWALE_EINVAL. */
 swale_status swale_set_adjoint_tape(swale_ctx* ctx, int32_t enable);
 
-/* Test hook for the bounded waits of the bulk (TMA) copies that stage the reconstruction's
- * tiles (the paper has no counterpart). With pad_bytes > 0, each tile of the next steps, after
- * its real copies have landed, also waits on a second barrier that expects pad_bytes which
- * never arrive, for `tries` polls (0: the default, about a million), so that wait runs out: the
+/* Test hook for the bounded waits (the paper has no counterpart). With pad_bytes > 0, each tile of the next steps, after
+ * the bulk (TMA) copies that stage it have landed, also waits on a second barrier that expects pad_bytes which
+ * never arrive, for `tries` polls (0: the default, about a million), so that wait runs out (small meshes take the
+ * stage kernels meanwhile). With pad_bytes = 0, a mesh of several blocks that runs whole steps in one launch polls
+ * at most `tries` times (0: the default, 2^22) for its other blocks: one poll runs out. Either way the
  * kernel then sets SWALE_BIT_TIMEOUT and returns, the step is not committed and reports
  * SWALE_ETIMEOUT, and the context stays usable (reset the hook with 0, 0; the instance keeps the
- * state of its last good step, a new problem clears the status). A block never returns while a
- * copy of its own may still write its shared memory. Nothing faults or hangs. (Small meshes take the stage kernels meanwhile.)
+ * state of its last good step: cells, widths, nodes, time and step count; a new problem clears the status). A block
+ * never returns while a copy of its own may still write its shared memory. Nothing faults or hangs.
  * Errors: SWALE_EINVAL, SWALE_ECUDA. */
 swale_status swale_set_wait_test(swale_ctx* ctx, int32_t tries, uint32_t pad_bytes);
 

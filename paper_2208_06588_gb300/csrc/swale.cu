@@ -56,8 +56,8 @@ struct swale_ctx {
   // swale_adjoint: keep every step's stage data from the segment recompute (1) instead of
   // recomputing each step before its reverse sweep (0).
   int32_t adjoint_tape = 0;
-  // swale_set_wait_test: polls of the bulk-copy waits (0: the default) and extra bytes they
-  // expect (0).
+  // swale_set_wait_test: polls of the bulk-copy waits and of k_steps' grid-wide waits (0: the defaults) and extra
+  // bytes that the former expect (0).
   int32_t wait_tries = 0;
   uint32_t tx_pad = 0;
   // Whole steps in one launch (k_steps), for meshes of few blocks: the blocks, 0 if there are too many,
@@ -152,6 +152,7 @@ StepConst step_const(const swale_ctx* ctx) {
   K.bot_coef = ctx->bot_coef;
   K.wait_tries = ctx->wait_tries > 0 ? ctx->wait_tries : kWaitTries;
   K.tx_pad = ctx->tx_pad;
+  K.barrier_tries = ctx->wait_tries > 0 ? ctx->wait_tries : kBarrierTries;
   K.wave_rel = ctx->cfg.alpha_bound ? 0 : 1;
   return K;
 }
@@ -741,7 +742,7 @@ swale_status set_instances(swale_ctx* ctx, const std::vector<int64_t>& off, cons
 
 swale_status status_from_bits(swale_ctx* ctx, unsigned int bits) {
   if (bits & swale::ST_TIMEOUT)
-    return fail(ctx, SWALE_ETIMEOUT, "a bounded wait for a bulk copy gave up; the stage was abandoned");
+    return fail(ctx, SWALE_ETIMEOUT, "a bounded wait gave up; the stage was abandoned");
   if (bits & swale::ST_NODT)
     return fail(ctx, SWALE_ENONFINITE, "no finite time step: zero wave speed, no mesh motion and t_end = 0");
   if (bits & swale::ST_NONFINITE) return fail(ctx, SWALE_ENONFINITE, "non-finite value in a stage");

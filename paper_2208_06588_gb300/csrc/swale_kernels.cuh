@@ -108,6 +108,7 @@ struct StepConst {
   // copies (0; swale_set_wait_test raises it so that the waits run out, to test that path).
   int32_t wait_tries;
   uint32_t tx_pad;
+  int32_t barrier_tries;  // polls of a grid-wide wait of k_steps
 };
 
 // Stage viscosity of instance i in stage s of step `step` (DevScalars::step_idx): the computed

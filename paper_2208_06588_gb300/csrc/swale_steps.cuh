@@ -13,7 +13,7 @@ constexpr int kStepCells = kStepThreads - 6;  // cells a block owns: three on ea
 // Per-instance scratch of k_steps, zero at its launch. The maxima and status words of a step live in
 // set (step mod 3); the next but one is cleared while a step runs.
 struct StepScratch {
-  unsigned int arrived;  // barrier arrivals since the launch
+  unsigned int arrived;  // barrier arrivals since the launch, and kGaveUp
   unsigned int pad_;
   unsigned long long mx[3][6];  // A of the three stages, max J^(1), max J^(2), complement of min J^(1)
   unsigned int st[3][6];        // status bits raised before each of the step's barriers
@@ -21,27 +21,34 @@ struct StepScratch {
 
 // Barrier of the nb blocks of an instance: arrivals are counted in global memory and every block
 // waits until all have come. All blocks are resident (a cooperative launch), so the wait ends; it is
-// bounded all the same (kBarrierTries polls, seconds) and returns false if it gives up.
-constexpr int kBarrierTries = 1 << 22;
-__device__ __forceinline__ bool inst_barrier(unsigned int* arrived, unsigned int nb, unsigned int& target) {
-  target += nb;
+// bounded all the same (`tries` polls). A block that runs out of them marks the counter, unless the last arrival has
+// come meanwhile (one compare-and-swap decides), and no block passes this barrier then: all of an instance's
+// blocks give up at the same one, so that they leave the state of the same step. (A mark set at the next barrier
+// follows an arrival there, a count above this barrier's.)
+constexpr int kBarrierTries = 1 << 22;  // (seconds)
+constexpr unsigned int kGaveUp = 0x80000000u;
+__device__ __forceinline__ bool meet(unsigned int* arrived, unsigned int target, int tries) {
+  // (the release and the acquire order the whole block's accesses through the two block barriers)
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
+  unsigned int v = 0;
+  for (int i = 0; i < tries && v < target; ++i)  // (ends on a mark too)
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
+  while (v < target) {  // (repeated once for every arrival at most: ends)
+    const unsigned int old = atomicCAS(arrived, v, v | kGaveUp);
+    v = old == v ? v | kGaveUp : old;
+    __threadfence();
+  }
+  return v < kGaveUp || (v & ~kGaveUp) > target;
+}
+__device__ __forceinline__ bool inst_barrier(unsigned int* arrived, unsigned int nb, unsigned int& target, int tries) {
+  target += nb;  // (at most 6 arrivals a step and block: far below kGaveUp)
   if (nb == 1) {
     __syncthreads();
     return true;
   }
   __shared__ bool ok;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // (the release and the acquire order the whole block's accesses through the two block barriers)
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrived) : "memory");
-    bool got = false;
-    for (int i = 0; i < kBarrierTries && !got; ++i) {
-      unsigned int v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
-      got = (int)(v - target) >= 0;
-    }
-    ok = got;
-  }
+  if (threadIdx.x == 0) ok = meet(arrived, target, tries);
   __syncthreads();
   return ok;
 }
@@ -118,7 +125,7 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
   const double Wbar = S->Wbar;
   long long taken = 0;
   unsigned int bits = 0;
-  bool timeout = false;
+  bool timeout = false, written = false;
   int done = 0;
   StepDt sd{S->dt, S->alpha1, S->sdiff, 0, 0};
   double amax[3] = {0.0, 0.0, 0.0}, jm1 = jmax, jm2 = jmax;
@@ -198,7 +205,7 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
       block_wave<T>(&X->mx[set][stage - 1], 0.0, K.sc.g, mine && c != -1, mine && c != N,
                     WaveEdge{o.hL, o.uL, rel ? w : 0.0}, WaveEdge{o.hR, o.uR, rel && tid < T - 1 ? sW[tid + 1] : 0.0});
       block_or_status(&X->st[set][2 * stage - 2], st);
-      if (!inst_barrier(&X->arrived, nb, target)) {
+      if (!inst_barrier(&X->arrived, nb, target, K.barrier_tries)) {
         timeout = true;
         break;
       }
@@ -312,8 +319,9 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
         kept_sr = sr;
         have_mesh = true;
       }
-      if (!inst_barrier(&X->arrived, nb, target)) {
+      if (!inst_barrier(&X->arrived, nb, target, K.barrier_tries)) {
         timeout = true;
+        written = stage == 3;
         break;
       }
       if (stage == 1) fetch(D.Ea, D.Ma, D.Ba, D.J1, D.iJ1);
@@ -354,9 +362,15 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
     tn = sd.clipped ? K.t_end : tn + sd.dt;
     ++taken;
   }
-  if (timeout) {
-    if (tid == 0) atomicOr(&S->status, (unsigned int)swale::ST_TIMEOUT);
-    return;
+  if (timeout) {  // (not folded into the steps' error path: that costs 100 bytes of spills a thread, 2 to 5 % of the time)
+    if (written && own) {  // the step's cells are written: q^n, J^n back
+      D.E0[g] = q0[0];
+      D.M0[g] = q0[1];
+      D.B0[g] = q0[2];
+      D.J0[g] = J0;
+    }
+    bits |= swale::ST_TIMEOUT;
+    done = 1;
   }
   if (own_node && taken > 0) D.x[nbase + c] = x;
   if (tl.c0 == 0 && tid == 0) {

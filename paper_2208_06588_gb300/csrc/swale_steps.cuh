@@ -392,6 +392,13 @@ __global__ void __launch_bounds__(kStepThreads, PER_SM) k_steps(StepConst K, Dev
   }
 }
 
+// A width as a candidate for the largest: its bit pattern, zero for a negative one or a NaN (whose patterns lie above
+// infinity's), so that a bad cell spoils its neighbours only.
+__device__ __forceinline__ unsigned long long width_bits(double J) {
+  const unsigned long long b = dbits(J);
+  return b <= 0x7ff0000000000000ull ? b : 0ull;
+}
+
 // Largest of n widths, by one block, into *out; *wave (if given) is cleared.
 __global__ void __launch_bounds__(1024) k_rhs_widths(const double* __restrict__ J, int32_t n, unsigned long long* out,
                                                      unsigned long long* wave) {
@@ -400,7 +407,7 @@ __global__ void __launch_bounds__(1024) k_rhs_widths(const double* __restrict__ 
   pdl_wait();
   pdl_trigger();
 #pragma unroll 8
-  for (int32_t i = threadIdx.x; i < n; i += 1024) m = umax64(m, dbits(J[i]));
+  for (int32_t i = threadIdx.x; i < n; i += 1024) m = umax64(m, width_bits(J[i]));
   m = warp_umax64(m);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
@@ -457,7 +464,7 @@ __global__ void __launch_bounds__(kStepThreads, 4) k_rhs(SchemeConst P, int bc, 
   } else {
     unsigned long long m = 0ull;
 #pragma unroll 4
-    for (int32_t i = tid; i < N; i += T) m = umax64(m, dbits(J[i]));
+    for (int32_t i = tid; i < N; i += T) m = umax64(m, width_bits(J[i]));
     m = warp_umax64(m);
     if ((tid & 31) == 0) red[tid >> 5] = m;
     __syncthreads();

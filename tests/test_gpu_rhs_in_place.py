@@ -77,3 +77,26 @@ def test_in_place(n, scheme):
             call(cfg, n, d, out, fl, False)
             for a, r in zip(out, ref):
                 assert torch.equal(a, r), (k, shift)
+
+
+@pytest.mark.parametrize("n", [300, 9000])
+@pytest.mark.parametrize("bad", [-1.0, -1e-300, float("nan")])
+def test_a_bad_width_spoils_its_neighbours_only(n, bad):
+    """One width is not positive, as an integrator's mesh may come out: cells away from it have the stage kernels'
+    values (the jump's indicators use the largest width)."""
+    import torch
+    d = inputs(n)
+    at = n // 2 + 20
+    d["J"][at] = bad if bad != -1.0 else -d["J"][at]
+    cfg = B.make_config(bc="reflective")
+    out = [torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(3)]
+    fl = torch.empty(n, dtype=torch.uint8, device="cuda")
+    call(cfg, n, {k: torch.from_numpy(v).cuda() for k, v in d.items()}, out, fl, False)
+    ctx = B.swale_create(cfg)
+    ref, fr = [np.zeros(n) for _ in range(3)], np.zeros(n, dtype=np.uint8)
+    B.swale_rhs(ctx, n, *(d[k] for k in "EMBJw"), 7.5, *ref, fr)
+    B.swale_destroy(ctx)
+    far = np.abs(np.arange(n) - at) > 8
+    assert fr[far].max() > 0 and np.array_equal(fl.cpu().numpy()[far], fr[far])
+    for a, r in zip(out, ref):
+        assert np.isfinite(r[far]).all() and np.array_equal(a.cpu().numpy()[far], r[far])

@@ -303,7 +303,7 @@ SWALE_HD bool sure_smooth1_f32(const float F[3], float c4, float c3, const float
 }
 
 // The test for a cell of the non-well-balanced scheme: both characteristic fields and the bottom
-// surely smooth, from the FP32 pair differences of eta, hu and h and the cell's averages hb, mb. The
+// surely smooth, from the FP32 pair differences of eta, hu and h (bottom_dd: of the bottom) and the cell's averages hb, mb. The
 // rows of R^-1 (nonwb_proj) are formed in FP32 too: u = mb / hb within 5 u, c within 4 u, 1 / (2c)
 // within 5 u, so the rows' entries within 12 u of (|u| + c) / (2c) and 5 u of 1 / (2c), and a
 // field's differences within 16 u of their magnitudes; the test gets three times these
@@ -312,7 +312,7 @@ SWALE_HD bool sure_smooth1_f32(const float F[3], float c4, float c3, const float
 // back is the identity.
 SWALE_HD bool sure_smooth_nonwb_f32(double g, double h_dry, double hb, double mb, const float F[3], float c4, float c3,
                                     const float d2e[4], const float d2m[4], const float d2h[4], const float it[3],
-                                    float eps) {
+                                    float eps, bool bottom_dd = false) {
   float a11 = 1.0f, a12 = 0.0f, a21 = 0.0f, a22 = 1.0f, m1 = 1.0f, m12 = 0.0f, m21 = 0.0f, m2 = 1.0f;
   if (hb > h_dry) {
     const float hf = f32_trunc(hb), uf = f32_trunc(mb) / hf, cf = sqrtf(f32_trunc(g) * hf), i2c = 0.5f / cf;
@@ -335,8 +335,8 @@ SWALE_HD bool sure_smooth_nonwb_f32(double g, double h_dry, double hb, double mb
   }
   if (!sure_smooth1_f32(F, c4, c3, fd, fm, it, eps)) return false;
   for (int a = 0; a < 4; ++a) {
-    fd[a] = d2e[a] - d2h[a];
-    fm[a] = fabsf(d2e[a]) + fabsf(d2h[a]);
+    fd[a] = bottom_dd ? d2h[a] : d2e[a] - d2h[a];
+    fm[a] = bottom_dd ? fabsf(d2h[a]) : fabsf(d2e[a]) + fabsf(d2h[a]);
   }
   return sure_smooth1_f32(F, c4, c3, fd, fm, it, eps);
 }
@@ -865,9 +865,10 @@ SWALE_HD NonwbProj nonwb_proj(const SchemeConst& P, const real v0[3][3]) {
 
 //   known_smooth[3] (may be null): fields whose smooth class the caller has established (the
 //   device's FP32 test, which implies it for the FP64 indicators); their indicators are not formed.
+//   bottom_dd: DD.D2[2], DD.D3[2] are differences of the bottom, not of the depth.
 SWALE_HD void recon_cell_nonwb_g(const SchemeConst& P, const CellGeom& G, const real v0[3][3], const StencilDD& DD,
                                  EdgeState& o, uint8_t& flag, uint32_t& st, const NonwbProj& pr,
-                                 const bool* known_smooth = nullptr) {
+                                 const bool* known_smooth = nullptr, bool bottom_dd = false) {
   const real hb = v0[2][2];
   const bool wet = pr.wet;
   const real a11 = pr.a11, a12 = pr.a12, a21 = pr.a21, a22 = pr.a22, u = pr.u, c = pr.c;
@@ -879,12 +880,12 @@ SWALE_HD void recon_cell_nonwb_g(const SchemeConst& P, const CellGeom& G, const 
     fv0[2][a] = v0[0][a] - v0[2][a];
     fD3[0][a] = a11 * DD.D3[0][a] + a12 * DD.D3[1][a];
     fD3[1][a] = a21 * DD.D3[0][a] + a22 * DD.D3[1][a];
-    fD3[2][a] = DD.D3[0][a] - DD.D3[2][a];
+    fD3[2][a] = bottom_dd ? DD.D3[2][a] : DD.D3[0][a] - DD.D3[2][a];
   }
   for (int a = 0; a < 4; ++a) {
     fD2[0][a] = a11 * DD.D2[0][a] + a12 * DD.D2[1][a];
     fD2[1][a] = a21 * DD.D2[0][a] + a22 * DD.D2[1][a];
-    fD2[2][a] = DD.D2[0][a] - DD.D2[2][a];
+    fD2[2][a] = bottom_dd ? DD.D2[2][a] : DD.D2[0][a] - DD.D2[2][a];
   }
   real fe[3][2];
   flag = 0;

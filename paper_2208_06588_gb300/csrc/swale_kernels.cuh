@@ -628,7 +628,7 @@ __device__ __noinline__ OpenOut recon_open_cell(const SchemeConst P, const TileR
   r.etaG[0] = r.etaG[1] = 0.0;
   swale::cell_geom(h, dxe, G, r.st);
   if (SCHEME == 1) {
-    swale::recon_cell_nonwb_g(P, G, v0, DD, r.o, r.flag, r.st, swale::nonwb_proj(P, v0));
+    swale::recon_cell_nonwb_g(P, G, v0, DD, r.o, r.flag, r.st, swale::nonwb_proj(P, v0), nullptr, true);
   } else {
     swale::recon_cell_special_g(P, G, h, v0, DD, r.o, r.flag, r.st, r.etaG);
   }
@@ -706,7 +706,7 @@ template <int T, int SCHEME>
 struct ReconRows {
   static constexpr int NV32 = SCHEME == 1 ? 3 : 2;
   double H[T + 2], P[T + 2], Q[T];            // depths; pair and quadruple sums of widths
-  double D2[3][T + 2], D3[3][T + 2], D4[3][T];  // divided differences of eta, hu, h
+  double D2[3][T + 2], D3[3][T + 2], D4[3][T];  // divided differences of eta, hu, h (non-well-balanced scheme: of the bottom)
   // FP32 copies for the smooth-class test: widths, triple reciprocals, pair differences (hu, h, and
   // for the non-well-balanced scheme eta)
   float Jf[T], ITf[T], D2f[NV32][T];
@@ -885,7 +885,9 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
     if (!g.all_pair) ip = g.pair ? g.ip : swale::recip(p);
     d2[0] = swale::mul_(de, ip);
     d2[1] = swale::mul_(dm, ip);
-    d2[2] = swale::mul_(dh, ip);
+    // (the non-well-balanced scheme reconstructs the bottom, and its edge depths are eta's less the bottom's: the other
+    // way round the rounding of eta's and h's edge values stays in the bottom's, and doubles the error of its right-hand side)
+    d2[2] = swale::mul_(SCHEME == 1 ? swale::sub_(de, dh) : dh, ip);
     R.P[tid] = p;
 #pragma unroll
     for (int v = 0; v < 3; ++v) R.D2[v][tid] = d2[v];
@@ -938,7 +940,7 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
       float d2e[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) d2e[a] = R.D2f[R.NV32 - 1][tid - 2 + a];
-      smooth = swale::sure_smooth_nonwb_f32(P.g, P.h_dry, hv, mv, F32, c4f, c3f, d2e, d2m, d2h, itf, epsf);
+      smooth = swale::sure_smooth_nonwb_f32(P.g, P.h_dry, hv, mv, F32, c4f, c3f, d2e, d2m, d2h, itf, epsf, true);
     } else {
       smooth = swale::sure_smooth_f32(F32, c4f, c3f, d2h, d2m, itf, epsf);
     }
@@ -980,7 +982,7 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
   double evl[3][2];
   if (smooth) {
     const swale::SmoothWidths w = {sJ[tid - 1], jv, sJ[tid + 1], R.P[tid - 2], R.P[tid - 1], p, R.P[tid + 1]};
-    const double vj[3] = {ev, mv, hv};
+    const double vj[3] = {ev, mv, SCHEME == 1 ? swale::sub_(ev, hv) : hv};
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
       const double d4l = R.D4[v][tid - 2], d4r = R.D4[v][tid - 1], d3c = R.D3[v][tid - 1];
@@ -989,6 +991,9 @@ __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, 
       evl[v][1] = swale::smooth_right(w, vj[v], d2[v], d3c, d4r, d5);
       if (SCHEME == 2 && v == 0) pts = swale::smooth_points(w, ev, evl[0][0], evl[0][1], d4r, d5);
     }
+    if (SCHEME == 1)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) evl[2][e] = swale::sub_(evl[0][e], evl[2][e]);
   } else {
 #pragma unroll
     for (int v = 0; v < 3; ++v) {

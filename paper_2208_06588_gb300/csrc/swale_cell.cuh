@@ -113,17 +113,6 @@ SWALE_HD double recip(double x) {
   return fma(fma(e, e, e), y, y);
 }
 SWALE_HD double dsqrt(double a) { return sqrt(a); }
-// Square root of a >= 0 for the wave speeds: the hardware's 20-bit reciprocal square root y refined
-// by one third-order step, a y (1 + e/2 + 3 e^2 / 8) with e = 1 - a y^2 (the binomial series of
-// (1 - e)^(-1/2)): 5 FP64 operations, within about one unit in the last place. Zero, subnormal and
-// huge arguments take sqrt().
-SWALE_HD double wave_sqrt(double a) {
-  if (!(a > 1e-300 && a < 1e300)) return sqrt(a);
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  const double r = a * y, e = fma(-r, y, 1.0);
-  return fma(r * e, fma(0.375, e, 0.5), r);
-}
 // NaN, infinite or of magnitude above 1e300, any of six (the high words first).
 SWALE_HD bool bad6(double a, double b, double c, double d, double e, double f) {
   const int m = 0x7fffffff;
@@ -148,10 +137,8 @@ SWALE_HD bool bad6(real a, real b, real c, real d, real e, real f) {
 }
 #ifdef SWALE_REAL
 SWALE_HD real dsqrt(real a) { return swale_sqrt(a); }
-SWALE_HD real wave_sqrt(real a) { return swale_sqrt(a); }
 #else
 SWALE_HD real dsqrt(real a) { return sqrt(a); }
-SWALE_HD real wave_sqrt(real a) { return sqrt(a); }
 #endif
 #endif
 
@@ -439,7 +426,7 @@ SWALE_HD double trig_pi(double x, bool want_sin) {
 }
 
 // Wave speed |u| + sqrt(g max(h, 0)) of one limited edge state (Eq. alpha2D).
-SWALE_HD real wave_speed(real g, real h, real u) { return add_(dabs(u), wave_sqrt(mul_(g, pos0(h)))); }
+SWALE_HD real wave_speed(real g, real h, real u) { return add_(dabs(u), dsqrt(mul_(g, pos0(h)))); }
 
 // ------------------------------------------------------------------------------------
 // Shared per-pair and per-triple terms (Step 1): reciprocal widths and divided differences.

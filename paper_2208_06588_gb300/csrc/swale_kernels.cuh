@@ -635,6 +635,16 @@ __device__ __noinline__ OpenOut recon_open_cell(const SchemeConst P, const TileR
   return r;
 }
 
+// a / b rounded once: the product with the reciprocal, corrected by its remainder (Markstein 1990), two operations where
+// the division is a chain of a dozen (an accuracy run at N = 50 takes 5 % longer with divisions). Operands and
+// quotients near the ends of the range take the division.
+__device__ __forceinline__ double quotient(double a, double b) {
+  const double y = swale::recip(b), q = a * y;
+  const auto mid = [](double v) { return swale::gt_pos(v, 1e-250) && swale::lt_pos(v, 1e250); };
+  if (!mid(a) || !mid(b) || !mid(q)) return a / b;
+  return fma(fma(-b, q, a), y, q);
+}
+
 // A step's dt and the secant factor of the prescribed motion from alpha_1, by whole warps (every
 // lane computes dt: an FP64 instruction costs the same for one lane as for 32). The secant factor
 // (sin(2 pi (t + dt) / T) - sin(2 pi t / T)) / dt is formed as
@@ -648,9 +658,8 @@ __device__ __noinline__ StepDt step_dt(double cfl, double alpha1, double dwmax, 
                                        double t_end, double inv_T) {
   StepDt r{dt_fixed, alpha1, 0.0, 0, 0};
   if (!(dt_fixed > 0.0)) {
-    // (zero and subnormal divisors take the division: the quotient is then infinite, or a NaN)
-    r.dt = alpha1 > 1e-290 ? cfl * jmin * swale::recip(alpha1) : cfl * jmin / alpha1;
-    if (dwmax > 0.0) r.dt = fmin(r.dt, dwmax > 1e-290 ? 0.5 * jmin * swale::recip(dwmax) : 0.5 * jmin / dwmax);
+    r.dt = quotient(cfl * jmin, alpha1);
+    if (dwmax > 0.0) r.dt = fmin(r.dt, quotient(0.5 * jmin, dwmax));
   }
   if (t_end > 0.0 && t_end - tn <= r.dt) {
     r.dt = t_end - tn;

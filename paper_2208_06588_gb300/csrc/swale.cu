@@ -1423,27 +1423,34 @@ typedef StateArrays StateCopy;
 // slack as every device array of the library has.
 uint64_t adj_block(uint64_t bytes) { return (bytes + 255) / 256 * 256 + 256; }
 
-// Bytes of the device block swale_adjoint carves its arrays from; the list follows the arrays in
-// swale_adjoint one for one.
-uint64_t adjoint_bytes(int64_t B, int64_t Nt, int64_t nsteps, int64_t ckpt_every, int32_t G, int32_t tape) {
+// Bytes of the arrays that swale_adjoint carves from its device block; the list follows the arrays there one for one (it
+// refuses to run if the two differ). spare: bytes of the block beyond them, a state copy with the tape, so
+// that the size is the documented one.
+uint64_t adjoint_bytes(int64_t B, int64_t Nt, int64_t nsteps, int64_t ckpt_every, int32_t G, int32_t tape,
+                       uint64_t* spare = nullptr) {
   const int64_t NN = Nt + B, NE = Nt + 2 * B;
   const int64_t C = std::min(ckpt_every, nsteps), nseg = (nsteps + C - 1) / C;
   auto a = [](uint64_t n, uint64_t size) { return adj_block(n * size); };
   const uint64_t copy = 4 * a(Nt, 8) + a(NN, 8) + a(B, sizeof(DevScalars));
-  const uint64_t state_set = 15 * a(Nt, 8) + 2 * a(NN, 8) + 10 * a(NE, 8) + a(NE, 1) + a(B, sizeof(DevScalars));
-  const uint64_t common = 15 * a(Nt, 8) + 8 * a(NE, 8) + state_set + 2 * a((uint64_t)B * G, 8) +
+  const uint64_t edges = 10 * a(NE, 8), adj = a(14 * (uint64_t)NE, 8);
+  // (with the tape every step's edge arrays are its slot's)
+  const uint64_t state_set = 17 * a(Nt, 8) + 2 * a(NN, 8) + (tape ? 0 : edges) + 3 * a(NE, 8) + a(NE, 1) + a(B, sizeof(DevScalars));
+  // lambda twice, the stage inputs' adjoints, the segment recomputes' set and mesh cache; the gauges
+  const uint64_t common = 12 * a(Nt, 8) + state_set + a((uint64_t)GEO_ARRAYS * NE, 8) + 2 * a((uint64_t)B * G, 8) +
                           a((uint64_t)nsteps * B * G, 8) + a(B, 8) + a((uint64_t)nsteps * B * 3, 8);
   // Segment buffers (per-step snapshots, and the tape's slots): two, one being recomputed while
-  // the other is reversed; one when a single segment covers every step.
-  const uint64_t nb = nseg == 1 ? 1 : 2;
+  // the other is reversed; one when a single segment covers every step. A checkpoint per segment and the final state.
+  const uint64_t nb = nseg == 1 ? 1 : 2, copies = (uint64_t)(nseg + nb * C + 1) * copy;
   if (tape) {
-    // per step of a segment: three stage edge sets with their smooth-class linear and source
-    // forms, q^(1), J^(1), q^(2), J^(2), node velocities
-    const uint64_t slot = 30 * a(NE, 8) + 3 * a(14 * (uint64_t)NE, 8) + 8 * a(Nt, 8) + a(NN, 8);
-    return common + (uint64_t)(nseg + nb * C + 1) * copy + (uint64_t)(nb * C) * slot;
+    // per step of a segment: q^(1), J^(1), q^(2), J^(2), node velocities, and three stages' edge sets and
+    // arrays of the reverse
+    const uint64_t slot = 8 * a(Nt, 8) + a(NN, 8) + 3 * (edges + adj);
+    if (spare) *spare = copy;
+    return common + copies + (uint64_t)(nb * C) * slot + copy;
   }
-  // two state sets of the step recompute: four further stage edge sets and six sets of forms
-  return common + state_set + 40 * a(NE, 8) + 6 * a(14 * (uint64_t)NE, 8) + (uint64_t)(nseg + nb * C + 3) * copy;
+  if (spare) *spare = 0;
+  // the step recompute's second state set, and for both stages 1 and 2 edge sets and all stages' arrays of the reverse
+  return common + copies + state_set + 4 * edges + 6 * adj;
 }
 
 }  // namespace
@@ -1559,7 +1566,8 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   // bytes: one cudaMalloc and one cudaFree per call, however many segment buffers and tape
   // slots it holds (at large checkpoint intervals the tape alone has tens of thousands of
   // arrays, whose separate allocations took longer than the gradient).
-  const uint64_t arena_bytes = adjoint_bytes(B, Nt, nsteps, ckpt_every, G, tape ? 1 : 0);
+  uint64_t spare = 0;
+  const uint64_t arena_bytes = adjoint_bytes(B, Nt, nsteps, ckpt_every, G, tape ? 1 : 0, &spare);
   char* arena = nullptr;
   uint64_t arena_off = 0;
   if (cudaError_t e0 = cudaMalloc(&arena, arena_bytes)) {
@@ -1715,6 +1723,7 @@ swale_status swale_adjoint(swale_ctx* ctx, int64_t nsteps, int64_t ckpt_every, i
   if (!s) s = carve(&alog, (size_t)nsteps * B * 3);
   int64_t* gcell = nullptr;  // last cell of each gauge (searched from, the mesh moves little per step)
   if (!s) s = carve(&gcell, (size_t)B * G);
+  if (!s && arena_off + spare != arena_bytes) s = fail(ctx, SWALE_ENOMEM, "adjoint: scratch layout differs from its block");
   if (s) return release(s);
   cudaError_t e = cudaSuccess;
   e = e ? e : cudaMemcpyAsync(gx, gauges_x, (size_t)B * G * sizeof(double), cudaMemcpyDefault, st);

@@ -53,8 +53,9 @@ METHOD_SOURCE_GEOM_FLOPS = 7.0
 # on the initial state of this workload (2^20 cells) and, cell-weighted, of the first 16
 # instances of the batched workload. The oracle builds the mesh-only coefficients by Gaussian
 # elimination, which is not a figure of the method; the method figures add the kernels'
-# closed-form count of that mesh-only part in every stage (no reuse across stages). These are
-# the roofline numerators, so a kernel change that removes work does not lower the fraction.
+# closed-form count of that mesh-only part in every stage (no reuse across stages). The kernels reach the same results
+# with fewer operations, so this count times the rate can pass the hardware's peak: it is reported as
+# method_count (a multiple of the peak), and is no roofline.
 ORACLE_RECON_FLOPS = 318.60
 ORACLE_STEP_FLOPS = 1891.80
 ORACLE_BATCH_STEP_FLOPS = 1893.17
@@ -66,6 +67,20 @@ ORACLE_VARIANT_FLOPS = {"nonwb": (583.01, 2613.02), "special": (366.61, 1780.82)
 UPDATE_DRAM_BYTES = (192_998_656 + 47_543_040 + 201_380_352 + 82_679_808 + 226_542_848 + 56_431_360) // 3
 UPDATE_FP64_PIPE_ACTIVE = (0.8680 + 0.8670 + 0.8604) / 3
 UPDATE_EXECUTED_FLOPS = (106.2 + 124.3 + 127.3) / 3
+# FP64 pipe instructions per cell and launch (ncu sm__inst_executed_pipe_fp64 x 32 lanes over the cells; stages 1, 2, 3), the
+# roofline numerators: every kernel is bound by their issue, one warp instruction per 64 cycles and sub-partition,
+# which a fused multiply-add fills with two FLOPs. By scheme (2^18-cell dam break for the variants, 2^18-cell bump):
+# (reconstruction, update).
+RECON_INSTR = (81.3 + 85.4 + 85.4) / 3
+UPDATE_INSTR = (73.6 + 92.7 + 93.7) / 3
+VARIANT_INSTR = {"nonwb": ((82.8 + 91.1 + 91.1) / 3, (71.6 + 90.7 + 91.7) / 3),
+                 "special": ((96.2 + 100.3 + 100.3) / 3, (110.9 + 108.9 + 105.8) / 3),
+                 "bump": ((75.8 + 89.9 + 89.9) / 3, (73.6 + 94.7 + 91.7) / 3)}
+MESH_INSTR = 13.8  # the fluid-driven mesh's filter
+BATCH_STEP_INSTR = (79.7 + 83.5 + 83.5) + (75.8 + 94.3 + 95.3)
+# A gradient's forward steps and its reverse of a step (65536-cell basin).
+BASIN_STEP_INSTR = (78.3 + 82.9 + 82.8) + (74.6 + 92.8 + 93.8)
+REVERSE_STEP_INSTR = 224.4 + 234.0 + 248.9
 
 
 def parse():
@@ -164,18 +179,19 @@ def op_counts(pr):
     return opcount.count_stage(pr.E, pr.hu, pr.b, pr.J, bc=pr.bc, sample=1 << 16)
 
 
-def fp64_roofline(flops_per_cell_step, cell_steps_per_s, scope, basis="kernel count", kernel_flops=None):
+def fp64_roofline(flops_per_cell_step, cell_steps_per_s, scope,
+                  basis="FP64 instructions issued per cell-step (ncu), two FLOPs of the peak each", method_flops=None):
     """Whole-job FP64 roofline: FLOPs of a cell-step times the measured cell-steps per second,
-    against the FP64 peak. Every kernel of the step is FP64-pipe bound (DRAM below 16 %), so this
-    is the slower of the two rooflines. basis: "method" (the oracle's count, see
-    ORACLE_STEP_FLOPS) or "kernel count" (the closed-form per-cell code counted on the host; the kernels need less);
-    with kernel_flops given, the kernel-count fraction is reported beside the method's."""
+    against the FP64 peak. Every kernel of the step is FP64-pipe bound (DRAM below 25 %), so this
+    is the slower of the two rooflines. Callers pass twice the FP64 instructions that the kernels issue, so frac is the
+    share of the pipe's issue slots; method_flops: the method's operations (the oracle's count, see ORACLE_STEP_FLOPS), reported
+    beside it as a multiple of the peak."""
     achieved = flops_per_cell_step * cell_steps_per_s / 1e12
     out = {"bound": "alu", "scope": scope, "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
            "frac": achieved / FP64_PEAK_TFLOPS, "flops_per_cell_step": flops_per_cell_step, "basis": basis}
-    if kernel_flops is not None:
-        out["kernel_count"] = {"flops_per_cell_step": kernel_flops,
-                               "frac": kernel_flops * cell_steps_per_s / 1e12 / FP64_PEAK_TFLOPS}
+    if method_flops is not None:
+        out["method_count"] = {"flops_per_cell_step": method_flops,
+                               "times_peak": method_flops * cell_steps_per_s / 1e12 / FP64_PEAK_TFLOPS}
     return out
 
 
@@ -185,23 +201,13 @@ def method_step_flops(oc, oracle_step=ORACLE_STEP_FLOPS):
     return oracle_step + 3.0 * (oc["geom_flops"] + METHOD_SOURCE_GEOM_FLOPS)
 
 
-def batch_step_flops(bt, n_inst=16):
-    """Forward-step FLOPs per cell of a batch, averaged (cell-weighted) over its first instances."""
-    from paper_2208_06588_gb300 import opcount
-    tot = cells = 0.0
-    for i in range(min(n_inst, bt.B)):
-        pr = bt.instance(i)
-        c = opcount.count_stage(pr.E, pr.hu, pr.b, pr.J, bc=pr.bc, sample=1 << 13)
-        tot += opcount.forward_step_flops(c) * pr.N
-        cells += pr.N
-    return tot / cells
-
-
-def adjoint_step_flops(pr, tape=False, runs=None):
-    from paper_2208_06588_gb300 import opcount
-    c = opcount.count_stage(pr.E, pr.hu, pr.b, pr.J, bc=pr.bc, sample=1 << 13)
-    r = opcount.count_reverse(pr.E, pr.hu, pr.b, pr.J, bc=pr.bc, sample=1 << 13)
-    return opcount.adjoint_step_flops(c, r, runs=runs if runs else (2 if tape else 3))
+def gradient_step_flops(nsteps, ckpt_every, tape):
+    """Twice the FP64 instructions per cell and step of a gradient: the forward run, the recomputes (a step's segment once
+    unless it is one of the last two, and the step itself once more without the tape) and the reverse."""
+    nseg = -(-nsteps // ckpt_every)
+    kept = nsteps - max(0, nseg - (1 if nseg == 1 else 2)) * ckpt_every
+    runs = 2.0 - kept / nsteps + (0.0 if tape else 1.0)
+    return 2.0 * (runs * BASIN_STEP_INSTR + REVERSE_STEP_INSTR)
 
 
 def cpu_oracle_rate(n_cells, steps):
@@ -300,12 +306,11 @@ def bench_batched(args, stream, dev, rank=0, ws=1):
            "value": ntot * args.batched_steps / (ms * 1e-3), "unit": UNIT, "steps": args.batched_steps,
            "ms_per_step": ms / args.batched_steps, "tiles": list(tiles), "status_bits": bits,
            "parallelism": f"instances sharded over {ws} ranks" if ws > 1 else "single", "scaling": "weak"}
-    kflops = batch_step_flops(bt_all)
     from paper_2208_06588_gb300 import opcount
     pr0 = bt_all.instance(0)
     oc0 = opcount.count_stage(pr0.E, pr0.hu, pr0.b, pr0.J, bc=pr0.bc, sample=1 << 13)
-    out["roofline"] = fp64_roofline(method_step_flops(oc0, ORACLE_BATCH_STEP_FLOPS), out["value"],
-                                    "whole step, all kernels", "method", kflops)
+    out["roofline"] = fp64_roofline(2.0 * BATCH_STEP_INSTR, out["value"], "whole step, all kernels",
+                                    method_flops=method_step_flops(oc0, ORACLE_BATCH_STEP_FLOPS))
     if args.no_loop_baseline:
         return out
     # Same work, batched vs one context per instance (launches per instance and step).
@@ -407,7 +412,7 @@ def bench_adjoint(args, stream, dev=None, ws=1):
                               dev)
     bits = s.status()[0]
     # The same gradient with the tape (swale_set_adjoint_tape): every step run twice, not three
-    # times, for about 39 doubles per cell and step of two segments.
+    # times, for about 81 doubles per cell and step of two segments.
     B.swale_set_adjoint_tape(s.ctx, 1)
     s.set_problem(pr.x, pr.E, pr.hu, pr.b, pr.profile, q0_is_eta=True)
     Jt, gEt = np.zeros(1), np.zeros(N)
@@ -418,8 +423,8 @@ def bench_adjoint(args, stream, dev=None, ws=1):
     tape = {"ms_per_gradient": ms_t, "value": ws * N * K / (ms_t * 1e-3), "ckpt_every": C,
             "adjoint_scratch_bytes": int(B.swale_adjoint_bytes(1, N, K, C, G, tape=1)),
             "grad_eta_rel_diff": float(np.abs(gEt - gE).max() / np.abs(gE).max()),
-            "roofline": fp64_roofline(adjoint_step_flops(pr, tape=True), ws * N * K / (ms_t * 1e-3),
-                                      "whole gradient: 2 forward steps + reverse sweep per step")}
+            "roofline": fp64_roofline(gradient_step_flops(K, C, True), ws * N * K / (ms_t * 1e-3),
+                                      "whole gradient: up to 2 forward steps + reverse sweep per step")}
     return {"workload": f"gaussian_basin N={N} [0,1] reflective, 4 Gaussian bumps, eta0 from 32 Gaussian basis "
                         f"functions, sine mesh motion A=0.02, fixed dt; {K} SSP-RK3 steps; 16 gauges",
             "metric": "cell-updates/s FP64 (forward + adjoint)", "unit": UNIT,
@@ -431,8 +436,8 @@ def bench_adjoint(args, stream, dev=None, ws=1):
             "J": float(J[0]), "grad_norms": [float(np.linalg.norm(v)) for v in (gE, gM, gB)], "status_bits": bits,
             "call": "swale_adjoint (host gauges, observations and gradients)", "mode": "recompute inside each step",
             "tape_mode": tape,
-            "roofline": fp64_roofline(adjoint_step_flops(pr), ws * N * K / (ms * 1e-3),
-                                      "whole gradient: 3 forward steps + reverse sweep per step")}
+            "roofline": fp64_roofline(gradient_step_flops(K, C, False), ws * N * K / (ms * 1e-3),
+                                      "whole gradient: up to 3 forward steps + reverse sweep per step")}
 
 
 def bench_batched_adjoint(args, stream, dev=None, rank=0, ws=1):
@@ -488,8 +493,8 @@ def bench_batched_adjoint(args, stream, dev=None, rank=0, ws=1):
                     "ckpt_every": Ct, "adjoint_over_forward": ms_t / ms_fwd,
                     "peak_device_bytes": int(state_bytes + B.swale_adjoint_bytes(bt.B, Nt, K, Ct, G, tape=1)),
                     "peak_device_bytes_2000_steps": int(state_bytes + cands[0][0]),
-                    "roofline": fp64_roofline(adjoint_step_flops(bt.instance(0), tape=True), Nt_all * K / (ms_t * 1e-3),
-                                              "whole gradient: 2 forward steps + reverse sweep per step")}
+                    "roofline": fp64_roofline(gradient_step_flops(K, Ct, True), Nt_all * K / (ms_t * 1e-3),
+                                              "whole gradient: up to 2 forward steps + reverse sweep per step")}
         except B.SwaleError as err:
             tape = {"unavailable": str(err)}
         B.swale_set_adjoint_tape(s.ctx, 0)
@@ -505,8 +510,8 @@ def bench_batched_adjoint(args, stream, dev=None, rank=0, ws=1):
            "forward_only_value": Nt * K / (ms_fwd * 1e-3), "adjoint_over_forward": ms / ms_fwd,
            "peak_device_bytes": int(state_bytes + adj_bytes), "peak_device_bytes_2000_steps": int(state_bytes + full_bytes),
            "status_bits": bits,
-           "roofline": fp64_roofline(adjoint_step_flops(bt.instance(0)), Nt_all * K / (ms * 1e-3),
-                                     "whole gradient: 3 forward steps + reverse sweep per step"),
+           "roofline": fp64_roofline(gradient_step_flops(K, C, False), Nt_all * K / (ms * 1e-3),
+                                     "whole gradient: up to 3 forward steps + reverse sweep per step"),
            "mode": "recompute inside each step", "tape_mode": tape}
     if args.no_loop_baseline:
         return out
@@ -567,18 +572,14 @@ def bench_variant(args, stream, pr, scheme="hydrostatic", bottom=None):
     B.swale_destroy(ctx)
     oc = opcount.count_stage(pr.E, pr.hu, pr.b, pr.J, bc=pr.bc, sample=1 << 16, scheme=scheme)
     dom = "reconstruction" if fam["reconstruction"][0] >= fam["update"][0] else "update"
-    kfl = oc["recon_flops"] - oc["geom_flops"] / 3.0 if dom == "reconstruction" else oc["update_flops"]
     o_rec, o_step = ORACLE_VARIANT_FLOPS.get(scheme, (ORACLE_RECON_FLOPS, ORACLE_STEP_FLOPS))
     fl = (o_rec + oc["geom_flops"]) if dom == "reconstruction" else (o_step - 3.0 * o_rec) / 3.0 + METHOD_SOURCE_GEOM_FLOPS
+    instr = VARIANT_INSTR.get(scheme, VARIANT_INSTR["bump"])[0 if dom == "reconstruction" else 1]
     ms_dom, n_dom = fam[dom]
     per_s = pr.N / (ms_dom / n_dom * 1e-3)
-    achieved = fl * per_s / 1e12
+    roof = fp64_roofline(2.0 * instr, per_s, "dominant kernel, per launch", method_flops=fl)
     return {"value": pr.N * K / (ms * 1e-3), "unit": UNIT, "steps": K, "ms_per_step": ms / K, "status_bits": bits,
-            "roofline": {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                         "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS, "flops_per_cell": fl,
-                         "flops_basis": "method (CPU oracle count + mesh-only geometry)",
-                         "kernel_count": {"flops_per_cell": kfl, "frac": kfl * per_s / 1e12 / FP64_PEAK_TFLOPS},
-                         "avg_launch_ms": ms_dom / n_dom},
+            "roofline": {**roof, "kernel": dom, "avg_launch_ms": ms_dom / n_dom},
             "fp64_flops_per_cell_stage": {"recon": oc["recon_flops"], "update": oc["update_flops"]}}
 
 
@@ -776,30 +777,25 @@ def main():
     ms_rec, n_rec = fam["reconstruction"]
     ms_upd, n_upd = fam["update"]
     dom = "reconstruction" if ms_rec >= ms_upd else "update"
-    # Stage 1 takes the mesh-only geometry from the previous step's stage 2 (same mesh), so a
-    # reconstruction launch does on average a third of that part less.
-    recon_avg = oc["recon_flops"] - oc["geom_flops"] / 3.0
-    from paper_2208_06588_gb300 import opcount
-    opcount_step = opcount.forward_step_flops(oc)
-    kernel_flops_cell = recon_avg if dom == "reconstruction" else oc["update_flops"]
     # The method's count per cell and launch (oracle count + mesh-only geometry of the stage).
     method_recon = ORACLE_RECON_FLOPS + oc["geom_flops"]
     method_update = (ORACLE_STEP_FLOPS - 3.0 * ORACLE_RECON_FLOPS) / 3.0 + METHOD_SOURCE_GEOM_FLOPS
     flops_cell = method_recon if dom == "reconstruction" else method_update
+    instr_cell = RECON_INSTR if dom == "reconstruction" else UPDATE_INSTR
     ms_dom, n_dom = fam[dom]
     per_s = N / (ms_dom / n_dom * 1e-3)
-    achieved = flops_cell * per_s / 1e12
+    achieved = 2.0 * instr_cell * per_s / 1e12
     roof = {"bound": "alu", "kernel": f"k_{'recon' if dom == 'reconstruction' else 'update'} (per stage)",
             "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS,
             "traffic": RECON_DRAM_BYTES if dom == "reconstruction" else UPDATE_DRAM_BYTES,
             "traffic_unit": "bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum of the kernel, "
                             "N = 2^20, the autotuned tiles, mean of the three stages)",
-            "flops_per_cell": flops_cell, "cells_per_launch": N,
-            "flops_basis": "method: the CPU oracle's count of the state arithmetic (operation-counting scalar) "
-                           "+ the mesh-only geometry in closed form; the kernels reach the same result with fewer "
-                           "operations (kernel_count, executed), so this fraction can exceed the hardware's",
-            "kernel_count": {"flops_per_cell": kernel_flops_cell,
-                             "frac": kernel_flops_cell * per_s / 1e12 / FP64_PEAK_TFLOPS},
+            "fp64_instructions_per_cell": instr_cell, "cells_per_launch": N,
+            "flops_basis": "FP64 instructions issued per cell (ncu), two FLOPs of the peak each: the share of the pipe's "
+                           "issue slots",
+            "method_count": {"flops_per_cell": flops_cell, "times_peak": flops_cell * per_s / 1e12 / FP64_PEAK_TFLOPS,
+                             "source": "the CPU oracle's count of the state arithmetic + the mesh-only geometry in closed "
+                                       "form; the kernels reach the same result with fewer operations"},
             "ncu_fp64_pipe_active": RECON_FP64_PIPE_ACTIVE if dom == "reconstruction" else UPDATE_FP64_PIPE_ACTIVE,
             "executed": {"flops_per_cell": RECON_EXECUTED_FLOPS if dom == "reconstruction" else UPDATE_EXECUTED_FLOPS,
                          "frac": (RECON_EXECUTED_FLOPS if dom == "reconstruction" else UPDATE_EXECUTED_FLOPS) * per_s
@@ -824,8 +820,8 @@ def main():
            "vs_baseline": None, "dtype": "f64", "data": "synthetic",
            "config": run_config(N, ws), "tiles": list(tiles),
            "e2e": e2e, "gpu_launches": launches, "clocks": clk, "roofline": roof,
-           "step_roofline": fp64_roofline(method_step_flops(oc), value, "whole step, all kernels", "method",
-                                          opcount_step),
+           "step_roofline": fp64_roofline(2.0 * (3.0 * (RECON_INSTR + UPDATE_INSTR) + MESH_INSTR), value,
+                                          "whole step, all kernels", method_flops=method_step_flops(oc)),
            "cpu_baseline": cpu,
            "status_bits": bits, "steps_done_device": steps_done, "last_dt": last_dt, "batched": batched,
            "adjoint": adjoint, "batched_adjoint": batched_adjoint, "variants": variants,

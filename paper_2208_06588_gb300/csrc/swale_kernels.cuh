@@ -875,11 +875,11 @@ __device__ __noinline__ void open_cells_split(const SchemeConst P, ReconRows<T, 
 // with mine set (2 <= i <= T - 3) get the limited edge state o, the class and, for the special scheme,
 // the interior points of eta. The sink is handed each thread's pair differences and reciprocals as
 // they are formed: pair(ip, de, dh), triple(it), quad(iq), quint(iv). SPLIT: up to how many open cells
-// open_cells_split takes them: 16 (one warp per sub-partition) where the block is alone on its SM; none where
+// open_cells_split takes them (dxmax, the stage's largest width, is read behind the first barrier): 16 (one warp per sub-partition) where the block is alone on its SM; none where
 // other blocks fill it (up to 4 cells, one warp: 8580 us instead of 8556 for 8 steps of 10^6 cells).
 template <int T, int SCHEME, int SPLIT, class Sink>
 __device__ __forceinline__ void recon_phases(const SchemeConst& P, ReconRows<T, SCHEME>& R, const double* sE, const double* sM,
-                                             const double* sJ, double jv, double ev, double mv, double hv, double dxmax,
+                                             const double* sJ, double jv, double ev, double mv, double hv, const double& dxmax,
                                              const MeshRecips& g, bool mine, Sink& sink, EdgeState& o, uint8_t& flag,
                                              swale::PointPair& pts, uint32_t& st, bool* limited = nullptr) {
   const int tid = threadIdx.x;

@@ -74,8 +74,8 @@ struct StepSink {
 // stage values. Bound by the chain of a warp's FP64 instructions (64 cycles each, whatever the
 // number of warps or lanes: about 170 a stage, 67 more where cells are open) and by
 // the six barriers (one to two microseconds each with several blocks). 16 steps at N = 200 take 830 us (1599 by
-// the stage kernels at first, 1077 by today's), at 16300 cells 867 (1554, 993); an accuracy run of N = 50 to
-// t = 0.1 36 ms (79). One block per SM runs a warp on each
+// the stage kernels at first, 1077 by today's), at 16300 cells 862 (1554, 993); an accuracy run of N = 50 to
+// t = 0.1 35 ms (79). One block per SM runs a warp on each
 // sub-partition; hydrostatic and non-well-balanced schemes, static, profile and linear motion. PER_SM:
 // blocks that an SM holds (2: 255 registers; 4: 128, 5: 96, the rest spilled).
 template <int SCHEME, int PER_SM>
